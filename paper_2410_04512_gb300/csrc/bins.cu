@@ -1599,6 +1599,7 @@ struct Scr {
     int nbuf = 0;
     int32_t *take(size_t count)
     {
+        if (nbuf >= SGP_BIN_SCRATCH) return nullptr;
         DBuf &b = B->scr[nbuf++];
         if (buf_ensure(ctx, b, sizeof(int32_t) * std::max<size_t>(count, 4)) != SGP_OK) return nullptr;
         return bp<int32_t>(b);

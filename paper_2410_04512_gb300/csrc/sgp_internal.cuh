@@ -276,6 +276,7 @@ struct sgp_tree {
 // them.  Per-bin arrays are padded to 4 entries so that every segment starts
 // on a 16-byte boundary (bulk copies).  Index [0] of the numeric arrays is
 // FP32, [1] FP64.
+#define SGP_BIN_SCRATCH 96
 struct BinLayout {
     int ok32 = 0, ok64 = 0;
     int32_t nb = 0, nt = 0, LV = 0, LVP = 0, bmax = 0;
@@ -297,7 +298,7 @@ struct BinLayout {
     DBuf i_of_t, t_of_i, rpt, ma32, mb32, m64, mc64;
     uint64_t mgen = 0;
     int mat32 = 0, mat64 = 0;
-    DBuf scr[64];
+    DBuf scr[SGP_BIN_SCRATCH];
 };
 
 struct sgp_factor {
