@@ -209,6 +209,7 @@ sgp_status sgp_friction_assemble(sgp_ctx *ctx, const sgp_graph *G, const double 
     M->m = m;
     M->gamma0 = gamma0;
     M->precision = precision;
+    M->batched = G->batched;
     M->jac_valid = 0;
     M->gen = next_generation();
     const int64_t ns = 2 * m;

@@ -1157,7 +1157,16 @@ sgp_status sgp_tree_factor(sgp_ctx *ctx, const sgp_matrix *M, const sgp_tree *T,
     int herr = 0;
     SGP_TRY(read_back(ctx, &herr, err, sizeof(int)));
     if (herr) return sgp_fail(ctx, SGP_ERR_NOT_SPD, "tree_factor: a pivot block is not positive definite");
-    SGP_TRY(bins_build(ctx, F, M));
+    // default tuning, one system: the grid solve's layout; else the bins
+    F->gl.ok = 0;
+    if (ctx->bin_cap == 0 && ctx->fused && !M->batched) SGP_TRY(grid_build(ctx, F, M));
+    if (F->gl.ok) {
+        F->bl.ok32 = F->bl.ok64 = 0;
+        F->bl.mgen = 0;
+        F->bl.NT = F->bl.nb = F->bl.nt = F->bl.nly = F->bl.bmax = 0;
+    } else {
+        SGP_TRY(bins_build(ctx, F, M));
+    }
     return SGP_OK;
 }
 
@@ -1225,6 +1234,7 @@ void sgp_factor_destroy(sgp_factor *F)
     }
     for (DBuf &b : B.scr)
         if (b.p) cudaFree(b.p);
+    grid_release(F->gl);
     delete F;
 }
 

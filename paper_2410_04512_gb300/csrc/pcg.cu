@@ -1141,9 +1141,11 @@ sgp_status pcg_core(sgp_ctx *ctx, const sgp_matrix *M, const sgp_factor *Fac, in
 template <typename T, typename X>
 sgp_status pcg_run(sgp_ctx *ctx, const sgp_matrix *M, const sgp_factor *Fac, int precond, const T *F, X *x,
                    int x_given, double tol, int64_t maxit, T *r, T *p, T *q, T *w, T *Ft, T *xt,
-                   double *partials, Scal *sc, Scal *hs, double mu = 0.0, int stopE = 0)
+                   double *partials, Scal *sc, void *gwork, Scal *hs, double mu = 0.0, int stopE = 0)
 {
     static_assert(sizeof(X) == sizeof(T), "iterate and vectors share one precision");
+    if (precond == SGP_PRECOND_TREE && grid_ready<T>(ctx, Fac, M))
+        return grid_pcg<T>(ctx, M, Fac->gl, F, reinterpret_cast<T *>(x), x_given, tol, maxit, gwork, hs, mu, stopE);
     const bool tree = precond == SGP_PRECOND_TREE && ctx->fused && Ft && xt && bins_tree_ready<T>(Fac, M);
     if (!tree)
         return pcg_core<T, X>(ctx, M, Fac, precond, make_blk<T>(M), bp<const int32_t>(M->row_ptr), M->n, false, F,
@@ -1310,7 +1312,8 @@ sgp_status sgp_pcg_solve(sgp_ctx *ctx, const sgp_matrix *M, const sgp_factor *Fa
     const int64_t nv = (opts->precond == SGP_PRECOND_TREE && Fac && Fac->bl.NT > n) ? Fac->bl.NT : n;
     const size_t v64 = sizeof(double) * 3 * nv, v32 = sizeof(float) * 3 * nv;
     size_t need = 8 * v64 + (mixed ? 8 * v32 : 0) + sizeof(double) * 2 * MAXP + 2 * sizeof(Scal) + 8192;
-    SGP_TRY(scratch_ensure(ctx, need + 4096));
+    const size_t gw = opts->precond == SGP_PRECOND_TREE ? grid_work_bytes(Fac->gl, mixed ? 4 : 8) : 0;
+    SGP_TRY(scratch_ensure(ctx, need + gw + 4096));
     char *base = reinterpret_cast<char *>(ctx->d_scratch) + 256;
     auto take = [&](size_t b) {
         char *p = base;
@@ -1320,6 +1323,7 @@ sgp_status sgp_pcg_solve(sgp_ctx *ctx, const sgp_matrix *M, const sgp_factor *Fa
     double *partials = reinterpret_cast<double *>(take(sizeof(double) * 2 * MAXP));
     Scal *sc = reinterpret_cast<Scal *>(take(sizeof(Scal)));
     double *o2 = reinterpret_cast<double *>(take(64));
+    char *gwork = take(gw);
     double *r = reinterpret_cast<double *>(take(v64));
     double *p = reinterpret_cast<double *>(take(v64));
     double *q = reinterpret_cast<double *>(take(v64));
@@ -1348,7 +1352,8 @@ sgp_status sgp_pcg_solve(sgp_ctx *ctx, const sgp_matrix *M, const sgp_factor *Fa
     double hres[2] = {0, 0};
     if (!mixed) {
         SGP_TRY(pcg_run<double, double>(ctx, M, Fac, opts->precond, F, v, opts->x0_given, opts->tol,
-                                        opts->maxit, r, p, q, w, Ft64, xt64, partials, sc, &hs, mu, stopE ? 1 : 0));
+                                        opts->maxit, r, p, q, w, Ft64, xt64, partials, sc, gwork, &hs, mu,
+                                        stopE ? 1 : 0));
         inf.iterations = hs.it;
         inf.err_bound = (mu > 0.0 && hs.gsum > 0.0) ? std::sqrt(std::max(hs.est, 0.0) / hs.gsum) : 0.0;
         inf.status = hs.status;
@@ -1408,7 +1413,7 @@ sgp_status sgp_pcg_solve(sgp_ctx *ctx, const sgp_matrix *M, const sgp_factor *Fa
             const double itol_k = std::max(itol, std::min(need, 0.5));
             SGP_TRY(pcg_run<float, float>(ctx, M, Fac, opts->precond, (const float *)r32, d32, 0, itol_k,
                                           opts->maxit - total, s32, p32, q32, w32, Ft32, xt32, partials, sc,
-                                          &hs));
+                                          gwork, &hs));
             total += hs.it;
             ++outer;
             if (hs.status == SGP_ERR_NOT_SPD || hs.status == SGP_ERR_TIMEOUT) {

@@ -221,6 +221,20 @@ template <typename T>
 sgp_status bins_pcg_step(sgp_ctx *ctx, const sgp_factor *F, T *r, const T *q, T *z, void *scal);
 sgp_status bins_check(sgp_ctx *ctx, const sgp_factor *F);
 
+// The grid solve (grid.cu): a whole PCG run in one persistent launch.
+// grid_build runs at the end of a factor build; grid_ready tells whether it
+// serves precision T of this matrix; grid_pcg runs it on internal-order
+// vectors with `work` (grid_work_bytes) and returns the final scalars.
+sgp_status grid_build(sgp_ctx *ctx, sgp_factor *F, const sgp_matrix *M);
+struct GridLayout;
+void grid_release(GridLayout &G);
+template <typename T>
+bool grid_ready(const sgp_ctx *ctx, const sgp_factor *F, const sgp_matrix *M);
+size_t grid_work_bytes(const GridLayout &G, size_t sz);
+template <typename T>
+sgp_status grid_pcg(sgp_ctx *ctx, const sgp_matrix *M, const GridLayout &G, const T *F, T *x, int x_given, double tol,
+                    int64_t maxit, void *work, void *hs, double mu, int stopE);
+
 // Kernel timing hooks (no-ops unless enabled on the context).
 sgp_status kt_begin(sgp_ctx *ctx, int kclass, cudaEvent_t *ev);
 sgp_status kt_end(sgp_ctx *ctx, int kclass, cudaEvent_t ev);
@@ -231,6 +245,7 @@ sgp_status kt_collect(sgp_ctx *ctx);  // after a stream synchronisation
 // ---------------------------------------------------------------------------
 struct sgp_graph {
     int64_t n = 0, m = 0;
+    int batched = 0;   // built from several instances
     DBuf ij;       // m x 2 int32, canonical (i < j), sorted
     DBuf up_ptr;   // n + 1 int32: edges of row i are [up_ptr[i], up_ptr[i+1])
     // cell-list scratch kept for reuse
@@ -244,6 +259,7 @@ struct sgp_matrix {
     int64_t n = 0, m = 0;
     double gamma0 = 0;
     int32_t precision = SGP_PREC_F64;
+    int batched = 0;   // assembled from a batched graph (solved per instance)
     DBuf ij;         // m x 2 int32 (copy of the graph's edge list)
     DBuf row_ptr;    // n + 1 int32 over 2m directed slots, columns ascending in a row
     DBuf col;        // 2m int32
@@ -301,6 +317,19 @@ struct BinLayout {
     DBuf scr[SGP_BIN_SCRATCH];
 };
 
+// The grid solve's layout (grid.cu): one part per thread block and the top,
+// in the factor's own precision, with the matrix's rows of generation mgen.
+#define SGP_GRID_SCRATCH 48
+struct GridLayout {
+    int ok = 0, prec = 0, halo = 0;
+    uint64_t mgen = 0;
+    int32_t P = 0, LV = 0;
+    int32_t tot[24] = {0}, top_slots[2] = {0, 0};   // totals and maxima over the parts; the top's programs
+    DBuf hdr, dtot, ws, glen, gso, perm, xflag, hl, zi, zslot, tlk, i_of_t, t_of_i;
+    DBuf prog[2], D, ma, mb;
+    DBuf scr[SGP_GRID_SCRATCH];
+};
+
 struct sgp_factor {
     uint64_t gen = 0;
     int64_t n = 0, npairs = 0;
@@ -329,6 +358,7 @@ struct sgp_factor {
     DBuf orig_of;   // n int32: the matrix's internal cell order (vectors are solved in it)
     DBuf small;     // counts of the short-tail contraction kernel (header + per-level records)
     BinLayout bl;
+    GridLayout gl;
     // structure-simulation scratch
     DBuf adj_ptr, nbr, twin, eref, deg, lev, nrec, rq, re, ren, pos, flag, alive_a, alive_b,
         acc, fill, sbuf, tmp, rflag, cnt;
