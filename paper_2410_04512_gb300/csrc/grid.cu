@@ -10,8 +10,8 @@
 //   q = Gamma p on its rows (its own p and the rows of other parts that its
 //     rows name, the "halo", in shared memory), p^T q
 //   r -= alpha q, x += alpha p, |r|^2, its part's forward levels
-//   the top's forward, diagonal and backward levels, computed by every block
-//     for itself (cheaper than one block solving it and the others waiting)
+//   z at the top vertices it reaches or owns: rows of the top's inverse times
+//     the top's right-hand side
 //   its part's backward levels, r^T z, p = z + beta p
 // Between the blocks travel p of the halo, the parts' sums for the top with
 // the top's r, and three sums (p^T q, |r|^2, r^T z).
@@ -28,15 +28,20 @@
 // k_gr_segments): records and blocks in the order of use, so that a level
 // costs its reads of the vector and a barrier.
 //
-// What bounds it: the levels (about 20 each way; 250-300 clocks each, a chain
-// of shared-memory reads, products and a barrier) and the exchanges (about
-// 1.2 us each) up to about 3e5 cells in FP32; FP64 by its issue rate (1/64 of
-// FP32's); at 1e6 cells also the stream of matrix rows and blocks from HBM.
+// The top's inverse (a few hundred vertices, computed once per factor by one
+// block per column) replaces its 2 x 10 levels, which every block ran for
+// itself: 5 us per iteration less at 1e4 to 3e5 cells.
+//
+// What bounds it: the levels of a part (about 10 each way; 200-300 clocks
+// each, a chain of shared-memory reads, products and a barrier), the
+// exchanges (about 1.2 us each) and the wait for the largest part, up to
+// about 3e5 cells in FP32; FP64 by its issue rate (1/64 of FP32's); at 1e6
+// cells also the stream of matrix rows and blocks from HBM.
 // Measured per iteration against the multi-launch paths it replaces (product,
 // vector kernels and level kernels or bins; tol 1e-10): FP64 lattice of 1e4
-// cells 39 us (104), FP32 spheroid of 1e5 31 us (63), FP32 sheet of 2.5e5 42
-// us (76), FP64 spheroid of 3e5 150 us (282), FP32 spheroid of 1e6 145 us
-// (181).
+// cells 30.8 us (104), FP32 spheroid of 1e5 27.2 us (63), FP32 sheet of 2.5e5
+// 36.2 us (76), FP64 spheroid of 3e5 138 us (282), FP32 spheroid of 1e6 132
+// us (181).
 #include <type_traits>
 
 #include "solver_common.cuh"
@@ -46,7 +51,7 @@ namespace {
 constexpr int GT = 512;          // threads of a part's block
 constexpr int GW = GT / 32;
 constexpr int PMAX = 160;        // parts
-constexpr int NTOP = 4096;       // top vertices
+constexpr int NTOP = 2048;       // top vertices
 constexpr int GRID_SMEM = 225 * 1024;   // beside about 1 KB of static shared memory
 constexpr int MS_ITEMS = 4096;   // items per block of the stable split
 
@@ -57,7 +62,7 @@ constexpr int NCLS = 8;          // segment classes: 8 sources or more, 7, ... 1
 enum { Q_SOFF, Q_NV, Q_ROFF, Q_NR, Q_T0, Q_NP, Q_POFF, Q_NZ, Q_ZOFF, Q_DOFF, Q_NSF, Q_SF, Q_NSB, Q_SB, Q_NS, Q_SLOT, Q_NH,
        Q_HOFF, Q_N = 24 };
 // totals and maxima over the parts
-enum { T_NT, T_NR, T_P, T_Z, T_D, T_SF, T_SB, T_S, T_H, T_MNR, T_MNZ, T_MNH, T_MSF, T_MSB, T_MDZ, T_MNF, T_MNB, T_ERR,
+enum { T_NT, T_NR, T_P, T_Z, T_D, T_SF, T_SB, T_S, T_H, T_MNR, T_MNZ, T_MNH, T_MSF, T_MSB, T_MDZ, T_MNF, T_MNB, T_MNO, T_ERR,
        T_N = 24 };
 // streams of a program: first slot of every warp's wide levels, of the narrow
 // levels, the end; wide levels
@@ -272,15 +277,15 @@ struct GBuild {
     int32_t *st;                             // first step of every (program, level): 2 x (LMAX + 1) per part
     int32_t *sp_slot[2], *sp_n[2];           // every step's first slot, and its slots | barriers before << 16
     int32_t *ws;                             // streams: 2 x W_N per part
-    int32_t lps;                             // receivers per step: 32, or 10 with a lane per row
+    int32_t lps;                             // receivers per step of a part: 32, or 10 with a lane per row (the top: 10)
     int32_t *glen, *gso;
     uint16_t *perm;
     uint32_t *hb;                            // halo bitmap
     int32_t *hpre;                           // its running count, per word
     int32_t *hl;                             // halo rows
     uint8_t *xflag;                          // rows other parts read
-    char *prog[2];                           // slots
-    int32_t *msrc[2];                        // source pair of every slot's lane
+    char *prog[2], *tprog[2];                // slots of the parts and of the top
+    int32_t *msrc[2], *tmsrc[2];             // source pair of every slot's lane
     int32_t *zi, *zslot, *tlk;
     int identity, halo;
 };
@@ -384,8 +389,8 @@ __global__ void __launch_bounds__(256) k_gr_offsets1(int32_t P, int32_t *hdr, in
 __global__ void __launch_bounds__(256) k_gr_offsets2(int32_t P, int32_t *hdr, int32_t *tot, const int32_t *ws)
 {
     __shared__ int32_t sh[8];
-    hdr_scan(P + 1, hdr, tot, Q_NSF, Q_SF, T_SF, 0, sh);
-    hdr_scan(P + 1, hdr, tot, Q_NSB, Q_SB, T_SB, 0, sh);
+    hdr_scan(P, hdr, tot, Q_NSF, Q_SF, T_SF, 0, sh);
+    hdr_scan(P, hdr, tot, Q_NSB, Q_SB, T_SB, 0, sh);
     hdr_scan(P, hdr, tot, Q_NS, Q_SLOT, T_S, 0, sh);
     hdr_scan(P, hdr, tot, Q_NH, Q_HOFF, T_H, 0, sh);
     if (threadIdx.x < P) {
@@ -396,6 +401,7 @@ __global__ void __launch_bounds__(256) k_gr_offsets2(int32_t P, int32_t *hdr, in
         atomicMax(tot + T_MSF, h[Q_NSF]);
         atomicMax(tot + T_MSB, h[Q_NSB]);
         atomicMax(tot + T_MDZ, h[Q_NR] + h[Q_NZ]);
+        atomicMax(tot + T_MNO, h[Q_NZ] + h[Q_NR] - h[Q_NV]);
         if (ws) {
             const int32_t *f = ws + (size_t)threadIdx.x * 2 * W_N;
             atomicMax(tot + T_MNF, f[W_END] - f[W_NARROW]);
@@ -432,7 +438,7 @@ __global__ void __launch_bounds__(GT) k_gr_segments(GBuild g)
     for (int i = threadIdx.x; i < LMAX; i += GT) lmax[i] = 0;
     const bool top = b == g.P;
     const int32_t so = h[Q_SOFF], nv = h[Q_NV], nr = h[Q_NR], nt = g.tot[T_NT], po = h[Q_POFF],
-                  nd = top ? nv : nr + h[Q_NZ];
+                  nd = top ? nv : nr + h[Q_NZ], lps = top ? 10 : g.lps;
     const int32_t *vm = g.vm + (size_t)b * nt;
     int32_t *dc = g.dcnt + h[Q_DOFF];
     for (int i = threadIdx.x; i < 2 * LMAX * NCLS; i += GT) (&hist[0][0])[i] = 0;
@@ -518,7 +524,7 @@ __global__ void __launch_bounds__(GT) k_gr_segments(GBuild g)
                 kb[l * NCLS + k] = c;
                 c += hist[q][l * NCLS + k];
             }
-            const int32_t ns = (c + g.lps - 1) / g.lps;
+            const int32_t ns = (c + lps - 1) / lps;
             if (ns > 1) {
                 wide0 = min(wide0, l);
                 wide1 = l + 1;
@@ -533,7 +539,7 @@ __global__ void __launch_bounds__(GT) k_gr_segments(GBuild g)
     __syncthreads();
     // slots of a step: its largest segment, the first one of its class order
     auto slots = [&](int q, int l, int32_t s) {
-        int32_t at = (s - lst[q][l]) * g.lps, k = 0;
+        int32_t at = (s - lst[q][l]) * lps, k = 0;
         while (k < NCLS - 1 && at >= hist[q][l * NCLS + k]) at -= hist[q][l * NCLS + k++];
         return k == 0 ? lmax[l] : NCLS - k;
     };
@@ -721,8 +727,8 @@ __global__ void __launch_bounds__(GT) k_gr_halo_list(GBuild g)
 
 // A slot: 32 records, then the blocks in planes of 32 values (all nine
 // entries, or the lane's row).  rec = source | receiver << 13 | block barriers
-// before the slot << 26 | last slot of its step << 31.  Idle lanes work on a
-// spare cell behind the vectors with a zero block.
+// before the slot << 26.  Idle lanes work on a spare cell behind the vectors
+// with a zero block.
 template <typename T>
 struct SlotSize;
 template <>
@@ -734,12 +740,12 @@ struct SlotSize<double> {
     static constexpr int B = 128 + 3 * 256, LPS = 10;
 };
 template <typename T>
-__global__ void __launch_bounds__(GT) k_gr_program(GBuild g)
+__global__ void __launch_bounds__(GT) k_gr_program(GBuild g, int32_t b0)
 {
     __shared__ uint16_t wc[GW][LMAX * NCLS];
     __shared__ int32_t base_s[LMAX * NCLS];
     constexpr int B = SlotSize<T>::B, LPS = SlotSize<T>::LPS, R = LPS == 32 ? 1 : 3;
-    const int b = blockIdx.x, q = blockIdx.y, w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int b = b0 + blockIdx.x, q = blockIdx.y, w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int32_t *h = g.hdr + (size_t)Q_N * b;
     const bool top = b == g.P;
     const int32_t so = h[Q_SOFF], nv = h[Q_NV], nr = h[Q_NR], nt = g.tot[T_NT], po = h[Q_POFF],
@@ -748,14 +754,13 @@ __global__ void __launch_bounds__(GT) k_gr_program(GBuild g)
     const int32_t *kb = g.kb + ((size_t)b * 2 + q) * LMAX * NCLS, *st = g.st + ((size_t)b * 2 + q) * (LMAX + 1);
     const int32_t *sslot = g.sp_slot[q] + po + b, *sn = g.sp_n[q] + po + b;
     const int32_t slot0 = h[q ? Q_SB : Q_SF], nsteps = st[LMAX];
-    char *prog = g.prog[q] + (size_t)B * slot0;
-    int32_t *msrc = g.msrc[q] + 32 * (size_t)slot0;
+    char *prog = top ? g.tprog[q] : g.prog[q] + (size_t)B * slot0;
+    int32_t *msrc = top ? g.tmsrc[q] : g.msrc[q] + 32 * (size_t)slot0;
     auto rec = [&](int32_t slot, int32_t ln) -> uint32_t & { return reinterpret_cast<uint32_t *>(prog + (size_t)B * slot)[ln]; };
     for (int32_t s = w; s < nsteps; s += GW) {
         const int32_t a = sslot[s], n = sn[s] & 0xffff, bars = sn[s] >> 16;
         for (int32_t j = 0; j < n; ++j) {
-            rec(a + j, lane) = (uint32_t)nd | (uint32_t)nd << 13 | (j == 0 ? (uint32_t)bars << 26 : 0u) |
-                               (j == n - 1 ? 1u << 31 : 0u);
+            rec(a + j, lane) = (uint32_t)nd | (uint32_t)nd << 13 | (j == 0 ? (uint32_t)bars << 26 : 0u);
             msrc[32 * (a + j) + lane] = -1;
         }
     }
@@ -861,7 +866,7 @@ __global__ void k_gr_pivots(int32_t cnt, const int32_t *__restrict__ src, const 
 #pragma unroll
     for (int a = 0; a < 6; ++a) o[32 * a] = s >= 0 ? (T)from[(size_t)6 * s + a] : T(0);
 }
-// The programs' blocks: L of the lane's pair, transposed in the backward
+// The programs' blocks: -L of the lane's pair, transposed in the backward
 // program (TR); FP64 lanes hold one row.
 template <typename T, bool TR>
 __global__ void k_gr_blocks(int32_t lanes, const int32_t *__restrict__ src, const double *__restrict__ L, char *prog)
@@ -872,11 +877,11 @@ __global__ void k_gr_blocks(int32_t lanes, const int32_t *__restrict__ src, cons
     T *o = reinterpret_cast<T *>(prog + (size_t)(i >> 5) * SlotSize<T>::B + 128) + ln;
     if (sizeof(T) == 4) {
 #pragma unroll
-        for (int a = 0; a < 9; ++a) o[32 * (TR ? 3 * (a % 3) + a / 3 : a)] = s >= 0 ? (T)L[(size_t)9 * s + a] : T(0);
+        for (int a = 0; a < 9; ++a) o[32 * (TR ? 3 * (a % 3) + a / 3 : a)] = s >= 0 ? (T)-L[(size_t)9 * s + a] : T(0);
     } else {
         const int r = ln % 3;
 #pragma unroll
-        for (int c = 0; c < 3; ++c) o[32 * c] = s >= 0 ? (T)L[(size_t)9 * s + (TR ? 3 * c + r : 3 * r + c)] : T(0);
+        for (int c = 0; c < 3; ++c) o[32 * c] = s >= 0 ? (T)-L[(size_t)9 * s + (TR ? 3 * c + r : 3 * r + c)] : T(0);
     }
 }
 
@@ -954,8 +959,8 @@ __global__ void __launch_bounds__(GT) k_gr_check(GBuild g)
     const bool top = b == g.P;
     const int32_t nv = h[Q_NV], nr = top ? 0 : h[Q_NR], nz = h[Q_NZ], nd = top ? nv : nr + nz, ro = h[Q_ROFF];
     for (int q = 0; q < 2 && !g.identity; ++q) {
-        const int32_t ns = h[q ? Q_NSB : Q_NSF], B = g.lps == 32 ? SlotSize<float>::B : SlotSize<double>::B;
-        const char *prog = g.prog[q] + (size_t)B * h[q ? Q_SB : Q_SF];
+        const int32_t ns = h[q ? Q_NSB : Q_NSF], B = !top && g.lps == 32 ? SlotSize<float>::B : SlotSize<double>::B;
+        const char *prog = top ? g.tprog[q] : g.prog[q] + (size_t)B * h[q ? Q_SB : Q_SF];
         for (int32_t i = threadIdx.x; i < 32 * ns; i += GT) {
             const uint32_t r = reinterpret_cast<const uint32_t *>(prog + (size_t)B * (i >> 5))[i & 31];
             if ((int32_t)(r & 8191) > nd || (int32_t)(r >> 13 & 8191) > nd) bad = 32;
@@ -997,16 +1002,16 @@ struct Mat<double> {
 // Placement: byte offsets into shared memory (-1: the array stays in global
 // memory).
 struct GridPlace {
-    int32_t o_p, o_w, o_t, o_misc, o_top[2], o_nar[2], o_all[2], o_D, o_tD, o_r, o_x, o_perm, o_hl;
+    int32_t o_p, o_w, o_t, o_tp, o_misc, o_inv, o_nar[2], o_all[2], o_D, o_r, o_x, o_perm, o_hl;
     int32_t bytes;
 };
 struct GridArgs {
-    int32_t P, nt, x_given, timing, halo, tD0, nslots;
+    int32_t P, nt, ntp, x_given, timing, halo, nslots;
     const int32_t *hdr, *ws, *glen, *gso, *i_of_t, *zi, *zslot, *tlk, *hl;
     const char *prog[2];
     const uint16_t *perm;
     const uint8_t *xflag;
-    const void *D;             // pivots, of the solve's type
+    const void *D, *inv;       // pivots and rows of the top's inverse, of the solve's type
     const void *jac;           // block-Jacobi inverses, part order planes
     const void *ma, *mb;       // the matrix's rows
     const void *F;             // right-hand side, internal order
@@ -1022,18 +1027,18 @@ struct GridArgs {
     GridPlace pl;
 };
 
-// Vectors addressed at random live in shared memory, FP32 padded to 16 bytes
-// per cell (one load), FP64 at 24 bytes.
-template <typename T>
+// Vectors addressed at random live in shared memory, VB bytes per cell: FP64
+// 24; FP32 16 (one load per cell), or 12 where that makes room for the halo
+// (1e6 cells: the product's gathers of other parts' rows then stay on chip).
+template <typename T, int VB>
 struct V3;
 template <>
-struct V3<float> {
-    static constexpr int B = 16;
+struct V3<float, 16> {
     static __device__ __forceinline__ void ld(uint32_t a, float *v)
     {
         float pad;
         asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(pad) : "r"(a) : "memory");
-        (void)pad;
+        asm volatile("" ::"f"(pad));
     }
     static __device__ __forceinline__ void st(uint32_t a, const float *v)
     {
@@ -1041,8 +1046,22 @@ struct V3<float> {
     }
 };
 template <>
-struct V3<double> {
-    static constexpr int B = 24;
+struct V3<float, 12> {
+    static __device__ __forceinline__ void ld(uint32_t a, float *v)
+    {
+        asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v[0]) : "r"(a) : "memory");
+        asm volatile("ld.shared.f32 %0, [%1+4];" : "=f"(v[1]) : "r"(a) : "memory");
+        asm volatile("ld.shared.f32 %0, [%1+8];" : "=f"(v[2]) : "r"(a) : "memory");
+    }
+    static __device__ __forceinline__ void st(uint32_t a, const float *v)
+    {
+        asm volatile("st.shared.f32 [%0], %1;" ::"r"(a), "f"(v[0]) : "memory");
+        asm volatile("st.shared.f32 [%0+4], %1;" ::"r"(a), "f"(v[1]) : "memory");
+        asm volatile("st.shared.f32 [%0+8], %1;" ::"r"(a), "f"(v[2]) : "memory");
+    }
+};
+template <>
+struct V3<double, 24> {
     static __device__ __forceinline__ void ld(uint32_t a, double *v)
     {
         asm volatile("ld.shared.f64 %0, [%1];" : "=d"(v[0]) : "r"(a) : "memory");
@@ -1072,7 +1091,8 @@ struct Acc<double> {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     }
-    __device__ __forceinline__ double2 pair() const { return make_double2(v, 0.0); }
+    __device__ __forceinline__ double pair() const { return v; }
+    __device__ __forceinline__ void join(double x) { v += x; }
 };
 template <>
 struct Acc<float> {
@@ -1098,16 +1118,36 @@ struct Acc<float> {
         }
     }
     __device__ __forceinline__ float2 pair() const { return make_float2(h, l); }
+    __device__ __forceinline__ void join(float2 x) { add(x.x, x.y); }
 };
 template <typename T>
-struct Part;   // a warp's partial sum in shared memory
+struct Part;   // a partial sum in shared memory and in packets
 template <>
 struct Part<float> {
     using type = float2;
+    static __device__ __forceinline__ void split(float2 v, unsigned &a, unsigned &b)
+    {
+        a = __float_as_uint(v.x);
+        b = __float_as_uint(v.y);
+    }
+    static __device__ __forceinline__ float2 unite(unsigned a, unsigned b)
+    {
+        return make_float2(__uint_as_float(a), __uint_as_float(b));
+    }
 };
 template <>
 struct Part<double> {
-    using type = double2;
+    using type = double;
+    static __device__ __forceinline__ void split(double v, unsigned &a, unsigned &b)
+    {
+        const unsigned long long x = (unsigned long long)__double_as_longlong(v);
+        a = (unsigned)x;
+        b = (unsigned)(x >> 32);
+    }
+    static __device__ __forceinline__ double unite(unsigned a, unsigned b)
+    {
+        return __longlong_as_double((long long)((unsigned long long)b << 32 | a));
+    }
 };
 
 __device__ __forceinline__ unsigned long long now_ns()
@@ -1208,8 +1248,8 @@ __device__ __forceinline__ bool wait_packet(const unsigned long long *p, unsigne
 // Two alternating packet sets are enough: a block writes exchange e only
 // after all blocks have written e - 1, that is, after they have read e - 2.
 constexpr int PK = (PMAX + 31) / 32;
-template <int NV>
-__device__ __forceinline__ bool exchange(unsigned long long *pk, int P, unsigned epoch, int *err, double *v)
+template <typename T, int NV>
+__device__ __forceinline__ bool exchange(unsigned long long *pk, int P, unsigned epoch, int *err, Acc<T> *v)
 {
     const int lane = threadIdx.x & 31;
     unsigned long long *set = pk + (size_t)(epoch & 1u) * PMAX * 4;
@@ -1217,8 +1257,9 @@ __device__ __forceinline__ bool exchange(unsigned long long *pk, int P, unsigned
     if (lane == 0) {
 #pragma unroll
         for (int k = 0; k < NV; ++k) {
-            const unsigned long long x = (unsigned long long)__double_as_longlong(v[k]);
-            st_words(set + 4 * blockIdx.x + 2 * k, e | (x & 0xffffffffull), e | (x >> 32));
+            unsigned x, y;
+            Part<T>::split(v[k].pair(), x, y);
+            st_words(set + 4 * blockIdx.x + 2 * k, e | x, e | y);
         }
     }
     // lanes without a packet of their own watch their block's
@@ -1245,30 +1286,25 @@ __device__ __forceinline__ bool exchange(unsigned long long *pk, int P, unsigned
     }
 #pragma unroll
     for (int k = 0; k < NV; ++k) {
-        double s = 0.0;
+        v[k] = Acc<T>();
 #pragma unroll
         for (int u = 0; u < PK; ++u)
-            if (lane + 32 * u < P) s += __longlong_as_double((long long)((a[k][u] & 0xffffffffull) | (b[k][u] << 32)));
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        v[k] = s;
+            if (lane + 32 * u < P) v[k].join(Part<T>::unite((unsigned)a[k][u], (unsigned)b[k][u]));
+        v[k].warp();
     }
     return ok;
 }
 
-// A lane's share of a slot: w[receiver] -= the sum over the step's slots of
-// M w[source]; FP32 lanes hold a whole block, FP64 lanes one row of it (an
-// FP64 instruction of one warp takes 64 clocks here, so a level's chain is
-// its number of FP64 instructions).
+// A lane's share of a slot: w[receiver] += M w[source] (M = -L); FP32 lanes
+// hold a whole block, FP64 lanes one row of it (an FP64 instruction of one
+// warp takes 64 clocks here, so a level's chain is its number of FP64
+// instructions).
 template <typename T>
 struct Lane;
 template <>
 struct Lane<float> {
     uint32_t rec;
     float M[9];
-    struct Sum {
-        float s[3] = {0.f, 0.f, 0.f};
-    };
     __device__ __forceinline__ void load(const char *slot, int lane)
     {
         rec = reinterpret_cast<const uint32_t *>(slot)[lane];
@@ -1276,31 +1312,22 @@ struct Lane<float> {
 #pragma unroll
         for (int a = 0; a < 9; ++a) M[a] = m[32 * a];
     }
-    __device__ __forceinline__ void step(uint32_t w, Sum &k) const
+    template <int VB>
+    __device__ __forceinline__ void step(uint32_t w) const
     {
-        float x[3];
-        V3<float>::ld(w + (rec & 8191u) * 16u, x);
+        float x[3], y[3];
+        const uint32_t d = w + (rec >> 13 & 8191u) * VB;
+        V3<float, VB>::ld(w + (rec & 8191u) * VB, x);
+        V3<float, VB>::ld(d, y);
 #pragma unroll
-        for (int r = 0; r < 3; ++r) k.s[r] += M[3 * r] * x[0] + M[3 * r + 1] * x[1] + M[3 * r + 2] * x[2];
-        if (rec >> 31) {
-            const uint32_t d = w + (rec >> 13 & 8191u) * 16u;
-            V3<float>::ld(d, x);
-#pragma unroll
-            for (int r = 0; r < 3; ++r) {
-                x[r] -= k.s[r];
-                k.s[r] = 0.f;
-            }
-            V3<float>::st(d, x);
-        }
+        for (int r = 0; r < 3; ++r) y[r] = fmaf(M[3 * r + 2], x[2], fmaf(M[3 * r + 1], x[1], fmaf(M[3 * r], x[0], y[r])));
+        V3<float, VB>::st(d, y);
     }
 };
 template <>
 struct Lane<double> {
     uint32_t rec;
     double M[3];
-    struct Sum {
-        double s = 0.0;
-    };
     __device__ __forceinline__ void load(const char *slot, int lane)
     {
         rec = reinterpret_cast<const uint32_t *>(slot)[lane];
@@ -1308,25 +1335,21 @@ struct Lane<double> {
 #pragma unroll
         for (int a = 0; a < 3; ++a) M[a] = m[32 * a];
     }
-    __device__ __forceinline__ void step(uint32_t w, Sum &k) const
+    template <int VB>
+    __device__ __forceinline__ void step(uint32_t w) const
     {
-        double x[3];
-        V3<double>::ld(w + (rec & 8191u) * 24u, x);
-        k.s += M[0] * x[0] + M[1] * x[1] + M[2] * x[2];
-        if (rec >> 31) {
-            const uint32_t d = w + (rec >> 13 & 8191u) * 24u + (threadIdx.x & 31) % 3 * 8u;
-            double y;
-            asm volatile("ld.shared.f64 %0, [%1];" : "=d"(y) : "r"(d) : "memory");
-            y -= k.s;
-            k.s = 0.0;
-            asm volatile("st.shared.f64 [%0], %1;" ::"r"(d), "d"(y) : "memory");
-        }
+        double x[3], y;
+        const uint32_t d = w + (rec >> 13 & 8191u) * VB + (threadIdx.x & 31) % 3 * 8u;
+        V3<double, VB>::ld(w + (rec & 8191u) * VB, x);
+        asm volatile("ld.shared.f64 %0, [%1];" : "=d"(y) : "r"(d) : "memory");
+        y = fma(M[2], x[2], fma(M[1], x[1], fma(M[0], x[0], y)));
+        asm volatile("st.shared.f64 [%0], %1;" ::"r"(d), "d"(y) : "memory");
     }
 };
 // n slots of a warp from `slot` on; NARROW: each step is a level, else the
 // records say where the block barriers lie (`levels` in all).  DEPTH slots
 // are in flight; each buffer is refilled as soon as it is used.
-template <typename T, bool NARROW>
+template <typename T, int VB, bool NARROW>
 __device__ __forceinline__ void run_stream(const char *slot, int32_t n, int levels, uint32_t w)
 {
     constexpr int D = 4, B = SlotSize<T>::B;
@@ -1334,7 +1357,6 @@ __device__ __forceinline__ void run_stream(const char *slot, int32_t n, int leve
     // zero first: a register that a skipped load might leave as it was would
     // count as live through the whole solve
     Lane<T> k[D] = {};
-    typename Lane<T>::Sum sum;
 #pragma unroll
     for (int d = 0; d < D; ++d)
         if (d < n) k[d].load(slot + d * B, lane);
@@ -1348,7 +1370,7 @@ __device__ __forceinline__ void run_stream(const char *slot, int32_t n, int leve
                     __syncthreads();
                     --levels;
                 }
-            k[d].step(w, sum);
+            k[d].template step<VB>(w);
             if (NARROW) __syncwarp();
             if (n > D) k[d].load(next, lane);
             next += B;
@@ -1363,19 +1385,19 @@ struct Prog {
     const int32_t *ws;
     const char *wide, *narrow;
 };
-template <typename T, bool FWD>
+template <typename T, int VB, bool FWD>
 __device__ __forceinline__ void run(const Prog &g, uint32_t w)
 {
     const int warp = threadIdx.x >> 5;
     constexpr int B = SlotSize<T>::B;
     if (!FWD) {
-        if (warp == 0) run_stream<T, true>(g.narrow, g.ws[W_END] - g.ws[W_NARROW], 0, w);
+        if (warp == 0) run_stream<T, VB, true>(g.narrow, g.ws[W_END] - g.ws[W_NARROW], 0, w);
         __syncthreads();
     }
     const int32_t a = g.ws[warp];
-    run_stream<T, false>(g.wide + (size_t)B * a, g.ws[warp + 1] - a, g.ws[W_LEVELS], w);
+    run_stream<T, VB, false>(g.wide + (size_t)B * a, g.ws[warp + 1] - a, g.ws[W_LEVELS], w);
     if (FWD) {
-        if (warp == 0) run_stream<T, true>(g.narrow, g.ws[W_END] - g.ws[W_NARROW], 0, w);
+        if (warp == 0) run_stream<T, VB, true>(g.narrow, g.ws[W_END] - g.ws[W_NARROW], 0, w);
         __syncthreads();
     }
 }
@@ -1426,7 +1448,7 @@ struct Slot<double> {
 // q = Gamma p on the part's rows (into w), p^T q: a warp takes 32 rows of
 // nearly equal length, U slots in flight per lane; p from shared memory (its
 // own rows and the halo), or the halo from global memory.
-template <typename T>
+template <typename T, int VB>
 __device__ __forceinline__ Acc<T> product(const GridArgs &a, const Mat<T> &M, int32_t ro, int32_t nr, int32_t slot0,
                                        const uint16_t *perm, const int32_t *glen, const int32_t *gso, const T *ps,
                                        uint32_t w)
@@ -1472,7 +1494,7 @@ __device__ __forceinline__ Acc<T> product(const GridArgs &a, const Mat<T> &M, in
                 y[c] = fma(g0, v[c], y[c]);
                 acc.mul(v[c], y[c]);
             }
-            V3<T>::st(w + l * V3<T>::B, y);
+            V3<T, VB>::st(w + l * VB, y);
         }
     }
     acc.warp();
@@ -1480,7 +1502,7 @@ __device__ __forceinline__ Acc<T> product(const GridArgs &a, const Mat<T> &M, in
 }
 
 // D^-1 w of every vertex
-template <typename T>
+template <typename T, int VB>
 __device__ __forceinline__ void pivots(const T *D, int32_t nv, uint32_t w)
 {
     for (int32_t i = threadIdx.x; i < nv; i += GT) {
@@ -1488,9 +1510,44 @@ __device__ __forceinline__ void pivots(const T *D, int32_t nv, uint32_t w)
         const T *d = D + (size_t)(i >> 5) * 192 + (i & 31);
 #pragma unroll
         for (int a = 0; a < 6; ++a) B[a] = d[32 * a];
-        V3<T>::ld(w + i * V3<T>::B, x);
+        V3<T, VB>::ld(w + i * VB, x);
         sym_mv(B, x, z);
-        V3<T>::st(w + i * V3<T>::B, z);
+        V3<T, VB>::st(w + i * VB, z);
+    }
+}
+
+// Rows of the top's inverse, in FP64: one column of it per block by the top's
+// programs (levels as in the solve), stored as the row it is by symmetry:
+// row 3 k + c of output vertex k, one plane of ntp inputs per (c, component).
+template <typename T>
+__global__ void __launch_bounds__(GT, 1) k_gr_top_inverse(int32_t nt, int32_t ntp, const int32_t *ws, const char *fwd,
+                                                          const char *bwd, const double *D, T *inv)
+{
+    extern __shared__ __align__(16) unsigned char sm[];
+    __shared__ int32_t s_ws[2][W_N];
+    const uint32_t w = (uint32_t)__cvta_generic_to_shared(sm);
+    constexpr int B = SlotSize<double>::B;
+    for (int i = threadIdx.x; i < 2 * W_N; i += GT) s_ws[i / W_N][i % W_N] = ws[i];
+    __syncthreads();
+    const Prog f{s_ws[0], fwd, fwd + (size_t)B * s_ws[0][W_NARROW]}, r{s_ws[1], bwd, bwd + (size_t)B * s_ws[1][W_NARROW]};
+    for (int32_t col = blockIdx.x; col < 3 * nt; col += gridDim.x) {
+        for (int32_t i = threadIdx.x; i <= nt; i += GT) {
+            const double e[3] = {col == 3 * i ? 1.0 : 0.0, col == 3 * i + 1 ? 1.0 : 0.0, col == 3 * i + 2 ? 1.0 : 0.0};
+            V3<double, 24>::st(w + i * 24, e);   // cell nt: the spare one, zero
+        }
+        __syncthreads();
+        run<double, 24, true>(f, w);
+        pivots<double, 24>(D, nt, w);
+        __syncthreads();
+        run<double, 24, false>(r, w);
+        T *o = inv + (size_t)col * 3 * ntp;
+        for (int32_t i = threadIdx.x; i < ntp; i += GT) {
+            double z[3] = {0.0, 0.0, 0.0};
+            if (i < nt) V3<double, 24>::ld(w + i * 24, z);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) o[(size_t)c * ntp + i] = (T)z[c];
+        }
+        __syncthreads();
     }
 }
 
@@ -1499,42 +1556,24 @@ template <typename T>
 struct Solve {
     Scal S;
     typename Part<T>::type red[2][GW];   // the warps' partial sums
+    typename Part<T>::type rho, stop2, rr;   // FP32 keeps these as pairs of floats
     T al, be;
     int go, bad;                         // the solve goes on; a wait gave up
     unsigned epoch;
 };
 enum { OP_START, OP_RHO, OP_PQ, OP_RR, OP_RR_RZ, OP_RZ, OP_NONE };
-// Warp 0, after the barrier behind the partial sums: their sums over the
-// grid, and the step's decision.
-template <typename T>
-__device__ __noinline__ void sums(const GridArgs &a, Solve<T> &Z, int op)
+
+// The decisions on a sum, in one thread.  FP64: on the Scal as in the
+// multi-launch solve.
+__device__ __forceinline__ void decide(const GridArgs &a, Solve<double> &Z, int op, double t, double t1)
 {
-    const int lane = threadIdx.x & 31;
-    const unsigned epoch = Z.epoch + 1;
-    double v[2] = {0.0, 0.0};
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-        if (k == 1 && op != OP_START && op != OP_RR_RZ) break;
-        if (lane < GW && op != OP_NONE) v[k] = (double)Z.red[k][lane].x + (double)Z.red[k][lane].y;
-#pragma unroll
-        for (int o = GW / 2; o > 0; o >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
-    }
-    const bool ok = op == OP_START || op == OP_RR_RZ ? exchange<2>(a.pk, a.P, epoch, a.err, v)
-                                                     : exchange<1>(a.pk, a.P, epoch, a.err, v);
-    if (lane) return;
     Scal &S = Z.S;
-    Z.epoch = epoch;
-    if (!ok) {
-        Z.bad = 1;
-        return;
-    }
-    const double t = v[0];
     switch (op) {
     case OP_START:
         S.FF = t;
-        S.rr = v[1];
+        S.rr = t1;
         S.stop2 = a.tol2 * t;
-        S.done = t == 0.0 || v[1] <= S.stop2;
+        S.done = t == 0.0 || t1 <= S.stop2;
         break;
     case OP_RHO:
         S.rho = S.rz = t;
@@ -1550,8 +1589,7 @@ __device__ __noinline__ void sums(const GridArgs &a, Solve<T> &Z, int op)
             S.status = SGP_ERR_NOT_SPD;
             S.done = 1;
         } else {
-            S.alpha = S.rho / t;
-            Z.al = (T)S.alpha;
+            Z.al = S.alpha = S.rho / t;
         }
         break;
     case OP_RR:
@@ -1565,32 +1603,119 @@ __device__ __noinline__ void sums(const GridArgs &a, Solve<T> &Z, int op)
             S.status = SGP_ERR_NO_CONVERGENCE;
         }
         if (op == OP_RR || S.done) break;
-        rz_finish(&S, v[1]);
-        Z.be = (T)S.beta;
+        rz_finish(&S, t1);
+        Z.be = S.beta;
         break;
     case OP_RZ:
         rz_finish(&S, t);
-        Z.be = (T)S.beta;
+        Z.be = S.beta;
         break;
     }
-    Z.go = S.done ? 0 : 1;
+}
+// FP32 (inner solves: no error bound): on pairs of floats, so that the chain
+// behind every exchange holds no FP64 instruction (64 clocks and more each
+// for one warp; a division is ten of them).
+__device__ __forceinline__ float pair_ratio(float2 x, float2 y)
+{
+    const float q = x.x / y.x;
+    return q + (fmaf(-q, y.x, x.x) + fmaf(-q, y.y, x.y)) / y.x;
+}
+__device__ __forceinline__ void decide(const GridArgs &a, Solve<float> &Z, int op, float2 t, float2 t1)
+{
+    Scal &S = Z.S;
+    switch (op) {
+    case OP_START: {
+        S.FF = (double)t.x + (double)t.y;
+        const double st = a.tol2 * S.FF;
+        Z.stop2.x = (float)st;
+        Z.stop2.y = (float)(st - (double)Z.stop2.x);
+        S.stop2 = st;
+        Z.rr = t1;
+        S.done = S.FF == 0.0 || (double)t1.x + (double)t1.y <= st;
+        break;
+    }
+    case OP_RHO:
+        Z.rho = t;
+        if (!(t.x > 0.f) || !isfinite(t.x)) {
+            S.status = SGP_ERR_NOT_SPD;
+            S.done = 1;
+        }
+        break;
+    case OP_PQ:
+        if (!(t.x > 0.f) || !isfinite(t.x)) {
+            S.status = SGP_ERR_NOT_SPD;
+            S.done = 1;
+        } else {
+            Z.al = pair_ratio(Z.rho, t);
+        }
+        break;
+    case OP_RR:
+    case OP_RR_RZ:
+        Z.rr = t;
+        S.it += 1;
+        if ((t.x - Z.stop2.x) + (t.y - Z.stop2.y) <= 0.f) {
+            S.done = 1;
+        } else if (S.it >= S.maxit) {
+            S.done = 1;
+            S.status = SGP_ERR_NO_CONVERGENCE;
+        }
+        if (op == OP_RR || S.done) break;
+        t = t1;
+        // fall through
+    case OP_RZ:
+        if (!(t.x > 0.f) || !isfinite(t.x)) {
+            S.status = SGP_ERR_NOT_SPD;
+            S.done = 1;
+        } else {
+            Z.be = pair_ratio(t, Z.rho);
+            Z.rho = t;
+        }
+        break;
+    }
+}
+__device__ __forceinline__ double pair_value(double x) { return x; }
+__device__ __forceinline__ double pair_value(float2 x) { return (double)x.x + (double)x.y; }
+
+// Warp 0, after the barrier behind the partial sums: their sums over the
+// grid, and the step's decision.
+template <typename T>
+__device__ __noinline__ void sums(const GridArgs &a, Solve<T> &Z, int op)
+{
+    const int lane = threadIdx.x & 31;
+    const unsigned epoch = Z.epoch + 1;
+    const bool two = op == OP_START || op == OP_RR_RZ;
+    Acc<T> v[2];
+    if (lane < GW && op != OP_NONE) v[0].join(Z.red[0][lane]);
+    v[0].warp();
+    if (two) {
+        if (lane < GW) v[1].join(Z.red[1][lane]);
+        v[1].warp();
+    }
+    const bool ok = two ? exchange<T, 2>(a.pk, a.P, epoch, a.err, v) : exchange<T, 1>(a.pk, a.P, epoch, a.err, v);
+    if (lane) return;
+    Z.epoch = epoch;
+    if (!ok) {
+        Z.bad = 1;
+        return;
+    }
+    decide(a, Z, op, v[0].pair(), v[1].pair());
+    Z.go = Z.S.done ? 0 : 1;
 }
 
-template <typename T, int PREC>
+template <typename T, int VB, int PREC>
 __global__ void __launch_bounds__(GT, 1) k_pcg_grid(const __grid_constant__ GridArgs a)
 {
     extern __shared__ __align__(16) unsigned char sm[];
     __shared__ Solve<T> Z;
-    __shared__ Prog s_prog[4];   // the part's forward and backward, the top's
-    __shared__ int32_t s_ws[4][W_N];
+    __shared__ Prog s_prog[2];   // the part's forward and backward programs
+    __shared__ int32_t s_ws[2][W_N];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int32_t *h = a.hdr + (size_t)Q_N * blockIdx.x, *ht = a.hdr + (size_t)Q_N * a.P;
+    const int32_t *h = a.hdr + (size_t)Q_N * blockIdx.x;
     const int32_t nv = h[Q_NV], nr = h[Q_NR], ro = h[Q_ROFF], t0 = h[Q_T0], nz = h[Q_NZ], zo = h[Q_ZOFF],
                   slot0 = h[Q_SLOT], nh = h[Q_NH], nt = a.nt;
     T *ps = reinterpret_cast<T *>(sm + a.pl.o_p);
     const uint32_t sm0 = (uint32_t)__cvta_generic_to_shared(sm);
     const uint32_t w = sm0 + a.pl.o_w, tw = sm0 + a.pl.o_t;
-    constexpr int VB = V3<T>::B;
     auto put = [&](auto *src, int32_t off, int32_t cnt) {
         using E = typename std::remove_const<typename std::remove_reference<decltype(*src)>::type>::type;
         if (off < 0) return (const E *)src;
@@ -1606,33 +1731,40 @@ __global__ void __launch_bounds__(GT, 1) k_pcg_grid(const __grid_constant__ Grid
         gso[i] = a.gso[ro / 32 + i];
     }
     const int32_t *hl = put(a.hl + h[Q_HOFF], a.pl.o_hl, a.halo ? nh : 0);
-    const T *D = nullptr, *tD = nullptr;
+    const T *D = nullptr, *inv = nullptr;
+    // top vertices the part needs: those it reaches, then those it owns
+    // and into how many pieces their rows are cut (about one item per warp)
+    const int32_t nout = nz + nr - nv, npc = (nt + 127) / 128,
+                  nch = nout > 0 ? max(1, min(npc, GW / nout)) : 1, chunk = (npc + nch - 1) / nch * 128;
     if (PREC == 0) {
         D = put(reinterpret_cast<const T *>(a.D) + 6 * (size_t)ro, a.pl.o_D, 6 * pad32(nv));
-        tD = put(reinterpret_cast<const T *>(a.D) + 6 * (size_t)a.tD0, a.pl.o_tD, 6 * pad32(nt));
         constexpr int B = SlotSize<T>::B;
-        for (int i = tid; i < 4 * W_N; i += GT)
-            s_ws[i / W_N][i % W_N] = a.ws[((size_t)(i / W_N < 2 ? blockIdx.x : a.P) * 2 + (i / W_N & 1)) * W_N + i % W_N];
+        for (int i = tid; i < 2 * W_N; i += GT) s_ws[i / W_N][i % W_N] = a.ws[(size_t)blockIdx.x * 2 * W_N + i];
         __syncthreads();
         for (int q = 0; q < 2; ++q) {
-            // slots in shared memory: the top's programs, the narrow levels,
-            // or the whole program
-            const char *pg = a.prog[q] + (size_t)B * h[q ? Q_SB : Q_SF], *tg = a.prog[q] + (size_t)B * ht[q ? Q_SB : Q_SF];
+            // slots in shared memory: the narrow levels, or the whole program
+            const char *pg = a.prog[q] + (size_t)B * h[q ? Q_SB : Q_SF];
             const int32_t nn = s_ws[q][W_END] - s_ws[q][W_NARROW];
             const int4 *all = put(reinterpret_cast<const int4 *>(pg), a.pl.o_all[q], (B / 16) * s_ws[q][W_END]);
             const int4 *nar = a.pl.o_all[q] >= 0 ? all + (size_t)(B / 16) * s_ws[q][W_NARROW]
                                                  : put(reinterpret_cast<const int4 *>(pg) + (size_t)(B / 16) * s_ws[q][W_NARROW],
                                                        a.pl.o_nar[q], (B / 16) * nn);
-            const int4 *top = put(reinterpret_cast<const int4 *>(tg), a.pl.o_top[q], (B / 16) * s_ws[2 + q][W_END]);
-            if (tid == 0) {
-                s_prog[q] = Prog{s_ws[q], reinterpret_cast<const char *>(all), reinterpret_cast<const char *>(nar)};
-                s_prog[2 + q] = Prog{s_ws[2 + q], reinterpret_cast<const char *>(top),
-                                     reinterpret_cast<const char *>(top) + (size_t)B * s_ws[2 + q][W_NARROW]};
-            }
+            if (tid == 0) s_prog[q] = Prog{s_ws[q], reinterpret_cast<const char *>(all), reinterpret_cast<const char *>(nar)};
         }
-        if (tid < 2) {   // the spare cells
+        if (tid == 0) {   // the spare cell
             const T zero[3] = {0, 0, 0};
-            V3<T>::st(tid ? tw + nt * VB : w + (nr + nz) * VB, zero);
+            V3<T, VB>::st(w + (nr + nz) * VB, zero);
+        }
+        // the rows of the top's inverse that the part needs, when they fit
+        inv = reinterpret_cast<const T *>(a.inv);
+        if (a.pl.o_inv >= 0) {
+            T *d = reinterpret_cast<T *>(sm + a.pl.o_inv);
+            for (int32_t o = 0; o < nout; ++o) {
+                const int32_t i = o < nz ? __ldg(a.zi + zo + o) : t0 + o - nz;
+                const T *f = inv + (size_t)i * 9 * a.ntp;
+                for (int32_t k = tid; k < 9 * a.ntp; k += GT) d[(size_t)o * 9 * a.ntp + k] = f[k];
+            }
+            inv = d;
         }
     }
     T *r = a.pl.o_r >= 0 ? reinterpret_cast<T *>(sm + a.pl.o_r) : reinterpret_cast<T *>(a.r) + 3 * (size_t)ro;
@@ -1717,7 +1849,7 @@ __global__ void __launch_bounds__(GT, 1) k_pcg_grid(const __grid_constant__ Grid
             }
             if (Z.bad) return;
             lap(t_vec);
-            Acc<T> pq = product<T>(a, M, ro, nr, slot0, perm, glen, gso, ps, w);
+            Acc<T> pq = product<T, VB>(a, M, ro, nr, slot0, perm, glen, gso, ps, w);
             if (lane == 0) Z.red[0][warp] = pq.pair();
             __syncthreads();
         }
@@ -1726,7 +1858,7 @@ __global__ void __launch_bounds__(GT, 1) k_pcg_grid(const __grid_constant__ Grid
             for (int32_t i = tid; i < nr; i += GT) {
                 const int32_t v = __ldg(a.i_of_t + ro + i);
                 T q[3] = {0, 0, 0}, z[3];
-                if (phase == 0) V3<T>::ld(w + i * VB, q);
+                if (phase == 0) V3<T, VB>::ld(w + i * VB, q);
 #pragma unroll
                 for (int c = 0; c < 3; ++c) {
                     const T f = F[3 * (size_t)v + c];
@@ -1736,7 +1868,7 @@ __global__ void __launch_bounds__(GT, 1) k_pcg_grid(const __grid_constant__ Grid
                     r[3 * i + c] = q[c];
                 }
                 diag(i, q, z);
-                V3<T>::st(w + i * VB, z);
+                V3<T, VB>::st(w + i * VB, z);
             }
             partial(0, ff);
             partial(1, rr);
@@ -1771,7 +1903,7 @@ __global__ void __launch_bounds__(GT, 1) k_pcg_grid(const __grid_constant__ Grid
                     const int32_t i = b + u * GT;
                     if (i >= nr) break;
                     T q[3], z[3];
-                    V3<T>::ld(w + i * VB, q);
+                    V3<T, VB>::ld(w + i * VB, q);
 #pragma unroll
                     for (int c = 0; c < 3; ++c) {
                         q[c] = fma(-al, q[c], rv[u][c]);
@@ -1784,7 +1916,7 @@ __global__ void __launch_bounds__(GT, 1) k_pcg_grid(const __grid_constant__ Grid
 #pragma unroll
                         for (int c = 0; c < 3; ++c) rz.mul(q[c], z[c]);
                     }
-                    V3<T>::st(w + i * VB, z);
+                    V3<T, VB>::st(w + i * VB, z);
                 }
             }
             partial(0, rr);
@@ -1795,20 +1927,20 @@ __global__ void __launch_bounds__(GT, 1) k_pcg_grid(const __grid_constant__ Grid
             // the part's sums for the top, its pivots
             const unsigned long long e = (unsigned long long)(ep + 1) << 32;
             const T zero[3] = {0, 0, 0};
-            for (int32_t z = tid; z < nz; z += GT) V3<T>::st(w + (nr + z) * VB, zero);
+            for (int32_t z = tid; z < nz; z += GT) V3<T, VB>::st(w + (nr + z) * VB, zero);
             __syncthreads();
             for (int32_t i = nv + tid; i < nr; i += GT) {
                 T v[3];
-                V3<T>::ld(w + i * VB, v);
+                V3<T, VB>::ld(w + i * VB, v);
                 Pkt<T>::put(trx + (size_t)Pkt<T>::W * (t0 + i - nv), e, v);
             }
-            run<T, true>(s_prog[0], w);
+            run<T, VB, true>(s_prog[0], w);
             for (int32_t z = tid; z < nz; z += GT) {
                 T v[3];
-                V3<T>::ld(w + (nr + z) * VB, v);
+                V3<T, VB>::ld(w + (nr + z) * VB, v);
                 Pkt<T>::put(a.lx + (size_t)Pkt<T>::W * __ldg(a.zslot + zo + z), e, v);
             }
-            pivots<T>(D, nv, w);
+            pivots<T, VB>(D, nv, w);
         } else {
             __syncthreads();
         }
@@ -1842,7 +1974,7 @@ __global__ void __launch_bounds__(GT, 1) k_pcg_grid(const __grid_constant__ Grid
                     ok = wait_packet<T>(a.lx + (size_t)Pkt<T>::W * k, ep + 1, y0, a.err);
                     v[0] += y0[0]; v[1] += y0[1]; v[2] += y0[2];
                 }
-                V3<T>::st(tw + i * VB, v);
+                V3<T, VB>::st(tw + i * VB, v);
             }
             if (!ok) Z.bad = 1;
         }
@@ -1853,27 +1985,57 @@ __global__ void __launch_bounds__(GT, 1) k_pcg_grid(const __grid_constant__ Grid
             break;
         }
         if (PREC == 0) {
-            // the top (every block for itself), then the part's backward levels
-            if (nt > 0) {
-                run<T, true>(s_prog[2], tw);
-                pivots<T>(tD, nt, tw);
-                __syncthreads();
-                run<T, false>(s_prog[3], tw);
-                for (int32_t z = tid; z < nz + nr - nv; z += GT) {
-                    T v[3];
-                    const int32_t i = z < nz ? __ldg(a.zi + zo + z) : t0 + z - nz;
-                    V3<T>::ld(tw + i * VB, v);
-                    V3<T>::st(w + (z < nz ? nr + z : nv + z - nz) * VB, v);
+            // the top, as far as the part needs it: the rows of its inverse
+            // times the top's right-hand side, a warp per row or piece of a
+            // row (several blocks per lane in flight), then the pieces in
+            // order; then the part's backward levels
+            T *tp = reinterpret_cast<T *>(sm + a.pl.o_tp);
+            for (int32_t it = warp; it < nout * nch; it += GW) {
+                const int32_t o = it / nch, k0 = (it - o * nch) * chunk, k1 = min(a.ntp, k0 + chunk);
+                const int32_t i = o < nz ? __ldg(a.zi + zo + o) : t0 + o - nz;
+                const T *f = inv + (size_t)(a.pl.o_inv >= 0 ? o : i) * 9 * a.ntp + lane;
+                T z[3] = {0, 0, 0};
+                constexpr int N = sizeof(T) == 4 ? 4 : 2;
+                for (int32_t k = k0; k < k1; k += 32 * N) {
+                    T m[N][9];
+#pragma unroll
+                    for (int u = 0; u < N; ++u)
+#pragma unroll
+                        for (int c = 0; c < 9; ++c) m[u][c] = k + 32 * u < k1 ? f[(size_t)c * a.ntp + k + 32 * u] : T(0);
+#pragma unroll
+                    for (int u = 0; u < N; ++u) {
+                        if (k + 32 * u >= k1) break;
+                        T y[3];
+                        V3<T, VB>::ld(tw + min(k + lane + 32 * u, nt - 1) * VB, y);
+#pragma unroll
+                        for (int c = 0; c < 3; ++c)
+                            z[c] = fma(m[u][3 * c + 2], y[2], fma(m[u][3 * c + 1], y[1], fma(m[u][3 * c], y[0], z[c])));
+                    }
                 }
-                __syncthreads();
+#pragma unroll
+                for (int b = 16; b > 0; b >>= 1)
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) z[c] += __shfl_xor_sync(0xffffffffu, z[c], b);
+                if (lane == 0) {
+                    tp[3 * it] = z[0]; tp[3 * it + 1] = z[1]; tp[3 * it + 2] = z[2];
+                }
             }
-            run<T, false>(s_prog[1], w);
+            __syncthreads();
+            for (int32_t o = tid; o < nout; o += GT) {
+                T z[3] = {0, 0, 0};
+                for (int32_t k = o * nch; k < (o + 1) * nch; ++k) {
+                    z[0] += tp[3 * k]; z[1] += tp[3 * k + 1]; z[2] += tp[3 * k + 2];
+                }
+                V3<T, VB>::st(w + (o < nz ? nr + o : nv + o - nz) * VB, z);
+            }
+            __syncthreads();
+            run<T, VB, false>(s_prog[1], w);
         }
         if (PREC == 0 || phase <= 0) {
             Acc<T> acc;
             for (int32_t i = tid; i < nr; i += GT) {
                 T z[3];
-                V3<T>::ld(w + i * VB, z);
+                V3<T, VB>::ld(w + i * VB, z);
                 const T r0 = r[3 * i], r1 = r[3 * i + 1], r2 = r[3 * i + 2];
                 acc.mul(r0, z[0]);
                 acc.mul(r1, z[1]);
@@ -1890,7 +2052,7 @@ __global__ void __launch_bounds__(GT, 1) k_pcg_grid(const __grid_constant__ Grid
         const T be = phase <= 0 ? T(0) : Z.be;
         for (int32_t i = tid; i < nr; i += GT) {
             T z[3];
-            V3<T>::ld(w + i * VB, z);
+            V3<T, VB>::ld(w + i * VB, z);
 #pragma unroll
             for (int c = 0; c < 3; ++c) ps[3 * i + c] = phase <= 0 ? z[c] : fma(be, ps[3 * i + c], z[c]);
         }
@@ -1903,6 +2065,7 @@ __global__ void __launch_bounds__(GT, 1) k_pcg_grid(const __grid_constant__ Grid
         for (int c = 0; c < 3; ++c) xo[3 * (size_t)v + c] = x[3 * i + c];
     }
     if (blockIdx.x == 0 && tid == 0) {
+        if (sizeof(T) == 4) Z.S.rr = pair_value(Z.rr);
         *a.sc = Z.S;
         if (a.timing) {
             a.ns[0] = t_spmv;
@@ -1920,10 +2083,10 @@ namespace {
 // Shared-memory placement (sized by the largest part, the same in every
 // block): what is addressed at random always; then, as far as it fits, what
 // is read most often.  False: the vectors alone do not fit.
-bool place(const GridLayout &G, size_t sz, bool tree, bool halo, GridPlace *pl)
+bool place(const GridLayout &G, size_t sz, size_t vb, bool tree, bool halo, GridPlace *pl)
 {
     const int32_t *t = G.tot;
-    const size_t vb = sz == 4 ? 16 : 24, mnr = (size_t)t[T_MNR], nt = tree ? (size_t)t[T_NT] : 0;
+    const size_t mnr = (size_t)t[T_MNR], nt = tree ? (size_t)t[T_NT] : 0;
     size_t at = 0;
     auto need = [&](size_t b) {
         const int32_t o = (int32_t)at;
@@ -1937,16 +2100,16 @@ bool place(const GridLayout &G, size_t sz, bool tree, bool halo, GridPlace *pl)
     const size_t B = sz == 4 ? SlotSize<float>::B : SlotSize<double>::B;
     pl->o_p = need(3 * sz * (mnr + (halo ? (size_t)t[T_MNH] : 0)));
     pl->o_w = need(vb * (size_t)(tree ? t[T_MDZ] + 1 : t[T_MNR]));
-    pl->o_t = need(vb * (nt + 1));
+    pl->o_t = need(vb * nt);
+    pl->o_tp = need(3 * sz * (tree ? (size_t)std::max(GW, t[T_MNO]) : 0));
     pl->o_misc = need(8 * (mnr / 32 + 1));
     if (at > (size_t)GRID_SMEM) return false;
-    for (int q = 0; q < 2; ++q) pl->o_top[q] = pl->o_nar[q] = pl->o_all[q] = -1;
-    pl->o_D = pl->o_tD = -1;
+    for (int q = 0; q < 2; ++q) pl->o_nar[q] = pl->o_all[q] = -1;
+    pl->o_D = pl->o_inv = -1;
     pl->o_perm = opt(2 * (size_t)pad32((int32_t)mnr));
     pl->o_hl = halo ? opt(4 * (size_t)t[T_MNH]) : -1;
     if (tree) {
-        for (int q = 0; q < 2; ++q) pl->o_top[q] = opt(B * (size_t)G.top_slots[q]);
-        pl->o_tD = opt(6 * sz * (size_t)pad32((int32_t)nt));
+        pl->o_inv = opt(9 * sz * (size_t)pad32((int32_t)nt) * (size_t)t[T_MNO]);
         // the whole programs when they fit beside r and x, else the narrow levels
         const size_t all = B * ((size_t)t[T_MSF] + (size_t)t[T_MSB]) + 6 * sz * mnr + 64;
         if (at + all <= (size_t)GRID_SMEM)
@@ -1967,16 +2130,6 @@ bool place(const GridLayout &G, size_t sz, bool tree, bool halo, GridPlace *pl)
     }
     pl->bytes = (int32_t)at;
     return true;
-}
-
-template <typename T, int PREC>
-sgp_status optin(sgp_ctx *ctx)
-{
-    static int done_dev[64] = {0};
-    if (ctx->device >= 0 && ctx->device < 64 && done_dev[ctx->device]) return SGP_OK;
-    SGP_CUDA(ctx, cudaFuncSetAttribute(k_pcg_grid<T, PREC>, cudaFuncAttributeMaxDynamicSharedMemorySize, GRID_SMEM));
-    if (ctx->device >= 0 && ctx->device < 64) done_dev[ctx->device] = 1;
-    return SGP_OK;
 }
 
 struct GScr {
@@ -2066,12 +2219,25 @@ sgp_status numeric(sgp_ctx *ctx, GridLayout &G, const sgp_factor *F, const GBuil
     const int32_t *t = G.tot;
     const double *L = bp<const double>(F->L), *Di = bp<const double>(F->Dinv);
     const int32_t nf = 32 * t[T_SF], nb = 32 * t[T_SB], nr = t[T_NR], nt = t[T_NT], B = SGP_BLOCK;
-    T *D;
-    SGP_TRY(ensure(ctx, G.D, 6 * ((size_t)nr + pad32(nt)), &D));
+    T *D, *inv;
+    double *tD;
+    const int32_t ntp = pad32(nt), us[2] = {G.top_slots[0], G.top_slots[1]};
+    SGP_TRY(ensure(ctx, G.D, 6 * (size_t)nr, &D));
+    SGP_TRY(ensure(ctx, G.inv, 9 * (size_t)ntp * nt, &inv));
+    SGP_TRY(ensure(ctx, G.tD, 6 * (size_t)ntp, &tD));
     LAUNCH(ctx, (k_gr_blocks<T, false>), grid_for(nf, B), B, 0, nf, (const int32_t *)g.msrc[0], L, g.prog[0]);
     LAUNCH(ctx, (k_gr_blocks<T, true>), grid_for(nb, B), B, 0, nb, (const int32_t *)g.msrc[1], L, g.prog[1]);
     LAUNCH(ctx, k_gr_pivots<T>, grid_for(nr, B), B, 0, nr, (const int32_t *)g.d_src, Di, D);
-    LAUNCH(ctx, k_gr_pivots<T>, grid_for(nt, B), B, 0, nt, td_src, Di, D + 6 * (size_t)nr);
+    if (nt == 0) return SGP_OK;
+    LAUNCH(ctx, (k_gr_blocks<double, false>), grid_for(32 * us[0], B), B, 0, 32 * us[0], (const int32_t *)g.tmsrc[0], L,
+           g.tprog[0]);
+    LAUNCH(ctx, (k_gr_blocks<double, true>), grid_for(32 * us[1], B), B, 0, 32 * us[1], (const int32_t *)g.tmsrc[1], L,
+           g.tprog[1]);
+    LAUNCH(ctx, k_gr_pivots<double>, grid_for(nt, B), B, 0, nt, td_src, Di, tD);
+    SGP_CUDA(ctx, cudaFuncSetAttribute(k_gr_top_inverse<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 24 * (NTOP + 1)));
+    LAUNCH(ctx, k_gr_top_inverse<T>, std::min(3 * nt, ctx->num_sms * 4), GT, 24 * (size_t)(nt + 1), nt, ntp,
+           (const int32_t *)(g.ws + (size_t)G.P * 2 * W_N), (const char *)g.tprog[0], (const char *)g.tprog[1],
+           (const double *)tD, inv);
     return SGP_OK;
 }
 
@@ -2095,15 +2261,16 @@ sgp_status grid_build(sgp_ctx *ctx, sgp_factor *F, const sgp_matrix *M)
     SGP_TRY(part_count(ctx, n, 128, &P));
     const int32_t U = (n + P - 1) / P;
     // p and w of the largest part must fit
-    if ((size_t)U * (f32 ? 28 : 48) > (size_t)GRID_SMEM) return SGP_OK;
-    // The subtree bound trades the size of the top, which every block solves,
-    // against the imbalance of the parts (half a subtree either way).
-    // Measured, us per iteration with bmax = U/4, U/2, 3U/4, U: FP32, U = 197
-    // 30.9, 28.1, -, 26.2; U = 658 34.5, 31.3, 31.6, 31.3; U = 1645 49.9,
-    // 45.1, 40.7, 43.8; FP64, U = 197 60.7, 54.1, -, 47.9; U = 658 80.0, 71.1,
-    // 75.3, 79.6; U = 1974 149.7, 156.2, 164.0, -.  Above 2048 (FP32, U = 6579)
-    // U/8 147.2, U/5 144.9, U/4 147.5.
-    const int32_t part = U <= 512 ? U : (f32 ? (U <= 2048 ? 3 * U / 4 : U / 5) : (U <= 1024 ? U / 2 : U / 4));
+    if ((size_t)U * (f32 ? 24 : 48) > (size_t)GRID_SMEM) return SGP_OK;
+    // The subtree bound trades the number of top vertices (every block reads
+    // its rows of their inverse) and the length of the narrow levels against
+    // the imbalance of the parts (half a subtree either way).  Measured, us
+    // per iteration: FP64, U = 128 rows per part: 32.9 with bmax = U, 31.1 with
+    // 3U/2; U = 197: 42.8, 39.2; U = 658: U/2 66.7, 0.6 U 63.3, U 69.3; U =
+    // 1974: U/4 163, U/2 141.5, 0.6 U 137.9, 3U/4 139.5.  FP32, U = 197: 23.1
+    // with U, 22.1 with 3U/2; U = 658: 28.5 with U/2, 28.8 with U; U = 1645:
+    // U/2 38.6, 3U/4 45.7; U = 6579: U/5 136.8, U/4 134.1, 0.3 U 135.8.
+    const int32_t part = U <= 512 ? 3 * U / 2 : (f32 ? (U <= 2048 ? U / 2 : U / 4) : 3 * U / 5);
     const int32_t bmax = std::max(32, part);
     G.P = P;
     G.LV = LV;
@@ -2200,21 +2367,30 @@ sgp_status grid_build(sgp_ctx *ctx, sgp_factor *F, const sgp_matrix *M)
         (int64_t)G.tot[T_S] * 32 > 4 * (int64_t)M->m + 64 * (int64_t)n + 65536)
         return SGP_OK;
     GridPlace pl;
+    // the halo on chip, in FP32 with packed vectors if need be
     G.halo = 1;
-    if (!place(G, sz, true, true, &pl)) {
-        G.halo = 0;
-        if (!place(G, sz, true, false, &pl)) return SGP_OK;
+    G.vb = f32 ? 16 : 24;
+    if (!place(G, sz, G.vb, true, true, &pl)) {
+        if (f32) G.vb = 12;
+        if (!f32 || !place(G, sz, G.vb, true, true, &pl)) {
+            G.halo = 0;
+            if (!place(G, sz, G.vb, true, false, &pl)) return SGP_OK;
+        }
     }
     g.halo = G.halo;
     for (int q = 0; q < 2; ++q) {
         const size_t slots = (size_t)G.tot[q ? T_SB : T_SF];
         SGP_TRY(ensure(ctx, G.prog[q], slots * (f32 ? SlotSize<float>::B : SlotSize<double>::B), &g.prog[q]));
         SGP_TRY(S.take(32 * slots, &g.msrc[q]));
+        SGP_TRY(S.take((size_t)G.top_slots[q] * SlotSize<double>::B, &g.tprog[q]));
+        SGP_TRY(S.take(32 * (size_t)G.top_slots[q], &g.tmsrc[q]));
     }
     SGP_TRY(ensure(ctx, G.zi, G.tot[T_Z], &g.zi));
     SGP_TRY(ensure(ctx, G.zslot, G.tot[T_Z], &g.zslot));
     SGP_TRY(ensure(ctx, G.tlk, (size_t)G.tot[T_NT] + 1, &g.tlk));
-    SGP_TRY(sgp_launch(ctx, "k_gr_program", f32 ? k_gr_program<float> : k_gr_program<double>, dim3(P + 1, 2), dim3(GT), 0, g));
+    SGP_TRY(sgp_launch(ctx, "k_gr_program", f32 ? k_gr_program<float> : k_gr_program<double>, dim3(P, 2), dim3(GT), 0, g, 0));
+    if (G.tot[T_NT] > 0)
+        SGP_TRY(sgp_launch(ctx, "k_gr_program", k_gr_program<double>, dim3(1, 2), dim3(GT), 0, g, P));
     LAUNCH(ctx, k_gr_slots, 1, 1024, 0, g);
     SGP_TRY(rows_fill(ctx, G, g, M, f32));
     LAUNCH(ctx, k_gr_check, P + 1, GT, 0, g);
@@ -2234,7 +2410,7 @@ sgp_status grid_build(sgp_ctx *ctx, sgp_factor *F, const sgp_matrix *M)
 void grid_release(GridLayout &G)
 {
     DBuf *b[] = {&G.hdr, &G.dtot, &G.ws, &G.glen, &G.gso, &G.perm, &G.xflag, &G.hl, &G.zi, &G.zslot, &G.tlk, &G.i_of_t,
-                 &G.t_of_i, &G.prog[0], &G.prog[1], &G.D, &G.ma, &G.mb};
+                 &G.t_of_i, &G.prog[0], &G.prog[1], &G.D, &G.inv, &G.tD, &G.ma, &G.mb};
     for (DBuf *d : b)
         if (d->p) cudaFree(d->p);
     for (DBuf &d : G.scr)
@@ -2268,8 +2444,7 @@ sgp_status grid_pcg(sgp_ctx *ctx, const sgp_matrix *M, const GridLayout &G, cons
 {
     const int32_t *t = G.tot;
     GridArgs a{};
-    if (!place(G, sizeof(T), true, G.halo != 0, &a.pl)) return sgp_fail(ctx, SGP_ERR_CUDA, "pcg: the grid layout does not fit");
-    SGP_TRY((optin<T, 0>(ctx)));
+    if (!place(G, sizeof(T), G.vb, true, G.halo != 0, &a.pl)) return sgp_fail(ctx, SGP_ERR_CUDA, "pcg: the grid layout does not fit");
     char *at = reinterpret_cast<char *>(work);
     auto take = [&](size_t b) {
         char *p = at;
@@ -2292,14 +2467,14 @@ sgp_status grid_pcg(sgp_ctx *ctx, const sgp_matrix *M, const GridLayout &G, cons
     if (a.pl.o_r < 0) a.r = take(3 * sizeof(T) * nr);
     if (a.pl.o_x < 0) a.xt = take(3 * sizeof(T) * nr);
     a.P = G.P; a.nt = t[T_NT]; a.x_given = x_given; a.timing = ctx->timing; a.halo = G.halo;
-    a.tD0 = t[T_NR]; a.nslots = t[T_Z];
+    a.ntp = pad32(t[T_NT]); a.nslots = t[T_Z];
     a.hdr = bp<const int32_t>(G.hdr); a.ws = bp<const int32_t>(G.ws);
     a.glen = bp<const int32_t>(G.glen); a.gso = bp<const int32_t>(G.gso); a.i_of_t = bp<const int32_t>(G.i_of_t);
     a.zi = bp<const int32_t>(G.zi); a.zslot = bp<const int32_t>(G.zslot); a.tlk = bp<const int32_t>(G.tlk);
     a.hl = bp<const int32_t>(G.hl);
     a.perm = bp<const uint16_t>(G.perm); a.xflag = bp<const uint8_t>(G.xflag);
     for (int q = 0; q < 2; ++q) a.prog[q] = bp<const char>(G.prog[q]);
-    a.D = G.D.p; a.ma = G.ma.p; a.mb = G.mb.p;
+    a.D = G.D.p; a.inv = G.inv.p; a.ma = G.ma.p; a.mb = G.mb.p;
     a.F = F; a.x = x;
     a.gamma0 = M->gamma0;
     a.tol2 = stopE ? -1.0 : tol * tol;
@@ -2312,8 +2487,16 @@ sgp_status grid_pcg(sgp_ctx *ctx, const sgp_matrix *M, const GridLayout &G, cons
     a.ns = out->ns;
     SGP_CUDA(ctx, cudaMemsetAsync(zero, 0, (size_t)(zend - zero), ctx->stream));
     void *args[] = {&a};
-    SGP_CUDA(ctx, cudaLaunchCooperativeKernel((const void *)k_pcg_grid<T, 0>, dim3(G.P), dim3(GT), args, (size_t)a.pl.bytes,
-                                              ctx->stream));
+    auto go = [&](auto kern) -> sgp_status {
+        SGP_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, GRID_SMEM));
+        SGP_CUDA(ctx, cudaLaunchCooperativeKernel((const void *)kern, dim3(G.P), dim3(GT), args, (size_t)a.pl.bytes,
+                                                  ctx->stream));
+        return SGP_OK;
+    };
+    if constexpr (sizeof(T) == 8)
+        SGP_TRY(go(k_pcg_grid<T, 24, 0>));
+    else
+        SGP_TRY(G.vb == 16 ? go(k_pcg_grid<T, 16, 0>) : go(k_pcg_grid<T, 12, 0>));
     ctx->launches++;
     Out h;
     SGP_TRY(read_back(ctx, &h, out, sizeof(h)));

@@ -1160,18 +1160,22 @@ sgp_status pcg_run(sgp_ctx *ctx, const sgp_matrix *M, const sgp_factor *Fac, int
 }  // namespace
 
 
-// The one-block solve applies: MIXED, tree preconditioner, residual
-// stopping, the factor's tail covering every level, and everything fitting
-// in one block's shared memory.
-static bool small_pcg_fits(const sgp_ctx *ctx, const sgp_matrix *M, const sgp_factor *Fac, const sgp_solve_opts *o)
+// The one-block solve serves a factor: MIXED, the tail covering every level,
+// and everything fitting in one block's shared memory.
+bool small_solve_fits(const sgp_ctx *ctx, const sgp_factor *Fac)
 {
-    if (!ctx->small_solve || o->precision != SGP_PREC_MIXED || o->precond != SGP_PRECOND_TREE ||
-        o->stop != SGP_STOP_RESIDUAL || !Fac || Fac->precision != SGP_PREC_MIXED || M->precision != SGP_PREC_MIXED)
-        return false;
+    if (!ctx->small_solve || Fac->precision != SGP_PREC_MIXED) return false;
     if (Fac->levels == 0 || Fac->tail_level != 0 || Fac->tail_P0 != 0 || !Fac->L32.p || !Fac->Dinv32.p) return false;
     const Tail tl = tail_of(Fac);
-    if (tl.n != M->n) return false;
-    return small_smem_bytes(tl.n, tl.np, tl.nr) <= (size_t)TREE_TAIL_SMEM;
+    return tl.n == Fac->n && small_smem_bytes(tl.n, tl.np, tl.nr) <= (size_t)TREE_TAIL_SMEM;
+}
+
+// The one-block solve applies: such a factor, the tree preconditioner, MIXED
+// and residual stopping.
+static bool small_pcg_fits(const sgp_ctx *ctx, const sgp_matrix *M, const sgp_factor *Fac, const sgp_solve_opts *o)
+{
+    return o->precision == SGP_PREC_MIXED && o->precond == SGP_PRECOND_TREE && o->stop == SGP_STOP_RESIDUAL && Fac &&
+           M->precision == SGP_PREC_MIXED && Fac->n == M->n && small_solve_fits(ctx, Fac);
 }
 
 static sgp_status small_pcg(sgp_ctx *ctx, const sgp_matrix *M, const sgp_factor *Fac, const double *F, double *v,

@@ -220,6 +220,8 @@ sgp_status bins_from_tree(sgp_ctx *ctx, const sgp_factor *F, const T *src, T *ds
 template <typename T>
 sgp_status bins_pcg_step(sgp_ctx *ctx, const sgp_factor *F, T *r, const T *q, T *z, void *scal);
 sgp_status bins_check(sgp_ctx *ctx, const sgp_factor *F);
+// The factor is solved whole by one thread block (pcg.cu).
+bool small_solve_fits(const sgp_ctx *ctx, const sgp_factor *F);
 
 // The grid solve (grid.cu): a whole PCG run in one persistent launch.
 // grid_build runs at the end of a factor build; grid_ready tells whether it
@@ -321,12 +323,12 @@ struct BinLayout {
 // in the factor's own precision, with the matrix's rows of generation mgen.
 #define SGP_GRID_SCRATCH 48
 struct GridLayout {
-    int ok = 0, prec = 0, halo = 0;
+    int ok = 0, prec = 0, halo = 0, vb = 16;   // vb: bytes per cell of the on-chip vectors
     uint64_t mgen = 0;
     int32_t P = 0, LV = 0;
-    int32_t tot[24] = {0}, top_slots[2] = {0, 0};   // totals and maxima over the parts; the top's programs
+    int32_t tot[24] = {0}, top_slots[2] = {0, 0};   // totals and maxima over the parts; slots of the top's programs
     DBuf hdr, dtot, ws, glen, gso, perm, xflag, hl, zi, zslot, tlk, i_of_t, t_of_i;
-    DBuf prog[2], D, ma, mb;
+    DBuf prog[2], D, inv, tD, ma, mb;
     DBuf scr[SGP_GRID_SCRATCH];
 };
 
