@@ -503,6 +503,8 @@ void sgp_destroy(sgp_ctx *ctx)
     for (auto e : ctx->ev_free) cudaEventDestroy(e);
     for (int k = 0; k < SGP_KT_COUNT; ++k)
         for (auto e : ctx->ev_pending[k]) cudaEventDestroy(e);
+    grid_release(ctx->grid_plain);
+    grid_rows_release(ctx->grid_rows);
     delete ctx;
 }
 

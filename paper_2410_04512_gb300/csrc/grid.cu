@@ -59,11 +59,12 @@ constexpr int LMAX = 64;         // contraction levels
 constexpr int NCLS = 8;          // segment classes: 8 sources or more, 7, ... 1
 
 // header of a part (entry P: the top); Q_NSF, Q_NSB: slots of its programs
-enum { Q_SOFF, Q_NV, Q_ROFF, Q_NR, Q_T0, Q_NP, Q_POFF, Q_NZ, Q_ZOFF, Q_DOFF, Q_NSF, Q_SF, Q_NSB, Q_SB, Q_NS, Q_SLOT, Q_NH,
-       Q_HOFF, Q_N = 24 };
+enum { Q_SOFF, Q_NV, Q_ROFF, Q_NR, Q_T0, Q_NP, Q_POFF, Q_NZ, Q_ZOFF, Q_DOFF, Q_NSF, Q_SF, Q_NSB, Q_SB, Q_N = 24 };
 // totals and maxima over the parts
-enum { T_NT, T_NR, T_P, T_Z, T_D, T_SF, T_SB, T_S, T_H, T_MNR, T_MNZ, T_MNH, T_MSF, T_MSB, T_MDZ, T_MNF, T_MNB, T_MNO, T_ERR,
-       T_N = 24 };
+enum { T_NT, T_NR, T_P, T_Z, T_D, T_SF, T_SB, T_MNR, T_MNZ, T_MSF, T_MSB, T_MDZ, T_MNF, T_MNB, T_MNO, T_ERR, T_N = 24 };
+// a matrix's rows on the parts: slots and halo cells of each part with their
+// offsets; behind the parts the totals and the largest halo
+enum { R_NS, R_SLOT, R_NH, R_HOFF, R_N };
 // streams of a program: first slot of every warp's wide levels, of the narrow
 // levels, the end; wide levels
 enum { W_NARROW = GW, W_END, W_LEVELS, W_N = GW + 4 };
@@ -261,6 +262,23 @@ __global__ void __launch_bounds__(256) k_gr_rows(int32_t P, int32_t nblk, const 
     }
 }
 
+// parts of U consecutive rows (no forest)
+__global__ void __launch_bounds__(256) k_gr_rows_plain(int32_t n, int32_t P, int32_t U, int32_t *hdr, int32_t *tot)
+{
+    const int b = threadIdx.x;
+    if (b > P) return;
+    int32_t *h = hdr + (size_t)Q_N * b;
+    for (int k = 0; k < Q_N; ++k) h[k] = 0;
+    const int32_t r0 = min(n, b * U), nr = b < P ? min(n, r0 + U) - r0 : 0;
+    h[Q_SOFF] = r0;
+    h[Q_NV] = h[Q_NR] = nr;
+    h[Q_ROFF] = b * pad32(U);
+    if (b == P) {
+        tot[T_NR] = P * pad32(U);
+        tot[T_MNR] = U;
+    }
+}
+
 struct GBuild {
     int32_t n, P, LV;
     int32_t NRW;                             // halo bitmap words per part
@@ -269,7 +287,7 @@ struct GBuild {
     const int32_t *seg, *sp, *lpos;
     const int32_t *row_ptr, *col;            // the matrix's rows (internal order)
     const float2 *col32;                     // MIXED: the column of a slot is in its record
-    int32_t *hdr, *tot, *vm;
+    int32_t *hdr, *tot, *vm, *rh;            // rh: R_N per part
     int32_t *i_of_t, *t_of_i, *d_src;
     int32_t *dcnt, *plist, *sgk, *sgd, *sgf, *sgn; // per receiver counts; pairs by receiver; segments
     int32_t *nseg;                           // segments of each part
@@ -391,13 +409,10 @@ __global__ void __launch_bounds__(256) k_gr_offsets2(int32_t P, int32_t *hdr, in
     __shared__ int32_t sh[8];
     hdr_scan(P, hdr, tot, Q_NSF, Q_SF, T_SF, 0, sh);
     hdr_scan(P, hdr, tot, Q_NSB, Q_SB, T_SB, 0, sh);
-    hdr_scan(P, hdr, tot, Q_NS, Q_SLOT, T_S, 0, sh);
-    hdr_scan(P, hdr, tot, Q_NH, Q_HOFF, T_H, 0, sh);
     if (threadIdx.x < P) {
         const int32_t *h = hdr + (size_t)Q_N * threadIdx.x;
         atomicMax(tot + T_MNR, h[Q_NR]);
         atomicMax(tot + T_MNZ, h[Q_NZ]);
-        atomicMax(tot + T_MNH, h[Q_NH]);
         atomicMax(tot + T_MSF, h[Q_NSF]);
         atomicMax(tot + T_MSB, h[Q_NSB]);
         atomicMax(tot + T_MDZ, h[Q_NR] + h[Q_NZ]);
@@ -593,7 +608,7 @@ __global__ void __launch_bounds__(GT) k_gr_part_rows(GBuild g)
 {
     __shared__ int32_t cls[64], wc[GW][64], sh[GW];
     const int b = blockIdx.x, w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    int32_t *h = g.hdr + (size_t)Q_N * b;
+    const int32_t *h = g.hdr + (size_t)Q_N * b;
     const int32_t nr = h[Q_NR], ro = h[Q_ROFF], ng = pad32(nr) / 32;
     for (int i = threadIdx.x; i < 64; i += GT) cls[i] = 0;
     __syncthreads();
@@ -653,7 +668,7 @@ __global__ void __launch_bounds__(GT) k_gr_part_rows(GBuild g)
         }
         carry += tot;
     }
-    if (threadIdx.x == 0) h[Q_NS] = carry;
+    if (threadIdx.x == 0) g.rh[R_N * b + R_NS] = carry;
 }
 
 // The rows of other parts that a part's rows name ("halo"): marked in a
@@ -705,14 +720,30 @@ __global__ void __launch_bounds__(1024) k_gr_halo_count(GBuild g)
         }
         carry += tot;
     }
-    if (threadIdx.x == 0) g.hdr[(size_t)Q_N * b + Q_NH] = carry;
+    if (threadIdx.x == 0) g.rh[R_N * b + R_NH] = carry;
+}
+__global__ void __launch_bounds__(256) k_gr_row_offsets(GBuild g)
+{
+    __shared__ int32_t sh[8];
+    const int b = threadIdx.x;
+    int32_t *rh = g.rh + R_N * b, *t = g.rh + R_N * g.P, total;
+    if (b < R_N) t[b] = 0;
+    int32_t o = gscan<256>(b < g.P ? rh[R_NS] : 0, sh, &total);
+    if (b < g.P) rh[R_SLOT] = o;
+    if (b == 0) t[0] = total;
+    o = gscan<256>(b < g.P ? rh[R_NH] : 0, sh, &total);
+    if (b < g.P) {
+        rh[R_HOFF] = o;
+        atomicMax(t + 2, rh[R_NH]);
+    }
+    if (b == 0) t[1] = total;
 }
 __global__ void __launch_bounds__(GT) k_gr_halo_list(GBuild g)
 {
     const int b = blockIdx.x;
     const uint32_t *hb = g.hb + (size_t)b * g.NRW;
     const int32_t *hp = g.hpre + (size_t)b * g.NRW;
-    int32_t *hl = g.hl + g.hdr[(size_t)Q_N * b + Q_HOFF];
+    int32_t *hl = g.hl + g.rh[R_N * b + R_HOFF];
     const int32_t nw = g.tot[T_NR] / 32;
     for (int32_t w = blockIdx.y * GT + threadIdx.x; w < nw; w += GT * gridDim.y) {
         uint32_t m = hb[w];
@@ -906,7 +937,7 @@ __global__ void __launch_bounds__(GT) k_gr_sell32(GBuild g, const float4 *__rest
         const int32_t l = g.perm[ro + 32 * gi + lane];
         const int32_t v = l != 0xffff ? g.i_of_t[ro + l] : -1;
         const int32_t b0 = v >= 0 ? g.row_ptr[v] : 0, n = v >= 0 ? g.row_ptr[v + 1] - b0 : 0;
-        const size_t o = (size_t)(h[Q_SLOT] + g.gso[ro / 32 + gi]) * 32 + lane;
+        const size_t o = (size_t)(g.rh[R_N * blockIdx.x + R_SLOT] + g.gso[ro / 32 + gi]) * 32 + lane;
         const int32_t gl = g.glen[ro / 32 + gi];
         for (int32_t k = 0; k < gl; ++k) {
             float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -930,7 +961,7 @@ __global__ void __launch_bounds__(GT) k_gr_sell64(GBuild g, const double *__rest
         const int32_t l = g.perm[ro + 32 * gi + lane];
         const int32_t v = l != 0xffff ? g.i_of_t[ro + l] : -1;
         const int32_t b0 = v >= 0 ? g.row_ptr[v] : 0, n = v >= 0 ? g.row_ptr[v + 1] - b0 : 0;
-        const size_t o = (size_t)(h[Q_SLOT] + g.gso[ro / 32 + gi]);
+        const size_t o = (size_t)(g.rh[R_N * blockIdx.x + R_SLOT] + g.gso[ro / 32 + gi]);
         const int32_t gl = g.glen[ro / 32 + gi];
         for (int32_t k = 0; k < gl; ++k) {
             double2 x[3] = {{0.0, 0.0}, {0.0, 0.0}, {0.0, 0.0}};
@@ -978,8 +1009,8 @@ __global__ void __launch_bounds__(GT) k_gr_check(GBuild g)
         if (q != 0xffff && q >= nr) bad = 1024;
     }
     if (!top && g.halo)
-        for (int32_t k = threadIdx.x; k < h[Q_NH]; k += GT) {
-            const int32_t t = g.hl[h[Q_HOFF] + k];
+        for (int32_t k = threadIdx.x; k < g.rh[R_N * b + R_NH]; k += GT) {
+            const int32_t t = g.hl[g.rh[R_N * b + R_HOFF] + k];
             if (t < 0 || t >= g.tot[T_NR] || !g.xflag[t]) bad = 2048;
         }
     if (bad) atomicOr(g.tot + T_ERR, bad);
@@ -1007,7 +1038,7 @@ struct GridPlace {
 };
 struct GridArgs {
     int32_t P, nt, ntp, x_given, timing, halo, nslots;
-    const int32_t *hdr, *ws, *glen, *gso, *i_of_t, *zi, *zslot, *tlk, *hl;
+    const int32_t *hdr, *rh, *ws, *glen, *gso, *i_of_t, *zi, *zslot, *tlk, *hl;
     const char *prog[2];
     const uint16_t *perm;
     const uint8_t *xflag;
@@ -1712,7 +1743,7 @@ __global__ void __launch_bounds__(GT, 1) k_pcg_grid(const __grid_constant__ Grid
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int32_t *h = a.hdr + (size_t)Q_N * blockIdx.x;
     const int32_t nv = h[Q_NV], nr = h[Q_NR], ro = h[Q_ROFF], t0 = h[Q_T0], nz = h[Q_NZ], zo = h[Q_ZOFF],
-                  slot0 = h[Q_SLOT], nh = h[Q_NH], nt = a.nt;
+                  slot0 = a.rh[R_N * blockIdx.x + R_SLOT], nh = a.rh[R_N * blockIdx.x + R_NH], nt = a.nt;
     T *ps = reinterpret_cast<T *>(sm + a.pl.o_p);
     const uint32_t sm0 = (uint32_t)__cvta_generic_to_shared(sm);
     const uint32_t w = sm0 + a.pl.o_w, tw = sm0 + a.pl.o_t;
@@ -1730,7 +1761,7 @@ __global__ void __launch_bounds__(GT, 1) k_pcg_grid(const __grid_constant__ Grid
         glen[i] = a.glen[ro / 32 + i];
         gso[i] = a.gso[ro / 32 + i];
     }
-    const int32_t *hl = put(a.hl + h[Q_HOFF], a.pl.o_hl, a.halo ? nh : 0);
+    const int32_t *hl = put(a.hl + a.rh[R_N * blockIdx.x + R_HOFF], a.pl.o_hl, a.halo ? nh : 0);
     const T *D = nullptr, *inv = nullptr;
     // top vertices the part needs: those it reaches, then those it owns
     // and into how many pieces their rows are cut (about one item per warp)
@@ -2083,7 +2114,7 @@ namespace {
 // Shared-memory placement (sized by the largest part, the same in every
 // block): what is addressed at random always; then, as far as it fits, what
 // is read most often.  False: the vectors alone do not fit.
-bool place(const GridLayout &G, size_t sz, size_t vb, bool tree, bool halo, GridPlace *pl)
+bool place(const GridLayout &G, int32_t mnh, size_t sz, size_t vb, bool tree, bool halo, GridPlace *pl)
 {
     const int32_t *t = G.tot;
     const size_t mnr = (size_t)t[T_MNR], nt = tree ? (size_t)t[T_NT] : 0;
@@ -2098,7 +2129,7 @@ bool place(const GridLayout &G, size_t sz, size_t vb, bool tree, bool halo, Grid
         return r > 0 && at + r <= (size_t)GRID_SMEM ? need(b) : -1;
     };
     const size_t B = sz == 4 ? SlotSize<float>::B : SlotSize<double>::B;
-    pl->o_p = need(3 * sz * (mnr + (halo ? (size_t)t[T_MNH] : 0)));
+    pl->o_p = need(3 * sz * (mnr + (halo ? (size_t)mnh : 0)));
     pl->o_w = need(vb * (size_t)(tree ? t[T_MDZ] + 1 : t[T_MNR]));
     pl->o_t = need(vb * nt);
     pl->o_tp = need(3 * sz * (tree ? (size_t)std::max(GW, t[T_MNO]) : 0));
@@ -2107,7 +2138,7 @@ bool place(const GridLayout &G, size_t sz, size_t vb, bool tree, bool halo, Grid
     for (int q = 0; q < 2; ++q) pl->o_nar[q] = pl->o_all[q] = -1;
     pl->o_D = pl->o_inv = -1;
     pl->o_perm = opt(2 * (size_t)pad32((int32_t)mnr));
-    pl->o_hl = halo ? opt(4 * (size_t)t[T_MNH]) : -1;
+    pl->o_hl = halo ? opt(4 * (size_t)mnh) : -1;
     if (tree) {
         pl->o_inv = opt(9 * sz * (size_t)pad32((int32_t)nt) * (size_t)t[T_MNO]);
         // the whole programs when they fit beside r and x, else the narrow levels
@@ -2164,17 +2195,19 @@ sgp_status part_count(sgp_ctx *ctx, int32_t n, int32_t umin, int32_t *P)
     return SGP_OK;
 }
 
-// The buffers of the row layout, and the kernels up to the counts.
-sgp_status rows_count(sgp_ctx *ctx, GridLayout &G, GScr &S, GBuild &g, const sgp_matrix *M, size_t NRmax)
+// The rows of a matrix on the parts of a layout, up to the counts (they go to
+// the host with the next read of `R.tot`).
+sgp_status rows_count(sgp_ctx *ctx, GridRows &R, GBuild &g, const sgp_matrix *M, size_t NRmax)
 {
     const int32_t P = g.P;
     g.NRW = (int32_t)(NRmax / 32);
-    SGP_TRY(ensure(ctx, G.glen, NRmax / 32 + 1, &g.glen));
-    SGP_TRY(ensure(ctx, G.gso, NRmax / 32 + 1, &g.gso));
-    SGP_TRY(ensure(ctx, G.perm, NRmax, &g.perm));
-    SGP_TRY(ensure(ctx, G.xflag, NRmax, &g.xflag));
-    SGP_TRY(S.take((size_t)P * g.NRW, &g.hb));
-    SGP_TRY(S.take((size_t)P * g.NRW, &g.hpre));
+    SGP_TRY(ensure(ctx, R.rh, R_N * ((size_t)P + 1), &g.rh));
+    SGP_TRY(ensure(ctx, R.glen, NRmax / 32 + 1, &g.glen));
+    SGP_TRY(ensure(ctx, R.gso, NRmax / 32 + 1, &g.gso));
+    SGP_TRY(ensure(ctx, R.perm, NRmax, &g.perm));
+    SGP_TRY(ensure(ctx, R.xflag, NRmax, &g.xflag));
+    SGP_TRY(ensure(ctx, R.hb, (size_t)P * g.NRW, &g.hb));
+    SGP_TRY(ensure(ctx, R.hpre, (size_t)P * g.NRW, &g.hpre));
     SGP_CUDA(ctx, cudaMemsetAsync(g.hb, 0, sizeof(uint32_t) * (size_t)P * g.NRW, ctx->stream));
     SGP_CUDA(ctx, cudaMemsetAsync(g.xflag, 0, NRmax, ctx->stream));
     g.row_ptr = bp<const int32_t>(M->row_ptr);
@@ -2183,33 +2216,55 @@ sgp_status rows_count(sgp_ctx *ctx, GridLayout &G, GScr &S, GBuild &g, const sgp
     const unsigned gy = (unsigned)std::max<size_t>(1, std::min<size_t>(8, NRmax / P / GT));
     SGP_TRY(sgp_launch(ctx, "k_gr_halo_mark", k_gr_halo_mark, dim3(P, gy), dim3(GT), 0, g));
     LAUNCH(ctx, k_gr_halo_count, P, 1024, 0, g);
+    LAUNCH(ctx, k_gr_row_offsets, 1, 256, 0, g);
     return SGP_OK;
 }
 
+// Where the halo goes: on chip, in FP32 with packed vectors if need be, else
+// read from memory.  False: nothing fits, or the padded rows are too many.
+bool rows_place(const GridLayout &G, GridRows &R, const sgp_matrix *M, bool f32, bool tree)
+{
+    const size_t sz = f32 ? 4 : 8;
+    GridPlace pl;
+    if (G.tot[T_MNR] + R.tot[2] > 65535 ||
+        (int64_t)R.tot[0] * 32 > 4 * (int64_t)M->m + 64 * (int64_t)M->n + 65536)
+        return false;
+    R.halo = 1;
+    R.vb = f32 ? 16 : 24;
+    if (place(G, R.tot[2], sz, R.vb, tree, true, &pl)) return true;
+    if (f32) R.vb = 12;
+    if (f32 && place(G, R.tot[2], sz, R.vb, tree, true, &pl)) return true;
+    R.halo = 0;
+    return place(G, R.tot[2], sz, R.vb, tree, false, &pl);
+}
+
 // The matrix's rows in part order (after the counts are known).
-sgp_status rows_fill(sgp_ctx *ctx, GridLayout &G, GBuild &g, const sgp_matrix *M, bool f32)
+sgp_status rows_fill(sgp_ctx *ctx, const GridLayout &G, GridRows &R, GBuild &g, const sgp_matrix *M, bool f32)
 {
     const int32_t P = g.P;
     const unsigned gy = (unsigned)std::max(1, std::min(8, G.tot[T_MNR] / GT));
-    SGP_TRY(ensure(ctx, G.hl, G.tot[T_H], &g.hl));
+    g.halo = R.halo;
+    SGP_TRY(ensure(ctx, R.hl, R.tot[1], &g.hl));
     if (g.halo) SGP_TRY(sgp_launch(ctx, "k_gr_halo_list", k_gr_halo_list, dim3(P, gy), dim3(GT), 0, g));
-    const size_t slots = 32 * (size_t)G.tot[T_S];
+    const size_t slots = 32 * (size_t)R.tot[0];
     if (f32) {
         float4 *at;
         float2 *bt;
-        SGP_TRY(ensure(ctx, G.ma, slots, &at));
-        SGP_TRY(ensure(ctx, G.mb, slots, &bt));
+        SGP_TRY(ensure(ctx, R.ma, slots, &at));
+        SGP_TRY(ensure(ctx, R.mb, slots, &bt));
         const float4 *a4 = bp<const float4>(M->blk32);
         SGP_TRY(sgp_launch(ctx, "k_gr_sell32", k_gr_sell32, dim3(P, gy), dim3(GT), 0, g, a4,
                            reinterpret_cast<const float2 *>(a4 + 2 * M->m), at, bt));
     } else {
         double2 *at;
         int32_t *bt;
-        SGP_TRY(ensure(ctx, G.ma, 3 * slots, &at));
-        SGP_TRY(ensure(ctx, G.mb, slots, &bt));
+        SGP_TRY(ensure(ctx, R.ma, 3 * slots, &at));
+        SGP_TRY(ensure(ctx, R.mb, slots, &bt));
         SGP_TRY(sgp_launch(ctx, "k_gr_sell64", k_gr_sell64, dim3(P, gy), dim3(GT), 0, g, bp<const double>(M->blk),
                            bp<const int32_t>(M->col), at, bt));
     }
+    R.mgen = M->gen;
+    R.ok = 1;
     return SGP_OK;
 }
 
@@ -2352,7 +2407,8 @@ sgp_status grid_build(sgp_ctx *ctx, sgp_factor *F, const sgp_matrix *M)
     LAUNCH(ctx, k_gr_part_count, P + 1, GT, 0, g);
     LAUNCH(ctx, k_gr_offsets1, 1, 256, 0, P, g.hdr, g.tot);
     LAUNCH(ctx, k_gr_segments, P + 1, GT, 0, g);
-    SGP_TRY(rows_count(ctx, G, S, g, M, NRmax));
+    GridRows &R = G.rows;
+    SGP_TRY(rows_count(ctx, R, g, M, NRmax));
     LAUNCH(ctx, k_gr_offsets2, 1, 256, 0, P, g.hdr, g.tot, (const int32_t *)g.ws);
     // sizes to the host
     struct {
@@ -2360,24 +2416,12 @@ sgp_status grid_build(sgp_ctx *ctx, sgp_factor *F, const sgp_matrix *M)
     } hs;
     SGP_TRY(read_back(ctx, hs.t, g.tot, sizeof(hs.t)));
     SGP_TRY(read_back(ctx, hs.top, g.hdr + (size_t)Q_N * P, sizeof(hs.top)));
+    SGP_TRY(read_back(ctx, R.tot, g.rh + R_N * P, sizeof(R.tot)));
     memcpy(G.tot, hs.t, sizeof(hs.t));
     G.top_slots[0] = hs.top[Q_NSF];
     G.top_slots[1] = hs.top[Q_NSB];
-    if (G.tot[T_ERR] || G.tot[T_MDZ] > 8190 || G.tot[T_MNR] + G.tot[T_MNH] > 65535 ||
-        (int64_t)G.tot[T_S] * 32 > 4 * (int64_t)M->m + 64 * (int64_t)n + 65536)
-        return SGP_OK;
-    GridPlace pl;
-    // the halo on chip, in FP32 with packed vectors if need be
-    G.halo = 1;
-    G.vb = f32 ? 16 : 24;
-    if (!place(G, sz, G.vb, true, true, &pl)) {
-        if (f32) G.vb = 12;
-        if (!f32 || !place(G, sz, G.vb, true, true, &pl)) {
-            G.halo = 0;
-            if (!place(G, sz, G.vb, true, false, &pl)) return SGP_OK;
-        }
-    }
-    g.halo = G.halo;
+    if (G.tot[T_ERR] || G.tot[T_MDZ] > 8190 || !rows_place(G, R, M, f32, true)) return SGP_OK;
+    G.nr_max = (int64_t)NRmax;
     for (int q = 0; q < 2; ++q) {
         const size_t slots = (size_t)G.tot[q ? T_SB : T_SF];
         SGP_TRY(ensure(ctx, G.prog[q], slots * (f32 ? SlotSize<float>::B : SlotSize<double>::B), &g.prog[q]));
@@ -2392,7 +2436,7 @@ sgp_status grid_build(sgp_ctx *ctx, sgp_factor *F, const sgp_matrix *M)
     if (G.tot[T_NT] > 0)
         SGP_TRY(sgp_launch(ctx, "k_gr_program", k_gr_program<double>, dim3(1, 2), dim3(GT), 0, g, P));
     LAUNCH(ctx, k_gr_slots, 1, 1024, 0, g);
-    SGP_TRY(rows_fill(ctx, G, g, M, f32));
+    SGP_TRY(rows_fill(ctx, G, R, g, M, f32));
     LAUNCH(ctx, k_gr_check, P + 1, GT, 0, g);
     const int32_t *td_src = sp + hs.top[Q_SOFF];
     if (f32)
@@ -2401,27 +2445,100 @@ sgp_status grid_build(sgp_ctx *ctx, sgp_factor *F, const sgp_matrix *M)
         SGP_TRY(numeric<double>(ctx, G, F, g, td_src));
     SGP_TRY(read_back(ctx, hs.t, g.tot, sizeof(hs.t)));
     if (hs.t[T_ERR]) return sgp_fail(ctx, SGP_ERR_CUDA, "tree_factor: inconsistent grid layout (0x%x)", hs.t[T_ERR]);
-    G.mgen = M->gen;
     G.prec = F->precision;
     G.ok = 1;
     return SGP_OK;
 }
 
+// The rows of another matrix on a factor's parts (the augmented forest's P':
+// its product, the factor's preconditioner).  R.ok is 0 when they do not fit.
+sgp_status grid_rows(sgp_ctx *ctx, const sgp_factor *F, const sgp_matrix *M, GridRows &R)
+{
+    const GridLayout &G = F->gl;
+    R.ok = 0;
+    const bool f32 = G.prec == SGP_PREC_MIXED;
+    if (!G.ok || M->n != F->n || (f32 && M->precision != SGP_PREC_MIXED)) return SGP_OK;
+    GBuild g{};
+    g.n = (int32_t)M->n; g.P = G.P;
+    g.hdr = bp<int32_t>(G.hdr); g.tot = bp<int32_t>(G.dtot);
+    g.i_of_t = bp<int32_t>(G.i_of_t); g.t_of_i = bp<int32_t>(G.t_of_i);
+    if (f32) g.col32 = reinterpret_cast<const float2 *>(bp<const float4>(M->blk32) + 2 * M->m);
+    SGP_TRY(rows_count(ctx, R, g, M, (size_t)G.nr_max));
+    SGP_TRY(read_back(ctx, R.tot, g.rh + R_N * g.P, sizeof(R.tot)));
+    if (!rows_place(G, R, M, f32, true)) return SGP_OK;
+    SGP_TRY(rows_fill(ctx, G, R, g, M, f32));
+    return SGP_OK;
+}
+
+// A matrix cut into parts of consecutive rows, for the row-wise
+// preconditioners, in FP64 or (MIXED matrices) FP32; G.ok is 0 when the parts
+// do not fit.  `jac`: the block-Jacobi inverses (internal order), or NULL.
+sgp_status grid_plain(sgp_ctx *ctx, const sgp_matrix *M, bool f32, const double *jac, GridLayout &G)
+{
+    const int32_t n = (int32_t)M->n;
+    GridRows &R = G.rows;
+    G.ok = 0;
+    G.prec = f32 ? SGP_PREC_MIXED : SGP_PREC_F64;
+    // FP64 is bound by its issue rate: all SMs from 64 rows each on; FP32 from 128
+    int32_t P = 1;
+    SGP_TRY(part_count(ctx, n, f32 ? 128 : 64, &P));
+    const int32_t U = (n + P - 1) / P;
+    P = (n + U - 1) / U;
+    if ((size_t)U * (f32 ? 24 : 48) > (size_t)GRID_SMEM) return SGP_OK;
+    G.P = P;
+    G.nr_max = (int64_t)P * pad32(U) + 32;
+    GBuild g{};
+    g.n = n; g.P = P; g.identity = 1;
+    SGP_TRY(ensure(ctx, G.hdr, (size_t)Q_N * (P + 1), &g.hdr));
+    SGP_TRY(ensure(ctx, G.dtot, T_N, &g.tot));
+    SGP_TRY(ensure(ctx, G.i_of_t, (size_t)G.nr_max, &g.i_of_t));
+    SGP_TRY(ensure(ctx, G.t_of_i, n, &g.t_of_i));
+    if (f32) g.col32 = reinterpret_cast<const float2 *>(bp<const float4>(M->blk32) + 2 * M->m);
+    SGP_CUDA(ctx, cudaMemsetAsync(g.tot, 0, sizeof(int32_t) * T_N, ctx->stream));
+    LAUNCH(ctx, k_gr_rows_plain, 1, 256, 0, n, P, U, g.hdr, g.tot);
+    const unsigned gy = (unsigned)std::max(1, std::min(8, U / GT));
+    SGP_TRY(sgp_launch(ctx, "k_gr_row_maps", k_gr_row_maps, dim3(P, gy), dim3(GT), 0, g));
+    SGP_TRY(rows_count(ctx, R, g, M, (size_t)G.nr_max));
+    SGP_TRY(read_back(ctx, R.tot, g.rh + R_N * P, sizeof(R.tot)));
+    memset(G.tot, 0, sizeof(G.tot));
+    G.tot[T_NR] = P * pad32(U);
+    G.tot[T_MNR] = U;
+    if (!rows_place(G, R, M, f32, false)) return SGP_OK;
+    SGP_TRY(rows_fill(ctx, G, R, g, M, f32));
+    if (jac) {
+        const int32_t nr = G.tot[T_NR];
+        SGP_TRY(buf_ensure(ctx, G.D, (f32 ? 4 : 8) * 6 * (size_t)nr));
+        if (f32)
+            LAUNCH(ctx, k_gr_pivots<float>, grid_for(nr, SGP_BLOCK), SGP_BLOCK, 0, nr, bp<const int32_t>(G.i_of_t), jac,
+                   bp<float>(G.D));
+        else
+            LAUNCH(ctx, k_gr_pivots<double>, grid_for(nr, SGP_BLOCK), SGP_BLOCK, 0, nr, bp<const int32_t>(G.i_of_t), jac,
+                   bp<double>(G.D));
+    }
+    G.ok = 1;
+    return SGP_OK;
+}
+
+void grid_rows_release(GridRows &R)
+{
+    for (DBuf *d : {&R.rh, &R.glen, &R.gso, &R.perm, &R.xflag, &R.hl, &R.ma, &R.mb, &R.hb, &R.hpre})
+        if (d->p) cudaFree(d->p);
+}
 void grid_release(GridLayout &G)
 {
-    DBuf *b[] = {&G.hdr, &G.dtot, &G.ws, &G.glen, &G.gso, &G.perm, &G.xflag, &G.hl, &G.zi, &G.zslot, &G.tlk, &G.i_of_t,
-                 &G.t_of_i, &G.prog[0], &G.prog[1], &G.D, &G.inv, &G.tD, &G.ma, &G.mb};
-    for (DBuf *d : b)
+    for (DBuf *d : {&G.hdr, &G.dtot, &G.ws, &G.zi, &G.zslot, &G.tlk, &G.i_of_t, &G.t_of_i, &G.prog[0], &G.prog[1], &G.D,
+                    &G.inv, &G.tD})
         if (d->p) cudaFree(d->p);
     for (DBuf &d : G.scr)
         if (d.p) cudaFree(d.p);
+    grid_rows_release(G.rows);
 }
 
 // The grid solve serves this matrix and precision.
 template <typename T>
 bool grid_ready(const sgp_ctx *ctx, const sgp_factor *F, const sgp_matrix *M)
 {
-    return ctx->fused && F && M && F->gl.ok && F->gl.mgen == M->gen &&
+    return ctx->fused && F && M && F->gl.ok && F->gl.rows.mgen == M->gen &&
            F->gl.prec == (sizeof(T) == 4 ? SGP_PREC_MIXED : SGP_PREC_F64);
 }
 template bool grid_ready<float>(const sgp_ctx *, const sgp_factor *, const sgp_matrix *);
@@ -2437,14 +2554,18 @@ size_t grid_work_bytes(const GridLayout &G, size_t sz)
 }
 
 // One PCG run on Gamma x = F (vectors in the matrix's internal order) in one
-// launch; the final scalars go to *hs (a Scal).
+// launch: the parts and the forest of `G` (precond TREE), or parts of rows
+// (block Jacobi, none), the matrix's rows `R`; the final scalars go to *hs (a
+// Scal).
 template <typename T>
-sgp_status grid_pcg(sgp_ctx *ctx, const sgp_matrix *M, const GridLayout &G, const T *F, T *x, int x_given, double tol,
-                    int64_t maxit, void *work, void *hs, double mu, int stopE)
+sgp_status grid_pcg(sgp_ctx *ctx, const sgp_matrix *M, const GridLayout &G, const GridRows &R, int precond, const T *F, T *x,
+                    int x_given, double tol, int64_t maxit, void *work, void *hs, double mu, int stopE)
 {
     const int32_t *t = G.tot;
+    const bool tree = precond == SGP_PRECOND_TREE;
     GridArgs a{};
-    if (!place(G, sizeof(T), G.vb, true, G.halo != 0, &a.pl)) return sgp_fail(ctx, SGP_ERR_CUDA, "pcg: the grid layout does not fit");
+    if (!place(G, R.tot[2], sizeof(T), R.vb, tree, R.halo != 0, &a.pl))
+        return sgp_fail(ctx, SGP_ERR_CUDA, "pcg: the grid layout does not fit");
     char *at = reinterpret_cast<char *>(work);
     auto take = [&](size_t b) {
         char *p = at;
@@ -2461,20 +2582,20 @@ sgp_status grid_pcg(sgp_ctx *ctx, const sgp_matrix *M, const GridLayout &G, cons
     a.pk = reinterpret_cast<unsigned long long *>(take(2 * PMAX * 4 * 8));
     a.lx = reinterpret_cast<unsigned long long *>(take(wb * ((size_t)t[T_Z] + (size_t)t[T_NT])));
     Out *out = reinterpret_cast<Out *>(take(sizeof(Out)));
-    if (G.halo) a.px = reinterpret_cast<unsigned long long *>(take(wb * nr));
+    if (R.halo) a.px = reinterpret_cast<unsigned long long *>(take(wb * nr));
     char *zend = take(0);
-    if (!G.halo) a.pg = take(3 * sizeof(T) * nr);
+    if (!R.halo) a.pg = take(3 * sizeof(T) * nr);
     if (a.pl.o_r < 0) a.r = take(3 * sizeof(T) * nr);
     if (a.pl.o_x < 0) a.xt = take(3 * sizeof(T) * nr);
-    a.P = G.P; a.nt = t[T_NT]; a.x_given = x_given; a.timing = ctx->timing; a.halo = G.halo;
-    a.ntp = pad32(t[T_NT]); a.nslots = t[T_Z];
-    a.hdr = bp<const int32_t>(G.hdr); a.ws = bp<const int32_t>(G.ws);
-    a.glen = bp<const int32_t>(G.glen); a.gso = bp<const int32_t>(G.gso); a.i_of_t = bp<const int32_t>(G.i_of_t);
+    a.P = G.P; a.nt = tree ? t[T_NT] : 0; a.x_given = x_given; a.timing = ctx->timing; a.halo = R.halo;
+    a.ntp = pad32(a.nt); a.nslots = t[T_Z];
+    a.hdr = bp<const int32_t>(G.hdr); a.rh = bp<const int32_t>(R.rh); a.ws = bp<const int32_t>(G.ws);
+    a.glen = bp<const int32_t>(R.glen); a.gso = bp<const int32_t>(R.gso); a.i_of_t = bp<const int32_t>(G.i_of_t);
     a.zi = bp<const int32_t>(G.zi); a.zslot = bp<const int32_t>(G.zslot); a.tlk = bp<const int32_t>(G.tlk);
-    a.hl = bp<const int32_t>(G.hl);
-    a.perm = bp<const uint16_t>(G.perm); a.xflag = bp<const uint8_t>(G.xflag);
+    a.hl = bp<const int32_t>(R.hl);
+    a.perm = bp<const uint16_t>(R.perm); a.xflag = bp<const uint8_t>(R.xflag);
     for (int q = 0; q < 2; ++q) a.prog[q] = bp<const char>(G.prog[q]);
-    a.D = G.D.p; a.inv = G.inv.p; a.ma = G.ma.p; a.mb = G.mb.p;
+    a.D = a.jac = G.D.p; a.inv = G.inv.p; a.ma = R.ma.p; a.mb = R.mb.p;
     a.F = F; a.x = x;
     a.gamma0 = M->gamma0;
     a.tol2 = stopE ? -1.0 : tol * tol;
@@ -2493,10 +2614,18 @@ sgp_status grid_pcg(sgp_ctx *ctx, const sgp_matrix *M, const GridLayout &G, cons
                                                   ctx->stream));
         return SGP_OK;
     };
+    auto pick = [&](auto vb) -> sgp_status {
+        constexpr int VB = decltype(vb)::value;
+        if (precond == SGP_PRECOND_BLOCK_JACOBI) return go(k_pcg_grid<T, VB, 1>);
+        if (precond == SGP_PRECOND_NONE) return go(k_pcg_grid<T, VB, 2>);
+        return go(k_pcg_grid<T, VB, 0>);
+    };
     if constexpr (sizeof(T) == 8)
-        SGP_TRY(go(k_pcg_grid<T, 24, 0>));
+        SGP_TRY(pick(std::integral_constant<int, 24>{}));
+    else if (R.vb == 16)
+        SGP_TRY(pick(std::integral_constant<int, 16>{}));
     else
-        SGP_TRY(G.vb == 16 ? go(k_pcg_grid<T, 16, 0>) : go(k_pcg_grid<T, 12, 0>));
+        SGP_TRY(pick(std::integral_constant<int, 12>{}));
     ctx->launches++;
     Out h;
     SGP_TRY(read_back(ctx, &h, out, sizeof(h)));
@@ -2508,13 +2637,18 @@ sgp_status grid_pcg(sgp_ctx *ctx, const sgp_matrix *M, const GridLayout &G, cons
     if (ctx->timing) {
         const int cls[3] = {SGP_KT_SPMV, SGP_KT_TREE_SOLVE, SGP_KT_PCG_VECTOR};
         for (int k = 0; k < 3; ++k) {
+            if (!tree && k == 1) {   // no tree solve: the vector work
+                ctx->kt_ms[SGP_KT_PCG_VECTOR] += 1e-6 * (double)h.ns[1];
+                continue;
+            }
             ctx->kt_ms[cls[k]] += 1e-6 * (double)h.ns[k];
             ctx->kt_n[cls[k]] += h.sc.it + (k == 1);
         }
     }
     return SGP_OK;
 }
-template sgp_status grid_pcg<float>(sgp_ctx *, const sgp_matrix *, const GridLayout &, const float *, float *, int, double,
-                                    int64_t, void *, void *, double, int);
-template sgp_status grid_pcg<double>(sgp_ctx *, const sgp_matrix *, const GridLayout &, const double *, double *, int,
-                                     double, int64_t, void *, void *, double, int);
+#define GRID_PCG(T)                                                                                                      \
+    template sgp_status grid_pcg<T>(sgp_ctx *, const sgp_matrix *, const GridLayout &, const GridRows &, int, const T *, \
+                                    T *, int, double, int64_t, void *, void *, double, int);
+GRID_PCG(float)
+GRID_PCG(double)

@@ -1134,6 +1134,15 @@ sgp_status pcg_core(sgp_ctx *ctx, const sgp_matrix *M, const sgp_factor *Fac, in
     return SGP_OK;
 }
 
+// The layout of the persistent solve that serves this run, or NULL.
+template <typename T>
+const GridLayout *grid_of(const sgp_ctx *ctx, const sgp_matrix *M, const sgp_factor *Fac, int precond)
+{
+    if (precond == SGP_PRECOND_TREE) return grid_ready<T>(ctx, Fac, M) ? &Fac->gl : nullptr;
+    const GridLayout &G = ctx->grid_plain;   // written for this call
+    return ctx->fused && ctx->bin_cap == 0 && G.ok ? &G : nullptr;
+}
+
 // One PCG run on Gamma x = F in the matrix's internal order.  With the
 // tree preconditioner and a binned factor built from this assembly, the run
 // takes F (and x) to the factor's tree order, solves there with the fused
@@ -1144,8 +1153,9 @@ sgp_status pcg_run(sgp_ctx *ctx, const sgp_matrix *M, const sgp_factor *Fac, int
                    double *partials, Scal *sc, void *gwork, Scal *hs, double mu = 0.0, int stopE = 0)
 {
     static_assert(sizeof(X) == sizeof(T), "iterate and vectors share one precision");
-    if (precond == SGP_PRECOND_TREE && grid_ready<T>(ctx, Fac, M))
-        return grid_pcg<T>(ctx, M, Fac->gl, F, reinterpret_cast<T *>(x), x_given, tol, maxit, gwork, hs, mu, stopE);
+    if (const GridLayout *G = grid_of<T>(ctx, M, Fac, precond))
+        return grid_pcg<T>(ctx, M, *G, G->rows, precond, F, reinterpret_cast<T *>(x), x_given, tol, maxit, gwork, hs, mu,
+                           stopE);
     const bool tree = precond == SGP_PRECOND_TREE && ctx->fused && Ft && xt && bins_tree_ready<T>(Fac, M);
     if (!tree)
         return pcg_core<T, X>(ctx, M, Fac, precond, make_blk<T>(M), bp<const int32_t>(M->row_ptr), M->n, false, F,
@@ -1316,7 +1326,18 @@ sgp_status sgp_pcg_solve(sgp_ctx *ctx, const sgp_matrix *M, const sgp_factor *Fa
     const int64_t nv = (opts->precond == SGP_PRECOND_TREE && Fac && Fac->bl.NT > n) ? Fac->bl.NT : n;
     const size_t v64 = sizeof(double) * 3 * nv, v32 = sizeof(float) * 3 * nv;
     size_t need = 8 * v64 + (mixed ? 8 * v32 : 0) + sizeof(double) * 2 * MAXP + 2 * sizeof(Scal) + 8192;
-    const size_t gw = opts->precond == SGP_PRECOND_TREE ? grid_work_bytes(Fac->gl, mixed ? 4 : 8) : 0;
+    // the persistent solve's layout: the factor's, or (row-wise
+    // preconditioners) parts of the matrix's rows
+    if (opts->precond != SGP_PRECOND_TREE && ctx->fused && ctx->bin_cap == 0) {
+        const double *jac = nullptr;
+        if (opts->precond == SGP_PRECOND_BLOCK_JACOBI) {
+            SGP_TRY(matrix_block_jacobi(ctx, const_cast<sgp_matrix *>(M)));
+            jac = bp<const double>(M->jac);
+        }
+        SGP_TRY(grid_plain(ctx, M, mixed, jac, ctx->grid_plain));
+    }
+    const GridLayout *G0 = mixed ? grid_of<float>(ctx, M, Fac, opts->precond) : grid_of<double>(ctx, M, Fac, opts->precond);
+    const size_t gw = G0 ? grid_work_bytes(*G0, mixed ? 4 : 8) : 0;
     SGP_TRY(scratch_ensure(ctx, need + gw + 4096));
     char *base = reinterpret_cast<char *>(ctx->d_scratch) + 256;
     auto take = [&](size_t b) {
@@ -1479,7 +1500,14 @@ sgp_status sgp_fcg_solve(sgp_ctx *ctx, const sgp_matrix *M, const sgp_aug *A, co
     }
     const double itol = opts->inner_tol > 0.0 ? opts->inner_tol : 0.1;
     const size_t v64 = sizeof(double) * 3 * n;
-    SGP_TRY(scratch_ensure(ctx, 10 * (v64 + 256) + sizeof(double) * 2 * MAXP + 4 * sizeof(Scal) + 8192));
+    // the inner solves: P' on the parts of the factor's persistent solve
+    bool grid = ctx->fused && Fac->gl.ok && Fac->gl.prec == SGP_PREC_F64;
+    if (grid) {
+        SGP_TRY(grid_rows(ctx, Fac, A->P, ctx->grid_rows));
+        grid = ctx->grid_rows.ok != 0;
+    }
+    const size_t gw = grid ? grid_work_bytes(Fac->gl, 8) : 0;
+    SGP_TRY(scratch_ensure(ctx, 10 * (v64 + 256) + sizeof(double) * 2 * MAXP + 4 * sizeof(Scal) + 8192 + gw + 256));
     char *base = reinterpret_cast<char *>(ctx->d_scratch) + 256;
     auto take = [&](size_t b) {
         char *p = base;
@@ -1490,6 +1518,7 @@ sgp_status sgp_fcg_solve(sgp_ctx *ctx, const sgp_matrix *M, const sgp_aug *A, co
     Scal *sco = reinterpret_cast<Scal *>(take(sizeof(Scal)));
     Scal *sci = reinterpret_cast<Scal *>(take(sizeof(Scal)));
     double *o2 = reinterpret_cast<double *>(take(64));
+    char *gwork = take(gw);
     double *r = reinterpret_cast<double *>(take(v64)), *p = reinterpret_cast<double *>(take(v64)),
            *q = reinterpret_cast<double *>(take(v64)), *z = reinterpret_cast<double *>(take(v64)),
            *Fi = reinterpret_cast<double *>(take(v64)), *x = reinterpret_cast<double *>(take(v64)),
@@ -1530,9 +1559,13 @@ sgp_status sgp_fcg_solve(sgp_ctx *ctx, const sgp_matrix *M, const sgp_aug *A, co
     for (int64_t k = 0; !h.done; ++k) {
         // z ~ P'^-1 r: PCG on P' with the forest factor, from z = 0
         Scal hi{};
-        SGP_TRY((pcg_core<double, double>(ctx, P, Fac, SGP_PRECOND_TREE, make_blk<double>(P),
-                                          bp<const int32_t>(P->row_ptr), n, false, (const double *)r, z, 0, itol,
-                                          inner_maxit, ri, pi, qi, wi, partials, sci, &hi)));
+        if (grid)
+            SGP_TRY(grid_pcg<double>(ctx, P, Fac->gl, ctx->grid_rows, SGP_PRECOND_TREE, r, z, 0, itol, inner_maxit, gwork, &hi, 0.0,
+                                     0));
+        else
+            SGP_TRY((pcg_core<double, double>(ctx, P, Fac, SGP_PRECOND_TREE, make_blk<double>(P),
+                                              bp<const int32_t>(P->row_ptr), n, false, (const double *)r, z, 0, itol,
+                                              inner_maxit, ri, pi, qi, wi, partials, sci, &hi)));
         inner += hi.it;
         if (hi.status == SGP_ERR_NOT_SPD || hi.status == SGP_ERR_TIMEOUT) {
             h.status = hi.status;

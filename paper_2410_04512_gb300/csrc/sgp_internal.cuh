@@ -37,6 +37,33 @@ struct GraphEntry {
     uint64_t last_use = 0;
 };
 
+// Stream-ordered device buffer owned by a handle.
+struct DBuf {
+    void *p = nullptr;
+    size_t bytes = 0;
+};
+
+// The rows of one matrix (generation mgen) on the parts of a grid layout; tot: slots / 32, halo cells, the largest halo.
+struct GridRows {
+    int ok = 0, halo = 0, vb = 16;   // vb: bytes per cell of the on-chip vectors
+    uint64_t mgen = 0;
+    int32_t tot[4] = {0};
+    DBuf rh, glen, gso, perm, xflag, hl, ma, mb, hb, hpre;
+};
+// The grid solve's layout (grid.cu): one part per thread block, and for the
+// forest the parts' programs and the top, in one precision.
+#define SGP_GRID_SCRATCH 48
+struct GridLayout {
+    int ok = 0, prec = 0;
+    int64_t nr_max = 0;
+    int32_t P = 0, LV = 0;
+    int32_t tot[24] = {0}, top_slots[2] = {0, 0};   // totals and maxima over the parts; slots of the top's programs
+    DBuf hdr, dtot, ws, zi, zslot, tlk, i_of_t, t_of_i;
+    DBuf prog[2], D, inv, tD;
+    DBuf scr[SGP_GRID_SCRATCH];
+    GridRows rows;                                  // of the matrix the layout was built from
+};
+
 struct sgp_ctx {
     int device = 0;
     cudaStream_t stream = nullptr;
@@ -80,6 +107,11 @@ struct sgp_ctx {
     std::vector<KtRec> *capture_sink = nullptr;
     std::vector<GraphEntry *> graphs;
     uint64_t graph_clock = 0;
+    // persistent solves whose layout belongs to one call, written anew by each:
+    // the parts of rows of the row-wise preconditioners, and P' of a flexible
+    // solve on its factor's parts
+    GridLayout grid_plain;
+    GridRows grid_rows;
 };
 
 // Grid of at most one full wave: min(want, SMs x resident blocks per SM of
@@ -167,11 +199,6 @@ static inline unsigned grid_for(int64_t n, int block)
     return (unsigned)(g < 1 ? 0 : g);
 }
 
-// Stream-ordered device buffer owned by a handle.
-struct DBuf {
-    void *p = nullptr;
-    size_t bytes = 0;
-};
 sgp_status buf_ensure(sgp_ctx *ctx, DBuf &b, size_t bytes);
 void buf_release(DBuf &b, cudaStream_t s);
 template <typename T>
@@ -225,17 +252,23 @@ bool small_solve_fits(const sgp_ctx *ctx, const sgp_factor *F);
 
 // The grid solve (grid.cu): a whole PCG run in one persistent launch.
 // grid_build runs at the end of a factor build; grid_ready tells whether it
-// serves precision T of this matrix; grid_pcg runs it on internal-order
-// vectors with `work` (grid_work_bytes) and returns the final scalars.
-sgp_status grid_build(sgp_ctx *ctx, sgp_factor *F, const sgp_matrix *M);
+// serves precision T of this matrix; grid_rows puts another matrix on a
+// factor's parts, grid_plain cuts a matrix into parts of rows; grid_pcg runs
+// it on internal-order vectors with `work` (grid_work_bytes) and returns the
+// final scalars.
 struct GridLayout;
+struct GridRows;
+sgp_status grid_build(sgp_ctx *ctx, sgp_factor *F, const sgp_matrix *M);
+sgp_status grid_rows(sgp_ctx *ctx, const sgp_factor *F, const sgp_matrix *M, GridRows &R);
+sgp_status grid_plain(sgp_ctx *ctx, const sgp_matrix *M, bool f32, const double *jac, GridLayout &G);
 void grid_release(GridLayout &G);
+void grid_rows_release(GridRows &R);
 template <typename T>
 bool grid_ready(const sgp_ctx *ctx, const sgp_factor *F, const sgp_matrix *M);
 size_t grid_work_bytes(const GridLayout &G, size_t sz);
 template <typename T>
-sgp_status grid_pcg(sgp_ctx *ctx, const sgp_matrix *M, const GridLayout &G, const T *F, T *x, int x_given, double tol,
-                    int64_t maxit, void *work, void *hs, double mu, int stopE);
+sgp_status grid_pcg(sgp_ctx *ctx, const sgp_matrix *M, const GridLayout &G, const GridRows &R, int precond, const T *F, T *x,
+                    int x_given, double tol, int64_t maxit, void *work, void *hs, double mu, int stopE);
 
 // Kernel timing hooks (no-ops unless enabled on the context).
 sgp_status kt_begin(sgp_ctx *ctx, int kclass, cudaEvent_t *ev);
@@ -317,19 +350,6 @@ struct BinLayout {
     uint64_t mgen = 0;
     int mat32 = 0, mat64 = 0;
     DBuf scr[SGP_BIN_SCRATCH];
-};
-
-// The grid solve's layout (grid.cu): one part per thread block and the top,
-// in the factor's own precision, with the matrix's rows of generation mgen.
-#define SGP_GRID_SCRATCH 48
-struct GridLayout {
-    int ok = 0, prec = 0, halo = 0, vb = 16;   // vb: bytes per cell of the on-chip vectors
-    uint64_t mgen = 0;
-    int32_t P = 0, LV = 0;
-    int32_t tot[24] = {0}, top_slots[2] = {0, 0};   // totals and maxima over the parts; slots of the top's programs
-    DBuf hdr, dtot, ws, glen, gso, perm, xflag, hl, zi, zslot, tlk, i_of_t, t_of_i;
-    DBuf prog[2], D, inv, tD, ma, mb;
-    DBuf scr[SGP_GRID_SCRATCH];
 };
 
 struct sgp_factor {

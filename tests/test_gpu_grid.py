@@ -70,6 +70,25 @@ def test_grid_solve_matches_level_kernels(cuda_device, name, precision):
     assert torch.equal(again, v)
 
 
+@pytest.mark.parametrize("precision", [sgp.PREC_F64, sgp.PREC_MIXED])
+@pytest.mark.parametrize("precond", [sgp.PRECOND_BLOCK_JACOBI, sgp.PRECOND_NONE])
+@pytest.mark.parametrize("name", ["one", "pair", "hub", "forest", "sheet", "cube129", "ball"])
+def test_grid_rows_match_multi_launch(cuda_device, name, precond, precision):
+    """The row-wise preconditioners on parts of rows; bound as above."""
+    c = _cells(name)
+    F = dev_tensor(c.forces())
+    out = []
+    for cap in (0, -1):
+        cx = sgp.Context(0)
+        cx.set_tuning(bin_cap=cap)
+        s = GpuSystem(cx, c, precision=precision)
+        v, info = cx.pcg_solve(s.M, None, F, tol=1e-10, precond=precond, precision=precision)
+        assert info.status == 0 and info.true_rel_residual <= 1.05e-10
+        out.append((v.cpu().numpy(), info))
+    assert abs(out[0][1].iterations - out[1][1].iterations) <= max(3, out[1][1].iterations // 20)
+    assert rel_err(out[0][0], out[1][0]) <= 1e-8
+
+
 def test_grid_iterates_at_equal_k(cuda_device):
     """FP64 iterates after k = 1, 5, 30 steps agree with the oracle's PCG to
     1e-9, from zero and from a given start (whose product the launch forms)."""
