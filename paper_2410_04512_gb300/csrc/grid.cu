@@ -274,7 +274,7 @@ __global__ void __launch_bounds__(256) k_gr_rows_plain(int32_t n, int32_t P, int
     h[Q_NV] = h[Q_NR] = nr;
     h[Q_ROFF] = b * pad32(U);
     if (b == P) {
-        tot[T_NR] = P * pad32(U);
+        tot[T_NR] = (P - 1) * pad32(U) + pad32(n - (P - 1) * U);
         tot[T_MNR] = U;
     }
 }
@@ -2501,7 +2501,7 @@ sgp_status grid_plain(sgp_ctx *ctx, const sgp_matrix *M, bool f32, const double 
     SGP_TRY(rows_count(ctx, R, g, M, (size_t)G.nr_max));
     SGP_TRY(read_back(ctx, R.tot, g.rh + R_N * P, sizeof(R.tot)));
     memset(G.tot, 0, sizeof(G.tot));
-    G.tot[T_NR] = P * pad32(U);
+    G.tot[T_NR] = (P - 1) * pad32(U) + pad32(n - (P - 1) * U);   // the rows that k_gr_row_maps writes
     G.tot[T_MNR] = U;
     if (!rows_place(G, R, M, f32, false)) return SGP_OK;
     SGP_TRY(rows_fill(ctx, G, R, g, M, f32));
