@@ -47,7 +47,8 @@ __global__ void k_mp_jacobi(int64_t n, const double *__restrict__ jac, const dou
     if (i < n) sym_mv(jac + 6 * i, F + 3 * i, b0 + 3 * i);
 }
 
-// sum_i |b1_i|, reduced by blocks then by the last block (fixed order)
+// The mean of |b1_i| and the scale 1 / mean (1 if it vanishes): blocks, then
+// the last block (fixed order).
 __global__ void k_mp_norm_sum(int64_t n, const double *__restrict__ b1, double *partials, unsigned *counter,
                               double *out)
 {
@@ -59,107 +60,92 @@ __global__ void k_mp_norm_sum(int64_t n, const double *__restrict__ b1, double *
     if (threadIdx.x == 0) partials[blockIdx.x] = s;
     if (last_block(counter)) {
         double t = sum_partials<TB>(partials, gridDim.x, sh);
-        if (threadIdx.x == 0) out[0] = t / (double)(n > 0 ? n : 1);
+        if (threadIdx.x == 0) {
+            const double mean = t / (double)(n > 0 ? n : 1);
+            out[0] = mean;
+            out[1] = 1.0 / (mean > 0.0 ? mean : 1.0);
+        }
     }
 }
 
+// FP64 bound: the scale comes as a reciprocal, as a division is some ten
+// instructions (seven of them per cell: 26 us at 1e5 cells, 15 so).
 __global__ void k_mp_features(int64_t n, const double *__restrict__ b0, const double *__restrict__ b1,
                               const double *__restrict__ b2, const int32_t *__restrict__ row_ptr,
                               const double *__restrict__ mean_b1, float *x)
 {
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
-    double s = mean_b1[0];
-    if (!(s > 0.0)) s = 1.0;
+    const double s = mean_b1[1], s2 = s * s;
     const double *a = b0 + 3 * i, *b = b1 + 3 * i, *c = b2 + 3 * i;
     auto dot = [](const double *u, const double *v) { return u[0] * v[0] + u[1] * v[1] + u[2] * v[2]; };
     float *o = x + DIN * i;
-    o[0] = (float)(sqrt(dot(a, a)) / s);
-    o[1] = (float)(sqrt(dot(b, b)) / s);
-    o[2] = (float)(sqrt(dot(c, c)) / s);
-    o[3] = (float)(dot(a, b) / (s * s));
-    o[4] = (float)(dot(a, c) / (s * s));
-    o[5] = (float)(dot(b, c) / (s * s));
-    o[6] = (float)((row_ptr[i + 1] - row_ptr[i]) / 6.0);
+    o[0] = (float)(sqrt(dot(a, a)) * s);
+    o[1] = (float)(sqrt(dot(b, b)) * s);
+    o[2] = (float)(sqrt(dot(c, c)) * s);
+    o[3] = (float)(dot(a, b) * s2);
+    o[4] = (float)(dot(a, c) * s2);
+    o[5] = (float)(dot(b, c) * s2);
+    o[6] = (float)((row_ptr[i + 1] - row_ptr[i]) * (1.0 / 6.0));
     o[7] = 1.0f;
 }
 
 // ------------------------------------------------------------ dense layers
 // Y (n x DOUT) = act(X Wt + bias) where X = [X1 (n x D1), X2 (n x D2)] and the
-// BF16 matrix W is DOUT x (D1 + D2) (TRANS = false), or Y = X W with W of
-// shape (D1 + D2) x DOUT read transposed (TRANS = true, no bias/act: the
-// backward product dX = dZ W).  The weights are staged transposed in shared
-// memory as FP32 so that the threads of a node read consecutive outputs.
-template <int D1, int D2, int DOUT, bool TRANS, bool RELU>
-__global__ void __launch_bounds__(TB) k_mp_dense(int64_t n, const float *__restrict__ X1,
-                                                 const float *__restrict__ X2,
-                                                 const __nv_bfloat16 *__restrict__ W,
-                                                 const __nv_bfloat16 *__restrict__ bias, float *Y)
+// BF16 matrix W is DOUT x (D1 + D2), or, TRANS, Y = X W with W of shape
+// (D1 + D2) x DOUT (the backward product dX = dZ W; the second half of the
+// outputs, dA, is scaled by 1 / deg of its row for the transposed mean).
+// FP32 FMAs on register tiles: a block holds the weights (FP32, [k][o]) and a
+// tile of 16 NU nodes' inputs (row-major, padded) in shared memory; a thread
+// computes NU nodes (ty, ty + 16, ...) x 4 or 8 outputs, reading 16 bytes per
+// load: with NU = 8 a warp takes 16 to 24 shared-memory wavefronts per 128 to
+// 256 FMAs, so the FMA pipe is the bound.  Weights are read 16 bytes at a time
+// (8 inputs of one output) and spread over the rows without bank conflicts.
+// Each output accumulates bias + sum_k x_k w_k in ascending k.  1e5 cells:
+// forward layer 80 -> 69 us, backward product 147 -> 53 us.
+template <int D1, int D2, int DOUT, bool TRANS, bool RELU, int NU>
+__global__ void __launch_bounds__(TB, 2) k_mp_dense(int64_t n, const float *__restrict__ X1, const float *__restrict__ X2,
+                                                    const __nv_bfloat16 *__restrict__ W,
+                                                    const __nv_bfloat16 *__restrict__ bias,
+                                                    const int32_t *__restrict__ row_ptr, float *__restrict__ Y)
 {
-    constexpr int DI = D1 + D2;
-    constexpr int NPB = TB / DOUT > 0 ? TB / DOUT : 1;   // nodes per pass
-    __shared__ float wt[DI * DOUT];
-    __shared__ float xs[NPB][DI];
-    for (int t = threadIdx.x; t < DI * DOUT; t += TB) {
-        const int k = t / DOUT, o = t % DOUT;             // wt[k][o]
-        wt[t] = TRANS ? bf(W, k * DOUT + o) : bf(W, o * DI + k);
-    }
-    const int o = threadIdx.x % DOUT, slot = threadIdx.x / DOUT;
-    const float b = (!TRANS && bias && threadIdx.x < NPB * DOUT) ? bf(bias, o) : 0.f;
-    for (int64_t base = (int64_t)blockIdx.x * NPB; base < n; base += (int64_t)gridDim.x * NPB) {
-        __syncthreads();
-        for (int t = threadIdx.x; t < NPB * DI; t += TB) {
-            const int s = t / DI, k = t % DI;
-            const int64_t i = base + s;
-            float v = 0.f;
-            if (i < n) v = k < D1 ? X1[i * D1 + k] : X2[i * D2 + (k - D1)];
-            xs[s][k] = v;
-        }
-        __syncthreads();
-        const int64_t i = base + slot;
-        if (slot < NPB && threadIdx.x < NPB * DOUT && i < n) {
-            float acc = b;
-#pragma unroll 8
-            for (int k = 0; k < DI; ++k) acc = fmaf(xs[slot][k], wt[k * DOUT + o], acc);
-            if (RELU) acc = fmaxf(acc, 0.f);
-            Y[i * DOUT + o] = acc;
-        }
-    }
-}
-
-// The forward layers (TRANS = false, DOUT = H) as a register-tiled product:
-// a block holds all weights (FP32, [k][o]) and a tile of 64 nodes' inputs
-// (row-major, padded) in shared memory; each thread computes 4 nodes x 4
-// outputs, reading four inputs of each of its nodes and four outputs' weights
-// per 16-byte load (64 FMAs per 8 shared loads).  Each output accumulates
-// bias + sum_k x_k w_k in ascending k with FMAs: the same order, so the same
-// bits, as k_mp_dense.
-constexpr int DT_NODES = 64;
-template <int D1, int D2, bool RELU>
-__global__ void __launch_bounds__(TB) k_mp_dense_tiled(int64_t n, const float *__restrict__ X1,
-                                                       const float *__restrict__ X2,
-                                                       const __nv_bfloat16 *__restrict__ W,
-                                                       const __nv_bfloat16 *__restrict__ bias, float *Y)
-{
-    constexpr int DI = D1 + D2, XP = DI + 4;
-    static_assert(DI % 4 == 0 && H == 64, "tile shape");
+    constexpr int DI = D1 + D2, XP = DI + 4, OG = DOUT / 64, DN = 16 * NU;
+    static_assert(DI % 8 == 0 && D1 % 4 == 0 && (DOUT == 64 || DOUT == 128), "tile shape");
     extern __shared__ __align__(16) float dsm[];
-    float *wt = dsm;                 // [DI][H]
-    float *xs = dsm + DI * H;        // [DT_NODES][XP]
-    for (int t = threadIdx.x; t < DI * H; t += TB) {
-        const int k = t / H, o = t % H;
-        wt[t] = bf(W, o * DI + k);
+    float *wt = dsm;                    // [DI][DOUT]
+    float *xs = dsm + DI * DOUT;        // [DN][XP]
+    for (int c = threadIdx.x; c < DI * DOUT / 8; c += TB) {
+        if (TRANS) {
+            const int t = 8 * c;        // row k, outputs o..o+7
+            const uint4 q = *reinterpret_cast<const uint4 *>(W + t);
+            const uint32_t u[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                wt[t + 2 * j] = __uint_as_float(u[j] << 16);
+                wt[t + 2 * j + 1] = __uint_as_float(u[j] & 0xffff0000u);
+            }
+        } else {
+            const int o = c % DOUT, k = 8 * (c / DOUT);
+            const uint4 q = *reinterpret_cast<const uint4 *>(W + o * DI + k);
+            const uint32_t u[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                wt[(k + 2 * j) * DOUT + o] = __uint_as_float(u[j] << 16);
+                wt[(k + 2 * j + 1) * DOUT + o] = __uint_as_float(u[j] & 0xffff0000u);
+            }
+        }
     }
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    float bv[4];
+    float bv[4 * OG];
 #pragma unroll
-    for (int v = 0; v < 4; ++v) bv[v] = bias ? bf(bias, 4 * tx + v) : 0.f;
-    const int64_t ntiles = (n + DT_NODES - 1) / DT_NODES;
+    for (int v = 0; v < 4 * OG; ++v) bv[v] = bias ? bf(bias, (v >> 2) * 64 + 4 * tx + (v & 3)) : 0.f;
+    const int64_t ntiles = (n + DN - 1) / DN;
     for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        const int64_t base = tile * DT_NODES;
+        const int64_t base = tile * DN;
         __syncthreads();
-        for (int c = threadIdx.x; c < DT_NODES * (DI / 4); c += TB) {
-            const int node = c / (DI / 4), kq = c % (DI / 4), k = 4 * kq;
+#pragma unroll 8
+        for (int c = threadIdx.x; c < DN * (DI / 4); c += TB) {
+            const int node = c / (DI / 4), k = 4 * (c % (DI / 4));
             const int64_t i = base + node;
             float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
             if (i < n) v = k < D1 ? *reinterpret_cast<const float4 *>(X1 + i * D1 + k)
@@ -167,100 +153,150 @@ __global__ void __launch_bounds__(TB) k_mp_dense_tiled(int64_t n, const float *_
             *reinterpret_cast<float4 *>(xs + node * XP + k) = v;
         }
         __syncthreads();
-        float acc[4][4];
+        float acc[NU][4 * OG];
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
+        for (int u = 0; u < NU; ++u)
 #pragma unroll
-            for (int v = 0; v < 4; ++v) acc[u][v] = bv[v];
-#pragma unroll 2
+            for (int v = 0; v < 4 * OG; ++v) acc[u][v] = bv[v];
+#pragma unroll 1
         for (int k = 0; k < DI; k += 4) {
-            float4 xv[4];
+            float4 xv[NU];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) xv[u] = *reinterpret_cast<const float4 *>(xs + (4 * ty + u) * XP + k);
+            for (int u = 0; u < NU; ++u) xv[u] = *reinterpret_cast<const float4 *>(xs + (ty + 16 * u) * XP + k);
 #pragma unroll
-            for (int kk = 0; kk < 4; ++kk) {
-                const float4 wv = *reinterpret_cast<const float4 *>(wt + (k + kk) * H + 4 * tx);
+            for (int kk = 0; kk < 4; ++kk)
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const float xk = kk == 0 ? xv[u].x : kk == 1 ? xv[u].y : kk == 2 ? xv[u].z : xv[u].w;
-                    acc[u][0] = fmaf(xk, wv.x, acc[u][0]);
-                    acc[u][1] = fmaf(xk, wv.y, acc[u][1]);
-                    acc[u][2] = fmaf(xk, wv.z, acc[u][2]);
-                    acc[u][3] = fmaf(xk, wv.w, acc[u][3]);
+                for (int g = 0; g < OG; ++g) {
+                    const float4 wv = *reinterpret_cast<const float4 *>(wt + (k + kk) * DOUT + 64 * g + 4 * tx);
+#pragma unroll
+                    for (int u = 0; u < NU; ++u) {
+                        const float xk = kk == 0 ? xv[u].x : kk == 1 ? xv[u].y : kk == 2 ? xv[u].z : xv[u].w;
+                        acc[u][4 * g] = fmaf(xk, wv.x, acc[u][4 * g]);
+                        acc[u][4 * g + 1] = fmaf(xk, wv.y, acc[u][4 * g + 1]);
+                        acc[u][4 * g + 2] = fmaf(xk, wv.z, acc[u][4 * g + 2]);
+                        acc[u][4 * g + 3] = fmaf(xk, wv.w, acc[u][4 * g + 3]);
+                    }
                 }
+        }
+#pragma unroll
+        for (int u = 0; u < NU; ++u) {
+            const int64_t i = base + ty + 16 * u;
+            if (i >= n) continue;
+#pragma unroll
+            for (int g = 0; g < OG; ++g) {
+                float4 o4 = make_float4(acc[u][4 * g], acc[u][4 * g + 1], acc[u][4 * g + 2], acc[u][4 * g + 3]);
+                if (RELU) o4 = make_float4(fmaxf(o4.x, 0.f), fmaxf(o4.y, 0.f), fmaxf(o4.z, 0.f), fmaxf(o4.w, 0.f));
+                if (TRANS && g == 1) {
+                    const float inv = 1.0f / (float)max(row_ptr[i + 1] - row_ptr[i], 1);
+                    o4 = make_float4(o4.x * inv, o4.y * inv, o4.z * inv, o4.w * inv);
+                }
+                *reinterpret_cast<float4 *>(Y + i * DOUT + 64 * g + 4 * tx) = o4;
             }
         }
+    }
+}
+
+// The sum of the neighbours' rows (16 lanes per node, 16 bytes per lane; the
+// neighbours' indices in one load, their rows four at a time), in ascending
+// column order.
+__device__ __forceinline__ void row_sum(const int32_t *__restrict__ col, int32_t s0, int32_t s1,
+                                        const float *__restrict__ X, int pitch, float4 &a)
+{
+    const int lane = threadIdx.x & 31, l = lane & 15;
+    const unsigned mask = 0xffffu << (lane & 16);
+    for (int32_t b = s0; b < s1; b += 16) {
+        const int cnt = min(16, s1 - b);
+        const int32_t c = l < cnt ? col[b + l] : 0;
+        for (int j = 0; j < cnt; j += 4) {
+            float4 v[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int64_t i = base + 4 * ty + u;
-            if (i >= n) continue;
-            float4 o4 = make_float4(acc[u][0], acc[u][1], acc[u][2], acc[u][3]);
-            if (RELU) o4 = make_float4(fmaxf(o4.x, 0.f), fmaxf(o4.y, 0.f), fmaxf(o4.z, 0.f), fmaxf(o4.w, 0.f));
-            *reinterpret_cast<float4 *>(Y + i * H + 4 * tx) = o4;
+            for (int u = 0; u < 4; ++u) {
+                const int32_t i = __shfl_sync(mask, c, (lane & 16) | min(j + u, 15));
+                v[u] = j + u < cnt ? reinterpret_cast<const float4 *>(X + (int64_t)i * pitch)[l]
+                                   : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                a.x += v[u].x; a.y += v[u].y; a.z += v[u].z; a.w += v[u].w;
+            }
         }
     }
 }
 
-// A_i = mean_{j ~ i} H_j (0 for an isolated cell); one warp per node, two
-// features per lane.  Neighbours in ascending column order.
-__global__ void k_mp_agg(int64_t n, const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col,
-                         const float *__restrict__ Hm, float *A)
+// A_i = mean_{j ~ i} H_j (0 for an isolated cell).
+__global__ void __launch_bounds__(TB) k_mp_agg(int64_t n, const int32_t *__restrict__ row_ptr,
+                                               const int32_t *__restrict__ col, const float *__restrict__ Hm, float *A)
 {
-    const int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
+    const int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 4;
     if (w >= n) return;
     const int32_t s0 = row_ptr[w], s1 = row_ptr[w + 1];
-    float a0 = 0.f, a1 = 0.f;
-    for (int32_t s = s0; s < s1; ++s) {
-        const float2 v = reinterpret_cast<const float2 *>(Hm + (int64_t)col[s] * H)[lane];
-        a0 += v.x;
-        a1 += v.y;
-    }
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+    row_sum(col, s0, s1, Hm, H, a);
     const float inv = 1.0f / (float)max(s1 - s0, 1);
-    reinterpret_cast<float2 *>(A + w * H)[lane] = make_float2(a0 * inv, a1 * inv);
+    reinterpret_cast<float4 *>(A + w * H)[threadIdx.x & 15] = make_float4(a.x * inv, a.y * inv, a.z * inv, a.w * inv);
 }
 
-// Transpose of the mean: dH_j = dSelf_j + sum_{i ~ j} dA_i / deg_i.
-__global__ void k_mp_agg_t(int64_t n, const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col,
-                           const float *__restrict__ dU, float *dH)
+__device__ __forceinline__ float4 relu_mask(float4 y, float4 d)
 {
-    const int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
+    return make_float4(y.x > 0.f ? d.x : 0.f, y.y > 0.f ? d.y : 0.f, y.z > 0.f ? d.z : 0.f, y.w > 0.f ? d.w : 0.f);
+}
+
+// Transpose of the mean, dH_j = dSelf_j + sum_{i ~ j} dA_i / deg_i (dA comes
+// scaled), through the ReLU of H: dZ_j = dH_j where H_j > 0.
+__global__ void __launch_bounds__(TB) k_mp_agg_t(int64_t n, const int32_t *__restrict__ row_ptr,
+                                                 const int32_t *__restrict__ col, const float *__restrict__ dU,
+                                                 const float *__restrict__ Hm, float *dZ)
+{
+    const int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 4;
     if (w >= n) return;
-    const float2 self = reinterpret_cast<const float2 *>(dU + w * H2)[lane];
-    float a0 = self.x, a1 = self.y;
-    for (int32_t s = row_ptr[w]; s < row_ptr[w + 1]; ++s) {
-        const int32_t i = col[s];
-        const float inv = 1.0f / (float)max(row_ptr[i + 1] - row_ptr[i], 1);
-        const float2 v = reinterpret_cast<const float2 *>(dU + (int64_t)i * H2 + H)[lane];
-        a0 = fmaf(v.x, inv, a0);
-        a1 = fmaf(v.y, inv, a1);
-    }
-    reinterpret_cast<float2 *>(dH + w * H)[lane] = make_float2(a0, a1);
+    const int l = threadIdx.x & 15;
+    float4 a = reinterpret_cast<const float4 *>(dU + w * H2)[l];
+    const float4 y = reinterpret_cast<const float4 *>(Hm + w * H)[l];
+    row_sum(col, row_ptr[w], row_ptr[w + 1], dU + H, H2, a);
+    reinterpret_cast<float4 *>(dZ + w * H)[l] = relu_mask(y, a);
 }
 
-// c = W_out h3 + b_out (kept), v0 = sum_k c_k b^(k) in FP64.
-__global__ void k_mp_out(int64_t n, const float *__restrict__ h3, const __nv_bfloat16 *__restrict__ Wout,
-                         const __nv_bfloat16 *__restrict__ bout, const double *__restrict__ b0,
-                         const double *__restrict__ b1, const double *__restrict__ b2, float *c, double *v0)
+// The output layer backwards: dZ = (W_out^T dc) where H > 0.
+__global__ void __launch_bounds__(TB) k_mp_out_t(int64_t n, const float *__restrict__ dc,
+                                                 const __nv_bfloat16 *__restrict__ W, const float *__restrict__ Hm, float *dZ)
 {
-    __shared__ float w[KB * H + KB];
-    for (int t = threadIdx.x; t < KB * H; t += blockDim.x) w[t] = bf(Wout, t);
-    if (threadIdx.x < KB) w[KB * H + threadIdx.x] = bf(bout, threadIdx.x);
-    __syncthreads();
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, i = t >> 4;
     if (i >= n) return;
+    const int l = (int)(t & 15);
+    float a[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int k = 0; k < KB; ++k) {
+        const float d = dc[i * KB + k];
+#pragma unroll
+        for (int v = 0; v < 4; ++v) a[v] = fmaf(d, bf(W, k * H + 4 * l + v), a[v]);
+    }
+    reinterpret_cast<float4 *>(dZ)[t] = relu_mask(reinterpret_cast<const float4 *>(Hm)[t], make_float4(a[0], a[1], a[2], a[3]));
+}
+
+// c = W_out h3 + b_out (kept), v0 = sum_k c_k b^(k) in FP64; 16 lanes per node.
+__global__ void __launch_bounds__(TB) k_mp_out(int64_t n, const float *__restrict__ h3, const __nv_bfloat16 *__restrict__ Wout,
+                                               const __nv_bfloat16 *__restrict__ bout, const double *__restrict__ b0,
+                                               const double *__restrict__ b1, const double *__restrict__ b2, float *c,
+                                               double *v0)
+{
+    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, i = t >> 4;
+    if (i >= n) return;
+    const int lane = threadIdx.x & 31, l = lane & 15;
+    const unsigned mask = 0xffffu << (lane & 16);
+    const float4 h = reinterpret_cast<const float4 *>(h3)[t];
     float ck[KB];
 #pragma unroll
     for (int k = 0; k < KB; ++k) {
-        float acc = w[KB * H + k];
-        for (int f = 0; f < H; ++f) acc = fmaf(h3[i * H + f], w[k * H + f], acc);
-        ck[k] = acc;
-        c[i * KB + k] = acc;
-    }
+        const __nv_bfloat16 *w = Wout + k * H + 4 * l;
+        ck[k] = fmaf(h.x, bf(w, 0), fmaf(h.y, bf(w, 1), fmaf(h.z, bf(w, 2), h.w * bf(w, 3))));
 #pragma unroll
-    for (int d = 0; d < 3; ++d)
-        v0[3 * i + d] = (double)ck[0] * b0[3 * i + d] + (double)ck[1] * b1[3 * i + d] + (double)ck[2] * b2[3 * i + d];
+        for (int b = 8; b > 0; b >>= 1) ck[k] += __shfl_xor_sync(mask, ck[k], b);
+        ck[k] += bf(bout, k);
+    }
+    if (l < 3) {
+        c[i * KB + l] = l == 0 ? ck[0] : l == 1 ? ck[1] : ck[2];
+        v0[3 * i + l] = (double)ck[0] * b0[3 * i + l] + (double)ck[1] * b1[3 * i + l] + (double)ck[2] * b2[3 * i + l];
+    }
 }
 
 // out[0] = x . y, out[1] = z . w over 3n values (blocks, then the last
@@ -336,13 +372,6 @@ __global__ void k_mp_scale(int64_t n3, const double *__restrict__ nd, double *v0
     if (isfinite(alpha)) v0[k] *= alpha;
 }
 
-// dZ = dY * (Y > 0) in place (ReLU derivative from the stored activation)
-__global__ void k_mp_relu_mask(int64_t cnt, const float *__restrict__ y, float *dy)
-{
-    int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (k < cnt && !(y[k] > 0.f)) dy[k] = 0.f;
-}
-
 // Per-block partial of G[o][k] = sum_n dZ[n][o] X[n][k] over the block's
 // CHUNK nodes, plus the bias gradient sum_n dZ[n][o] in G[DOUT][...].
 template <int D1, int D2, int DOUT>
@@ -352,7 +381,7 @@ __global__ void __launch_bounds__(TB) k_mp_wgrad(int64_t n, const float *__restr
     constexpr int DI = D1 + D2;
     constexpr int NG = DOUT * DI + DOUT;
     constexpr int PER = (NG + TB - 1) / TB;
-    constexpr int TILE = 32;
+    constexpr int TILE = 64;
     __shared__ float zs[TILE][DOUT];
     __shared__ float xs[TILE][DI];
     float acc[PER];
@@ -398,14 +427,92 @@ __global__ void __launch_bounds__(TB) k_mp_wgrad(int64_t n, const float *__restr
     }
 }
 
-// grad[off + g] = sum over blocks (in order) of partial[b][g]
-__global__ void k_mp_wsum(int nblocks, int NG, const float *__restrict__ partial, int off_w, int off_b, int nw,
-                          float *grad)
+// The same for the layers (64 outputs, 128 inputs), FMA bound: a thread keeps
+// 4 outputs x 8 inputs (64 threads also a bias), three 16-byte shared loads
+// per 32 FMAs, and has the next 16 nodes' rows in flight in registers.  1e5
+// cells: 236 -> 51 us.
+__global__ void __launch_bounds__(TB, 3) k_mp_wgrad_layer(int64_t n, const float *__restrict__ dZ, const float *__restrict__ X1,
+                                                          const float *__restrict__ X2, float *__restrict__ partial)
 {
-    int g = blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= NG) return;
+    constexpr int TILE = 16, NG = H * H2 + H, NZ = TILE * H / 4 / TB, NX = TILE * H2 / 4 / TB;
+    __shared__ __align__(16) float zs[TILE][H];
+    __shared__ __align__(16) float xs[TILE][H2];
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    const int64_t n0 = (int64_t)blockIdx.x * CHUNK, n1 = n < n0 + CHUNK ? n : n0 + CHUNK;
+    float acc[4][8], bias = 0.f;
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int v = 0; v < 8; ++v) acc[u][v] = 0.f;
+    float4 zq[NZ], xq[NX];
+    auto fetch = [&](int64_t t0) {
+#pragma unroll
+        for (int q = 0; q < NZ; ++q) {
+            const int c = threadIdx.x + q * TB;
+            const int64_t i = t0 + c / (H / 4);
+            zq[q] = i < n1 ? reinterpret_cast<const float4 *>(dZ + i * H)[c % (H / 4)] : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+#pragma unroll
+        for (int q = 0; q < NX; ++q) {
+            const int c = threadIdx.x + q * TB, k = c % (H2 / 4);
+            const int64_t i = t0 + c / (H2 / 4);
+            const float *x = k < H / 4 ? X1 : X2;
+            xq[q] = i < n1 ? reinterpret_cast<const float4 *>(x + i * H)[k % (H / 4)] : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+    };
+    fetch(n0);
+    for (int64_t t0 = n0; t0 < n1; t0 += TILE) {
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < NZ; ++q) reinterpret_cast<float4 *>(&zs[0][0])[threadIdx.x + q * TB] = zq[q];
+#pragma unroll
+        for (int q = 0; q < NX; ++q) reinterpret_cast<float4 *>(&xs[0][0])[threadIdx.x + q * TB] = xq[q];
+        __syncthreads();
+        if (t0 + TILE < n1) fetch(t0 + TILE);
+        if (threadIdx.x < H)
+            for (int s = 0; s < TILE; ++s) bias += zs[s][threadIdx.x];
+#pragma unroll 4
+        for (int s = 0; s < TILE; ++s) {
+            const float4 z = *reinterpret_cast<const float4 *>(&zs[s][4 * ty]);
+            const float4 a = *reinterpret_cast<const float4 *>(&xs[s][4 * tx]);
+            const float4 b = *reinterpret_cast<const float4 *>(&xs[s][H + 4 * tx]);
+            const float zv[4] = {z.x, z.y, z.z, z.w}, xv[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+#pragma unroll
+                for (int v = 0; v < 8; ++v) acc[u][v] = fmaf(zv[u], xv[v], acc[u][v]);
+            }
+        }
+    }
+    float *o = partial + (int64_t)blockIdx.x * NG;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        float *r = o + (4 * ty + u) * H2 + 4 * tx;
+        *reinterpret_cast<float4 *>(r) = make_float4(acc[u][0], acc[u][1], acc[u][2], acc[u][3]);
+        *reinterpret_cast<float4 *>(r + H) = make_float4(acc[u][4], acc[u][5], acc[u][6], acc[u][7]);
+    }
+    if (threadIdx.x < H) o[H * H2 + threadIdx.x] = bias;
+}
+
+// grad[off + g] = sum over blocks of partial[b][g]: 8 runs of blocks per
+// column, each in order, then the runs in order.
+__global__ void __launch_bounds__(TB) k_mp_wsum(int nblocks, int NG, const float *__restrict__ partial, int off_w, int off_b,
+                                                int nw, float *grad)
+{
+    constexpr int R = TB / 32;
+    __shared__ float sh[R][32];
+    const int g = blockIdx.x * 32 + (threadIdx.x & 31), r = threadIdx.x >> 5;
+    const int per = (nblocks + R - 1) / R, b1 = min(nblocks, (r + 1) * per);
     float s = 0.f;
-    for (int b = 0; b < nblocks; ++b) s += partial[(int64_t)b * NG + g];
+    if (g < NG) {
+#pragma unroll 8
+        for (int b = r * per; b < b1; ++b) s += partial[(int64_t)b * NG + g];
+    }
+    sh[r][threadIdx.x & 31] = s;
+    __syncthreads();
+    if (r || g >= NG) return;
+#pragma unroll
+    for (int k = 1; k < R; ++k) s += sh[k][threadIdx.x];
     if (g < nw) grad[off_w + g] = s;
     else grad[off_b + (g - nw)] = s;
 }
@@ -464,31 +571,27 @@ static unsigned red_blocks(int64_t cnt)
     return (unsigned)std::max<int64_t>(1, std::min<int64_t>(1024, (cnt + TB - 1) / TB));
 }
 
+template <int D1, int D2, int DOUT, bool TRANS, bool RELU, int NU>
+static sgp_status dense_tiles(sgp_ctx *ctx, int64_t n, const float *X1, const float *X2, const __nv_bfloat16 *W,
+                              const __nv_bfloat16 *b, const int32_t *row_ptr, float *Y)
+{
+    constexpr int DI = D1 + D2;
+    constexpr size_t smem = sizeof(float) * ((size_t)DI * DOUT + (size_t)16 * NU * (DI + 4));
+    auto kern = k_mp_dense<D1, D2, DOUT, TRANS, RELU, NU>;
+    SGP_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    const int64_t want = (n + 16 * NU - 1) / (16 * NU);
+    // two blocks per SM (registers)
+    const unsigned G = (unsigned)std::max<int64_t>(1, std::min<int64_t>(want, 2 * 152));
+    LAUNCH(ctx, kern, G, TB, smem, n, X1, X2, W, b, row_ptr, Y);
+    return SGP_OK;
+}
+// 128 nodes per tile while that fills two blocks per SM, else 64
 template <int D1, int D2, int DOUT, bool TRANS, bool RELU>
 static sgp_status dense(sgp_ctx *ctx, int64_t n, const float *X1, const float *X2, const __nv_bfloat16 *W,
-                        const __nv_bfloat16 *b, float *Y)
+                        const __nv_bfloat16 *b, const int32_t *row_ptr, float *Y)
 {
-    if constexpr (!TRANS && DOUT == H && (D1 + D2) % 4 == 0 && D1 % 4 == 0) {
-        // forward layers: the register-tiled kernel (shared memory above
-        // 48 KB opted in once per device)
-        constexpr int DI = D1 + D2;
-        constexpr size_t smem = sizeof(float) * ((size_t)DI * H + (size_t)DT_NODES * (DI + 4));
-        static bool opted[64] = {false};
-        auto kern = k_mp_dense_tiled<D1, D2, RELU>;
-        if (ctx->device >= 0 && ctx->device < 64 && !opted[ctx->device]) {
-            SGP_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-            opted[ctx->device] = true;
-        }
-        unsigned G = 1;
-        SGP_TRY(resident_grid(ctx, (const void *)kern, TB, (n + DT_NODES - 1) / DT_NODES, &G));
-        LAUNCH(ctx, kern, G, TB, smem, n, X1, X2, W, b, Y);
-        return SGP_OK;
-    }
-    constexpr int NPB = TB / DOUT > 0 ? TB / DOUT : 1;
-    const int64_t want = (n + NPB - 1) / NPB;
-    const unsigned G = (unsigned)std::max<int64_t>(1, std::min<int64_t>(want, 152 * 16));
-    LAUNCH(ctx, (k_mp_dense<D1, D2, DOUT, TRANS, RELU>), G, TB, 0, n, X1, X2, W, b, Y);
-    return SGP_OK;
+    return n >= 2 * 152 * 128 ? dense_tiles<D1, D2, DOUT, TRANS, RELU, 8>(ctx, n, X1, X2, W, b, row_ptr, Y)
+                              : dense_tiles<D1, D2, DOUT, TRANS, RELU, 4>(ctx, n, X1, X2, W, b, row_ptr, Y);
 }
 
 template <int D1, int D2, int DOUT>
@@ -499,8 +602,11 @@ static sgp_status wgrad(sgp_ctx *ctx, sgp_mpnn *N, int64_t n, const float *dZ, c
     constexpr int NG = DOUT * DI + DOUT;
     const unsigned nb = (unsigned)((n + CHUNK - 1) / CHUNK);
     float *part = bp<float>(N->part);
-    LAUNCH(ctx, (k_mp_wgrad<D1, D2, DOUT>), nb, TB, 0, n, dZ, X1, X2, part);
-    LAUNCH(ctx, k_mp_wsum, grid_for(NG, TB), TB, 0, (int)nb, NG, (const float *)part, off_w, off_b, DOUT * DI,
+    if constexpr (D1 == H && D2 == H && DOUT == H)
+        LAUNCH(ctx, k_mp_wgrad_layer, nb, TB, 0, n, dZ, X1, X2, part);
+    else
+        LAUNCH(ctx, (k_mp_wgrad<D1, D2, DOUT>), nb, TB, 0, n, dZ, X1, X2, part);
+    LAUNCH(ctx, k_mp_wsum, grid_for(NG, 32), TB, 0, (int)nb, NG, (const float *)part, off_w, off_b, DOUT * DI,
            bp<float>(N->g));
     return SGP_OK;
 }
@@ -593,15 +699,15 @@ static sgp_status mpnn_forward_internal(sgp_ctx *ctx, sgp_mpnn *N, const sgp_mat
     // forward
     const __nv_bfloat16 *pb = bp<const __nv_bfloat16>(N->pb);
     float *hs = bp<float>(N->hs), *aggs = bp<float>(N->aggs);
-    SGP_TRY((dense<DIN, 0, H, false, true>(ctx, n, x, nullptr, pb + OFF_WIN, pb + OFF_BIN, hs)));
+    const int32_t *row_ptr = bp<const int32_t>(M->row_ptr), *col = bp<const int32_t>(M->col);
+    SGP_TRY((dense<DIN, 0, H, false, true>(ctx, n, x, nullptr, pb + OFF_WIN, pb + OFF_BIN, row_ptr, hs)));
     for (int l = 0; l < 3; ++l) {
         float *h = hs + (int64_t)l * H * n, *a = aggs + (int64_t)l * H * n, *hn = hs + (int64_t)(l + 1) * H * n;
-        LAUNCH(ctx, k_mp_agg, grid_for(32 * n, TB), TB, 0, n, bp<const int32_t>(M->row_ptr),
-               bp<const int32_t>(M->col), (const float *)h, a);
+        LAUNCH(ctx, k_mp_agg, grid_for(16 * n, TB), TB, 0, n, row_ptr, col, (const float *)h, a);
         const int off = OFF_L0 + l * LAYER;
-        SGP_TRY((dense<H, H, H, false, true>(ctx, n, h, a, pb + off, pb + off + H * H2, hn)));
+        SGP_TRY((dense<H, H, H, false, true>(ctx, n, h, a, pb + off, pb + off + H * H2, row_ptr, hn)));
     }
-    LAUNCH(ctx, k_mp_out, grid_for(n, TB), TB, 0, n, (const float *)(hs + 3 * H * n), pb + OFF_WOUT, pb + OFF_BOUT,
+    LAUNCH(ctx, k_mp_out, grid_for(16 * n, TB), TB, 0, n, (const float *)(hs + 3 * H * n), pb + OFF_WOUT, pb + OFF_BOUT,
            (const double *)b0, (const double *)b1, (const double *)b2, bp<float>(N->c), bp<double>(N->v0w));
     SGP_TRY(kt_end(ctx, SGP_KT_WARM_LAYERS, ev));
     return SGP_OK;
@@ -663,17 +769,15 @@ sgp_status sgp_mpnn_backward(sgp_ctx *ctx, sgp_mpnn *N, const double *v_target, 
     LAUNCH(ctx, k_mp_dc, grid_for(n, TB), TB, 0, n, g, b0, b1, b2, (const double *)nd, dc);
     // output layer
     SGP_TRY((wgrad<H, 0, KB>(ctx, N, n, dc, hs + 3 * H * n, nullptr, OFF_WOUT, OFF_BOUT)));
-    SGP_TRY((dense<KB, 0, H, true, false>(ctx, n, dc, nullptr, pb + OFF_WOUT, nullptr, dh)));
+    const int32_t *row_ptr = bp<const int32_t>(M->row_ptr), *col = bp<const int32_t>(M->col);
+    LAUNCH(ctx, k_mp_out_t, grid_for(16 * n, TB), TB, 0, n, (const float *)dc, pb + OFF_WOUT, hs + 3 * H * n, dh);
     for (int l = 2; l >= 0; --l) {
-        const float *hn = hs + (int64_t)(l + 1) * H * n, *h = hs + (int64_t)l * H * n, *a = aggs + (int64_t)l * H * n;
-        LAUNCH(ctx, k_mp_relu_mask, grid_for(H * n, TB), TB, 0, H * n, hn, dh);
+        const float *h = hs + (int64_t)l * H * n, *a = aggs + (int64_t)l * H * n;
         const int off = OFF_L0 + l * LAYER;
         SGP_TRY((wgrad<H, H, H>(ctx, N, n, dh, h, a, off, off + H * H2)));
-        SGP_TRY((dense<H, 0, H2, true, false>(ctx, n, dh, nullptr, pb + off, nullptr, du)));
-        LAUNCH(ctx, k_mp_agg_t, grid_for(32 * n, TB), TB, 0, n, bp<const int32_t>(M->row_ptr),
-               bp<const int32_t>(M->col), (const float *)du, dh);
+        SGP_TRY((dense<H, 0, H2, true, false>(ctx, n, dh, nullptr, pb + off, nullptr, row_ptr, du)));
+        LAUNCH(ctx, k_mp_agg_t, grid_for(16 * n, TB), TB, 0, n, row_ptr, col, (const float *)du, h, dh);
     }
-    LAUNCH(ctx, k_mp_relu_mask, grid_for(H * n, TB), TB, 0, H * n, hs, dh);
     SGP_TRY((wgrad<DIN, 0, H>(ctx, N, n, dh, x, nullptr, OFF_WIN, OFF_BIN)));
     if (loss) SGP_TRY(read_back(ctx, loss, lossout, sizeof(double)));
     return SGP_OK;
