@@ -807,6 +807,8 @@ Tail tail_of(const sgp_factor *F)
 template <typename T>
 sgp_status tree_apply_inplace(sgp_ctx *ctx, const sgp_factor *F, T *w, const int *done)
 {
+    if constexpr (sizeof(T) == 8)
+        if (grid_apply_ready(ctx, F)) return grid_apply(ctx, F, w, w, nullptr, done);
     if (bins_usable<T>(F)) return bins_apply<T>(ctx, F, w, done);
     const bool f64 = sizeof(T) == 8;
     const T *L = reinterpret_cast<const T *>(f64 ? F->L.p : F->L32.p);
@@ -1161,7 +1163,7 @@ sgp_status sgp_tree_factor(sgp_ctx *ctx, const sgp_matrix *M, const sgp_tree *T,
     // cells: not where the one-block solve serves the factor); else the bins
     F->gl.ok = 0;
     if (ctx->bin_cap == 0 && ctx->fused && !M->batched && !small_solve_fits(ctx, F)) SGP_TRY(grid_build(ctx, F, M));
-    if (F->gl.ok) {
+    if (F->gl.ok && F->gl.rows.ok) {
         F->bl.ok32 = F->bl.ok64 = 0;
         F->bl.mgen = 0;
         F->bl.NT = F->bl.nb = F->bl.nt = F->bl.nly = F->bl.bmax = 0;
@@ -1176,6 +1178,9 @@ sgp_status sgp_tree_apply(sgp_ctx *ctx, const sgp_factor *F, const double *b, do
     if (!ctx || !F || (F->n > 0 && (!b || !x))) return SGP_ERR_INVALID_ARG;
     if (F->n == 0) return SGP_OK;
     SGP_CUDA(ctx, cudaSetDevice(ctx->device));
+    // (in place is fine in one launch, as every part writes the rows it has read)
+    const bool apart = b == x || b + 3 * F->n <= x || x + 3 * F->n <= b;
+    if (apart && grid_apply_ready(ctx, F)) return grid_apply(ctx, F, b, x, bp<const int32_t>(F->orig_of), nullptr);
     // caller order -> internal order (the factor's workspace) -> caller order
     double *wi = bp<double>(F->work);
     const int32_t *orig_of = bp<const int32_t>(F->orig_of);

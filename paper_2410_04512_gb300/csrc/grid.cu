@@ -1733,6 +1733,135 @@ __device__ __noinline__ void sums(const GridArgs &a, Solve<T> &Z, int op)
     Z.go = Z.S.done ? 0 : 1;
 }
 
+// A part's numbers: its vertices, rows (with its top vertices), the top
+// vertices that it reaches and their offset, its first top vertex.  It needs
+// z of `nout` top vertices (those it reaches, then those it owns); a row of
+// their inverse is cut into nch pieces, about one per warp.
+struct PartDims {
+    int32_t nv, nr, ro, t0, nz, zo, nout, nch, chunk;
+};
+__device__ __forceinline__ PartDims part_of(const GridArgs &a)
+{
+    const int32_t *h = a.hdr + (size_t)Q_N * blockIdx.x;
+    PartDims g{h[Q_NV], h[Q_NR], h[Q_ROFF], h[Q_T0], h[Q_NZ], h[Q_ZOFF], 0, 1, 0};
+    const int32_t npc = (a.nt + 127) / 128;
+    g.nout = g.nz + g.nr - g.nv;
+    g.nch = g.nout > 0 ? max(1, min(npc, GW / g.nout)) : 1;
+    g.chunk = (npc + g.nch - 1) / g.nch * 128;
+    return g;
+}
+
+// One forest solve, in three steps (w: the right-hand side in, the solution
+// out).  First the r of the part's top rows to the others, the forward levels,
+// the part's sums for the top, its pivots.
+template <typename T, int VB>
+__device__ __forceinline__ void tree_up(const GridArgs &a, const PartDims &g, const Prog *s_prog, const T *D, uint32_t w,
+                                        unsigned long long *trx, unsigned ep)
+{
+    const unsigned long long e = (unsigned long long)ep << 32;
+    const T zero[3] = {0, 0, 0};
+    for (int32_t z = (int)threadIdx.x; z < g.nz; z += GT) V3<T, VB>::st(w + (g.nr + z) * VB, zero);
+    __syncthreads();
+    for (int32_t i = g.nv + (int)threadIdx.x; i < g.nr; i += GT) {
+        T v[3];
+        V3<T, VB>::ld(w + i * VB, v);
+        Pkt<T>::put(trx + (size_t)Pkt<T>::W * (g.t0 + i - g.nv), e, v);
+    }
+    run<T, VB, true>(s_prog[0], w);
+    for (int32_t z = (int)threadIdx.x; z < g.nz; z += GT) {
+        T v[3];
+        V3<T, VB>::ld(w + (g.nr + z) * VB, v);
+        Pkt<T>::put(a.lx + (size_t)Pkt<T>::W * __ldg(a.zslot + g.zo + z), e, v);
+    }
+    pivots<T, VB>(D, g.nv, w);
+}
+
+// Then, by the threads from `first` on, the parts' sums and the top's r.
+template <typename T, int VB>
+__device__ __forceinline__ bool gather_top(const GridArgs &a, uint32_t tw, const unsigned long long *trx, unsigned ep,
+                                           int first)
+{
+    const int tid = threadIdx.x;
+    bool ok = true;
+    for (int32_t i = tid - first; i < a.nt; i += GT - first) {
+        const int32_t k0 = __ldg(a.tlk + i), k1 = __ldg(a.tlk + i + 1);
+        // r and the first two sums in flight together
+        const unsigned long long *pv = trx + (size_t)Pkt<T>::W * i, *p0 = a.lx + (size_t)Pkt<T>::W * k0,
+                                 *p1 = k0 + 1 < k1 ? p0 + Pkt<T>::W : p0;
+        if (k0 >= k1) p0 = p1 = pv;
+        T v[3], y0[3], y1[3];
+        for (int it = 0; ok; ++it) {
+            const bool a0 = Pkt<T>::get(pv, ep, v), a1 = Pkt<T>::get(p0, ep, y0),
+                       a2 = Pkt<T>::get(p1, ep, y1);
+            if (a0 && a1 && a2) break;
+            ok = !give_up(it, a.err);
+        }
+        if (k0 < k1) {
+            v[0] += y0[0]; v[1] += y0[1]; v[2] += y0[2];
+        }
+        if (k0 + 1 < k1) {
+            v[0] += y1[0]; v[1] += y1[1]; v[2] += y1[2];
+        }
+        for (int32_t k = k0 + 2; k < k1 && ok; ++k) {
+            ok = wait_packet<T>(a.lx + (size_t)Pkt<T>::W * k, ep, y0, a.err);
+            v[0] += y0[0]; v[1] += y0[1]; v[2] += y0[2];
+        }
+        V3<T, VB>::st(tw + i * VB, v);
+    }
+    return ok;
+}
+
+// Then (after a barrier) the top, as far as the part needs it: the rows of its
+// inverse times the top's right-hand side, a warp per row or piece of a row
+// (several blocks per lane in flight), then the pieces in order; then the
+// part's backward levels.
+template <typename T, int VB>
+__device__ __forceinline__ void tree_down(const GridArgs &a, const PartDims &g, const Prog *s_prog, const T *inv, uint32_t w,
+                                          uint32_t tw, T *tp)
+{
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    for (int32_t it = warp; it < g.nout * g.nch; it += GW) {
+        const int32_t o = it / g.nch, k0 = (it - o * g.nch) * g.chunk, k1 = min(a.ntp, k0 + g.chunk);
+        const int32_t i = o < g.nz ? __ldg(a.zi + g.zo + o) : g.t0 + o - g.nz;
+        const T *f = inv + (size_t)(a.pl.o_inv >= 0 ? o : i) * 9 * a.ntp + lane;
+        T z[3] = {0, 0, 0};
+        constexpr int N = sizeof(T) == 4 ? 4 : 2;
+        for (int32_t k = k0; k < k1; k += 32 * N) {
+            T m[N][9];
+#pragma unroll
+            for (int u = 0; u < N; ++u)
+#pragma unroll
+                for (int c = 0; c < 9; ++c) m[u][c] = k + 32 * u < k1 ? f[(size_t)c * a.ntp + k + 32 * u] : T(0);
+#pragma unroll
+            for (int u = 0; u < N; ++u) {
+                if (k + 32 * u >= k1) break;
+                T y[3];
+                V3<T, VB>::ld(tw + min(k + lane + 32 * u, a.nt - 1) * VB, y);
+#pragma unroll
+                for (int c = 0; c < 3; ++c)
+                    z[c] = fma(m[u][3 * c + 2], y[2], fma(m[u][3 * c + 1], y[1], fma(m[u][3 * c], y[0], z[c])));
+            }
+        }
+#pragma unroll
+        for (int b = 16; b > 0; b >>= 1)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) z[c] += __shfl_xor_sync(0xffffffffu, z[c], b);
+        if (lane == 0) {
+            tp[3 * it] = z[0]; tp[3 * it + 1] = z[1]; tp[3 * it + 2] = z[2];
+        }
+    }
+    __syncthreads();
+    for (int32_t o = tid; o < g.nout; o += GT) {
+        T z[3] = {0, 0, 0};
+        for (int32_t k = o * g.nch; k < (o + 1) * g.nch; ++k) {
+            z[0] += tp[3 * k]; z[1] += tp[3 * k + 1]; z[2] += tp[3 * k + 2];
+        }
+        V3<T, VB>::st(w + (o < g.nz ? g.nr + o : g.nv + o - g.nz) * VB, z);
+    }
+    __syncthreads();
+    run<T, VB, false>(s_prog[1], w);
+}
+
 template <typename T, int VB, int PREC>
 __global__ void __launch_bounds__(GT, 1) k_pcg_grid(const __grid_constant__ GridArgs a)
 {
@@ -1742,8 +1871,9 @@ __global__ void __launch_bounds__(GT, 1) k_pcg_grid(const __grid_constant__ Grid
     __shared__ int32_t s_ws[2][W_N];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int32_t *h = a.hdr + (size_t)Q_N * blockIdx.x;
-    const int32_t nv = h[Q_NV], nr = h[Q_NR], ro = h[Q_ROFF], t0 = h[Q_T0], nz = h[Q_NZ], zo = h[Q_ZOFF],
-                  slot0 = a.rh[R_N * blockIdx.x + R_SLOT], nh = a.rh[R_N * blockIdx.x + R_NH], nt = a.nt;
+    const PartDims g = part_of(a);
+    const int32_t nv = g.nv, nr = g.nr, ro = g.ro, slot0 = a.rh[R_N * blockIdx.x + R_SLOT],
+                  nh = a.rh[R_N * blockIdx.x + R_NH];
     T *ps = reinterpret_cast<T *>(sm + a.pl.o_p);
     const uint32_t sm0 = (uint32_t)__cvta_generic_to_shared(sm);
     const uint32_t w = sm0 + a.pl.o_w, tw = sm0 + a.pl.o_t;
@@ -1763,10 +1893,6 @@ __global__ void __launch_bounds__(GT, 1) k_pcg_grid(const __grid_constant__ Grid
     }
     const int32_t *hl = put(a.hl + a.rh[R_N * blockIdx.x + R_HOFF], a.pl.o_hl, a.halo ? nh : 0);
     const T *D = nullptr, *inv = nullptr;
-    // top vertices the part needs: those it reaches, then those it owns
-    // and into how many pieces their rows are cut (about one item per warp)
-    const int32_t nout = nz + nr - nv, npc = (nt + 127) / 128,
-                  nch = nout > 0 ? max(1, min(npc, GW / nout)) : 1, chunk = (npc + nch - 1) / nch * 128;
     if (PREC == 0) {
         D = put(reinterpret_cast<const T *>(a.D) + 6 * (size_t)ro, a.pl.o_D, 6 * pad32(nv));
         constexpr int B = SlotSize<T>::B;
@@ -1784,14 +1910,14 @@ __global__ void __launch_bounds__(GT, 1) k_pcg_grid(const __grid_constant__ Grid
         }
         if (tid == 0) {   // the spare cell
             const T zero[3] = {0, 0, 0};
-            V3<T, VB>::st(w + (nr + nz) * VB, zero);
+            V3<T, VB>::st(w + (nr + g.nz) * VB, zero);
         }
         // the rows of the top's inverse that the part needs, when they fit
         inv = reinterpret_cast<const T *>(a.inv);
         if (a.pl.o_inv >= 0) {
             T *d = reinterpret_cast<T *>(sm + a.pl.o_inv);
-            for (int32_t o = 0; o < nout; ++o) {
-                const int32_t i = o < nz ? __ldg(a.zi + zo + o) : t0 + o - nz;
+            for (int32_t o = 0; o < g.nout; ++o) {
+                const int32_t i = o < g.nz ? __ldg(a.zi + g.zo + o) : g.t0 + o - g.nz;
                 const T *f = inv + (size_t)i * 9 * a.ntp;
                 for (int32_t k = tid; k < 9 * a.ntp; k += GT) d[(size_t)o * 9 * a.ntp + k] = f[k];
             }
@@ -1954,24 +2080,7 @@ __global__ void __launch_bounds__(GT, 1) k_pcg_grid(const __grid_constant__ Grid
             if (PREC != 0) partial(1, rz);
         }
         if (PREC == 0) {
-            // the r of the part's top rows to the others, the forward levels,
-            // the part's sums for the top, its pivots
-            const unsigned long long e = (unsigned long long)(ep + 1) << 32;
-            const T zero[3] = {0, 0, 0};
-            for (int32_t z = tid; z < nz; z += GT) V3<T, VB>::st(w + (nr + z) * VB, zero);
-            __syncthreads();
-            for (int32_t i = nv + tid; i < nr; i += GT) {
-                T v[3];
-                V3<T, VB>::ld(w + i * VB, v);
-                Pkt<T>::put(trx + (size_t)Pkt<T>::W * (t0 + i - nv), e, v);
-            }
-            run<T, VB, true>(s_prog[0], w);
-            for (int32_t z = tid; z < nz; z += GT) {
-                T v[3];
-                V3<T, VB>::ld(w + (nr + z) * VB, v);
-                Pkt<T>::put(a.lx + (size_t)Pkt<T>::W * __ldg(a.zslot + zo + z), e, v);
-            }
-            pivots<T, VB>(D, nv, w);
+            tree_up<T, VB>(a, g, s_prog, D, w, trx, ep + 1);
         } else {
             __syncthreads();
         }
@@ -1981,33 +2090,7 @@ __global__ void __launch_bounds__(GT, 1) k_pcg_grid(const __grid_constant__ Grid
         if (warp == 0 && phase > 0) {
             sums<T>(a, Z, PREC == 0 ? OP_RR : OP_RR_RZ);
         } else if (PREC == 0) {
-            bool ok = true;
-            for (int32_t i = tid - first; i < nt; i += GT - first) {
-                const int32_t k0 = __ldg(a.tlk + i), k1 = __ldg(a.tlk + i + 1);
-                // r and the first two sums in flight together
-                const unsigned long long *pv = trx + (size_t)Pkt<T>::W * i, *p0 = a.lx + (size_t)Pkt<T>::W * k0,
-                                         *p1 = k0 + 1 < k1 ? p0 + Pkt<T>::W : p0;
-                if (k0 >= k1) p0 = p1 = pv;
-                T v[3], y0[3], y1[3];
-                for (int it = 0; ok; ++it) {
-                    const bool a0 = Pkt<T>::get(pv, ep + 1, v), a1 = Pkt<T>::get(p0, ep + 1, y0),
-                               a2 = Pkt<T>::get(p1, ep + 1, y1);
-                    if (a0 && a1 && a2) break;
-                    ok = !give_up(it, a.err);
-                }
-                if (k0 < k1) {
-                    v[0] += y0[0]; v[1] += y0[1]; v[2] += y0[2];
-                }
-                if (k0 + 1 < k1) {
-                    v[0] += y1[0]; v[1] += y1[1]; v[2] += y1[2];
-                }
-                for (int32_t k = k0 + 2; k < k1 && ok; ++k) {
-                    ok = wait_packet<T>(a.lx + (size_t)Pkt<T>::W * k, ep + 1, y0, a.err);
-                    v[0] += y0[0]; v[1] += y0[1]; v[2] += y0[2];
-                }
-                V3<T, VB>::st(tw + i * VB, v);
-            }
-            if (!ok) Z.bad = 1;
+            if (!gather_top<T, VB>(a, tw, trx, ep + 1, first)) Z.bad = 1;
         }
         __syncthreads();
         if (Z.bad) return;
@@ -2016,51 +2099,7 @@ __global__ void __launch_bounds__(GT, 1) k_pcg_grid(const __grid_constant__ Grid
             break;
         }
         if (PREC == 0) {
-            // the top, as far as the part needs it: the rows of its inverse
-            // times the top's right-hand side, a warp per row or piece of a
-            // row (several blocks per lane in flight), then the pieces in
-            // order; then the part's backward levels
-            T *tp = reinterpret_cast<T *>(sm + a.pl.o_tp);
-            for (int32_t it = warp; it < nout * nch; it += GW) {
-                const int32_t o = it / nch, k0 = (it - o * nch) * chunk, k1 = min(a.ntp, k0 + chunk);
-                const int32_t i = o < nz ? __ldg(a.zi + zo + o) : t0 + o - nz;
-                const T *f = inv + (size_t)(a.pl.o_inv >= 0 ? o : i) * 9 * a.ntp + lane;
-                T z[3] = {0, 0, 0};
-                constexpr int N = sizeof(T) == 4 ? 4 : 2;
-                for (int32_t k = k0; k < k1; k += 32 * N) {
-                    T m[N][9];
-#pragma unroll
-                    for (int u = 0; u < N; ++u)
-#pragma unroll
-                        for (int c = 0; c < 9; ++c) m[u][c] = k + 32 * u < k1 ? f[(size_t)c * a.ntp + k + 32 * u] : T(0);
-#pragma unroll
-                    for (int u = 0; u < N; ++u) {
-                        if (k + 32 * u >= k1) break;
-                        T y[3];
-                        V3<T, VB>::ld(tw + min(k + lane + 32 * u, nt - 1) * VB, y);
-#pragma unroll
-                        for (int c = 0; c < 3; ++c)
-                            z[c] = fma(m[u][3 * c + 2], y[2], fma(m[u][3 * c + 1], y[1], fma(m[u][3 * c], y[0], z[c])));
-                    }
-                }
-#pragma unroll
-                for (int b = 16; b > 0; b >>= 1)
-#pragma unroll
-                    for (int c = 0; c < 3; ++c) z[c] += __shfl_xor_sync(0xffffffffu, z[c], b);
-                if (lane == 0) {
-                    tp[3 * it] = z[0]; tp[3 * it + 1] = z[1]; tp[3 * it + 2] = z[2];
-                }
-            }
-            __syncthreads();
-            for (int32_t o = tid; o < nout; o += GT) {
-                T z[3] = {0, 0, 0};
-                for (int32_t k = o * nch; k < (o + 1) * nch; ++k) {
-                    z[0] += tp[3 * k]; z[1] += tp[3 * k + 1]; z[2] += tp[3 * k + 2];
-                }
-                V3<T, VB>::st(w + (o < nz ? nr + o : nv + o - nz) * VB, z);
-            }
-            __syncthreads();
-            run<T, VB, false>(s_prog[1], w);
+            tree_down<T, VB>(a, g, s_prog, inv, w, tw, reinterpret_cast<T *>(sm + a.pl.o_tp));
         }
         if (PREC == 0 || phase <= 0) {
             Acc<T> acc;
@@ -2102,6 +2141,84 @@ __global__ void __launch_bounds__(GT, 1) k_pcg_grid(const __grid_constant__ Grid
             a.ns[0] = t_spmv;
             a.ns[1] = t_tree;
             a.ns[2] = t_vec;
+        }
+    }
+}
+
+// One forest solve alone: x = P^-1 b in the caller's order (orig_of) or the
+// internal one, the forest's part of one iteration above.  Everything is read once, so only what warp 0 reads
+// in sequence (the narrow levels) is brought on chip first, while the right-
+// hand side arrives.
+template <typename T, int VB>
+__global__ void __launch_bounds__(GT, 1) k_apply_grid(const __grid_constant__ GridArgs a, const int32_t *__restrict__ orig_of,
+                                                    const int *__restrict__ done)
+{
+    extern __shared__ __align__(16) unsigned char sm[];
+    __shared__ Prog s_prog[2];
+    __shared__ int32_t s_ws[2][W_N];
+    __shared__ int s_bad;
+    const int tid = threadIdx.x;
+    const int32_t *h = a.hdr + (size_t)Q_N * blockIdx.x;
+    const PartDims g = part_of(a);
+    const uint32_t sm0 = (uint32_t)__cvta_generic_to_shared(sm);
+    const uint32_t w = sm0 + a.pl.o_w, tw = sm0 + a.pl.o_t;
+    constexpr int B = SlotSize<T>::B;
+    if (done && *done) return;
+    const T *F = reinterpret_cast<const T *>(a.F);
+    T *x = reinterpret_cast<T *>(a.x);
+    for (int i = tid; i < 2 * W_N; i += GT) s_ws[i / W_N][i % W_N] = a.ws[(size_t)blockIdx.x * 2 * W_N + i];
+    if (tid == 0) s_bad = 0;
+    __syncthreads();
+    for (int q = 0; q < 2; ++q) {
+        const char *pg = a.prog[q] + (size_t)B * h[q ? Q_SB : Q_SF], *nar = pg + (size_t)B * s_ws[q][W_NARROW];
+        if (a.pl.o_nar[q] >= 0) {
+            const int32_t cnt = (B / 16) * (s_ws[q][W_END] - s_ws[q][W_NARROW]);
+            int4 *d = reinterpret_cast<int4 *>(sm + a.pl.o_nar[q]);
+            for (int32_t i = tid; i < cnt; i += GT) d[i] = reinterpret_cast<const int4 *>(nar)[i];
+            nar = reinterpret_cast<const char *>(d);
+        }
+        if (tid == 0) s_prog[q] = Prog{s_ws[q], pg, nar};
+    }
+    constexpr int N = 4;   // rows in flight per thread
+    for (int32_t b = tid; b < g.nr; b += N * GT) {
+        int32_t v[N];
+#pragma unroll
+        for (int u = 0; u < N; ++u) v[u] = __ldg(a.i_of_t + g.ro + min(b + u * GT, g.nr - 1));
+#pragma unroll
+        for (int u = 0; u < N; ++u)
+            if (orig_of) v[u] = __ldg(orig_of + v[u]);
+        T q[N][3];
+#pragma unroll
+        for (int u = 0; u < N; ++u)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) q[u][c] = F[3 * (size_t)v[u] + c];
+#pragma unroll
+        for (int u = 0; u < N; ++u)
+            if (b + u * GT < g.nr) V3<T, VB>::st(w + (b + u * GT) * VB, q[u]);
+    }
+    const T zero[3] = {0, 0, 0};
+    if (tid == 0) V3<T, VB>::st(w + (g.nr + g.nz) * VB, zero);   // the spare cell
+    unsigned long long *trx = a.lx + (size_t)Pkt<T>::W * a.nslots;
+    tree_up<T, VB>(a, g, s_prog, reinterpret_cast<const T *>(a.D) + 6 * (size_t)g.ro, w, trx, 1u);
+    if (!gather_top<T, VB>(a, tw, trx, 1u, 0)) s_bad = 1;
+    __syncthreads();
+    const bool bad = s_bad != 0;
+    if (!bad)
+        tree_down<T, VB>(a, g, s_prog, reinterpret_cast<const T *>(a.inv), w, tw, reinterpret_cast<T *>(sm + a.pl.o_tp));
+    for (int32_t b = tid; b < g.nr; b += N * GT) {
+        int32_t v[N];
+#pragma unroll
+        for (int u = 0; u < N; ++u) v[u] = __ldg(a.i_of_t + g.ro + min(b + u * GT, g.nr - 1));
+#pragma unroll
+        for (int u = 0; u < N; ++u)
+            if (orig_of) v[u] = __ldg(orig_of + v[u]);
+#pragma unroll
+        for (int u = 0; u < N; ++u) {
+            if (b + u * GT >= g.nr) break;
+            T q[3];
+            V3<T, VB>::ld(w + (b + u * GT) * VB, q);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) x[3 * (size_t)v[u] + c] = bad ? T(NAN) : q[c];
         }
     }
 }
@@ -2158,6 +2275,31 @@ bool place(const GridLayout &G, int32_t mnh, size_t sz, size_t vb, bool tree, bo
                 const int32_t o = opt(B * (size_t)(q ? t[T_MSB] : t[T_MSF]));
                 if (o >= 0) pl->o_all[q] = o;
             }
+    }
+    pl->bytes = (int32_t)at;
+    return true;
+}
+
+// The same for one forest solve alone.
+bool place_apply(const GridLayout &G, size_t sz, size_t vb, GridPlace *pl)
+{
+    const int32_t *t = G.tot;
+    size_t at = 0;
+    auto need = [&](size_t b) {
+        const int32_t o = (int32_t)at;
+        at += (b + 15) & ~size_t(15);
+        return o;
+    };
+    const size_t B = sz == 4 ? SlotSize<float>::B : SlotSize<double>::B;
+    *pl = GridPlace{};
+    pl->o_inv = -1;
+    pl->o_w = need(vb * (size_t)(t[T_MDZ] + 1));
+    pl->o_t = need(vb * (size_t)t[T_NT]);
+    pl->o_tp = need(3 * sz * (size_t)std::max(GW, t[T_MNO]));
+    if (at > (size_t)GRID_SMEM) return false;
+    for (int q = 0; q < 2; ++q) {
+        const size_t b = B * (size_t)(q ? t[T_MNB] : t[T_MNF]);
+        pl->o_nar[q] = b > 0 && at + b + 16 <= (size_t)GRID_SMEM ? need(b) : -1;
     }
     pl->bytes = (int32_t)at;
     return true;
@@ -2304,7 +2446,7 @@ sgp_status numeric(sgp_ctx *ctx, GridLayout &G, const sgp_factor *F, const GBuil
 sgp_status grid_build(sgp_ctx *ctx, sgp_factor *F, const sgp_matrix *M)
 {
     GridLayout &G = F->gl;
-    G.ok = 0;
+    G.ok = G.rows.ok = 0;
     const int32_t n = (int32_t)F->n, LV = F->levels;
     if (n == 0 || LV == 0 || LV > LMAX || !M || M->n != n || M->precision != F->precision) return SGP_OK;
     const bool f32 = F->precision == SGP_PREC_MIXED;
@@ -2315,8 +2457,9 @@ sgp_status grid_build(sgp_ctx *ctx, sgp_factor *F, const sgp_matrix *M)
     int32_t P = 1;
     SGP_TRY(part_count(ctx, n, 128, &P));
     const int32_t U = (n + P - 1) / P;
-    // p and w of the largest part must fit
-    if ((size_t)U * (f32 ? 24 : 48) > (size_t)GRID_SMEM) return SGP_OK;
+    // p and w of the largest part must fit; in FP64 w alone serves the forest
+    // solve, whose launch has no p
+    if ((size_t)U * 24 > (size_t)GRID_SMEM) return SGP_OK;
     // The subtree bound trades the number of top vertices (every block reads
     // its rows of their inverse) and the length of the narrow levels against
     // the imbalance of the parts (half a subtree either way).  Measured, us
@@ -2420,7 +2563,10 @@ sgp_status grid_build(sgp_ctx *ctx, sgp_factor *F, const sgp_matrix *M)
     memcpy(G.tot, hs.t, sizeof(hs.t));
     G.top_slots[0] = hs.top[Q_NSF];
     G.top_slots[1] = hs.top[Q_NSB];
-    if (G.tot[T_ERR] || G.tot[T_MDZ] > 8190 || !rows_place(G, R, M, f32, true)) return SGP_OK;
+    if (G.tot[T_ERR] || G.tot[T_MDZ] > 8190) return SGP_OK;
+    GridPlace pl;
+    const bool rows = rows_place(G, R, M, f32, true), apply = !f32 && place_apply(G, 8, 24, &pl);
+    if (!rows && !apply) return SGP_OK;
     G.nr_max = (int64_t)NRmax;
     for (int q = 0; q < 2; ++q) {
         const size_t slots = (size_t)G.tot[q ? T_SB : T_SF];
@@ -2436,7 +2582,7 @@ sgp_status grid_build(sgp_ctx *ctx, sgp_factor *F, const sgp_matrix *M)
     if (G.tot[T_NT] > 0)
         SGP_TRY(sgp_launch(ctx, "k_gr_program", k_gr_program<double>, dim3(1, 2), dim3(GT), 0, g, P));
     LAUNCH(ctx, k_gr_slots, 1, 1024, 0, g);
-    SGP_TRY(rows_fill(ctx, G, R, g, M, f32));
+    if (rows) SGP_TRY(rows_fill(ctx, G, R, g, M, f32));
     LAUNCH(ctx, k_gr_check, P + 1, GT, 0, g);
     const int32_t *td_src = sp + hs.top[Q_SOFF];
     if (f32)
@@ -2446,6 +2592,13 @@ sgp_status grid_build(sgp_ctx *ctx, sgp_factor *F, const sgp_matrix *M)
     SGP_TRY(read_back(ctx, hs.t, g.tot, sizeof(hs.t)));
     if (hs.t[T_ERR]) return sgp_fail(ctx, SGP_ERR_CUDA, "tree_factor: inconsistent grid layout (0x%x)", hs.t[T_ERR]);
     G.prec = F->precision;
+    // packets of a forest solve alone (its callers' vectors are FP64)
+    G.apply_bytes = 0;
+    if (apply) {
+        const size_t b = 8 * (size_t)Pkt<double>::W * ((size_t)G.tot[T_Z] + (size_t)G.tot[T_NT]) + 16;
+        SGP_TRY(buf_ensure(ctx, G.apply, b));
+        G.apply_bytes = b;
+    }
     G.ok = 1;
     return SGP_OK;
 }
@@ -2527,7 +2680,7 @@ void grid_rows_release(GridRows &R)
 void grid_release(GridLayout &G)
 {
     for (DBuf *d : {&G.hdr, &G.dtot, &G.ws, &G.zi, &G.zslot, &G.tlk, &G.i_of_t, &G.t_of_i, &G.prog[0], &G.prog[1], &G.D,
-                    &G.inv, &G.tD})
+                    &G.inv, &G.tD, &G.apply})
         if (d->p) cudaFree(d->p);
     for (DBuf &d : G.scr)
         if (d.p) cudaFree(d.p);
@@ -2538,7 +2691,7 @@ void grid_release(GridLayout &G)
 template <typename T>
 bool grid_ready(const sgp_ctx *ctx, const sgp_factor *F, const sgp_matrix *M)
 {
-    return ctx->fused && F && M && F->gl.ok && F->gl.rows.mgen == M->gen &&
+    return ctx->fused && F && M && F->gl.ok && F->gl.rows.ok && F->gl.rows.mgen == M->gen &&
            F->gl.prec == (sizeof(T) == 4 ? SGP_PREC_MIXED : SGP_PREC_F64);
 }
 template bool grid_ready<float>(const sgp_ctx *, const sgp_factor *, const sgp_matrix *);
@@ -2551,6 +2704,37 @@ size_t grid_work_bytes(const GridLayout &G, size_t sz)
     const int32_t *t = G.tot;
     const size_t wb = sz == 4 ? 32 : 48, nr = (size_t)t[T_NR];
     return 3 * (3 * sz * nr + 256) + wb * (nr + (size_t)t[T_NT] + (size_t)t[T_Z]) + 512 + 2 * PMAX * 4 * 8 + 2048;
+}
+
+// x = P^-1 b of an FP64 factor in one launch, without a host synchronisation;
+// a wait that gives up leaves NaN.  orig_of: the caller's order, or NULL for
+// the internal one; nothing is done when *done is set.
+bool grid_apply_ready(const sgp_ctx *ctx, const sgp_factor *F)
+{
+    return ctx->fused && F->gl.ok && F->gl.prec == SGP_PREC_F64 && F->gl.apply_bytes > 0;
+}
+sgp_status grid_apply(sgp_ctx *ctx, const sgp_factor *F, const double *b, double *x, const int32_t *orig_of, const int *done)
+{
+    const GridLayout &G = F->gl;
+    const int32_t *t = G.tot;
+    GridArgs a{};
+    if (!place_apply(G, 8, 24, &a.pl)) return sgp_fail(ctx, SGP_ERR_CUDA, "tree solve: the grid layout does not fit");
+    a.P = G.P; a.nt = t[T_NT]; a.ntp = pad32(a.nt); a.nslots = t[T_Z];
+    a.hdr = bp<const int32_t>(G.hdr); a.ws = bp<const int32_t>(G.ws);
+    a.i_of_t = bp<const int32_t>(G.i_of_t);
+    a.zi = bp<const int32_t>(G.zi); a.zslot = bp<const int32_t>(G.zslot); a.tlk = bp<const int32_t>(G.tlk);
+    for (int q = 0; q < 2; ++q) a.prog[q] = bp<const char>(G.prog[q]);
+    a.D = G.D.p; a.inv = G.inv.p;
+    a.F = b; a.x = x;
+    a.err = bp<int>(G.apply);
+    a.lx = reinterpret_cast<unsigned long long *>(G.apply.p) + 2;
+    SGP_CUDA(ctx, cudaMemsetAsync(G.apply.p, 0, G.apply_bytes, ctx->stream));
+    void *args[] = {&a, &orig_of, &done};
+    const auto kern = k_apply_grid<double, 24>;
+    SGP_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, GRID_SMEM));
+    SGP_CUDA(ctx, cudaLaunchCooperativeKernel((const void *)kern, dim3(G.P), dim3(GT), args, (size_t)a.pl.bytes, ctx->stream));
+    ctx->launches++;
+    return SGP_OK;
 }
 
 // One PCG run on Gamma x = F (vectors in the matrix's internal order) in one

@@ -60,6 +60,8 @@ struct GridLayout {
     int32_t tot[24] = {0}, top_slots[2] = {0, 0};   // totals and maxima over the parts; slots of the top's programs
     DBuf hdr, dtot, ws, zi, zslot, tlk, i_of_t, t_of_i;
     DBuf prog[2], D, inv, tD;
+    DBuf apply;                                     // error word and packets of a forest solve alone
+    size_t apply_bytes = 0;
     DBuf scr[SGP_GRID_SCRATCH];
     GridRows rows;                                  // of the matrix the layout was built from
 };
@@ -265,6 +267,8 @@ void grid_release(GridLayout &G);
 void grid_rows_release(GridRows &R);
 template <typename T>
 bool grid_ready(const sgp_ctx *ctx, const sgp_factor *F, const sgp_matrix *M);
+bool grid_apply_ready(const sgp_ctx *ctx, const sgp_factor *F);
+sgp_status grid_apply(sgp_ctx *ctx, const sgp_factor *F, const double *b, double *x, const int32_t *orig_of, const int *done);
 size_t grid_work_bytes(const GridLayout &G, size_t sz);
 template <typename T>
 sgp_status grid_pcg(sgp_ctx *ctx, const sgp_matrix *M, const GridLayout &G, const GridRows &R, int precond, const T *F, T *x,
