@@ -40,16 +40,105 @@ __device__ __forceinline__ void row_product(const Blk<T> &B, const int32_t *__re
     }
 }
 
-// y = Gamma v  (plain)
-template <typename T>
-__global__ void k_spmv(Blk<T> B, const int32_t *__restrict__ row_ptr, T gamma0, int64_t n,
-                       const T *__restrict__ v, T *y)
+// y = Gamma v, FP64, a lane per row.  Bound by the FP64 pipe (2 fused multiply-
+// adds per clock and SM; 12 operations per slot: three differences, nine
+// multiply-adds; 98 us of it at 1e6 cells and 4.7e6 slots), and a warp runs as
+// long as its longest row: rows in memory order keep 49% of the lanes busy at
+// 4.7 slots a row, so the block deals its R rows out in order of length (76%
+// with R = 128, 92% with 512, 95% with 1024).  The result goes straight to the
+// caller's order (orig_of) when given.  1e6 cells, with the gather of v: 363 ->
+// 172 us.
+template <int R, int NT>
+__global__ void __launch_bounds__(NT, 1024 / NT) k_product64(Blk<double> B, const int32_t *__restrict__ row_ptr, double gamma0,
+                                                  int64_t n, const double *__restrict__ v,
+                                                  const int32_t *__restrict__ orig_of, double *__restrict__ y)
 {
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    T vi[3], yi[3];
-    row_product(B, row_ptr, gamma0, v, i, vi, yi);
-    y[3 * i] = yi[0]; y[3 * i + 1] = yi[1]; y[3 * i + 2] = yi[2];
+    __shared__ int32_t cnt[64], row[R];
+    const int tid = threadIdx.x;
+    const int64_t i0 = blockIdx.x * (int64_t)R;
+    constexpr int K = R / NT;
+    for (int k = tid; k < 64; k += NT) cnt[k] = 0;
+    __syncthreads();
+    int len[K], rank[K];
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        const int64_t i = i0 + k * NT + tid;
+        len[k] = i < n ? 63 - min(row_ptr[i + 1] - row_ptr[i], 63) : 63;   // the longest first
+    }
+#pragma unroll
+    for (int k = 0; k < K; ++k) rank[k] = atomicAdd(&cnt[len[k]], 1);
+    __syncthreads();
+    if (tid < 32) {
+        const int32_t a = cnt[2 * tid], b = cnt[2 * tid + 1];
+        int32_t s = a + b;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const int32_t t = __shfl_up_sync(0xffffffffu, s, d);
+            if (tid >= d) s += t;
+        }
+        cnt[2 * tid] = s - a - b;
+        cnt[2 * tid + 1] = s - b;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < K; ++k) row[cnt[len[k]] + rank[k]] = k * NT + tid;
+    __syncthreads();
+    for (int k = 0; k < K; ++k) {
+        // a warp's groups of 32 rows: long and short ones
+        const int64_t i = i0 + row[k & 1 ? (k + 1) * NT - 32 - (tid & ~31) + (tid & 31) : k * NT + tid];
+        if (i >= n) continue;
+        const double v0 = v[3 * i], v1 = v[3 * i + 1], v2 = v[3 * i + 2];
+        double y0 = gamma0 * v0, y1 = gamma0 * v1, y2 = gamma0 * v2;
+        int32_t s = row_ptr[i];
+        const int32_t e = row_ptr[i + 1];
+        // two slots a turn in sums of their own (one chain of fused multiply-
+        // adds over all slots rounds a fifth worse); the next blocks are loaded
+        // while these ones' gathers and products run
+        double z0 = 0.0, z1 = 0.0, z2 = 0.0;
+        typename Blk<double>::Raw Q{}, R2{};
+        if (s < e) {
+            Q = B.fetch(s);
+            R2 = B.fetch(min(s + 1, e - 1));
+        }
+        for (; s < e; s += 2) {
+            const bool two = s + 1 < e;
+            double S[6], U[6];
+            int32_t j, k;
+            B.expand(Q, S, j);
+            B.expand(R2, U, k);
+            const double w0 = v[3 * (int64_t)j], w1 = v[3 * (int64_t)j + 1], w2 = v[3 * (int64_t)j + 2];
+            const double x0 = v[3 * (int64_t)k], x1 = v[3 * (int64_t)k + 1], x2 = v[3 * (int64_t)k + 2];
+            Q = B.fetch(min(s + 2, e - 1));
+            R2 = B.fetch(min(s + 3, e - 1));
+            const double d0 = v0 - w0, d1 = v1 - w1, d2 = v2 - w2;
+            y0 = fma(S[0], d0, y0); y0 = fma(S[1], d1, y0); y0 = fma(S[2], d2, y0);
+            y1 = fma(S[1], d0, y1); y1 = fma(S[3], d1, y1); y1 = fma(S[4], d2, y1);
+            y2 = fma(S[2], d0, y2); y2 = fma(S[4], d1, y2); y2 = fma(S[5], d2, y2);
+            if (two) {
+                const double c0 = v0 - x0, c1 = v1 - x1, c2 = v2 - x2;
+                z0 = fma(U[0], c0, z0); z0 = fma(U[1], c1, z0); z0 = fma(U[2], c2, z0);
+                z1 = fma(U[1], c0, z1); z1 = fma(U[3], c1, z1); z1 = fma(U[4], c2, z1);
+                z2 = fma(U[2], c0, z2); z2 = fma(U[4], c1, z2); z2 = fma(U[5], c2, z2);
+            }
+        }
+        y0 += z0; y1 += z1; y2 += z2;
+        const int64_t o = orig_of ? orig_of[i] : i;
+        y[3 * o] = y0; y[3 * o + 1] = y1; y[3 * o + 2] = y2;
+    }
+}
+sgp_status product64(sgp_ctx *ctx, const sgp_matrix *M, const double *v, const int32_t *orig_of, double *y)
+{
+    const Blk<double> B = make_blk<double>(M);
+    const int32_t *rp = bp<const int32_t>(M->row_ptr);
+    const int64_t n = M->n;
+    // from about 100 blocks of 1024 rows on (us a call with the gather of v,
+    // 1024 rows against 128: 40,000 cells 36 and 25, 80,000 37.5 and 33.4,
+    // 100,000 37.5 both, 150,000 40 and 48, 300,000 64 and 76, 1e6 175 and 210)
+    if (n >= 100000)
+        LAUNCH(ctx, (k_product64<1024, 512>), (unsigned)((n + 1023) / 1024), 512, 0, B, rp, M->gamma0, n, v, orig_of, y);
+    else
+        LAUNCH(ctx, (k_product64<128, 128>), (unsigned)((n + 127) / 128), 128, 0, B, rp, M->gamma0, n, v, orig_of, y);
+    return SGP_OK;
 }
 
 // PCG product q = Gamma p with p^T q; the last block sets alpha = rho / p^T q.
@@ -1226,8 +1315,7 @@ static sgp_status small_pcg(sgp_ctx *ctx, const sgp_matrix *M, const sgp_factor 
 // network's loss and scaling).
 sgp_status spmv64(sgp_ctx *ctx, const sgp_matrix *M, const double *v, double *y)
 {
-    LAUNCH(ctx, k_spmv<double>, grid_for(M->n, 128), 128, 0, make_blk<double>(M), bp<const int32_t>(M->row_ptr),
-           M->gamma0, M->n, v, y);
+    SGP_TRY(product64(ctx, M, v, nullptr, y));
     return SGP_OK;
 }
 
@@ -1268,16 +1356,14 @@ sgp_status sgp_spmv(sgp_ctx *ctx, const sgp_matrix *M, const double *v, double *
     const int64_t n = M->n;
     if (n == 0) return SGP_OK;
     // caller order -> internal order -> product -> caller order
-    SGP_TRY(scratch_ensure(ctx, sizeof(double) * 6 * n + 1024));
-    double *vi = reinterpret_cast<double *>(ctx->d_scratch), *yi = vi + 3 * n;
+    SGP_TRY(scratch_ensure(ctx, sizeof(double) * 3 * n + 1024));
+    double *vi = reinterpret_cast<double *>(ctx->d_scratch);
     const int32_t *orig_of = bp<const int32_t>(M->orig_of);
     LAUNCH(ctx, k_to_internal<double>, grid_for(n, SGP_BLOCK), SGP_BLOCK, 0, n, orig_of, v, vi);
     cudaEvent_t ev;
     SGP_TRY(kt_begin(ctx, SGP_KT_SPMV, &ev));
-    LAUNCH(ctx, k_spmv<double>, grid_for(n, 128), 128, 0, make_blk<double>(M), bp<const int32_t>(M->row_ptr),
-           M->gamma0, n, (const double *)vi, yi);
+    SGP_TRY(product64(ctx, M, vi, orig_of, y));
     SGP_TRY(kt_end(ctx, SGP_KT_SPMV, ev));
-    LAUNCH(ctx, k_to_caller<double>, grid_for(n, SGP_BLOCK), SGP_BLOCK, 0, n, orig_of, (const double *)yi, y);
     return SGP_OK;
 }
 
