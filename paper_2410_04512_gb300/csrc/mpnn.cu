@@ -273,30 +273,50 @@ __global__ void __launch_bounds__(TB) k_mp_out_t(int64_t n, const float *__restr
     reinterpret_cast<float4 *>(dZ)[t] = relu_mask(reinterpret_cast<const float4 *>(Hm)[t], make_float4(a[0], a[1], a[2], a[3]));
 }
 
-// c = W_out h3 + b_out (kept), v0 = sum_k c_k b^(k) in FP64; 16 lanes per node.
+// c = W_out h3 + b_out (kept), v0 = sum_k c_k b^(k) in FP64.  16 lanes per node
+// for c, four nodes each; then a lane per component of v0, so that the FP64
+// instructions run on full warps (with three of 16 lanes: 22 us at 1e5
+// cells).
+constexpr int ON = 64;   // nodes per block
 __global__ void __launch_bounds__(TB) k_mp_out(int64_t n, const float *__restrict__ h3, const __nv_bfloat16 *__restrict__ Wout,
                                                const __nv_bfloat16 *__restrict__ bout, const double *__restrict__ b0,
                                                const double *__restrict__ b1, const double *__restrict__ b2, float *c,
                                                double *v0)
 {
-    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, i = t >> 4;
-    if (i >= n) return;
-    const int lane = threadIdx.x & 31, l = lane & 15;
-    const unsigned mask = 0xffffu << (lane & 16);
-    const float4 h = reinterpret_cast<const float4 *>(h3)[t];
-    float ck[KB];
+    __shared__ float cs[ON * KB];
+    const int64_t base = blockIdx.x * (int64_t)ON;
+    const int l = threadIdx.x & 15, node = threadIdx.x >> 4;
+    const int nn = (int)min((int64_t)ON, n - base);
+    float w[KB][4], bk[KB];
 #pragma unroll
     for (int k = 0; k < KB; ++k) {
-        const __nv_bfloat16 *w = Wout + k * H + 4 * l;
-        ck[k] = fmaf(h.x, bf(w, 0), fmaf(h.y, bf(w, 1), fmaf(h.z, bf(w, 2), h.w * bf(w, 3))));
+        bk[k] = bf(bout, k);
 #pragma unroll
-        for (int b = 8; b > 0; b >>= 1) ck[k] += __shfl_xor_sync(mask, ck[k], b);
-        ck[k] += bf(bout, k);
+        for (int v = 0; v < 4; ++v) w[k][v] = bf(Wout, k * H + 4 * l + v);
     }
-    if (l < 3) {
-        c[i * KB + l] = l == 0 ? ck[0] : l == 1 ? ck[1] : ck[2];
-        v0[3 * i + l] = (double)ck[0] * b0[3 * i + l] + (double)ck[1] * b1[3 * i + l] + (double)ck[2] * b2[3 * i + l];
+    float4 h[ON / 16];
+#pragma unroll
+    for (int u = 0; u < ON / 16; ++u)
+        h[u] = node + 16 * u < nn ? reinterpret_cast<const float4 *>(h3 + (base + node + 16 * u) * H)[l]
+                                  : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int u = 0; u < ON / 16; ++u) {
+        float ck[KB];
+#pragma unroll
+        for (int k = 0; k < KB; ++k) {
+            ck[k] = fmaf(h[u].x, w[k][0], fmaf(h[u].y, w[k][1], fmaf(h[u].z, w[k][2], h[u].w * w[k][3])));
+#pragma unroll
+            for (int b = 8; b > 0; b >>= 1) ck[k] += __shfl_xor_sync(0xffffffffu, ck[k], b);
+            ck[k] += bk[k];
+        }
+        if (l < KB) cs[(node + 16 * u) * KB + l] = l == 0 ? ck[0] : l == 1 ? ck[1] : ck[2];
     }
+    __syncthreads();
+    if (threadIdx.x >= 3 * nn) return;
+    const float *q = cs + threadIdx.x / 3 * KB;
+    const int64_t at = 3 * base + threadIdx.x;
+    c[at] = cs[threadIdx.x];
+    v0[at] = (double)q[0] * b0[at] + (double)q[1] * b1[at] + (double)q[2] * b2[at];
 }
 
 // out[0] = x . y, out[1] = z . w over 3n values (blocks, then the last
@@ -372,58 +392,42 @@ __global__ void k_mp_scale(int64_t n3, const double *__restrict__ nd, double *v0
     if (isfinite(alpha)) v0[k] *= alpha;
 }
 
-// Per-block partial of G[o][k] = sum_n dZ[n][o] X[n][k] over the block's
-// CHUNK nodes, plus the bias gradient sum_n dZ[n][o] in G[DOUT][...].
-template <int D1, int D2, int DOUT>
-__global__ void __launch_bounds__(TB) k_mp_wgrad(int64_t n, const float *__restrict__ dZ, const float *__restrict__ X1,
-                                                 const float *__restrict__ X2, float *partial)
+// Per-block partial of a weight gradient over the block's CHUNK nodes.  The
+// first and the last layer, one side A of 64 columns and one side B of K: G =
+// sum_n A[n][f] B[n][k] (AZ: A is dZ, f the output; else B is), and the bias
+// gradient, the sum of dZ, behind it.  A thread keeps column f against all K,
+// over every fourth node, straight from memory.
+template <int K, bool AZ>
+__global__ void __launch_bounds__(TB) k_mp_wgrad_thin(int64_t n, const float *__restrict__ A, const float *__restrict__ B,
+                                                      float *__restrict__ partial)
 {
-    constexpr int DI = D1 + D2;
-    constexpr int NG = DOUT * DI + DOUT;
-    constexpr int PER = (NG + TB - 1) / TB;
-    constexpr int TILE = 64;
-    __shared__ float zs[TILE][DOUT];
-    __shared__ float xs[TILE][DI];
-    float acc[PER];
+    constexpr int NS = TB / H, NG = K * H + (AZ ? H : K);
+    __shared__ float sh[NS][(K + 1) * H];
+    const int f = threadIdx.x % H, s = threadIdx.x / H;
+    const int64_t n0 = (int64_t)blockIdx.x * CHUNK, n1 = n < n0 + CHUNK ? n : n0 + CHUNK;
+    float acc[K + 1];
 #pragma unroll
-    for (int q = 0; q < PER; ++q) acc[q] = 0.f;
-    const int64_t n0 = (int64_t)blockIdx.x * CHUNK;
-    const int64_t n1 = n < n0 + CHUNK ? n : n0 + CHUNK;
-    for (int64_t t0 = n0; t0 < n1; t0 += TILE) {
-        __syncthreads();
-        for (int t = threadIdx.x; t < TILE * DOUT; t += TB) {
-            const int s = t / DOUT, o = t % DOUT;
-            const int64_t i = t0 + s;
-            zs[s][o] = i < n1 ? dZ[i * DOUT + o] : 0.f;
-        }
-        for (int t = threadIdx.x; t < TILE * DI; t += TB) {
-            const int s = t / DI, k = t % DI;
-            const int64_t i = t0 + s;
-            float v = 0.f;
-            if (i < n1) v = k < D1 ? X1[i * D1 + k] : X2[i * D2 + (k - D1)];
-            xs[s][k] = v;
-        }
-        __syncthreads();
+    for (int k = 0; k <= K; ++k) acc[k] = 0.f;
+#pragma unroll 4
+    for (int64_t i = n0 + s; i < n1; i += NS) {
+        const float a = A[i * H + f];
 #pragma unroll
-        for (int q = 0; q < PER; ++q) {
-            const int g = threadIdx.x + q * TB;
-            if (g < NG) {
-                float a = acc[q];
-                if (g < DOUT * DI) {
-                    const int o = g / DI, k = g % DI;
-                    for (int s = 0; s < TILE; ++s) a = fmaf(zs[s][o], xs[s][k], a);
-                } else {
-                    const int o = g - DOUT * DI;
-                    for (int s = 0; s < TILE; ++s) a += zs[s][o];
-                }
-                acc[q] = a;
-            }
-        }
+        for (int k = 0; k < K; ++k) acc[k] = fmaf(a, B[i * K + k], acc[k]);
+        if (AZ) acc[K] += a;
+        else if (f < K) acc[K] += B[i * K + f];
     }
 #pragma unroll
-    for (int q = 0; q < PER; ++q) {
-        const int g = threadIdx.x + q * TB;
-        if (g < NG) partial[(int64_t)blockIdx.x * NG + g] = acc[q];
+    for (int k = 0; k <= K; ++k) sh[s][k * H + f] = acc[k];
+    __syncthreads();
+    float *o = partial + (int64_t)blockIdx.x * NG;
+    for (int g = threadIdx.x; g < NG; g += TB) {
+        // G index: AZ: f * K + k, bias f; else k * H + f, bias k
+        const bool bias = g >= K * H;
+        const int at = bias ? K * H + g - K * H : AZ ? (g % K) * H + g / K : g;
+        float t = 0.f;
+#pragma unroll
+        for (int q = 0; q < NS; ++q) t += sh[q][at];
+        o[g] = t;
     }
 }
 
@@ -604,8 +608,10 @@ static sgp_status wgrad(sgp_ctx *ctx, sgp_mpnn *N, int64_t n, const float *dZ, c
     float *part = bp<float>(N->part);
     if constexpr (D1 == H && D2 == H && DOUT == H)
         LAUNCH(ctx, k_mp_wgrad_layer, nb, TB, 0, n, dZ, X1, X2, part);
+    else if constexpr (DOUT == H)
+        LAUNCH(ctx, (k_mp_wgrad_thin<DI, true>), nb, TB, 0, n, dZ, X1, part);
     else
-        LAUNCH(ctx, (k_mp_wgrad<D1, D2, DOUT>), nb, TB, 0, n, dZ, X1, X2, part);
+        LAUNCH(ctx, (k_mp_wgrad_thin<DOUT, false>), nb, TB, 0, n, X1, dZ, part);
     LAUNCH(ctx, k_mp_wsum, grid_for(NG, 32), TB, 0, (int)nb, NG, (const float *)part, off_w, off_b, DOUT * DI,
            bp<float>(N->g));
     return SGP_OK;
@@ -707,7 +713,7 @@ static sgp_status mpnn_forward_internal(sgp_ctx *ctx, sgp_mpnn *N, const sgp_mat
         const int off = OFF_L0 + l * LAYER;
         SGP_TRY((dense<H, H, H, false, true>(ctx, n, h, a, pb + off, pb + off + H * H2, row_ptr, hn)));
     }
-    LAUNCH(ctx, k_mp_out, grid_for(16 * n, TB), TB, 0, n, (const float *)(hs + 3 * H * n), pb + OFF_WOUT, pb + OFF_BOUT,
+    LAUNCH(ctx, k_mp_out, (unsigned)((n + ON - 1) / ON), TB, 0, n, (const float *)(hs + 3 * H * n), pb + OFF_WOUT, pb + OFF_BOUT,
            (const double *)b0, (const double *)b1, (const double *)b2, bp<float>(N->c), bp<double>(N->v0w));
     SGP_TRY(kt_end(ctx, SGP_KT_WARM_LAYERS, ev));
     return SGP_OK;
