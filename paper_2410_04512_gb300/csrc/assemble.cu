@@ -210,6 +210,7 @@ sgp_status sgp_friction_assemble(sgp_ctx *ctx, const sgp_graph *G, const double 
     M->gamma0 = gamma0;
     M->precision = precision;
     M->batched = G->batched;
+    M->inst_row = G->inst_row;
     M->jac_valid = 0;
     M->gen = next_generation();
     const int64_t ns = 2 * m;

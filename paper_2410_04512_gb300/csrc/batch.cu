@@ -480,6 +480,18 @@ sgp_status pcg_b_run(sgp_ctx *ctx, const sgp_matrix *M, const sgp_factor *Fac, i
     return SGP_OK;
 }
 
+// the persistent solve's scalars in the form of the launches'
+void take_scalars(std::vector<BScal> &hs, const std::vector<Scal> &gs)
+{
+    for (size_t s = 0; s < hs.size(); ++s) {
+        hs[s] = BScal{};
+        hs[s].it = gs[s].it;
+        hs[s].status = gs[s].status;
+        hs[s].FF = gs[s].FF;
+        hs[s].rr = gs[s].rr;
+    }
+}
+
 }  // namespace
 
 extern "C" {
@@ -544,7 +556,14 @@ sgp_status sgp_pcg_solve_batched(sgp_ctx *ctx, const sgp_matrix *M, const sgp_fa
     // workspace
     const size_t v64 = sizeof(double) * 3 * n, v32 = sizeof(float) * 3 * n;
     const size_t tbl = sizeof(int32_t) * (2 * nch + 2 * n_inst + 4 + n);
-    size_t need = 6 * v64 + (mixed ? 6 * v32 : 0) + sizeof(double) * 2 * nch + sizeof(BScal) * n_inst +
+    // the persistent solve, all systems in one launch, where the factor's layout
+    // has their boundaries
+    std::vector<int32_t> grp;
+    const bool grid = opts->precond == SGP_PRECOND_TREE &&
+                      (mixed ? grid_ready<float>(ctx, Fac, M) : grid_ready<double>(ctx, Fac, M)) &&
+                      grid_groups(Fac->gl, n_inst, offsets, grp);
+    const size_t gw = grid ? grid_work_bytes(Fac->gl, mixed ? 4 : 8, (int)n_inst) + sizeof(int32_t) * grp.size() + 1024 : 0;
+    size_t need = gw + 6 * v64 + (mixed ? 6 * v32 : 0) + sizeof(double) * 2 * nch + sizeof(BScal) * n_inst +
                   sizeof(double) * 6 * n_inst + tbl + 18 * 4096;
     SGP_TRY(scratch_ensure(ctx, need));
     char *base = reinterpret_cast<char *>(ctx->d_scratch) + 256;
@@ -565,6 +584,8 @@ sgp_status sgp_pcg_solve_batched(sgp_ctx *ctx, const sgp_matrix *M, const sgp_fa
     double *d_nrm = reinterpret_cast<double *>(take(sizeof(double) * n_inst));
     double *d_tol2 = reinterpret_cast<double *>(take(sizeof(double) * n_inst));
     int *d_flags = reinterpret_cast<int *>(take(64));
+    int32_t *d_grp = reinterpret_cast<int32_t *>(take(sizeof(int32_t) * grp.size()));
+    char *gwork = take(gw);
     double *r = reinterpret_cast<double *>(take(v64));
     double *p = reinterpret_cast<double *>(take(v64));
     double *q = reinterpret_cast<double *>(take(v64));
@@ -601,6 +622,13 @@ sgp_status sgp_pcg_solve_batched(sgp_ctx *ctx, const sgp_matrix *M, const sgp_fa
     F = F_in;
     v = v_in;
 
+    GridGroups groups;
+    std::vector<Scal> gs(grid ? n_inst : 0);
+    if (grid) {
+        SGP_CUDA(ctx, cudaMemcpyAsync(d_grp, grp.data(), sizeof(int32_t) * grp.size(), cudaMemcpyHostToDevice, ctx->stream));
+        groups.n = (int)n_inst;
+        groups.grp = d_grp;
+    }
     Batch b{d_chunk_inst, d_chunk_row, d_inst_chunk, d_sc, d_part, d_flags, d_flags + 1, (int)n_inst};
     const unsigned G = (unsigned)nch;
     Blk<double> B64 = make_blk<double>(M);
@@ -610,9 +638,16 @@ sgp_status sgp_pcg_solve_batched(sgp_ctx *ctx, const sgp_matrix *M, const sgp_fa
     std::vector<sgp_solve_info> inf(n_inst);
     std::memset(inf.data(), 0, sizeof(sgp_solve_info) * n_inst);
     if (!mixed) {
-        SGP_TRY(pcg_b_run<double>(ctx, M, Fac, opts->precond, b, G, F, v, opts->x0_given, opts->tol, nullptr,
-                                  opts->maxit, r, p, q, w));
-        SGP_TRY(read_back(ctx, hs.data(), d_sc, sizeof(BScal) * n_inst));
+        if (grid) {
+            if (!opts->x0_given) SGP_CUDA(ctx, cudaMemsetAsync(v, 0, v64, ctx->stream));
+            SGP_TRY(grid_pcg<double>(ctx, M, Fac->gl, Fac->gl.rows, SGP_PRECOND_TREE, F, v, opts->x0_given, opts->tol,
+                                     opts->maxit, gwork, gs.data(), 0.0, 0, &groups));
+            take_scalars(hs, gs);
+        } else {
+            SGP_TRY(pcg_b_run<double>(ctx, M, Fac, opts->precond, b, G, F, v, opts->x0_given, opts->tol, nullptr,
+                                      opts->maxit, r, p, q, w));
+            SGP_TRY(read_back(ctx, hs.data(), d_sc, sizeof(BScal) * n_inst));
+        }
         for (int64_t s = 0; s < n_inst; ++s) {
             inf[s].iterations = hs[s].it;
             inf[s].status = hs[s].status;
@@ -661,6 +696,9 @@ sgp_status sgp_pcg_solve_batched(sgp_ctx *ctx, const sgp_matrix *M, const sgp_fa
             if (n_active == 0) break;
             SGP_CUDA(ctx, cudaMemcpyAsync(d_scale, scale.data(), sizeof(double) * n_inst, cudaMemcpyHostToDevice, ctx->stream));
             SGP_CUDA(ctx, cudaMemcpyAsync(d_nrm, nrm.data(), sizeof(double) * n_inst, cudaMemcpyHostToDevice, ctx->stream));
+            if (grid)
+                for (int64_t s = 0; s < n_inst; ++s)
+                    if (!active[s]) tol2[s] = -1.0;
             SGP_CUDA(ctx, cudaMemcpyAsync(d_tol2, tol2.data(), sizeof(double) * n_inst, cudaMemcpyHostToDevice, ctx->stream));
             // per-instance skip flags for the inner solve
             for (int64_t s = 0; s < n_inst; ++s) {
@@ -669,9 +707,16 @@ sgp_status sgp_pcg_solve_batched(sgp_ctx *ctx, const sgp_matrix *M, const sgp_fa
             }
             SGP_CUDA(ctx, cudaMemcpyAsync(d_sc, hs.data(), sizeof(BScal) * n_inst, cudaMemcpyHostToDevice, ctx->stream));
             LAUNCH(ctx, k_b_scale, G, BB, 0, b, (const double *)r, (const double *)d_scale, r32, d32);
-            SGP_TRY(pcg_b_run<float>(ctx, M, Fac, opts->precond, b, G, (const float *)r32, d32, 0, itol, d_tol2,
-                                     opts->maxit, s32, p32, q32, w32));
-            SGP_TRY(read_back(ctx, hs.data(), d_sc, sizeof(BScal) * n_inst));
+            if (grid) {
+                groups.tol2 = d_tol2;
+                SGP_TRY(grid_pcg<float>(ctx, M, Fac->gl, Fac->gl.rows, SGP_PRECOND_TREE, (const float *)r32, d32, 0, itol,
+                                        opts->maxit, gwork, gs.data(), 0.0, 0, &groups));
+                take_scalars(hs, gs);
+            } else {
+                SGP_TRY(pcg_b_run<float>(ctx, M, Fac, opts->precond, b, G, (const float *)r32, d32, 0, itol, d_tol2,
+                                         opts->maxit, s32, p32, q32, w32));
+                SGP_TRY(read_back(ctx, hs.data(), d_sc, sizeof(BScal) * n_inst));
+            }
             for (int64_t s = 0; s < n_inst; ++s)
                 if (active[s]) {
                     inf[s].iterations += hs[s].it;

@@ -1159,10 +1159,10 @@ sgp_status sgp_tree_factor(sgp_ctx *ctx, const sgp_matrix *M, const sgp_tree *T,
     int herr = 0;
     SGP_TRY(read_back(ctx, &herr, err, sizeof(int)));
     if (herr) return sgp_fail(ctx, SGP_ERR_NOT_SPD, "tree_factor: a pivot block is not positive definite");
-    // default tuning, one system: the grid solve's layout (0.25 ms at 1000
-    // cells: not where the one-block solve serves the factor); else the bins
+    // default tuning: the grid solve's layout (0.25 ms at 1000 cells: not where
+    // the one-block solve serves the factor); else the bins
     F->gl.ok = 0;
-    if (ctx->bin_cap == 0 && ctx->fused && !M->batched && !small_solve_fits(ctx, F)) SGP_TRY(grid_build(ctx, F, M));
+    if (ctx->bin_cap == 0 && ctx->fused && (M->batched || !small_solve_fits(ctx, F))) SGP_TRY(grid_build(ctx, F, M));
     if (F->gl.ok && F->gl.rows.ok) {
         F->bl.ok32 = F->bl.ok64 = 0;
         F->bl.mgen = 0;

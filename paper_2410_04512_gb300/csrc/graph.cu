@@ -306,6 +306,7 @@ static sgp_status collision_graph(sgp_ctx *ctx, int64_t n, int64_t n_inst, const
     G->n = n;
     G->m = 0;
     G->batched = n_inst > 1;
+    G->inst_row.assign(offsets, offsets + n_inst + 1);
     SGP_TRY(buf_ensure(ctx, G->up_ptr, sizeof(int32_t) * (size_t)(n + 1)));
     if (n == 0) {
         SGP_CUDA(ctx, cudaMemsetAsync(G->up_ptr.p, 0, sizeof(int32_t), ctx->stream));

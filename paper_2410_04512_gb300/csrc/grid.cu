@@ -42,6 +42,9 @@
 // cells 30.8 us (104), FP32 spheroid of 1e5 27.2 us (63), FP32 sheet of 2.5e5
 // 36.2 us (76), FP64 spheroid of 3e5 138 us (282), FP32 spheroid of 1e6 132
 // us (181).
+#include <algorithm>
+#include <cstddef>
+#include <cstring>
 #include <type_traits>
 
 #include "solver_common.cuh"
@@ -147,7 +150,10 @@ __global__ void k_gr_class(int32_t n, int32_t bmax, const int32_t *__restrict__ 
 }
 // part of every root: the subtree's middle in the running total of sizes;
 // anc: itself for roots and top vertices (seg: P for the top), else its parent
-__global__ void k_gr_roots(int32_t n, int32_t bmax, int32_t P, const int32_t *__restrict__ sz,
+// (a batch: instance s has the vertices [irow[s], irow[s+1]) and the parts
+// [ipart[s], ipart[s+1]), and its top vertices are segment P + s)
+__global__ void k_gr_roots(int32_t n, int32_t bmax, int32_t P, int32_t NI, const int32_t *__restrict__ irow,
+                           const int32_t *__restrict__ ipart, const int32_t *__restrict__ sz,
                            const int32_t *__restrict__ par, const int32_t *__restrict__ ord,
                            const int32_t *__restrict__ pre, int32_t *anc, int32_t *seg)
 {
@@ -157,10 +163,20 @@ __global__ void k_gr_roots(int32_t n, int32_t bmax, int32_t P, const int32_t *__
     const bool tp = s > bmax, rt = !tp && (u < 0 || sz[u] > bmax);
     anc[t] = (tp || rt) ? t : u;
     int32_t b = -1;
-    if (tp) b = P;
-    if (rt) {
-        const int64_t total = max(pre[n], 1);
-        b = (int32_t)min((int64_t)P - 1, ((int64_t)pre[ord[t]] + s / 2) * P / total);
+    if (tp || rt) {
+        const int32_t v = ord[t];
+        int32_t lo = 0, hi = NI;   // the instance: the last one that starts at or before v
+        while (hi - lo > 1) {
+            const int32_t mid = (lo + hi) >> 1;
+            if (irow[mid] <= v) lo = mid; else hi = mid;
+        }
+        if (tp) {
+            b = P + lo;
+        } else {
+            const int32_t p0 = ipart[lo], np = ipart[lo + 1] - p0, before = pre[irow[lo]];
+            const int64_t total = max(pre[irow[lo + 1]] - before, 1);
+            b = p0 + (int32_t)min((int64_t)np - 1, ((int64_t)(pre[v] - before) + s / 2) * np / total);
+        }
     }
     seg[t] = b;
 }
@@ -180,7 +196,7 @@ __global__ void k_gr_seg(int32_t n, const int32_t *__restrict__ anc, const int32
 __global__ void __launch_bounds__(GT) k_gr_split_count(int32_t n, int32_t ns, const int32_t *__restrict__ seg,
                                                        int32_t *hist)
 {
-    __shared__ int32_t h[PMAX + 1];
+    __shared__ int32_t h[2 * PMAX];
     for (int i = threadIdx.x; i < ns; i += GT) h[i] = 0;
     __syncthreads();
     const int32_t i0 = blockIdx.x * MS_ITEMS;
@@ -191,9 +207,9 @@ __global__ void __launch_bounds__(GT) k_gr_split_count(int32_t n, int32_t ns, co
 __global__ void __launch_bounds__(GT) k_gr_split_place(int32_t n, int32_t ns, const int32_t *__restrict__ seg,
                                                        const int32_t *__restrict__ off, int32_t *out, int32_t *lpos)
 {
-    __shared__ int32_t wc[GW][PMAX + 1];
+    __shared__ int32_t wc[GW][2 * PMAX];
     const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-    for (int i = threadIdx.x; i < GW * (PMAX + 1); i += GT) (&wc[0][0])[i] = 0;
+    for (int i = threadIdx.x; i < GW * 2 * PMAX; i += GT) (&wc[0][0])[i] = 0;
     __syncthreads();
     constexpr int PER = MS_ITEMS / GW;   // consecutive items of a warp
     const int32_t i0 = blockIdx.x * MS_ITEMS + w * PER;
@@ -228,21 +244,37 @@ __global__ void __launch_bounds__(GT) k_gr_split_place(int32_t n, int32_t ns, co
     }
 }
 
+// a batch: the instances' top segments become one, in order
+__global__ void k_gr_top_merge(int32_t n, int32_t P, int32_t nblk, const int32_t *__restrict__ off, int32_t *seg, int32_t *lpos)
+{
+    int32_t t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= n || seg[t] <= P) return;
+    lpos[t] += off[(size_t)seg[t] * nblk] - off[(size_t)P * nblk];
+    seg[t] = P;
+}
+
 // Row segments: part b's vertices, then the top vertices it owns, padded to
 // 32 rows; the top's own header.
-__global__ void __launch_bounds__(256) k_gr_rows(int32_t P, int32_t nblk, const int32_t *__restrict__ off, int32_t *hdr,
-                                                 int32_t *tot)
+__global__ void __launch_bounds__(256) k_gr_rows(int32_t P, int32_t NI, const int32_t *__restrict__ ipart, int32_t nblk,
+                                                 const int32_t *__restrict__ off, int32_t *hdr, int32_t *tot)
 {
     __shared__ int32_t sh[8];
     const int b = threadIdx.x;
-    const int32_t s0 = off[(size_t)P * nblk], s1 = off[(size_t)(P + 1) * nblk];
-    const int32_t nt = s1 - s0, tc = (nt + P - 1) / max(P, 1);
+    const int32_t s0 = off[(size_t)P * nblk], s1 = off[(size_t)(P + NI) * nblk];
+    const int32_t nt = s1 - s0;
     int32_t nv = 0, nto = 0, t0 = 0, so = 0;
     if (b < P) {
         so = off[(size_t)b * nblk];
         nv = off[(size_t)(b + 1) * nblk] - so;
-        t0 = min(nt, b * tc);
-        nto = min(nt, t0 + tc) - t0;
+        int32_t lo = 0, hi = NI;   // the part's instance and its top vertices
+        while (hi - lo > 1) {
+            const int32_t mid = (lo + hi) >> 1;
+            if (ipart[mid] <= b) lo = mid; else hi = mid;
+        }
+        const int32_t ta = off[(size_t)(P + lo) * nblk] - s0, te = off[(size_t)(P + lo + 1) * nblk] - s0,
+                      np = ipart[lo + 1] - ipart[lo], tc = (te - ta + np - 1) / max(np, 1);
+        t0 = min(te, ta + (b - ipart[lo]) * tc);
+        nto = min(te, t0 + tc) - t0;
     }
     int32_t total;
     const int32_t ro = gscan<256>(pad32(nv + nto), sh, &total);
@@ -1038,6 +1070,8 @@ struct GridPlace {
 };
 struct GridArgs {
     int32_t P, nt, ntp, x_given, timing, halo, nslots;
+    const int32_t *grp;        // per part: first and end part of its system, the system (NULL: one system)
+    const double *gtol2;       // per system: tol^2, or below 0 for none to solve (NULL: tol2 for all)
     const int32_t *hdr, *rh, *ws, *glen, *gso, *i_of_t, *zi, *zslot, *tlk, *hl;
     const char *prog[2];
     const uint16_t *perm;
@@ -1280,7 +1314,7 @@ __device__ __forceinline__ bool wait_packet(const unsigned long long *p, unsigne
 // after all blocks have written e - 1, that is, after they have read e - 2.
 constexpr int PK = (PMAX + 31) / 32;
 template <typename T, int NV>
-__device__ __forceinline__ bool exchange(unsigned long long *pk, int P, unsigned epoch, int *err, Acc<T> *v)
+__device__ __forceinline__ bool exchange(unsigned long long *pk, int p0, int P, unsigned epoch, int *err, Acc<T> *v)
 {
     const int lane = threadIdx.x & 31;
     unsigned long long *set = pk + (size_t)(epoch & 1u) * PMAX * 4;
@@ -1296,7 +1330,7 @@ __device__ __forceinline__ bool exchange(unsigned long long *pk, int P, unsigned
     // lanes without a packet of their own watch their block's
     const unsigned long long *at[PK];
 #pragma unroll
-    for (int u = 0; u < PK; ++u) at[u] = set + 4 * (lane + 32 * u < P ? lane + 32 * u : (int)blockIdx.x);
+    for (int u = 0; u < PK; ++u) at[u] = set + 4 * (lane + 32 * u < P ? p0 + lane + 32 * u : (int)blockIdx.x);
     unsigned long long a[NV][PK], b[NV][PK];
     bool ok = true;
     for (int it = 0;; ++it) {
@@ -1590,6 +1624,8 @@ struct Solve {
     typename Part<T>::type rho, stop2, rr;   // FP32 keeps these as pairs of floats
     T al, be;
     int go, bad;                         // the solve goes on; a wait gave up
+    int p0, np;                          // the system's parts
+    double tol2;
     unsigned epoch;
 };
 enum { OP_START, OP_RHO, OP_PQ, OP_RR, OP_RR_RZ, OP_RZ, OP_NONE };
@@ -1603,7 +1639,7 @@ __device__ __forceinline__ void decide(const GridArgs &a, Solve<double> &Z, int 
     case OP_START:
         S.FF = t;
         S.rr = t1;
-        S.stop2 = a.tol2 * t;
+        S.stop2 = Z.tol2 * t;
         S.done = t == 0.0 || t1 <= S.stop2;
         break;
     case OP_RHO:
@@ -1657,7 +1693,7 @@ __device__ __forceinline__ void decide(const GridArgs &a, Solve<float> &Z, int o
     switch (op) {
     case OP_START: {
         S.FF = (double)t.x + (double)t.y;
-        const double st = a.tol2 * S.FF;
+        const double st = Z.tol2 * S.FF;
         Z.stop2.x = (float)st;
         Z.stop2.y = (float)(st - (double)Z.stop2.x);
         S.stop2 = st;
@@ -1722,7 +1758,7 @@ __device__ __noinline__ void sums(const GridArgs &a, Solve<T> &Z, int op)
         if (lane < GW) v[1].join(Z.red[1][lane]);
         v[1].warp();
     }
-    const bool ok = two ? exchange<T, 2>(a.pk, a.P, epoch, a.err, v) : exchange<T, 1>(a.pk, a.P, epoch, a.err, v);
+    const bool ok = two ? exchange<T, 2>(a.pk, Z.p0, Z.np, epoch, a.err, v) : exchange<T, 1>(a.pk, Z.p0, Z.np, epoch, a.err, v);
     if (lane) return;
     Z.epoch = epoch;
     if (!ok) {
@@ -1736,15 +1772,21 @@ __device__ __noinline__ void sums(const GridArgs &a, Solve<T> &Z, int op)
 // A part's numbers: its vertices, rows (with its top vertices), the top
 // vertices that it reaches and their offset, its first top vertex.  It needs
 // z of `nout` top vertices (those it reaches, then those it owns); a row of
-// their inverse is cut into nch pieces, about one per warp.
+// their inverse, from tb to te (its own system's top vertices), is cut into
+// nch pieces, about one per warp.
 struct PartDims {
-    int32_t nv, nr, ro, t0, nz, zo, nout, nch, chunk;
+    int32_t nv, nr, ro, t0, nz, zo, nout, nch, chunk, tb, te;
 };
 __device__ __forceinline__ PartDims part_of(const GridArgs &a)
 {
     const int32_t *h = a.hdr + (size_t)Q_N * blockIdx.x;
-    PartDims g{h[Q_NV], h[Q_NR], h[Q_ROFF], h[Q_T0], h[Q_NZ], h[Q_ZOFF], 0, 1, 0};
-    const int32_t npc = (a.nt + 127) / 128;
+    PartDims g{h[Q_NV], h[Q_NR], h[Q_ROFF], h[Q_T0], h[Q_NZ], h[Q_ZOFF], 0, 1, 0, 0, a.nt};
+    if (a.grp && a.nt > 0) {
+        const int32_t *h0 = a.hdr + (size_t)Q_N * a.grp[3 * blockIdx.x], *h1 = a.hdr + (size_t)Q_N * (a.grp[3 * blockIdx.x + 1] - 1);
+        g.tb = h0[Q_T0];
+        g.te = h1[Q_T0] + h1[Q_NR] - h1[Q_NV];
+    }
+    const int32_t npc = (pad32(g.te) - (g.tb & ~31) + 127) / 128;
     g.nout = g.nz + g.nr - g.nv;
     g.nch = g.nout > 0 ? max(1, min(npc, GW / g.nout)) : 1;
     g.chunk = (npc + g.nch - 1) / g.nch * 128;
@@ -1758,32 +1800,36 @@ template <typename T, int VB>
 __device__ __forceinline__ void tree_up(const GridArgs &a, const PartDims &g, const Prog *s_prog, const T *D, uint32_t w,
                                         unsigned long long *trx, unsigned ep)
 {
+    // (in registers: the cells' accesses below are volatile, so that a field
+    // read from shared memory is read again at every use)
+    const int32_t nv = g.nv, nr = g.nr, nz = g.nz, zo = g.zo, t0 = g.t0;
     const unsigned long long e = (unsigned long long)ep << 32;
     const T zero[3] = {0, 0, 0};
-    for (int32_t z = (int)threadIdx.x; z < g.nz; z += GT) V3<T, VB>::st(w + (g.nr + z) * VB, zero);
+    for (int32_t z = (int)threadIdx.x; z < nz; z += GT) V3<T, VB>::st(w + (nr + z) * VB, zero);
     __syncthreads();
-    for (int32_t i = g.nv + (int)threadIdx.x; i < g.nr; i += GT) {
+    for (int32_t i = nv + (int)threadIdx.x; i < nr; i += GT) {
         T v[3];
         V3<T, VB>::ld(w + i * VB, v);
-        Pkt<T>::put(trx + (size_t)Pkt<T>::W * (g.t0 + i - g.nv), e, v);
+        Pkt<T>::put(trx + (size_t)Pkt<T>::W * (t0 + i - nv), e, v);
     }
     run<T, VB, true>(s_prog[0], w);
-    for (int32_t z = (int)threadIdx.x; z < g.nz; z += GT) {
+    for (int32_t z = (int)threadIdx.x; z < nz; z += GT) {
         T v[3];
-        V3<T, VB>::ld(w + (g.nr + z) * VB, v);
-        Pkt<T>::put(a.lx + (size_t)Pkt<T>::W * __ldg(a.zslot + g.zo + z), e, v);
+        V3<T, VB>::ld(w + (nr + z) * VB, v);
+        Pkt<T>::put(a.lx + (size_t)Pkt<T>::W * __ldg(a.zslot + zo + z), e, v);
     }
-    pivots<T, VB>(D, g.nv, w);
+    pivots<T, VB>(D, nv, w);
 }
 
 // Then, by the threads from `first` on, the parts' sums and the top's r.
 template <typename T, int VB>
-__device__ __forceinline__ bool gather_top(const GridArgs &a, uint32_t tw, const unsigned long long *trx, unsigned ep,
+__device__ __forceinline__ bool gather_top(const GridArgs &a, const PartDims &g, uint32_t tw, const unsigned long long *trx, unsigned ep,
                                            int first)
 {
     const int tid = threadIdx.x;
+    const int32_t te = g.te;
     bool ok = true;
-    for (int32_t i = tid - first; i < a.nt; i += GT - first) {
+    for (int32_t i = g.tb + tid - first; i < te; i += GT - first) {
         const int32_t k0 = __ldg(a.tlk + i), k1 = __ldg(a.tlk + i + 1);
         // r and the first two sums in flight together
         const unsigned long long *pv = trx + (size_t)Pkt<T>::W * i, *p0 = a.lx + (size_t)Pkt<T>::W * k0,
@@ -1820,9 +1866,11 @@ __device__ __forceinline__ void tree_down(const GridArgs &a, const PartDims &g, 
                                           uint32_t tw, T *tp)
 {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    for (int32_t it = warp; it < g.nout * g.nch; it += GW) {
-        const int32_t o = it / g.nch, k0 = (it - o * g.nch) * g.chunk, k1 = min(a.ntp, k0 + g.chunk);
-        const int32_t i = o < g.nz ? __ldg(a.zi + g.zo + o) : g.t0 + o - g.nz;
+    const int32_t nout = g.nout, nch = g.nch, chunk = g.chunk, nz = g.nz, zo = g.zo, t0 = g.t0, nr = g.nr, nv = g.nv,
+                  kb = g.tb & ~31, ke = pad32(g.te);
+    for (int32_t it = warp; it < nout * nch; it += GW) {
+        const int32_t o = it / nch, k0 = kb + (it - o * nch) * chunk, k1 = min(ke, k0 + chunk);
+        const int32_t i = o < nz ? __ldg(a.zi + zo + o) : t0 + o - nz;
         const T *f = inv + (size_t)(a.pl.o_inv >= 0 ? o : i) * 9 * a.ntp + lane;
         T z[3] = {0, 0, 0};
         constexpr int N = sizeof(T) == 4 ? 4 : 2;
@@ -1836,7 +1884,7 @@ __device__ __forceinline__ void tree_down(const GridArgs &a, const PartDims &g, 
             for (int u = 0; u < N; ++u) {
                 if (k + 32 * u >= k1) break;
                 T y[3];
-                V3<T, VB>::ld(tw + min(k + lane + 32 * u, a.nt - 1) * VB, y);
+                V3<T, VB>::ld(tw + (k + lane + 32 * u) * VB, y);   // 0 outside [tb, te)
 #pragma unroll
                 for (int c = 0; c < 3; ++c)
                     z[c] = fma(m[u][3 * c + 2], y[2], fma(m[u][3 * c + 1], y[1], fma(m[u][3 * c], y[0], z[c])));
@@ -1851,12 +1899,12 @@ __device__ __forceinline__ void tree_down(const GridArgs &a, const PartDims &g, 
         }
     }
     __syncthreads();
-    for (int32_t o = tid; o < g.nout; o += GT) {
+    for (int32_t o = tid; o < nout; o += GT) {
         T z[3] = {0, 0, 0};
-        for (int32_t k = o * g.nch; k < (o + 1) * g.nch; ++k) {
+        for (int32_t k = o * nch; k < (o + 1) * nch; ++k) {
             z[0] += tp[3 * k]; z[1] += tp[3 * k + 1]; z[2] += tp[3 * k + 2];
         }
-        V3<T, VB>::st(w + (o < g.nz ? g.nr + o : g.nv + o - g.nz) * VB, z);
+        V3<T, VB>::st(w + (o < nz ? nr + o : nv + o - nz) * VB, z);
     }
     __syncthreads();
     run<T, VB, false>(s_prog[1], w);
@@ -1871,7 +1919,17 @@ __global__ void __launch_bounds__(GT, 1) k_pcg_grid(const __grid_constant__ Grid
     __shared__ int32_t s_ws[2][W_N];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int32_t *h = a.hdr + (size_t)Q_N * blockIdx.x;
-    const PartDims g = part_of(a);
+    const int32_t p0 = a.grp ? a.grp[3 * blockIdx.x] : 0, gid = a.grp ? a.grp[3 * blockIdx.x + 2] : 0;
+    const double tol2 = a.gtol2 ? a.gtol2[gid] : a.tol2;
+    if (a.gtol2 && tol2 < 0.0) return;   // nothing to solve
+    // in registers, but where those are shortest (VB = 12; us per iteration in
+    // registers and in shared memory: 1e5 cells FP32 27.1 and 27.9, 3e5 FP64
+    // 136.1 and 136.2, 1e6 FP32 133.9 and 130.8)
+    __shared__ PartDims sg;
+    const PartDims rg = part_of(a);
+    if (VB == 12 && tid == 0) sg = rg;
+    if (VB == 12) __syncthreads();
+    const PartDims &g = VB == 12 ? sg : rg;
     const int32_t nv = g.nv, nr = g.nr, ro = g.ro, slot0 = a.rh[R_N * blockIdx.x + R_SLOT],
                   nh = a.rh[R_N * blockIdx.x + R_NH];
     T *ps = reinterpret_cast<T *>(sm + a.pl.o_p);
@@ -1911,6 +1969,10 @@ __global__ void __launch_bounds__(GT, 1) k_pcg_grid(const __grid_constant__ Grid
         if (tid == 0) {   // the spare cell
             const T zero[3] = {0, 0, 0};
             V3<T, VB>::st(w + (nr + g.nz) * VB, zero);
+        }
+        for (int i = tid; i < a.ntp; i += GT) {   // lanes beside the system's top vertices
+            const T zero[3] = {0, 0, 0};
+            V3<T, VB>::st(tw + i * VB, zero);
         }
         // the rows of the top's inverse that the part needs, when they fit
         inv = reinterpret_cast<const T *>(a.inv);
@@ -1961,6 +2023,9 @@ __global__ void __launch_bounds__(GT, 1) k_pcg_grid(const __grid_constant__ Grid
     if (tid == 0) {
         memset(&Z.S, 0, sizeof(Z.S));
         Z.S.maxit = a.maxit;
+        Z.tol2 = tol2;
+        Z.p0 = p0;
+        Z.np = (a.grp ? a.grp[3 * blockIdx.x + 1] : a.P) - p0;
         Z.S.mu = a.mu;
         Z.S.phi = a.mu > 0.0 ? 1.0 / a.mu : 0.0;
         Z.S.stopE = a.stopE;
@@ -2090,7 +2155,7 @@ __global__ void __launch_bounds__(GT, 1) k_pcg_grid(const __grid_constant__ Grid
         if (warp == 0 && phase > 0) {
             sums<T>(a, Z, PREC == 0 ? OP_RR : OP_RR_RZ);
         } else if (PREC == 0) {
-            if (!gather_top<T, VB>(a, tw, trx, ep + 1, first)) Z.bad = 1;
+            if (!gather_top<T, VB>(a, g, tw, trx, ep + 1, first)) Z.bad = 1;
         }
         __syncthreads();
         if (Z.bad) return;
@@ -2134,10 +2199,10 @@ __global__ void __launch_bounds__(GT, 1) k_pcg_grid(const __grid_constant__ Grid
 #pragma unroll
         for (int c = 0; c < 3; ++c) xo[3 * (size_t)v + c] = x[3 * i + c];
     }
-    if (blockIdx.x == 0 && tid == 0) {
+    if (blockIdx.x == p0 && tid == 0) {
         if (sizeof(T) == 4) Z.S.rr = pair_value(Z.rr);
-        *a.sc = Z.S;
-        if (a.timing) {
+        a.sc[gid] = Z.S;
+        if (a.timing && blockIdx.x == 0) {
             a.ns[0] = t_spmv;
             a.ns[1] = t_tree;
             a.ns[2] = t_vec;
@@ -2198,9 +2263,10 @@ __global__ void __launch_bounds__(GT, 1) k_apply_grid(const __grid_constant__ Gr
     }
     const T zero[3] = {0, 0, 0};
     if (tid == 0) V3<T, VB>::st(w + (g.nr + g.nz) * VB, zero);   // the spare cell
+    for (int i = a.nt + tid; i < a.ntp; i += GT) V3<T, VB>::st(tw + i * VB, zero);
     unsigned long long *trx = a.lx + (size_t)Pkt<T>::W * a.nslots;
     tree_up<T, VB>(a, g, s_prog, reinterpret_cast<const T *>(a.D) + 6 * (size_t)g.ro, w, trx, 1u);
-    if (!gather_top<T, VB>(a, tw, trx, 1u, 0)) s_bad = 1;
+    if (!gather_top<T, VB>(a, g, tw, trx, 1u, 0)) s_bad = 1;
     __syncthreads();
     const bool bad = s_bad != 0;
     if (!bad)
@@ -2248,7 +2314,7 @@ bool place(const GridLayout &G, int32_t mnh, size_t sz, size_t vb, bool tree, bo
     const size_t B = sz == 4 ? SlotSize<float>::B : SlotSize<double>::B;
     pl->o_p = need(3 * sz * (mnr + (halo ? (size_t)mnh : 0)));
     pl->o_w = need(vb * (size_t)(tree ? t[T_MDZ] + 1 : t[T_MNR]));
-    pl->o_t = need(vb * nt);
+    pl->o_t = need(vb * pad32((int32_t)nt));
     pl->o_tp = need(3 * sz * (tree ? (size_t)std::max(GW, t[T_MNO]) : 0));
     pl->o_misc = need(8 * (mnr / 32 + 1));
     if (at > (size_t)GRID_SMEM) return false;
@@ -2294,7 +2360,7 @@ bool place_apply(const GridLayout &G, size_t sz, size_t vb, GridPlace *pl)
     *pl = GridPlace{};
     pl->o_inv = -1;
     pl->o_w = need(vb * (size_t)(t[T_MDZ] + 1));
-    pl->o_t = need(vb * (size_t)t[T_NT]);
+    pl->o_t = need(vb * (size_t)pad32(t[T_NT]));
     pl->o_tp = need(3 * sz * (size_t)std::max(GW, t[T_MNO]));
     if (at > (size_t)GRID_SMEM) return false;
     for (int q = 0; q < 2; ++q) {
@@ -2456,7 +2522,34 @@ sgp_status grid_build(sgp_ctx *ctx, sgp_factor *F, const sgp_matrix *M)
     // 256, 53.9 with 512: more parts share the FP64 work, fewer exchange less.
     int32_t P = 1;
     SGP_TRY(part_count(ctx, n, 128, &P));
-    const int32_t U = (n + P - 1) / P;
+    int32_t U = (n + P - 1) / P;
+    // a batch: no part holds rows of two instances, and U is the smallest at
+    // which the instances' parts fit the device
+    std::vector<int64_t> &irow = G.irow;
+    irow.assign({0, (int64_t)n});
+    if (M->batched) irow = M->inst_row;
+    const int32_t NI = (int32_t)irow.size() - 1;
+    if (NI < 1 || irow[0] != 0 || irow[NI] != n || NI > PMAX) return SGP_OK;
+    G.ipart.assign(NI + 1, 0);
+    if (NI > 1) {
+        const int32_t most = std::min(ctx->num_sms, PMAX);
+        auto parts = [&](int64_t u) {
+            int64_t c = 0;
+            for (int32_t s = 0; s < NI; ++s) c += (irow[s + 1] - irow[s] + u - 1) / u;
+            return c;
+        };
+        int64_t lo = 127, hi = n;
+        if (parts(hi) > most) return SGP_OK;   // more instances than SMs
+        while (hi - lo > 1) {
+            const int64_t mid = (lo + hi) / 2;
+            if (parts(mid) <= most) hi = mid; else lo = mid;
+        }
+        U = (int32_t)hi;
+        P = (int32_t)parts(U);
+        for (int32_t s = 0; s < NI; ++s) G.ipart[s + 1] = G.ipart[s] + (int32_t)((irow[s + 1] - irow[s] + U - 1) / U);
+    } else {
+        G.ipart[1] = P;
+    }
     // p and w of the largest part must fit; in FP64 w alone serves the forest
     // solve, whose launch has no p
     if ((size_t)U * 24 > (size_t)GRID_SMEM) return SGP_OK;
@@ -2484,7 +2577,9 @@ sgp_status grid_build(sgp_ctx *ctx, sgp_factor *F, const sgp_matrix *M)
     g.pr_q = bp<const int32_t>(F->pr_q);
     g.pr_c = bp<const int32_t>(F->pr_c);
     int32_t *lp, *par, *sz_, *wv, *pre, *anc, *anc2, *rseg, *seg, *hist, *off, *sp, *lpos;
-    SGP_TRY(S.take((size_t)LV + 1, &lp));
+    SGP_TRY(S.take((size_t)LV + 1 + 2 * ((size_t)NI + 1), &lp));
+    const int32_t *d_irow = lp + LV + 1, *d_ipart = d_irow + NI + 1;
+    const int32_t NS = P + NI;   // segments: parts, then the instances' tops
     SGP_TRY(S.take(n, &par));
     SGP_TRY(S.take(n, &sz_));
     SGP_TRY(S.take(n, &wv));
@@ -2493,12 +2588,14 @@ sgp_status grid_build(sgp_ctx *ctx, sgp_factor *F, const sgp_matrix *M)
     SGP_TRY(S.take(n, &anc2));
     SGP_TRY(S.take(n, &rseg));
     SGP_TRY(S.take(n, &seg));
-    SGP_TRY(S.take((size_t)(P + 1) * nblk + 1, &hist));
-    SGP_TRY(S.take((size_t)(P + 1) * nblk + 1, &off));
+    SGP_TRY(S.take((size_t)NS * nblk + 1, &hist));
+    SGP_TRY(S.take((size_t)NS * nblk + 1, &off));
     SGP_TRY(S.take(n, &sp));
     SGP_TRY(S.take(n, &lpos));
-    SGP_CUDA(ctx, cudaMemcpyAsync(lp, F->lvl_ptr.data(), sizeof(int32_t) * ((size_t)LV + 1), cudaMemcpyHostToDevice,
-                                  ctx->stream));
+    std::vector<int32_t> tab(F->lvl_ptr.begin(), F->lvl_ptr.begin() + LV + 1);
+    tab.insert(tab.end(), irow.begin(), irow.end());
+    tab.insert(tab.end(), G.ipart.begin(), G.ipart.end());
+    SGP_CUDA(ctx, cudaMemcpyAsync(lp, tab.data(), sizeof(int32_t) * tab.size(), cudaMemcpyHostToDevice, ctx->stream));
     LAUNCH(ctx, k_gr_parent, grid_for(n, B), B, 0, n, g.pr_ptr, g.pr_q, g.pos, par, sz_);
     int l0 = 0;
     while (l0 < LV && F->lvl_ptr[l0 + 1] - F->lvl_ptr[l0] > 4096) {
@@ -2509,16 +2606,17 @@ sgp_status grid_build(sgp_ctx *ctx, sgp_factor *F, const sgp_matrix *M)
     if (l0 < LV) LAUNCH(ctx, k_gr_size_rest, 1, 1024, 0, (const int32_t *)lp, l0, LV, (const int32_t *)par, sz_);
     LAUNCH(ctx, k_gr_class, grid_for(n, B), B, 0, n, bmax, (const int32_t *)sz_, (const int32_t *)par, g.ord, wv);
     SGP_TRY(scan_exclusive_i32(ctx, wv, pre, n));
-    LAUNCH(ctx, k_gr_roots, grid_for(n, B), B, 0, n, bmax, P, (const int32_t *)sz_, (const int32_t *)par, g.ord,
+    LAUNCH(ctx, k_gr_roots, grid_for(n, B), B, 0, n, bmax, P, NI, d_irow, d_ipart, (const int32_t *)sz_, (const int32_t *)par, g.ord,
            (const int32_t *)pre, anc, rseg);
     for (int r = 0; (1 << r) <= LV + 1; ++r) {
         LAUNCH(ctx, k_gr_jump, grid_for(n, B), B, 0, n, (const int32_t *)anc, anc2);
         std::swap(anc, anc2);
     }
     LAUNCH(ctx, k_gr_seg, grid_for(n, B), B, 0, n, (const int32_t *)anc, (const int32_t *)rseg, seg);
-    LAUNCH(ctx, k_gr_split_count, nblk, GT, 0, n, P + 1, (const int32_t *)seg, hist);
-    SGP_TRY(scan_exclusive_i32(ctx, hist, off, (int64_t)(P + 1) * nblk));
-    LAUNCH(ctx, k_gr_split_place, nblk, GT, 0, n, P + 1, (const int32_t *)seg, (const int32_t *)off, sp, lpos);
+    LAUNCH(ctx, k_gr_split_count, nblk, GT, 0, n, NS, (const int32_t *)seg, hist);
+    SGP_TRY(scan_exclusive_i32(ctx, hist, off, (int64_t)NS * nblk));
+    LAUNCH(ctx, k_gr_split_place, nblk, GT, 0, n, NS, (const int32_t *)seg, (const int32_t *)off, sp, lpos);
+    if (NI > 1) LAUNCH(ctx, k_gr_top_merge, grid_for(n, B), B, 0, n, P, nblk, (const int32_t *)off, seg, lpos);
     const size_t NRmax = (size_t)pad32(n) + 32 * (size_t)P + 32, PB = (size_t)P + 1;
     SGP_TRY(ensure(ctx, G.hdr, (size_t)Q_N * PB, &g.hdr));
     SGP_TRY(ensure(ctx, G.dtot, T_N, &g.tot));
@@ -2544,7 +2642,7 @@ sgp_status grid_build(sgp_ctx *ctx, sgp_factor *F, const sgp_matrix *M)
     g.lp = lp; g.seg = seg; g.sp = sp; g.lpos = lpos;
     if (f32) g.col32 = reinterpret_cast<const float2 *>(bp<const float4>(M->blk32) + 2 * M->m);
     SGP_CUDA(ctx, cudaMemsetAsync(g.tot, 0, sizeof(int32_t) * T_N, ctx->stream));
-    LAUNCH(ctx, k_gr_rows, 1, 256, 0, P, nblk, (const int32_t *)off, g.hdr, g.tot);
+    LAUNCH(ctx, k_gr_rows, 1, 256, 0, P, NI, d_ipart, nblk, (const int32_t *)off, g.hdr, g.tot);
     const unsigned gy = (unsigned)std::max(1, std::min(8, U / GT));
     SGP_TRY(sgp_launch(ctx, "k_gr_row_maps", k_gr_row_maps, dim3(P, gy), dim3(GT), 0, g));
     LAUNCH(ctx, k_gr_part_count, P + 1, GT, 0, g);
@@ -2697,13 +2795,35 @@ bool grid_ready(const sgp_ctx *ctx, const sgp_factor *F, const sgp_matrix *M)
 template bool grid_ready<float>(const sgp_ctx *, const sgp_factor *, const sgp_matrix *);
 template bool grid_ready<double>(const sgp_ctx *, const sgp_factor *, const sgp_matrix *);
 
-// Device workspace of one grid solve in bytes (element size sz).
-size_t grid_work_bytes(const GridLayout &G, size_t sz)
+// The systems of a batched solve, offsets[0..n_inst], on the parts of a
+// factor: per part its system's parts and the system.  False where a system
+// does not begin and end with instances of the layout.
+bool grid_groups(const GridLayout &G, int64_t n_inst, const int64_t *offsets, std::vector<int32_t> &grp)
+{
+    grp.assign(3 * (size_t)G.P, 0);
+    for (int64_t s = 0; s < n_inst; ++s) {
+        if (offsets[s] == offsets[s + 1]) continue;
+        const auto a = std::upper_bound(G.irow.begin(), G.irow.end(), offsets[s]) - 1,
+                   e = std::lower_bound(G.irow.begin(), G.irow.end(), offsets[s + 1]);
+        if (a < G.irow.begin() || *a != offsets[s] || e == G.irow.end() || *e != offsets[s + 1]) return false;
+        const int32_t p0 = G.ipart[a - G.irow.begin()], p1 = G.ipart[e - G.irow.begin()];
+        for (int32_t p = p0; p < p1; ++p) {
+            grp[3 * p] = p0;
+            grp[3 * p + 1] = p1;
+            grp[3 * p + 2] = (int32_t)s;
+        }
+    }
+    return true;
+}
+
+// Device workspace of one grid solve in bytes (element size sz, ng systems).
+size_t grid_work_bytes(const GridLayout &G, size_t sz, int ng)
 {
     if (!G.ok) return 0;
     const int32_t *t = G.tot;
     const size_t wb = sz == 4 ? 32 : 48, nr = (size_t)t[T_NR];
-    return 3 * (3 * sz * nr + 256) + wb * (nr + (size_t)t[T_NT] + (size_t)t[T_Z]) + 512 + 2 * PMAX * 4 * 8 + 2048;
+    return 3 * (3 * sz * nr + 256) + wb * (nr + (size_t)t[T_NT] + (size_t)t[T_Z]) + 512 + 2 * PMAX * 4 * 8 + 2048 +
+           sizeof(Scal) * (size_t)ng;
 }
 
 // x = P^-1 b of an FP64 factor in one launch, without a host synchronisation;
@@ -2743,8 +2863,10 @@ sgp_status grid_apply(sgp_ctx *ctx, const sgp_factor *F, const double *b, double
 // Scal).
 template <typename T>
 sgp_status grid_pcg(sgp_ctx *ctx, const sgp_matrix *M, const GridLayout &G, const GridRows &R, int precond, const T *F, T *x,
-                    int x_given, double tol, int64_t maxit, void *work, void *hs, double mu, int stopE)
+                    int x_given, double tol, int64_t maxit, void *work, void *hs, double mu, int stopE,
+                    const GridGroups *groups)
 {
+    const int ng = groups ? groups->n : 1;
     const int32_t *t = G.tot;
     const bool tree = precond == SGP_PRECOND_TREE;
     GridArgs a{};
@@ -2757,15 +2879,16 @@ sgp_status grid_pcg(sgp_ctx *ctx, const sgp_matrix *M, const GridLayout &G, cons
         return p;
     };
     struct Out {
-        Scal sc;
         unsigned long long ns[4];
         int err, pad;
+        Scal sc[1];
     };
+    const size_t out_bytes = sizeof(Out) + sizeof(Scal) * (size_t)(ng - 1);
     const size_t wb = 8 * (size_t)Pkt<T>::W, nr = (size_t)t[T_NR];
     char *zero = take(0);
     a.pk = reinterpret_cast<unsigned long long *>(take(2 * PMAX * 4 * 8));
     a.lx = reinterpret_cast<unsigned long long *>(take(wb * ((size_t)t[T_Z] + (size_t)t[T_NT])));
-    Out *out = reinterpret_cast<Out *>(take(sizeof(Out)));
+    Out *out = reinterpret_cast<Out *>(take(out_bytes));
     if (R.halo) a.px = reinterpret_cast<unsigned long long *>(take(wb * nr));
     char *zend = take(0);
     if (!R.halo) a.pg = take(3 * sizeof(T) * nr);
@@ -2788,7 +2911,11 @@ sgp_status grid_pcg(sgp_ctx *ctx, const sgp_matrix *M, const GridLayout &G, cons
     a.maxit = maxit;
     a.stopE = stopE;
     a.err = &out->err;
-    a.sc = &out->sc;
+    a.sc = out->sc;
+    if (groups) {
+        a.grp = groups->grp;
+        a.gtol2 = groups->tol2;
+    }
     a.ns = out->ns;
     SGP_CUDA(ctx, cudaMemsetAsync(zero, 0, (size_t)(zend - zero), ctx->stream));
     void *args[] = {&a};
@@ -2811,13 +2938,17 @@ sgp_status grid_pcg(sgp_ctx *ctx, const sgp_matrix *M, const GridLayout &G, cons
     else
         SGP_TRY(pick(std::integral_constant<int, 12>{}));
     ctx->launches++;
+    std::vector<char> hb(out_bytes);
+    SGP_TRY(read_back(ctx, hb.data(), out, out_bytes));
     Out h;
-    SGP_TRY(read_back(ctx, &h, out, sizeof(h)));
-    if (h.err) {
-        h.sc.status = SGP_ERR_TIMEOUT;
-        h.sc.done = 1;
-    }
-    *reinterpret_cast<Scal *>(hs) = h.sc;
+    std::memcpy(&h, hb.data(), sizeof(h));
+    Scal *so = reinterpret_cast<Scal *>(hs);
+    std::memcpy(so, hb.data() + offsetof(Out, sc), sizeof(Scal) * (size_t)ng);
+    if (h.err)
+        for (int k = 0; k < ng; ++k) {
+            so[k].status = SGP_ERR_TIMEOUT;
+            so[k].done = 1;
+        }
     if (ctx->timing) {
         const int cls[3] = {SGP_KT_SPMV, SGP_KT_TREE_SOLVE, SGP_KT_PCG_VECTOR};
         for (int k = 0; k < 3; ++k) {
@@ -2826,13 +2957,13 @@ sgp_status grid_pcg(sgp_ctx *ctx, const sgp_matrix *M, const GridLayout &G, cons
                 continue;
             }
             ctx->kt_ms[cls[k]] += 1e-6 * (double)h.ns[k];
-            ctx->kt_n[cls[k]] += h.sc.it + (k == 1);
+            ctx->kt_n[cls[k]] += so[0].it + (k == 1);
         }
     }
     return SGP_OK;
 }
 #define GRID_PCG(T)                                                                                                      \
     template sgp_status grid_pcg<T>(sgp_ctx *, const sgp_matrix *, const GridLayout &, const GridRows &, int, const T *, \
-                                    T *, int, double, int64_t, void *, void *, double, int);
+                                    T *, int, double, int64_t, void *, void *, double, int, const GridGroups *);
 GRID_PCG(float)
 GRID_PCG(double)

@@ -64,6 +64,8 @@ struct GridLayout {
     size_t apply_bytes = 0;
     DBuf scr[SGP_GRID_SCRATCH];
     GridRows rows;                                  // of the matrix the layout was built from
+    std::vector<int64_t> irow;                      // instances: first rows
+    std::vector<int32_t> ipart;                     // and first parts
 };
 
 struct sgp_ctx {
@@ -258,6 +260,14 @@ bool small_solve_fits(const sgp_ctx *ctx, const sgp_factor *F);
 // factor's parts, grid_plain cuts a matrix into parts of rows; grid_pcg runs
 // it on internal-order vectors with `work` (grid_work_bytes) and returns the
 // final scalars.
+// Several systems in one solve (device arrays): grp, per part the system's
+// first and end part and the system; tol2, per system tol^2, below 0 to leave
+// it out (NULL: the call's for all).
+struct GridGroups {
+    int n = 0;
+    const int32_t *grp = nullptr;
+    const double *tol2 = nullptr;
+};
 struct GridLayout;
 struct GridRows;
 sgp_status grid_build(sgp_ctx *ctx, sgp_factor *F, const sgp_matrix *M);
@@ -269,10 +279,12 @@ template <typename T>
 bool grid_ready(const sgp_ctx *ctx, const sgp_factor *F, const sgp_matrix *M);
 bool grid_apply_ready(const sgp_ctx *ctx, const sgp_factor *F);
 sgp_status grid_apply(sgp_ctx *ctx, const sgp_factor *F, const double *b, double *x, const int32_t *orig_of, const int *done);
-size_t grid_work_bytes(const GridLayout &G, size_t sz);
+size_t grid_work_bytes(const GridLayout &G, size_t sz, int ng = 1);
 template <typename T>
 sgp_status grid_pcg(sgp_ctx *ctx, const sgp_matrix *M, const GridLayout &G, const GridRows &R, int precond, const T *F, T *x,
-                    int x_given, double tol, int64_t maxit, void *work, void *hs, double mu, int stopE);
+                    int x_given, double tol, int64_t maxit, void *work, void *hs, double mu, int stopE,
+                    const GridGroups *groups = nullptr);
+bool grid_groups(const GridLayout &G, int64_t n_inst, const int64_t *offsets, std::vector<int32_t> &grp);
 
 // Kernel timing hooks (no-ops unless enabled on the context).
 sgp_status kt_begin(sgp_ctx *ctx, int kclass, cudaEvent_t *ev);
@@ -285,6 +297,7 @@ sgp_status kt_collect(sgp_ctx *ctx);  // after a stream synchronisation
 struct sgp_graph {
     int64_t n = 0, m = 0;
     int batched = 0;   // built from several instances
+    std::vector<int64_t> inst_row;   // their offsets
     DBuf ij;       // m x 2 int32, canonical (i < j), sorted
     DBuf up_ptr;   // n + 1 int32: edges of row i are [up_ptr[i], up_ptr[i+1])
     // cell-list scratch kept for reuse
@@ -299,6 +312,7 @@ struct sgp_matrix {
     double gamma0 = 0;
     int32_t precision = SGP_PREC_F64;
     int batched = 0;   // assembled from a batched graph (solved per instance)
+    std::vector<int64_t> inst_row;   // its instances' offsets
     DBuf ij;         // m x 2 int32 (copy of the graph's edge list)
     DBuf row_ptr;    // n + 1 int32 over 2m directed slots, columns ascending in a row
     DBuf col;        // 2m int32

@@ -12,6 +12,7 @@ import oracle
 import paper_2410_04512_gb300 as sgp
 import workloads
 from gpu_common import GpuSystem, dev_tensor, oracle_system, rel_err, small_cube
+from test_gpu_batched import GpuBatch
 
 pytestmark = pytest.mark.gpu
 
@@ -87,6 +88,29 @@ def test_grid_rows_match_multi_launch(cuda_device, name, precond, precision):
         out.append((v.cpu().numpy(), info))
     assert abs(out[0][1].iterations - out[1][1].iterations) <= max(3, out[1][1].iterations // 20)
     assert rel_err(out[0][0], out[1][0]) <= 1e-8
+
+
+@pytest.mark.parametrize("precision", [sgp.PREC_F64, sgp.PREC_MIXED])
+@pytest.mark.parametrize("sizes,ends", [([300, 1200, 0, 1, 2500, 700, 2], None), ([300, 1200, 0, 1, 2500, 700, 2], [0, 1, 4, 5, 7]),
+                                        ([900, 20], [0, 2]), ([5] * 170, None)])
+def test_grid_batched(cuda_device, sizes, ends, precision):
+    """A batch on its instances' parts (or, the last, more instances than
+    thread blocks) against the level kernels; `ends`: the solve's systems as
+    runs of the graph's instances.  Bound as in the first test."""
+    out = []
+    for cap in (0, -1):
+        cx = sgp.Context(0)
+        cx.set_tuning(bin_cap=cap)
+        b = GpuBatch(cx, sizes, precision=precision)
+        off = b.off if ends is None else b.off[np.asarray(ends)]
+        v, infos = cx.pcg_solve_batched(b.M, b.Fh, off, dev_tensor(b.F), tol=1e-10, precision=precision)
+        assert all(i.status == 0 and i.true_rel_residual <= 1.05e-10 for i in infos)
+        out.append((v.cpu().numpy(), infos))
+    for s in range(len(off) - 1):
+        lo, hi = int(off[s]), int(off[s + 1])
+        assert abs(out[0][1][s].iterations - out[1][1][s].iterations) <= max(3, out[1][1][s].iterations // 20)
+        if hi > lo:
+            assert rel_err(out[0][0][lo:hi], out[1][0][lo:hi]) <= 1e-8
 
 
 def test_grid_iterates_at_equal_k(cuda_device):
