@@ -505,6 +505,7 @@ void sgp_destroy(sgp_ctx *ctx)
         for (auto e : ctx->ev_pending[k]) cudaEventDestroy(e);
     grid_release(ctx->grid_plain);
     grid_rows_release(ctx->grid_rows);
+    if (ctx->grid_apply.p) cudaFree(ctx->grid_apply.p);
     delete ctx;
 }
 

@@ -442,7 +442,7 @@ sgp_status pcg_b_run(sgp_ctx *ctx, const sgp_matrix *M, const sgp_factor *Fac, i
                                  M->gen, Fac ? Fac->gen : 0ull, (uint64_t)(uintptr_t)x, (uint64_t)(uintptr_t)r,
                                  (uint64_t)(uintptr_t)p, (uint64_t)(uintptr_t)q, (uint64_t)(uintptr_t)w,
                                  (uint64_t)(uintptr_t)b.sc, (uint64_t)(uintptr_t)jac, (uint64_t)wchunk,
-                                 (uint64_t)lpr};
+                                 (uint64_t)lpr, (uint64_t)(uintptr_t)ctx->grid_apply.p};
         GraphEntry *we = nullptr;
         SGP_TRY(graph_lookup(ctx, wkey, sizeof(wkey) / sizeof(wkey[0]), &we));
         if (!we->exec &&
@@ -467,7 +467,7 @@ sgp_status pcg_b_run(sgp_ctx *ctx, const sgp_matrix *M, const sgp_factor *Fac, i
                             M->gen, Fac ? Fac->gen : 0ull, (uint64_t)(uintptr_t)x, (uint64_t)(uintptr_t)r,
                             (uint64_t)(uintptr_t)p, (uint64_t)(uintptr_t)q, (uint64_t)(uintptr_t)w,
                             (uint64_t)(uintptr_t)b.sc, (uint64_t)(uintptr_t)jac, (uint64_t)ctx->timing,
-                            (uint64_t)lpr};
+                            (uint64_t)lpr, (uint64_t)(uintptr_t)ctx->grid_apply.p};
     GraphEntry *ge = nullptr;
     SGP_TRY(graph_lookup(ctx, key, sizeof(key) / sizeof(key[0]), &ge));
     if (!ge->exec) SGP_TRY(graph_capture(ctx, ge, [&]() { return iterate(chunk); }));

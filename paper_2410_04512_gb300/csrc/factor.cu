@@ -805,10 +805,16 @@ Tail tail_of(const sgp_factor *F)
 // contraction level below the tail, the tail kernel, one launch per level
 // back down.
 template <typename T>
-sgp_status tree_apply_inplace(sgp_ctx *ctx, const sgp_factor *F, T *w, const int *done)
+sgp_status tree_apply_inplace(sgp_ctx *ctx, const sgp_factor *F, T *w, const int *done, DBuf *ws)
 {
     if constexpr (sizeof(T) == 8)
-        if (grid_apply_ready(ctx, F)) return grid_apply(ctx, F, w, w, nullptr, done);
+        if (grid_apply_ready(ctx, F)) {
+            // not the factor's own buffer: solves only read the factor.  A
+            // caller under capture has had one call before it
+            DBuf &b = ws ? *ws : ctx->grid_apply;
+            SGP_TRY(buf_ensure(ctx, b, F->gl.apply_bytes));
+            return grid_apply(ctx, F, b, w, w, nullptr, done);
+        }
     if (bins_usable<T>(F)) return bins_apply<T>(ctx, F, w, done);
     const bool f64 = sizeof(T) == 8;
     const T *L = reinterpret_cast<const T *>(f64 ? F->L.p : F->L32.p);
@@ -844,8 +850,8 @@ sgp_status tree_apply_inplace(sgp_ctx *ctx, const sgp_factor *F, T *w, const int
     }
     return SGP_OK;
 }
-template sgp_status tree_apply_inplace<double>(sgp_ctx *, const sgp_factor *, double *, const int *);
-template sgp_status tree_apply_inplace<float>(sgp_ctx *, const sgp_factor *, float *, const int *);
+template sgp_status tree_apply_inplace<double>(sgp_ctx *, const sgp_factor *, double *, const int *, DBuf *);
+template sgp_status tree_apply_inplace<float>(sgp_ctx *, const sgp_factor *, float *, const int *, DBuf *);
 
 // Shared memory of the tail kernel must be opted in above 48 KB, once per device.
 static sgp_status tail_smem_optin(sgp_ctx *ctx)
@@ -1180,7 +1186,7 @@ sgp_status sgp_tree_apply(sgp_ctx *ctx, const sgp_factor *F, const double *b, do
     SGP_CUDA(ctx, cudaSetDevice(ctx->device));
     // (in place is fine in one launch, as every part writes the rows it has read)
     const bool apart = b == x || b + 3 * F->n <= x || x + 3 * F->n <= b;
-    if (apart && grid_apply_ready(ctx, F)) return grid_apply(ctx, F, b, x, bp<const int32_t>(F->orig_of), nullptr);
+    if (apart && grid_apply_ready(ctx, F)) return grid_apply(ctx, F, F->gl.apply, b, x, bp<const int32_t>(F->orig_of), nullptr);
     // caller order -> internal order (the factor's workspace) -> caller order
     double *wi = bp<double>(F->work);
     const int32_t *orig_of = bp<const int32_t>(F->orig_of);

@@ -2833,7 +2833,8 @@ bool grid_apply_ready(const sgp_ctx *ctx, const sgp_factor *F)
 {
     return ctx->fused && F->gl.ok && F->gl.prec == SGP_PREC_F64 && F->gl.apply_bytes > 0;
 }
-sgp_status grid_apply(sgp_ctx *ctx, const sgp_factor *F, const double *b, double *x, const int32_t *orig_of, const int *done)
+sgp_status grid_apply(sgp_ctx *ctx, const sgp_factor *F, const DBuf &ws, const double *b, double *x, const int32_t *orig_of,
+                      const int *done)
 {
     const GridLayout &G = F->gl;
     const int32_t *t = G.tot;
@@ -2846,9 +2847,9 @@ sgp_status grid_apply(sgp_ctx *ctx, const sgp_factor *F, const double *b, double
     for (int q = 0; q < 2; ++q) a.prog[q] = bp<const char>(G.prog[q]);
     a.D = G.D.p; a.inv = G.inv.p;
     a.F = b; a.x = x;
-    a.err = bp<int>(G.apply);
-    a.lx = reinterpret_cast<unsigned long long *>(G.apply.p) + 2;
-    SGP_CUDA(ctx, cudaMemsetAsync(G.apply.p, 0, G.apply_bytes, ctx->stream));
+    a.err = bp<int>(ws);
+    a.lx = reinterpret_cast<unsigned long long *>(ws.p) + 2;
+    SGP_CUDA(ctx, cudaMemsetAsync(ws.p, 0, G.apply_bytes, ctx->stream));
     void *args[] = {&a, &orig_of, &done};
     const auto kern = k_apply_grid<double, 24>;
     SGP_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, GRID_SMEM));

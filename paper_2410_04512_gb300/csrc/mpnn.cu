@@ -547,6 +547,7 @@ struct sgp_mpnn {
     DBuf basis, x, hs, aggs, c, v0w;  // activations of the last prediction
     DBuf dh, du, dc, part, red;
     DBuf tmp;                         // 3 x 3n float64: e, Gamma e, Gamma v*
+    DBuf forest;                      // workspace of the forest solve
     const sgp_matrix *M = nullptr;
 };
 
@@ -648,7 +649,7 @@ void sgp_mpnn_destroy(sgp_mpnn *N)
     if (!N) return;
     cudaDeviceSynchronize();
     DBuf *bufs[] = {&N->p, &N->pb, &N->g, &N->m, &N->v, &N->basis, &N->x, &N->hs, &N->aggs,
-                    &N->c, &N->v0w, &N->dh, &N->du, &N->dc, &N->part, &N->red, &N->tmp};
+                    &N->c, &N->v0w, &N->dh, &N->du, &N->dc, &N->part, &N->red, &N->tmp, &N->forest};
     for (DBuf *b : bufs)
         if (b->p) cudaFree(b->p);
     delete N;
@@ -688,7 +689,7 @@ static sgp_status mpnn_forward_internal(sgp_ctx *ctx, sgp_mpnn *N, const sgp_mat
     SGP_TRY(matrix_block_jacobi(ctx, const_cast<sgp_matrix *>(M)));
     LAUNCH(ctx, k_mp_jacobi, grid_for(n, TB), TB, 0, n, bp<const double>(M->jac), (const double *)Fi, b0);
     SGP_CUDA(ctx, cudaMemcpyAsync(b1, Fi, sizeof(double) * 3 * n, cudaMemcpyDeviceToDevice, ctx->stream));
-    SGP_TRY(tree_apply_inplace<double>(ctx, Fh, b1, nullptr));
+    SGP_TRY(tree_apply_inplace<double>(ctx, Fh, b1, nullptr, &N->forest));
     if (v_prev) LAUNCH(ctx, k_to_internal<double>, grid_for(n, TB), TB, 0, n, orig_of, v_prev, b2);
     else SGP_CUDA(ctx, cudaMemsetAsync(b2, 0, sizeof(double) * 3 * n, ctx->stream));
     double *red = bp<double>(N->red);

@@ -1182,7 +1182,7 @@ sgp_status pcg_core(sgp_ctx *ctx, const sgp_matrix *M, const sgp_factor *Fac, in
                                  (uint64_t)(uintptr_t)r, (uint64_t)(uintptr_t)p, (uint64_t)(uintptr_t)q,
                                  (uint64_t)(uintptr_t)w, (uint64_t)(uintptr_t)partials, (uint64_t)(uintptr_t)sc,
                                  (uint64_t)(uintptr_t)jac, (uint64_t)wchunk, (uint64_t)ctx->spmv_lpr,
-                                 (uint64_t)ctx->spmv_ilp, (uint64_t)fused};
+                                 (uint64_t)ctx->spmv_ilp, (uint64_t)fused, (uint64_t)(uintptr_t)ctx->grid_apply.p};
         GraphEntry *we = nullptr;
         SGP_TRY(graph_lookup(ctx, wkey, sizeof(wkey) / sizeof(wkey[0]), &we));
         if (!we->exec &&
@@ -1209,7 +1209,8 @@ sgp_status pcg_core(sgp_ctx *ctx, const sgp_matrix *M, const sgp_factor *Fac, in
                             (uint64_t)(uintptr_t)p, (uint64_t)(uintptr_t)q, (uint64_t)(uintptr_t)w,
                             (uint64_t)(uintptr_t)partials, (uint64_t)(uintptr_t)sc,
                             (uint64_t)(uintptr_t)jac, (uint64_t)ctx->timing, (uint64_t)chunk,
-                            (uint64_t)ctx->spmv_lpr, (uint64_t)ctx->spmv_ilp, (uint64_t)fused};
+                            (uint64_t)ctx->spmv_lpr, (uint64_t)ctx->spmv_ilp, (uint64_t)fused,
+                            (uint64_t)(uintptr_t)ctx->grid_apply.p};
     GraphEntry *ge = nullptr;
     SGP_TRY(graph_lookup(ctx, key, sizeof(key) / sizeof(key[0]), &ge));
     if (!ge->exec) SGP_TRY(graph_capture(ctx, ge, [&]() { return iterate(chunk); }));

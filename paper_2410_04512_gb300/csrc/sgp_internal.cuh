@@ -116,6 +116,7 @@ struct sgp_ctx {
     // solve on its factor's parts
     GridLayout grid_plain;
     GridRows grid_rows;
+    DBuf grid_apply;   // packets of the forest solves inside this context's solves
 };
 
 // Grid of at most one full wave: min(want, SMs x resident blocks per SM of
@@ -220,7 +221,7 @@ sgp_status scan_exclusive_i32(sgp_ctx *ctx, const int32_t *in, int32_t *out, int
 // z = P^-1 w in place (internal cell order); kernels return at once when
 // *done is set.
 template <typename T>
-sgp_status tree_apply_inplace(sgp_ctx *ctx, const sgp_factor *F, T *w, const int *done);
+sgp_status tree_apply_inplace(sgp_ctx *ctx, const sgp_factor *F, T *w, const int *done, DBuf *ws = nullptr);
 
 // The binned tree solve (bins.cu).  bins_build runs at the end of a factor
 // build; bins_usable tells whether precision T has a layout that fits;
@@ -278,7 +279,9 @@ void grid_rows_release(GridRows &R);
 template <typename T>
 bool grid_ready(const sgp_ctx *ctx, const sgp_factor *F, const sgp_matrix *M);
 bool grid_apply_ready(const sgp_ctx *ctx, const sgp_factor *F);
-sgp_status grid_apply(sgp_ctx *ctx, const sgp_factor *F, const double *b, double *x, const int32_t *orig_of, const int *done);
+// (ws: the packets' buffer, at least gl.apply_bytes)
+sgp_status grid_apply(sgp_ctx *ctx, const sgp_factor *F, const DBuf &ws, const double *b, double *x, const int32_t *orig_of,
+                      const int *done);
 size_t grid_work_bytes(const GridLayout &G, size_t sz, int ng = 1);
 template <typename T>
 sgp_status grid_pcg(sgp_ctx *ctx, const sgp_matrix *M, const GridLayout &G, const GridRows &R, int precond, const T *F, T *x,
