@@ -39,9 +39,9 @@
 // cells also the stream of matrix rows and blocks from HBM.
 // Measured per iteration against the multi-launch paths it replaces (product,
 // vector kernels and level kernels or bins; tol 1e-10): FP64 lattice of 1e4
-// cells 30.8 us (104), FP32 spheroid of 1e5 27.2 us (63), FP32 sheet of 2.5e5
-// 36.2 us (76), FP64 spheroid of 3e5 138 us (282), FP32 spheroid of 1e6 132
-// us (181).
+// cells 31 us (104), FP32 spheroid of 1e5 26.4 us (63), FP32 sheet of 2.5e5
+// 34 us (76), FP64 spheroid of 3e5 125 us (282), FP32 spheroid of 1e6 122 us
+// (181); block Jacobi, FP64, 2e5 cells 54 us (81).
 #include <algorithm>
 #include <cstddef>
 #include <cstring>
@@ -54,6 +54,7 @@ namespace {
 constexpr int GT = 512;          // threads of a part's block
 constexpr int GW = GT / 32;
 constexpr int PMAX = 160;        // parts
+constexpr int NBIG = 32, NSWEEP = 24;   // large subtrees of a part; rounds of handing them over
 constexpr int NTOP = 2048;       // top vertices
 constexpr int GRID_SMEM = 225 * 1024;   // beside about 1 KB of static shared memory
 constexpr int MS_ITEMS = 4096;   // items per block of the stable split
@@ -139,23 +140,33 @@ __global__ void __launch_bounds__(1024) k_gr_size_rest(const int32_t *__restrict
         __syncthreads();
     }
 }
-// top: subtree above bmax; roots carry their subtree's size, by vertex
-__global__ void k_gr_class(int32_t n, int32_t bmax, const int32_t *__restrict__ sz, const int32_t *__restrict__ par,
-                           const int32_t *__restrict__ ord, int32_t *wv)
+// top: subtree above bmax; roots carry their subtree's size, by vertex (and
+// again those of at most `small` vertices alone)
+__global__ void k_gr_class(int32_t n, int32_t bmax, int32_t small, const int32_t *__restrict__ sz,
+                           const int32_t *__restrict__ par, const int32_t *__restrict__ ord, int32_t *wv, int32_t *wsm)
 {
     int32_t t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= n) return;
-    const int32_t s = sz[t], u = par[t];
-    wv[ord[t]] = (s <= bmax && (u < 0 || sz[u] > bmax)) ? s : 0;
+    const int32_t s = sz[t], u = par[t], w = (s <= bmax && (u < 0 || sz[u] > bmax)) ? s : 0;
+    wv[ord[t]] = w;
+    wsm[ord[t]] = w <= small ? w : 0;
 }
-// part of every root: the subtree's middle in the running total of sizes;
+// The parts of the roots.  A root goes by its subtree's middle in the running
+// total of sizes (vertices are in spatial order, so parts are compact), which
+// leaves a part short or over by half a subtree at either end.  Then
+// neighbouring parts hand large subtrees over (k_gr_balance), and the small
+// ones fill all parts up to a common level, in order (k_gr_fill, k_gr_small).
+// The parts run in step, so the largest one sets the pace.  Largest part by
+// the middles alone and so (rows; the mean): FP32 1e5 cells 838 and 725 (658),
+// sheet of 2.5e5 2174 and 1767 (1645), FP64 3e5 2757 and 2208 (1974).
 // anc: itself for roots and top vertices (seg: P for the top), else its parent
 // (a batch: instance s has the vertices [irow[s], irow[s+1]) and the parts
 // [ipart[s], ipart[s+1]), and its top vertices are segment P + s)
 __global__ void k_gr_roots(int32_t n, int32_t bmax, int32_t P, int32_t NI, const int32_t *__restrict__ irow,
                            const int32_t *__restrict__ ipart, const int32_t *__restrict__ sz,
                            const int32_t *__restrict__ par, const int32_t *__restrict__ ord,
-                           const int32_t *__restrict__ pre, int32_t *anc, int32_t *seg)
+                           const int32_t *__restrict__ pre, int32_t small, int32_t *load, int32_t *cnt, int32_t *list,
+                           int32_t *anc, int32_t *seg)
 {
     int32_t t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= n) return;
@@ -176,9 +187,159 @@ __global__ void k_gr_roots(int32_t n, int32_t bmax, int32_t P, int32_t NI, const
             const int32_t p0 = ipart[lo], np = ipart[lo + 1] - p0, before = pre[irow[lo]];
             const int64_t total = max(pre[irow[lo + 1]] - before, 1);
             b = p0 + (int32_t)min((int64_t)np - 1, ((int64_t)(pre[v] - before) + s / 2) * np / total);
+            atomicAdd(load + b, s);
+            if (s <= small) {
+                b = -2 - lo;
+            } else {
+                const int32_t k = atomicAdd(cnt + b, 1);
+                if (k < NBIG) list[b * NBIG + k] = t;
+            }
         }
     }
     seg[t] = b;
+}
+// Large subtrees move between neighbouring parts of one instance, from the
+// heavier to the lighter, alone or against a smaller one, a warp per pair:
+// whatever leaves the smallest difference.  load: all the parts' sizes in, the large subtrees' sizes out.
+__global__ void __launch_bounds__(1024) k_gr_balance(int32_t P, int32_t NI, const int32_t *__restrict__ ipart,
+                                                     const int32_t *__restrict__ sz, const int32_t *__restrict__ cnt,
+                                                     const int32_t *__restrict__ list, int32_t *load, int32_t *seg)
+{
+    __shared__ int32_t st[PMAX][NBIG], ss[PMAX][NBIG], sc[PMAX], sl[PMAX], first[PMAX];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int32_t b = w; b < P; b += 32) {
+        // in the order of their vertices (the list's depends on timing)
+        const int32_t c = cnt[b] <= NBIG ? cnt[b] : 0, t = lane < c ? list[b * NBIG + lane] : INT32_MAX;
+        int32_t rank = 0;
+        for (int k = 0; k < c; ++k) rank += __shfl_sync(0xffffffffu, t, k) < t;
+        if (lane < c) {
+            st[b][rank] = t;
+            ss[b][rank] = sz[t];
+        }
+        if (lane == 0) {
+            sc[b] = c;
+            sl[b] = load[b];
+            first[b] = 0;
+        }
+    }
+    __syncthreads();
+    for (int32_t s = threadIdx.x; s < NI; s += 1024)
+        if (ipart[s + 1] > ipart[s]) first[ipart[s]] = 1;
+    __syncthreads();
+    for (int r = 0; r < NSWEEP; ++r) {
+        for (int32_t b = 2 * w + (r & 1); b + 1 < P; b += 64) {
+            if (first[b + 1]) continue;
+            const int32_t d = sl[b] - sl[b + 1], from = d > 0 ? b : b + 1, to = d > 0 ? b + 1 : b, D = abs(d), c = sc[from],
+                          c2 = sc[to];
+            const int32_t x = lane < c ? ss[from][lane] : 0;
+            int32_t left = INT32_MAX, other = -1;   // the best against this lane's subtree: none, or one of the lighter part
+            if (x > 0)
+                for (int32_t k = c2 < NBIG ? -1 : 0; k < c2; ++k) {
+                    const int32_t y = x - (k < 0 ? 0 : ss[to][k]);
+                    if (y > 0 && y < D && abs(D - 2 * y) < left) {
+                        left = abs(D - 2 * y);
+                        other = k;
+                    }
+                }
+            const int32_t best = __reduce_min_sync(0xffffffffu, left);
+            if (best >= D) continue;
+            const int k = __ffs(__ballot_sync(0xffffffffu, left == best)) - 1;
+            if (lane == k) {
+                const int32_t t = st[from][k];
+                if (other >= 0) {
+                    const int32_t y = ss[to][other];
+                    st[from][k] = st[to][other];
+                    ss[from][k] = y;
+                    st[to][other] = t;
+                    ss[to][other] = x;
+                    sl[from] -= x - y;
+                    sl[to] += x - y;
+                } else {
+                    st[from][k] = st[from][c - 1];
+                    ss[from][k] = ss[from][c - 1];
+                    st[to][c2] = t;
+                    ss[to][c2] = x;
+                    sc[from] = c - 1;
+                    sc[to] = c2 + 1;
+                    sl[from] -= x;
+                    sl[to] += x;
+                }
+            }
+            __syncwarp();
+        }
+        __syncthreads();
+    }
+    for (int32_t b = w; b < P; b += 32) {
+        // a part with more large subtrees than the list holds keeps them all
+        const bool over = cnt[b] > NBIG;
+        int32_t x = 0;
+        if (lane < sc[b]) {
+            seg[st[b][lane]] = b;
+            x = ss[b][lane];
+        }
+        x = __reduce_add_sync(0xffffffffu, x);
+        if (lane == 0) load[b] = over ? sl[b] : x;
+    }
+}
+// A warp per instance: the level up to which its small subtrees fill its
+// parts, and each part's room, as a running total.
+__global__ void __launch_bounds__(256) k_gr_fill(int32_t NI, const int32_t *__restrict__ irow, const int32_t *__restrict__ ipart,
+                                                 const int32_t *__restrict__ psm, const int32_t *__restrict__ load,
+                                                 int32_t *room)
+{
+    const int lane = threadIdx.x & 31;
+    for (int32_t s = threadIdx.x >> 5; s < NI; s += 8) {
+        const int32_t p0 = ipart[s], np = ipart[s + 1] - p0, want = psm[irow[s + 1]] - psm[irow[s]];
+        constexpr int K = (PMAX + 31) / 32;   // parts per lane, consecutive
+        int32_t l[K] = {}, hi = 0;
+        const int32_t k = (np + 31) / 32, b0 = lane * k;
+#pragma unroll
+        for (int u = 0; u < K; ++u) {
+            l[u] = u < k && b0 + u < np ? load[p0 + b0 + u] : INT32_MAX;
+            hi = max(hi, l[u] == INT32_MAX ? 0 : l[u]);
+        }
+        int32_t lo = -1;   // the lowest level with room for all of them
+        hi = __reduce_max_sync(0xffffffffu, hi) + want;
+        while (hi - lo > 1) {
+            const int32_t mid = lo + (hi - lo) / 2;
+            int32_t c = 0;
+#pragma unroll
+            for (int u = 0; u < K; ++u) c += min(max(mid - l[u], 0), want);
+            c = __reduce_add_sync(0xffffffffu, min(c, want));
+            if (c >= want) hi = mid; else lo = mid;
+        }
+        int32_t c = 0, own = 0;
+#pragma unroll
+        for (int u = 0; u < K; ++u) own += max(hi - l[u], 0);
+        int32_t x = own;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int32_t y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        c = x - own;
+#pragma unroll
+        for (int u = 0; u < K; ++u) {
+            if (u >= k || b0 + u >= np) break;
+            room[p0 + b0 + u] = c;
+            c += max(hi - l[u], 0);
+        }
+    }
+}
+// small roots: the part in whose room the subtree's middle lies
+__global__ void k_gr_small(int32_t n, const int32_t *__restrict__ irow, const int32_t *__restrict__ ipart,
+                           const int32_t *__restrict__ sz, const int32_t *__restrict__ ord, const int32_t *__restrict__ psm,
+                           const int32_t *__restrict__ room, int32_t *seg)
+{
+    int32_t t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= n || seg[t] > -2) return;
+    const int32_t s = -2 - seg[t], x = psm[ord[t]] - psm[irow[s]] + sz[t] / 2;
+    int32_t lo = ipart[s], hi = ipart[s + 1];
+    while (hi - lo > 1) {
+        const int32_t mid = (lo + hi) >> 1;
+        if (room[mid] <= x) lo = mid; else hi = mid;
+    }
+    seg[t] = lo;
 }
 __global__ void k_gr_jump(int32_t n, const int32_t *__restrict__ a, int32_t *b)
 {
@@ -2555,13 +2716,15 @@ sgp_status grid_build(sgp_ctx *ctx, sgp_factor *F, const sgp_matrix *M)
     if ((size_t)U * 24 > (size_t)GRID_SMEM) return SGP_OK;
     // The subtree bound trades the number of top vertices (every block reads
     // its rows of their inverse) and the length of the narrow levels against
-    // the imbalance of the parts (half a subtree either way).  Measured, us
-    // per iteration: FP64, U = 128 rows per part: 32.9 with bmax = U, 31.1 with
-    // 3U/2; U = 197: 42.8, 39.2; U = 658: U/2 66.7, 0.6 U 63.3, U 69.3; U =
-    // 1974: U/4 163, U/2 141.5, 0.6 U 137.9, 3U/4 139.5.  FP32, U = 197: 23.1
-    // with U, 22.1 with 3U/2; U = 658: 28.5 with U/2, 28.8 with U; U = 1645:
-    // U/2 38.6, 3U/4 45.7; U = 6579: U/5 136.8, U/4 134.1, 0.3 U 135.8.
-    const int32_t part = U <= 512 ? 3 * U / 2 : (f32 ? (U <= 2048 ? U / 2 : U / 4) : 3 * U / 5);
+    // what balancing can do (a part cannot be smaller than its largest
+    // subtree).  Measured, us per iteration: FP64, U = 127 rows per part: 31.8
+    // with bmax = U, 31.1 with 3U/2, 30.7 with 2U; U = 395: U/2 61, 3U/4 50, 3U/2
+    // 49; U = 658: 0.6 U 63.4, 3U/4 57.8, U 57.8, 1.3 U 60.2; U = 1974: U/2 133,
+    // 3U/4 125, U 124-130, 1.3 U 131.  FP32, U = 197: 20.7 with U, 20.2 with
+    // 3U/2; U = 395: U/2 24, 3U/2 22.4; U = 658: U/2 25.8, U 26.1; U = 1645: U/2
+    // 35, U 40; U = 3290: U/4 80, U/2 67-71, U 71-77; U = 6579: U/4 131, 0.35 U
+    // 121-127, U/2 120-125, U 182 (the halo no longer fits on chip).
+    const int32_t part = U <= 512 ? 3 * U / 2 : (f32 ? U / 2 : 3 * U / 4);
     const int32_t bmax = std::max(32, part);
     G.P = P;
     G.LV = LV;
@@ -2576,7 +2739,7 @@ sgp_status grid_build(sgp_ctx *ctx, sgp_factor *F, const sgp_matrix *M)
     g.pr_ptr = bp<const int32_t>(F->pr_ptr);
     g.pr_q = bp<const int32_t>(F->pr_q);
     g.pr_c = bp<const int32_t>(F->pr_c);
-    int32_t *lp, *par, *sz_, *wv, *pre, *anc, *anc2, *rseg, *seg, *hist, *off, *sp, *lpos;
+    int32_t *lp, *par, *sz_, *wv, *pre, *wsm, *psm, *load, *anc, *anc2, *rseg, *seg, *hist, *off, *sp, *lpos;
     SGP_TRY(S.take((size_t)LV + 1 + 2 * ((size_t)NI + 1), &lp));
     const int32_t *d_irow = lp + LV + 1, *d_ipart = d_irow + NI + 1;
     const int32_t NS = P + NI;   // segments: parts, then the instances' tops
@@ -2584,6 +2747,9 @@ sgp_status grid_build(sgp_ctx *ctx, sgp_factor *F, const sgp_matrix *M)
     SGP_TRY(S.take(n, &sz_));
     SGP_TRY(S.take(n, &wv));
     SGP_TRY(S.take((size_t)n + 1, &pre));
+    SGP_TRY(S.take(n, &wsm));
+    SGP_TRY(S.take((size_t)n + 1, &psm));
+    SGP_TRY(S.take((3 + NBIG) * (size_t)P, &load));
     SGP_TRY(S.take(n, &anc));
     SGP_TRY(S.take(n, &anc2));
     SGP_TRY(S.take(n, &rseg));
@@ -2604,10 +2770,21 @@ sgp_status grid_build(sgp_ctx *ctx, sgp_factor *F, const sgp_matrix *M)
         ++l0;
     }
     if (l0 < LV) LAUNCH(ctx, k_gr_size_rest, 1, 1024, 0, (const int32_t *)lp, l0, LV, (const int32_t *)par, sz_);
-    LAUNCH(ctx, k_gr_class, grid_for(n, B), B, 0, n, bmax, (const int32_t *)sz_, (const int32_t *)par, g.ord, wv);
+    // (U/8 against U/16: U = 658 FP64 57.8 and 59.6 us, FP32 25.8 and 26.4; U =
+    // 1645 35.6 and 34.3, U = 3290 71.1 and 67.1, U = 6579 125.5 and 122.3)
+    const int32_t small = U <= 1024 ? U / 8 : U / 16;
+    int32_t *cnt = load + P, *room = cnt + P, *list = room + P;
+    SGP_CUDA(ctx, cudaMemsetAsync(load, 0, 2 * sizeof(int32_t) * P, ctx->stream));
+    LAUNCH(ctx, k_gr_class, grid_for(n, B), B, 0, n, bmax, small, (const int32_t *)sz_, (const int32_t *)par, g.ord, wv, wsm);
     SGP_TRY(scan_exclusive_i32(ctx, wv, pre, n));
+    SGP_TRY(scan_exclusive_i32(ctx, wsm, psm, n));
     LAUNCH(ctx, k_gr_roots, grid_for(n, B), B, 0, n, bmax, P, NI, d_irow, d_ipart, (const int32_t *)sz_, (const int32_t *)par, g.ord,
-           (const int32_t *)pre, anc, rseg);
+           (const int32_t *)pre, small, load, cnt, list, anc, rseg);
+    LAUNCH(ctx, k_gr_balance, 1, 1024, 0, P, NI, d_ipart, (const int32_t *)sz_, (const int32_t *)cnt, (const int32_t *)list,
+           load, rseg);
+    LAUNCH(ctx, k_gr_fill, 1, 256, 0, NI, d_irow, d_ipart, (const int32_t *)psm, (const int32_t *)load, room);
+    LAUNCH(ctx, k_gr_small, grid_for(n, B), B, 0, n, d_irow, d_ipart, (const int32_t *)sz_, g.ord, (const int32_t *)psm,
+           (const int32_t *)room, rseg);
     for (int r = 0; (1 << r) <= LV + 1; ++r) {
         LAUNCH(ctx, k_gr_jump, grid_for(n, B), B, 0, n, (const int32_t *)anc, anc2);
         std::swap(anc, anc2);
