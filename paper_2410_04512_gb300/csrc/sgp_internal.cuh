@@ -91,7 +91,6 @@ struct sgp_ctx {
     int *d_flags = nullptr;
     // scan workspace (grows; only the scan touches it)
     void *d_scan = nullptr;
-    size_t d_scan_bytes = 0;
     // tuning knobs (0 = built-in default)
     int spmv_lpr = 0;
     int spmv_ilp = 0;       // row groups in flight per lane in the product (0: 1)
