@@ -16,6 +16,9 @@
 // batch until every instance has converged.
 #include "solver_common.cuh"
 
+// y = Gamma v, FP64 (pcg.cu)
+sgp_status spmv64(sgp_ctx *ctx, const sgp_matrix *M, const double *v, double *y);
+
 
 namespace {
 
@@ -288,27 +291,22 @@ __global__ void __launch_bounds__(BB) k_b_pupd(Batch b, const T *__restrict__ w,
         p[k] = fma(beta, p[k], w[k]);
 }
 
-// FP64 residual r = F - Gamma v per instance: out[2s] = |r_s|^2, out[2s+1] = |F_s|^2.
-__global__ void __launch_bounds__(BB) k_b_resid64(Blk<double> B, const int32_t *__restrict__ row_ptr, double g0,
-                                                  Batch b, const double *__restrict__ F,
-                                                  const double *__restrict__ v, double *r, double *out)
+// FP64 residual r = F - y, y = Gamma v (NULL: 0), per instance: out[2s] =
+// |r_s|^2, out[2s+1] = |F_s|^2.  The product is a launch of its own, whose lanes
+// are full (3e5 cells: 189 us in one launch with a lane per row in
+// memory order; the product of its own takes 60 us there)
+__global__ void __launch_bounds__(BB) k_b_resid64(Batch b, const double *__restrict__ F, const double *__restrict__ y,
+                                                  double *r, double *out)
 {
     __shared__ double sh[BB / 32];
     const int c = blockIdx.x, s = b.chunk_inst[c];
     double rr = 0.0, ff = 0.0;
-    for (int32_t i = b.chunk_row[c] + threadIdx.x; i < b.chunk_row[c + 1]; i += BB) {
-        const double v0 = v[3 * (int64_t)i], v1 = v[3 * (int64_t)i + 1], v2 = v[3 * (int64_t)i + 2];
-        double y0 = g0 * v0, y1 = g0 * v1, y2 = g0 * v2;
-        row_accumulate(B, row_ptr[i], row_ptr[i + 1], 1, v, v0, v1, v2, y0, y1, y2);
-        const double yy[3] = {y0, y1, y2};
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            const double f = F[3 * (int64_t)i + a];
-            const double rc = f - yy[a];
-            if (r) r[3 * (int64_t)i + a] = rc;
-            rr += rc * rc;
-            ff += f * f;
-        }
+#pragma unroll 4
+    for (int64_t k = 3 * (int64_t)b.chunk_row[c] + threadIdx.x; k < 3 * (int64_t)b.chunk_row[c + 1]; k += BB) {
+        const double f = F[k], rc = y ? f - y[k] : f;
+        if (r) r[k] = rc;
+        rr += rc * rc;
+        ff += f * f;
     }
     double s1 = block_sum<BB>(rr, sh);
     if (threadIdx.x == 0) b.part[2 * c] = s1;
@@ -631,8 +629,6 @@ sgp_status sgp_pcg_solve_batched(sgp_ctx *ctx, const sgp_matrix *M, const sgp_fa
     }
     Batch b{d_chunk_inst, d_chunk_row, d_inst_chunk, d_sc, d_part, d_flags, d_flags + 1, (int)n_inst};
     const unsigned G = (unsigned)nch;
-    Blk<double> B64 = make_blk<double>(M);
-    const int32_t *row_ptr = bp<const int32_t>(M->row_ptr);
     std::vector<BScal> hs(n_inst);
     std::vector<double> hres(2 * n_inst);
     std::vector<sgp_solve_info> inf(n_inst);
@@ -667,7 +663,10 @@ sgp_status sgp_pcg_solve_batched(sgp_ctx *ctx, const sgp_matrix *M, const sgp_fa
         std::vector<int> active(n_inst, 1);
         for (int outer = 0;; ++outer) {
             SGP_CUDA(ctx, cudaMemsetAsync(d_out, 0, sizeof(double) * 2 * n_inst, ctx->stream));
-            LAUNCH(ctx, k_b_resid64, G, BB, 0, B64, row_ptr, M->gamma0, b, F, (const double *)v, r, d_out);
+            // (r = F when v is zero)
+            const bool zero = outer == 0 && !opts->x0_given;
+            if (!zero) SGP_TRY(spmv64(ctx, M, v, q));
+            LAUNCH(ctx, k_b_resid64, G, BB, 0, b, F, zero ? (const double *)nullptr : (const double *)q, r, d_out);
             SGP_TRY(read_back(ctx, hres.data(), d_out, sizeof(double) * 2 * n_inst));
             int n_active = 0;
             for (int64_t s = 0; s < n_inst; ++s) {
@@ -732,7 +731,8 @@ sgp_status sgp_pcg_solve_batched(sgp_ctx *ctx, const sgp_matrix *M, const sgp_fa
     }
     // true FP64 residual per instance
     SGP_CUDA(ctx, cudaMemsetAsync(d_out, 0, sizeof(double) * 2 * n_inst, ctx->stream));
-    LAUNCH(ctx, k_b_resid64, G, BB, 0, B64, row_ptr, M->gamma0, b, F, (const double *)v, (double *)nullptr, d_out);
+    SGP_TRY(spmv64(ctx, M, v, q));
+    LAUNCH(ctx, k_b_resid64, G, BB, 0, b, F, (const double *)q, (double *)nullptr, d_out);
     SGP_TRY(read_back(ctx, hres.data(), d_out, sizeof(double) * 2 * n_inst));
     LAUNCH(ctx, k_to_caller<double>, grid_for(n, SGP_BLOCK), SGP_BLOCK, 0, n, orig_of, (const double *)v, v_user);
     sgp_status rc = SGP_OK;

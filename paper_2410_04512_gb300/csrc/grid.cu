@@ -226,7 +226,9 @@ __global__ void __launch_bounds__(1024) k_gr_balance(int32_t P, int32_t NI, cons
     for (int32_t s = threadIdx.x; s < NI; s += 1024)
         if (ipart[s + 1] > ipart[s]) first[ipart[s]] = 1;
     __syncthreads();
-    for (int r = 0; r < NSWEEP; ++r) {
+    int still = 0;   // sweeps without a move, both parities in turn
+    for (int r = 0; r < NSWEEP && still < 2; ++r) {
+        int moved = 0;
         for (int32_t b = 2 * w + (r & 1); b + 1 < P; b += 64) {
             if (first[b + 1]) continue;
             const int32_t d = sl[b] - sl[b + 1], from = d > 0 ? b : b + 1, to = d > 0 ? b + 1 : b, D = abs(d), c = sc[from],
@@ -243,6 +245,7 @@ __global__ void __launch_bounds__(1024) k_gr_balance(int32_t P, int32_t NI, cons
                 }
             const int32_t best = __reduce_min_sync(0xffffffffu, left);
             if (best >= D) continue;
+            moved = 1;
             const int k = __ffs(__ballot_sync(0xffffffffu, left == best)) - 1;
             if (lane == k) {
                 const int32_t t = st[from][k];
@@ -267,7 +270,7 @@ __global__ void __launch_bounds__(1024) k_gr_balance(int32_t P, int32_t NI, cons
             }
             __syncwarp();
         }
-        __syncthreads();
+        still = __syncthreads_or(moved) ? 0 : still + 1;
     }
     for (int32_t b = w; b < P; b += 32) {
         // a part with more large subtrees than the list holds keeps them all
@@ -2772,7 +2775,10 @@ sgp_status grid_build(sgp_ctx *ctx, sgp_factor *F, const sgp_matrix *M)
     if (l0 < LV) LAUNCH(ctx, k_gr_size_rest, 1, 1024, 0, (const int32_t *)lp, l0, LV, (const int32_t *)par, sz_);
     // (U/8 against U/16: U = 658 FP64 57.8 and 59.6 us, FP32 25.8 and 26.4; U =
     // 1645 35.6 and 34.3, U = 3290 71.1 and 67.1, U = 6579 125.5 and 122.3)
-    const int32_t small = U <= 1024 ? U / 8 : U / 16;
+    // A batch keeps the middles' parts: an instance has a few only, and the halo
+    // that moved subtrees add costs more (48 instances of 3e5 cells, two draws:
+    // solve 8.9 and 9.3 ms so, 8.4 and 10.6 ms balanced).
+    const int32_t small = NI > 1 ? 0 : U <= 1024 ? U / 8 : U / 16;
     int32_t *cnt = load + P, *room = cnt + P, *list = room + P;
     SGP_CUDA(ctx, cudaMemsetAsync(load, 0, 2 * sizeof(int32_t) * P, ctx->stream));
     LAUNCH(ctx, k_gr_class, grid_for(n, B), B, 0, n, bmax, small, (const int32_t *)sz_, (const int32_t *)par, g.ord, wv, wsm);
@@ -2780,8 +2786,9 @@ sgp_status grid_build(sgp_ctx *ctx, sgp_factor *F, const sgp_matrix *M)
     SGP_TRY(scan_exclusive_i32(ctx, wsm, psm, n));
     LAUNCH(ctx, k_gr_roots, grid_for(n, B), B, 0, n, bmax, P, NI, d_irow, d_ipart, (const int32_t *)sz_, (const int32_t *)par, g.ord,
            (const int32_t *)pre, small, load, cnt, list, anc, rseg);
-    LAUNCH(ctx, k_gr_balance, 1, 1024, 0, P, NI, d_ipart, (const int32_t *)sz_, (const int32_t *)cnt, (const int32_t *)list,
-           load, rseg);
+    if (NI == 1)
+        LAUNCH(ctx, k_gr_balance, 1, 1024, 0, P, NI, d_ipart, (const int32_t *)sz_, (const int32_t *)cnt,
+               (const int32_t *)list, load, rseg);
     LAUNCH(ctx, k_gr_fill, 1, 256, 0, NI, d_irow, d_ipart, (const int32_t *)psm, (const int32_t *)load, room);
     LAUNCH(ctx, k_gr_small, grid_for(n, B), B, 0, n, d_irow, d_ipart, (const int32_t *)sz_, g.ord, (const int32_t *)psm,
            (const int32_t *)room, rseg);
