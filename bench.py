@@ -380,8 +380,8 @@ def run_gpu(args):
 
     def form_rooflines(form, kres, label=""):
         """Rooflines of a form's kernel classes from its timed repeat: the
-        product, the tree step (fused binned solve, or the level kernels),
-        and the vector updates (per iteration)."""
+        product, the tree step (phase of the persistent solve, fused binned
+        solve, or the level kernels), and the vector updates (per iteration)."""
         H = form.H
         fpx = 4 if form.precision == sgp.PREC_MIXED else 8
         tn = "float" if fpx == 4 else "double"
@@ -391,7 +391,14 @@ def run_gpu(args):
         tree_ms, tree_n = kres["kt"][sgp.KT_TREE_SOLVE]
         vec_ms, _ = kres["kt"][sgp.KT_PCG_VECTOR]
         its = max(int(kres["iters_total"]), 1)   # iterations of every timed step
-        out = {"spmv": roof(label + "k_spmv_pq<%s>" % tn, spmv_bytes(n, mm, fpx), spmv_ms, spmv_n,
+        # fewer than two launches an iteration, setup included (the multi-launch
+        # forms have three to six): the whole run is one launch, and the classes
+        # are its phases by the first thread block's clock
+        grid = kres["launches"] < 2 * its
+        if grid:
+            traffic = {}
+        phase = "k_pcg_grid<%s>, " % tn if spmv_n else "k_pcg_small (no phases), "
+        out = {"spmv": roof(label + (phase + "product phase" if grid else "k_spmv_pq<%s>" % tn), spmv_bytes(n, mm, fpx), spmv_ms, spmv_n,
                             "one product Gamma p + p^T q over all rows", traffic.get("spmv"))}
         if fpx == 8:
             # FP64 is issue-bound on this GPU: the product against the FP64
@@ -423,16 +430,18 @@ def run_gpu(args):
                                      "x += alpha p, p = z + beta p, per iteration", traffic.get("vector"))
             else:
                 tb = tree_bytes(n, npairs, nrecv, fpx)
-                out["tree"] = roof(label + "tree solve (level kernels <%s>, %d levels)" % (tn, levels), tb,
+                out["tree"] = roof(label + (phase + "forest phase (with the sums around it)" if grid else
+                                            "tree solve (level kernels <%s>, %d levels)" % (tn, levels)), tb,
                                    tree_ms, tree_n, "one application of P^-1 (all levels)")
                 vb = vector_bytes(n, fpx, "tree")
-                out["vector"] = roof(label + "PCG vector kernels <%s>" % tn, vb, vec_ms, its,
+                out["vector"] = roof(label + (phase + "direction and halo exchange" if grid else
+                                              "PCG vector kernels <%s>" % tn), vb, vec_ms, its,
                                      "update, r^T z and direction kernels, per iteration")
             it_bytes += tb + vb
         else:
             vb = vector_bytes(n, fpx, "jacobi")
-            out["vector"] = roof(label + "PCG vector kernels <%s>" % tn, vb, vec_ms, its,
-                                 "update with the block-Jacobi product, per iteration")
+            out["vector"] = roof(label + (phase + "vector phase" if grid else "PCG vector kernels <%s>" % tn), vb, vec_ms,
+                                 its, "update with the block-Jacobi product, per iteration")
             it_bytes += vb
         return out, it_bytes
 

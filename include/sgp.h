@@ -428,10 +428,12 @@ typedef struct {
     int32_t bin_cap;     /* the tree solve's thread-block bins: contraction subtrees
                             of at most bin_cap vertices are solved by one thread
                             block each (three launches per application); 0 =
-                            default (single systems whose parts fit on chip,
-                            about 1e6 cells in MIXED and 5e5 in FP64: a whole
-                            PCG run is one persistent launch; larger ones and
-                            batches: bins of 1024 for the FP32 solve of a MIXED
+                            default (systems whose parts fit on chip, about 1e6
+                            cells in MIXED and 4.5e5 in FP64, and batches of no
+                            more instances than SMs: a whole PCG run is one
+                            persistent launch, with every preconditioner; FP64
+                            forest solves alone too, up to about 7e5 cells;
+                            otherwise bins of 1024 for the FP32 solve of a MIXED
                             factor, one launch per contraction level for FP64),
                             -1 = off in both precisions, 64..8192 = that cap in
                             both precisions; read when a factor is built */
