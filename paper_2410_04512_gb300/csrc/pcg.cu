@@ -40,6 +40,19 @@ __device__ __forceinline__ void row_product(const Blk<T> &B, const int32_t *__re
     }
 }
 
+// alpha = rho / p^T q, or a breakdown
+__device__ __forceinline__ void pq_finish(Scal *sc, double pq)
+{
+    sc->pq = pq;
+    if (!(pq > 0.0) || !isfinite(pq)) {
+        sc->status = SGP_ERR_NOT_SPD;
+        sc->done = 1;
+    } else {
+        sc->alpha = sc->rho / pq;
+        sc->xpend = 1;
+    }
+}
+
 // y = Gamma v, FP64, a lane per row.  Bound by the FP64 pipe (2 fused multiply-
 // adds per clock and SM; 12 operations per slot: three differences, nine
 // multiply-adds; 98 us of it at 1e6 cells and 4.7e6 slots), and a warp runs as
@@ -48,11 +61,17 @@ __device__ __forceinline__ void row_product(const Blk<T> &B, const int32_t *__re
 // with R = 128, 92% with 512, 95% with 1024).  The result goes straight to the
 // caller's order (orig_of) when given.  1e6 cells, with the gather of v: 363 ->
 // 172 us.
-template <int R, int NT>
+// DOT: inside a PCG step, with v^T y; the last block sets alpha = rho / v^T y
+// (in place of k_spmv_pq<double, 1, 1>, 238 us at 1e6 cells: FP64 steps of
+// 700,000 and 800,000 cells 129.7 -> 111.5 and 143.9 -> 124.9 ms).
+template <int R, int NT, bool DOT>
 __global__ void __launch_bounds__(NT, 1024 / NT) k_product64(Blk<double> B, const int32_t *__restrict__ row_ptr, double gamma0,
                                                   int64_t n, const double *__restrict__ v,
-                                                  const int32_t *__restrict__ orig_of, double *__restrict__ y)
+                                                  const int32_t *__restrict__ orig_of, double *__restrict__ y,
+                                                  double *partials, Scal *sc)
 {
+    if (DOT && sc->done) return;
+    double dot = 0.0;
     __shared__ int32_t cnt[64], row[R];
     const int tid = threadIdx.x;
     const int64_t i0 = blockIdx.x * (int64_t)R;
@@ -124,6 +143,16 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_product64(Blk<double> B, cons
         y0 += z0; y1 += z1; y2 += z2;
         const int64_t o = orig_of ? orig_of[i] : i;
         y[3 * o] = y0; y[3 * o + 1] = y1; y[3 * o + 2] = y2;
+        if (DOT) dot += fma(v2, y2, fma(v1, y1, v0 * y0));
+    }
+    if (DOT) {
+        __shared__ double sh[NT / 32];
+        const double s = block_sum<NT>(dot, sh);
+        if (tid == 0) partials[blockIdx.x] = s;
+        if (last_block(&sc->cnt)) {
+            const double pq = sum_partials<NT>(partials, gridDim.x, sh);
+            if (tid == 0) pq_finish(sc, pq);
+        }
     }
 }
 sgp_status product64(sgp_ctx *ctx, const sgp_matrix *M, const double *v, const int32_t *orig_of, double *y)
@@ -135,9 +164,11 @@ sgp_status product64(sgp_ctx *ctx, const sgp_matrix *M, const double *v, const i
     // 1024 rows against 128: 40,000 cells 36 and 25, 80,000 37.5 and 33.4,
     // 100,000 37.5 both, 150,000 40 and 48, 300,000 64 and 76, 1e6 175 and 210)
     if (n >= 100000)
-        LAUNCH(ctx, (k_product64<1024, 512>), (unsigned)((n + 1023) / 1024), 512, 0, B, rp, M->gamma0, n, v, orig_of, y);
+        LAUNCH(ctx, (k_product64<1024, 512, false>), (unsigned)((n + 1023) / 1024), 512, 0, B, rp, M->gamma0, n, v,
+               orig_of, y, (double *)nullptr, (Scal *)nullptr);
     else
-        LAUNCH(ctx, (k_product64<128, 128>), (unsigned)((n + 127) / 128), 128, 0, B, rp, M->gamma0, n, v, orig_of, y);
+        LAUNCH(ctx, (k_product64<128, 128, false>), (unsigned)((n + 127) / 128), 128, 0, B, rp, M->gamma0, n, v,
+               orig_of, y, (double *)nullptr, (Scal *)nullptr);
     return SGP_OK;
 }
 
@@ -236,16 +267,7 @@ __global__ void __launch_bounds__(RB, sizeof(T) == 4 ? (ILP == 1 ? 6 : 4) : (ILP
     if (threadIdx.x == 0) partials[blockIdx.x] = s;
     if (last_block(&sc->cnt)) {
         double pq = sum_partials<RB>(partials, gridDim.x, sh);
-        if (threadIdx.x == 0) {
-            sc->pq = pq;
-            if (!(pq > 0.0) || !isfinite(pq)) {
-                sc->status = SGP_ERR_NOT_SPD;
-                sc->done = 1;
-            } else {
-                sc->alpha = sc->rho / pq;
-                sc->xpend = 1;
-            }
-        }
+        if (threadIdx.x == 0) pq_finish(sc, pq);
     }
 }
 
@@ -1015,6 +1037,14 @@ template <typename T>
 sgp_status launch_spmv_pq(sgp_ctx *ctx, Blk<T> B, const int32_t *row_ptr, T g0, int64_t n, const T *p,
                           T *q, double *partials, Scal *sc)
 {
+    // FP64 with a lane per row: rows by length (from 100,000 rows on, see
+    // product64; as many partials as blocks)
+    if constexpr (sizeof(T) == 8)
+        if (ctx->spmv_lpr <= 1 && ctx->spmv_ilp <= 1 && n >= 100000 && n <= (int64_t)1024 * MAXP) {
+            LAUNCH(ctx, (k_product64<1024, 512, true>), (unsigned)((n + 1023) / 1024), 512, 0, B, row_ptr, g0, n, p,
+                   (const int32_t *)nullptr, q, partials, sc);
+            return SGP_OK;
+        }
     const int lpr = ctx->spmv_lpr > 0 ? ctx->spmv_lpr : (sizeof(T) == 8 ? 1 : 2);
     const int ilp = ctx->spmv_ilp > 0 ? ctx->spmv_ilp : 1;
     const int64_t want = (n * lpr + RB - 1) / RB;

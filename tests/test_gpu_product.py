@@ -53,3 +53,20 @@ def test_forest_solve_alone(cuda_device, name):
         cx.tree_apply(s.Fac, w, w)
         assert torch.equal(w, out[-1])
     assert rel_err(out[0].cpu().numpy(), out[1].cpu().numpy()) <= 1e-10
+
+
+def test_product_inside_multi_launch_steps(cuda_device):
+    """From 100,000 rows on the multi-launch FP64 step takes the sorted product
+    with p^T q: 20 unpreconditioned steps against the one-launch solve, equal
+    but for the order of sums (1e-10 of the iterate)."""
+    c = _shape("sheet100k")
+    F = dev_tensor(c.forces())
+    out = []
+    for cap in (0, -1):
+        cx = sgp.Context(0)
+        cx.set_tuning(bin_cap=cap)
+        s = GpuSystem(cx, c, tree=False)
+        v, info = cx.pcg_solve(s.M, None, F, tol=1e-300, maxit=20, precond=sgp.PRECOND_NONE, raise_on_error=False)
+        assert info.iterations == 20
+        out.append(v.cpu().numpy())
+    assert rel_err(out[0], out[1]) <= 1e-10
