@@ -429,7 +429,7 @@ typedef struct {
                             of at most bin_cap vertices are solved by one thread
                             block each (three launches per application); 0 =
                             default (systems whose parts fit on chip, about 1e6
-                            cells in MIXED and 4.5e5 in FP64, and batches of no
+                            cells in MIXED and 5e5 in FP64, and batches of no
                             more instances than SMs: a whole PCG run is one
                             persistent launch, with every preconditioner; FP64
                             forest solves alone too, up to about 7e5 cells;
