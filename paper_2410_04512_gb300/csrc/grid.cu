@@ -10,8 +10,8 @@
 //   q = Gamma p on its rows (its own p and the rows of other parts that its
 //     rows name, the "halo", in shared memory), p^T q
 //   r -= alpha q, x += alpha p, |r|^2, its part's forward levels
-//   z at the top vertices it reaches or owns: rows of the top's inverse times
-//     the top's right-hand side
+//   z at the top vertices it reaches or owns, from the rows and columns of the
+//     top's L^-1 that these need
 //   its part's backward levels, r^T z, p = z + beta p
 // Between the blocks travel p of the halo, the parts' sums for the top with
 // the top's r, and three sums (p^T q, |r|^2, r^T z).
@@ -28,9 +28,8 @@
 // k_gr_segments): records and blocks in the order of use, so that a level
 // costs its reads of the vector and a barrier.
 //
-// The top's inverse (a few hundred vertices, computed once per factor by one
-// block per column) replaces its 2 x 10 levels, which every block ran for
-// itself: 5 us per iteration less at 1e4 to 3e5 cells.
+// The top's rows and columns of L^-1 (a few hundred vertices, once per factor)
+// replace its 2 x 10 levels, which every block ran for itself.
 //
 // What bounds it: the levels of a part (about 10 each way; 200-300 clocks
 // each, a chain of shared-memory reads, products and a barrier), the
@@ -56,16 +55,22 @@ constexpr int GW = GT / 32;
 constexpr int PMAX = 160;        // parts
 constexpr int NBIG = 32, NSWEEP = 24;   // large subtrees of a part; rounds of handing them over
 constexpr int NTOP = 2048;       // top vertices
+constexpr int CMAX = 48;         // entries of a column of the top's X
+constexpr int TLONG = 32;        // a row of X with more entries has a warp, others 8 lanes
 constexpr int GRID_SMEM = 225 * 1024;   // beside about 1 KB of static shared memory
 constexpr int MS_ITEMS = 4096;   // items per block of the stable split
 
 constexpr int LMAX = 64;         // contraction levels
 constexpr int NCLS = 8;          // segment classes: 8 sources or more, 7, ... 1
 
-// header of a part (entry P: the top); Q_NSF, Q_NSB: slots of its programs
-enum { Q_SOFF, Q_NV, Q_ROFF, Q_NR, Q_T0, Q_NP, Q_POFF, Q_NZ, Q_ZOFF, Q_DOFF, Q_NSF, Q_SF, Q_NSB, Q_SB, Q_N = 24 };
+// header of a part (entry P: the top); Q_NSF, Q_NSB: slots of its programs;
+// Q_NA, Q_NL: rows of the top that it forms and how many are long; Q_XR, Q_XC:
+// entries of those rows and of the columns of its outputs (padded)
+enum { Q_SOFF, Q_NV, Q_ROFF, Q_NR, Q_T0, Q_NP, Q_POFF, Q_NZ, Q_ZOFF, Q_DOFF, Q_NSF, Q_SF, Q_NSB, Q_SB,
+       Q_NA, Q_AOFF, Q_NL, Q_XR, Q_XC, Q_N = 24 };
 // totals and maxima over the parts
-enum { T_NT, T_NR, T_P, T_Z, T_D, T_SF, T_SB, T_MNR, T_MNZ, T_MSF, T_MSB, T_MDZ, T_MNF, T_MNB, T_MNO, T_ERR, T_N = 24 };
+enum { T_NT, T_NR, T_P, T_Z, T_D, T_SF, T_SB, T_MNR, T_MNZ, T_MSF, T_MSB, T_MDZ, T_MNF, T_MNB, T_MNO,
+       T_RE, T_CE, T_A, T_MNA, T_MX, T_ERR, T_N = 32 };
 // a matrix's rows on the parts: slots and halo cells of each part with their
 // offsets; behind the parts the totals and the largest halo
 enum { R_NS, R_SLOT, R_NH, R_HOFF, R_N };
@@ -74,6 +79,7 @@ enum { R_NS, R_SLOT, R_NH, R_HOFF, R_N };
 enum { W_NARROW = GW, W_END, W_LEVELS, W_N = GW + 4 };
 
 __host__ __device__ __forceinline__ int32_t pad32(int32_t x) { return (x + 31) & ~31; }
+__host__ __device__ __forceinline__ int32_t pad8(int32_t x) { return (x + 7) & ~7; }
 
 // Block-wide exclusive scan of one int per thread; *total gets the sum.
 template <int BS>
@@ -491,16 +497,21 @@ struct GBuild {
     int32_t *st;                             // first step of every (program, level): 2 x (LMAX + 1) per part
     int32_t *sp_slot[2], *sp_n[2];           // every step's first slot, and its slots | barriers before << 16
     int32_t *ws;                             // streams: 2 x W_N per part
-    int32_t lps;                             // receivers per step of a part: 32, or 10 with a lane per row (the top: 10)
+    int32_t lps;                             // receivers per step of a part: 32, or 10 with a lane per row
     int32_t *glen, *gso;
     uint16_t *perm;
     uint32_t *hb;                            // halo bitmap
     int32_t *hpre;                           // its running count, per word
     int32_t *hl;                             // halo rows
     uint8_t *xflag;                          // rows other parts read
-    char *prog[2], *tprog[2];                // slots of the parts and of the top
-    int32_t *msrc[2], *tmsrc[2];             // source pair of every slot's lane
-    int32_t *zi, *zslot, *tlk;
+    char *prog[2];                           // slots of the parts
+    int32_t *msrc[2];                        // source pair of every slot's lane
+    int32_t *zslot, *tlk;
+    int32_t *clen, *rlen, *cptr, *rptr;      // the top's X: entries of its columns and rows, and where they start
+    int32_t *cidx;                           // rows of every column's entries, CMAX per column
+    double *cx;                              // and their blocks
+    int32_t *xi;                             // the other index of every entry: rows, then columns
+    int4 *alist, *outs;                      // per part: rows of X, outputs (see k_gr_part_top)
     int identity, halo;
 };
 
@@ -536,8 +547,8 @@ __global__ void __launch_bounds__(GT) k_gr_row_maps(GBuild g)
     }
 }
 
-// One part (or the top): its pairs and the distinct top vertices it reaches,
-// numbered in top order.
+// One part: its pairs and the distinct top vertices it reaches, numbered in
+// top order.
 __global__ void __launch_bounds__(GT) k_gr_part_count(GBuild g)
 {
     __shared__ int32_t sh[GW];
@@ -548,8 +559,7 @@ __global__ void __launch_bounds__(GT) k_gr_part_count(GBuild g)
     if (g.tot[T_ERR]) return;
     int32_t *vm = g.vm + (size_t)b * nt;
     if (threadIdx.x == 0) s_np = 0;
-    if (b < g.P)
-        for (int32_t i = threadIdx.x; i < nt; i += GT) vm[i] = 0;
+    for (int32_t i = threadIdx.x; i < nt; i += GT) vm[i] = 0;
     __syncthreads();
     int32_t c = 0;
     for (int32_t l = threadIdx.x; l < nv; l += GT) {
@@ -557,13 +567,13 @@ __global__ void __launch_bounds__(GT) k_gr_part_count(GBuild g)
         for (int32_t p = g.pr_ptr[t]; p < g.pr_ptr[t + 1]; ++p) {
             ++c;
             const int32_t u = g.pos[g.pr_q[p]];
-            if (b < g.P && g.seg[u] == g.P) vm[g.lpos[u]] = 1;
+            if (g.seg[u] == g.P) vm[g.lpos[u]] = 1;
         }
     }
     if (c) atomicAdd(&s_np, c);
     __syncthreads();
     int32_t cz = 0;
-    for (int32_t base = 0; b < g.P && base < nt; base += GT) {
+    for (int32_t base = 0; base < nt; base += GT) {
         const int32_t i = base + threadIdx.x;
         const int32_t f = i < nt ? vm[i] : 0;
         int32_t tz;
@@ -577,7 +587,7 @@ __global__ void __launch_bounds__(GT) k_gr_part_count(GBuild g)
     }
 }
 
-// running offsets of one header field over the parts (and the top)
+// running offsets of one header field over the parts
 __device__ __forceinline__ void hdr_scan(int32_t n, int32_t *hdr, int32_t *tot, int f, int fo, int t, int extra, int32_t *sh)
 {
     const int b = threadIdx.x;
@@ -590,14 +600,13 @@ __device__ __forceinline__ void hdr_scan(int32_t n, int32_t *hdr, int32_t *tot, 
 __global__ void __launch_bounds__(256) k_gr_offsets1(int32_t P, int32_t *hdr, int32_t *tot)
 {
     __shared__ int32_t sh[8];
-    hdr_scan(P + 1, hdr, tot, Q_NP, Q_POFF, T_P, 0, sh);
-    hdr_scan(P + 1, hdr, tot, Q_NZ, Q_ZOFF, T_Z, 0, sh);
+    hdr_scan(P, hdr, tot, Q_NP, Q_POFF, T_P, 0, sh);
+    hdr_scan(P, hdr, tot, Q_NZ, Q_ZOFF, T_Z, 0, sh);
     const int b = threadIdx.x;
     int32_t *h = hdr + (size_t)Q_N * b;
     int32_t total;
-    const int32_t nd = b < P ? h[Q_NR] + h[Q_NZ] : (b == P ? h[Q_NV] : 0);
-    const int32_t o = gscan<256>(b <= P ? nd + 1 : 0, sh, &total);
-    if (b <= P) h[Q_DOFF] = o;
+    const int32_t o = gscan<256>(b < P ? h[Q_NR] + h[Q_NZ] + 1 : 0, sh, &total);
+    if (b < P) h[Q_DOFF] = o;
     if (b == 0) tot[T_D] = total;
 }
 __global__ void __launch_bounds__(256) k_gr_offsets2(int32_t P, int32_t *hdr, int32_t *tot, const int32_t *ws)
@@ -605,6 +614,7 @@ __global__ void __launch_bounds__(256) k_gr_offsets2(int32_t P, int32_t *hdr, in
     __shared__ int32_t sh[8];
     hdr_scan(P, hdr, tot, Q_NSF, Q_SF, T_SF, 0, sh);
     hdr_scan(P, hdr, tot, Q_NSB, Q_SB, T_SB, 0, sh);
+    hdr_scan(P, hdr, tot, Q_NA, Q_AOFF, T_A, 0, sh);
     if (threadIdx.x < P) {
         const int32_t *h = hdr + (size_t)Q_N * threadIdx.x;
         atomicMax(tot + T_MNR, h[Q_NR]);
@@ -613,6 +623,8 @@ __global__ void __launch_bounds__(256) k_gr_offsets2(int32_t P, int32_t *hdr, in
         atomicMax(tot + T_MSB, h[Q_NSB]);
         atomicMax(tot + T_MDZ, h[Q_NR] + h[Q_NZ]);
         atomicMax(tot + T_MNO, h[Q_NZ] + h[Q_NR] - h[Q_NV]);
+        atomicMax(tot + T_MNA, h[Q_NA]);
+        atomicMax(tot + T_MX, h[Q_XR] + h[Q_XC]);
         if (ws) {
             const int32_t *f = ws + (size_t)threadIdx.x * 2 * W_N;
             atomicMax(tot + T_MNF, f[W_END] - f[W_NARROW]);
@@ -629,8 +641,7 @@ __device__ __forceinline__ int32_t pair_dst(const GBuild &g, int b, int32_t nr, 
     return g.seg[u] == b ? g.lpos[u] : nr + vm[g.lpos[u]] - 1;
 }
 
-// The programs of one part (or the top): w[dst] -= sum M w[src], level by
-// level.  The pairs of one receiver (forward) or vertex (backward) in one
+// The programs of one part: w[dst] -= sum M w[src], level by level.  The pairs of one receiver (forward) or vertex (backward) in one
 // level are a segment; the segments of a level, by descending size, are cut
 // into steps of lps receivers, one lane (or three, one per row) each; a step
 // is as many slots as its largest segment has pairs, and a slot holds one
@@ -647,9 +658,8 @@ __global__ void __launch_bounds__(GT) k_gr_segments(GBuild g)
     int32_t *h = g.hdr + (size_t)Q_N * b;
     if (g.tot[T_ERR]) return;
     for (int i = threadIdx.x; i < LMAX; i += GT) lmax[i] = 0;
-    const bool top = b == g.P;
-    const int32_t so = h[Q_SOFF], nv = h[Q_NV], nr = h[Q_NR], nt = g.tot[T_NT], po = h[Q_POFF],
-                  nd = top ? nv : nr + h[Q_NZ], lps = top ? 10 : g.lps;
+    const int32_t so = h[Q_SOFF], nv = h[Q_NV], nr = h[Q_NR], nt = g.tot[T_NT], po = h[Q_POFF], nd = nr + h[Q_NZ],
+                  lps = g.lps;
     const int32_t *vm = g.vm + (size_t)b * nt;
     int32_t *dc = g.dcnt + h[Q_DOFF];
     for (int i = threadIdx.x; i < 2 * LMAX * NCLS; i += GT) (&hist[0][0])[i] = 0;
@@ -967,22 +977,20 @@ struct SlotSize<double> {
     static constexpr int B = 128 + 3 * 256, LPS = 10;
 };
 template <typename T>
-__global__ void __launch_bounds__(GT) k_gr_program(GBuild g, int32_t b0)
+__global__ void __launch_bounds__(GT) k_gr_program(GBuild g)
 {
     __shared__ uint16_t wc[GW][LMAX * NCLS];
     __shared__ int32_t base_s[LMAX * NCLS];
     constexpr int B = SlotSize<T>::B, LPS = SlotSize<T>::LPS, R = LPS == 32 ? 1 : 3;
-    const int b = b0 + blockIdx.x, q = blockIdx.y, w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int b = blockIdx.x, q = blockIdx.y, w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int32_t *h = g.hdr + (size_t)Q_N * b;
-    const bool top = b == g.P;
-    const int32_t so = h[Q_SOFF], nv = h[Q_NV], nr = h[Q_NR], nt = g.tot[T_NT], po = h[Q_POFF],
-                  nd = top ? nv : nr + h[Q_NZ];
+    const int32_t so = h[Q_SOFF], nv = h[Q_NV], nr = h[Q_NR], nt = g.tot[T_NT], po = h[Q_POFF], nd = nr + h[Q_NZ];
     const int32_t *vm = g.vm + (size_t)b * nt;
     const int32_t *kb = g.kb + ((size_t)b * 2 + q) * LMAX * NCLS, *st = g.st + ((size_t)b * 2 + q) * (LMAX + 1);
     const int32_t *sslot = g.sp_slot[q] + po + b, *sn = g.sp_n[q] + po + b;
     const int32_t slot0 = h[q ? Q_SB : Q_SF], nsteps = st[LMAX];
-    char *prog = top ? g.tprog[q] : g.prog[q] + (size_t)B * slot0;
-    int32_t *msrc = top ? g.tmsrc[q] : g.msrc[q] + 32 * (size_t)slot0;
+    char *prog = g.prog[q] + (size_t)B * slot0;
+    int32_t *msrc = g.msrc[q] + 32 * (size_t)slot0;
     auto rec = [&](int32_t slot, int32_t ln) -> uint32_t & { return reinterpret_cast<uint32_t *>(prog + (size_t)B * slot)[ln]; };
     for (int32_t s = w; s < nsteps; s += GW) {
         const int32_t a = sslot[s], n = sn[s] & 0xffff, bars = sn[s] >> 16;
@@ -1046,9 +1054,192 @@ __global__ void __launch_bounds__(GT) k_gr_program(GBuild g, int32_t b0)
         }
         __syncthreads();
     }
-    if (!top && q == 0)
-        for (int32_t i = threadIdx.x; i < nt; i += GT)
-            if (vm[i]) g.zi[h[Q_ZOFF] + vm[i] - 1] = i;
+}
+
+// ---- the top.  Its forest solve is z = X^T D^-1 X r with X = L^-1 of the top
+// alone: row j has an entry for every vertex whose elimination reaches j, the
+// column of a vertex one for itself and for each of its receivers' columns.  A
+// vertex has two receivers at most and meets two at a time on its way up, so
+// columns are short (6 or 7 entries, 11 at most, at 1e4 to 1e6 cells).  A part
+// forms the rows that its outputs' columns name (30 of some 340) and these
+// columns: a third of the work of the same outputs' rows of the inverse
+// X^T D^-1 X, which this replaces because in the inverse the 1 / gamma0 of the
+// roots swamps the rest (rounded to FP32 it is no longer positive definite:
+// sheets with gamma0 = 1e-10 broke down).  In this form the operator is
+// positive definite however X is rounded.
+// Whole steps with the inverse's rows and so: FP64 lattice of 1e4 cells 7.7 and
+// 7.7 ms, MIXED 1e5 13.0 and 13.4, 1e6 59.0 and 59.4, 48 instances 13.8 and 12.6.
+
+// One lane per component of a column, by its elimination steps in FP64.
+__global__ void k_gr_cols(GBuild g, const double *__restrict__ L)
+{
+    const int32_t k = blockIdx.x * blockDim.x + threadIdx.x, i = k / 3, c = k % 3;
+    if (g.tot[T_ERR] || i >= g.tot[T_NT]) return;
+    constexpr int W = 4;
+    int32_t f[W], n = 1, len = 0;   // vertices met, by position, and X's column c in their rows
+    double y[W][3] = {};
+    f[0] = g.sp[g.hdr[(size_t)Q_N * g.P + Q_SOFF] + i];
+    y[0][0] = c == 0; y[0][1] = c == 1; y[0][2] = c == 2;
+    bool bad = false;
+    while (n > 0 && !bad) {
+        int m = 0;
+        for (int a = 1; a < n; ++a)
+            if (f[a] < f[m]) m = a;
+        const int32_t t = f[m];
+        const double y0 = y[m][0], y1 = y[m][1], y2 = y[m][2];
+        --n;
+        f[m] = f[n];
+        for (int r = 0; r < 3; ++r) y[m][r] = y[n][r];
+        if (len == CMAX) {
+            bad = true;
+            break;
+        }
+        const int32_t j = g.lpos[t];
+        double *x = g.cx + ((size_t)i * CMAX + len) * 9 + c;
+        x[0] = y0; x[3] = y1; x[6] = y2;
+        if (c == 0) {
+            g.cidx[(size_t)i * CMAX + len] = j;
+            atomicAdd(g.rlen + j, 1);
+        }
+        ++len;
+        for (int32_t p = g.pr_ptr[t]; p < g.pr_ptr[t + 1]; ++p) {
+            const int32_t u = g.pos[g.pr_q[p]];
+            int a = 0;
+            while (a < n && f[a] != u) ++a;
+            if (a == W) {
+                bad = true;
+                break;
+            }
+            if (a == n) {
+                f[n] = u;
+                y[n][0] = y[n][1] = y[n][2] = 0.0;
+                ++n;
+            }
+            const double *l = L + 9 * (size_t)p;
+            for (int r = 0; r < 3; ++r) y[a][r] = fma(-l[3 * r + 2], y2, fma(-l[3 * r + 1], y1, fma(-l[3 * r], y0, y[a][r])));
+        }
+    }
+    if (c == 0) g.clen[i] = len;
+    if (bad) atomicOr(g.tot + T_ERR, 8);
+}
+// where the rows and columns start (padded to 8 entries)
+__global__ void __launch_bounds__(1024) k_gr_top_offsets(GBuild g)
+{
+    __shared__ int32_t sh[32];
+    const int32_t nt = min(g.tot[T_NT], NTOP);
+    int32_t cr = 0, cc = 0;
+    for (int32_t base = 0; base < nt; base += 1024) {
+        const int32_t i = base + threadIdx.x;
+        int32_t tr, tc;
+        const int32_t er = gscan<1024>(i < nt ? pad8(g.rlen[i]) : 0, sh, &tr);
+        const int32_t ec = gscan<1024>(i < nt ? pad8(g.clen[i]) : 0, sh, &tc);
+        if (i < nt) {
+            g.rptr[i] = cr + er;
+            g.cptr[i] = cc + ec;
+        }
+        cr += tr;
+        cc += tc;
+    }
+    if (threadIdx.x == 0) {
+        g.tot[T_RE] = cr;
+        g.tot[T_CE] = cc;
+    }
+}
+// A part's share: its outputs (the top vertices that it reaches, then those
+// that it owns) and the rows that their columns name, the long ones first.  On
+// chip the part's rows, then its columns, are packed ("local" starts).
+//   alist: row, start, local start, length
+//   outs:  column's start, local start, length
+template <bool FILL>
+__global__ void __launch_bounds__(GT) k_gr_part_top(GBuild g)
+{
+    __shared__ int32_t sh[GW];
+    __shared__ uint8_t in[NTOP];
+    const int b = blockIdx.x;
+    int32_t *h = g.hdr + (size_t)Q_N * b;
+    if (g.tot[T_ERR]) return;   // (nothing of this launch writes it)
+    const int32_t nt = g.tot[T_NT], nz = h[Q_NZ], nout = nz + h[Q_NR] - h[Q_NV], t0 = h[Q_T0];
+    const int32_t *vm = g.vm + (size_t)b * nt;
+    int4 *outs = FILL ? g.outs + h[Q_ZOFF] + t0 : nullptr;
+    for (int32_t i = threadIdx.x; i < nt; i += GT) in[i] = 0;
+    __syncthreads();
+    int32_t xc = 0;
+    for (int32_t base = 0; base < nt; base += GT) {
+        const int32_t i = base + threadIdx.x;
+        const bool own = i < nt && i >= t0 && i - t0 < nout - nz;
+        const bool reach = i < nt && vm[i] != 0;
+        int32_t n = 0;
+        if (own || reach) {
+            n = g.clen[i];
+            for (int32_t k = 0; k < n; ++k) in[g.cidx[(size_t)i * CMAX + k]] = 1;
+        }
+        // a vertex that is reached and owned has two outputs
+        const int32_t e = pad8(n) * ((own ? 1 : 0) + (reach ? 1 : 0));
+        int32_t tot;
+        const int32_t at = xc + gscan<GT>(e, sh, &tot);
+        if (FILL) {
+            const int32_t st = (own || reach) ? g.tot[T_RE] + g.cptr[i] : 0;
+            if (reach) outs[vm[i] - 1] = make_int4(st, h[Q_XR] + at, n, 0);
+            if (own) outs[nz + i - t0] = make_int4(st, h[Q_XR] + at + (reach ? pad8(n) : 0), n, 0);
+        }
+        xc += tot;
+    }
+    __syncthreads();
+    int32_t nl = 0, ns = 0, xr = 0;
+    for (int32_t base = 0; base < nt; base += GT) {
+        const int32_t j = base + threadIdx.x;
+        const int32_t n = j < nt && in[j] ? g.rlen[j] : 0;
+        int32_t tl, ts, tx;
+        const int32_t l = nl + gscan<GT>(n > TLONG, sh, &tl), k = ns + gscan<GT>(n > 0 && n <= TLONG, sh, &ts),
+                      x0 = xr + gscan<GT>(pad8(n), sh, &tx);
+        if (FILL && n > 0) g.alist[h[Q_AOFF] + (n > TLONG ? l : h[Q_NL] + k)] = make_int4(j, g.rptr[j], x0, n);
+        nl += tl;
+        ns += ts;
+        xr += tx;
+    }
+    if (!FILL && threadIdx.x == 0) {
+        h[Q_NA] = nl + ns;
+        h[Q_NL] = nl;
+        h[Q_XR] = xr;
+        h[Q_XC] = xc;
+    }
+}
+// X by rows (a block each: the columns that hold it, in order) and by columns:
+// planes of the nine entries over the padded length
+template <typename T>
+__global__ void __launch_bounds__(128) k_gr_top_fill(GBuild g, T *X)
+{
+    __shared__ int32_t sh[4];
+    const int32_t nt = g.tot[T_NT], re = g.tot[T_RE];
+    for (int32_t j = blockIdx.x; j < nt; j += gridDim.x) {
+        const int32_t st = g.rptr[j], lp = pad8(g.rlen[j]);
+        int32_t done = 0;
+        for (int32_t base = 0; base <= j; base += 128) {
+            const int32_t i = base + threadIdx.x;
+            int32_t k = -1;
+            if (i <= j)
+                for (int32_t e = g.clen[i] - 1; e >= 0 && k < 0; --e)
+                    if (g.cidx[(size_t)i * CMAX + e] == j) k = e;
+            int32_t tot;
+            const int32_t at = done + gscan<128>(k >= 0 ? 1 : 0, sh, &tot);
+            if (k >= 0) {
+                g.xi[st + at] = i;
+                const double *x = g.cx + ((size_t)i * CMAX + k) * 9;
+                T *o = X + 9 * (size_t)st + at;
+#pragma unroll
+                for (int a = 0; a < 9; ++a) o[(size_t)a * lp] = (T)x[a];
+            }
+            done += tot;
+        }
+        const int32_t cs = re + g.cptr[j], n = g.clen[j], lc = pad8(n);
+        for (int32_t e = threadIdx.x; e < n; e += 128) {
+            g.xi[cs + e] = g.cidx[(size_t)j * CMAX + e];
+            const double *x = g.cx + ((size_t)j * CMAX + e) * 9;
+            T *o = X + 9 * (size_t)cs + e;
+#pragma unroll
+            for (int a = 0; a < 9; ++a) o[(size_t)a * lc] = (T)x[a];
+        }
+    }
 }
 
 // Slots of the parts' sums for the top, grouped by top vertex, parts ascending.
@@ -1181,13 +1372,13 @@ __global__ void __launch_bounds__(GT) k_gr_check(GBuild g)
 {
     const int b = blockIdx.x;
     int bad = 0;
-    const int32_t nt = g.tot[T_NT];
+    const int32_t nt = g.tot[T_NT], xe = g.tot[T_RE] + g.tot[T_CE];
     const int32_t *h = g.hdr + (size_t)Q_N * b;
-    const bool top = b == g.P;
-    const int32_t nv = h[Q_NV], nr = top ? 0 : h[Q_NR], nz = h[Q_NZ], nd = top ? nv : nr + nz, ro = h[Q_ROFF];
-    for (int q = 0; q < 2 && !g.identity; ++q) {
-        const int32_t ns = h[q ? Q_NSB : Q_NSF], B = !top && g.lps == 32 ? SlotSize<float>::B : SlotSize<double>::B;
-        const char *prog = top ? g.tprog[q] : g.prog[q] + (size_t)B * h[q ? Q_SB : Q_SF];
+    const int32_t nv = h[Q_NV], nr = h[Q_NR], nz = h[Q_NZ], nd = nr + nz, ro = h[Q_ROFF], nout = nz + nr - nv,
+                  xl = h[Q_XR] + h[Q_XC];
+    for (int q = 0; q < 2; ++q) {
+        const int32_t ns = h[q ? Q_NSB : Q_NSF], B = g.lps == 32 ? SlotSize<float>::B : SlotSize<double>::B;
+        const char *prog = g.prog[q] + (size_t)B * h[q ? Q_SB : Q_SF];
         for (int32_t i = threadIdx.x; i < 32 * ns; i += GT) {
             const uint32_t r = reinterpret_cast<const uint32_t *>(prog + (size_t)B * (i >> 5))[i & 31];
             if ((int32_t)(r & 8191) > nd || (int32_t)(r >> 13 & 8191) > nd) bad = 32;
@@ -1196,15 +1387,29 @@ __global__ void __launch_bounds__(GT) k_gr_check(GBuild g)
         for (int k = threadIdx.x; k < W_END; k += GT)
             if (ws[k] < 0 || ws[k] > ws[k + 1] || ws[k + 1] > ns) bad = 64;
     }
+    // the top: every row and column that the part reads, and its entries
+    auto entries = [&](int32_t st, int32_t n, int32_t lp, int32_t loc) {
+        bool in = n >= 0 && n <= lp && st >= 0 && st + lp <= xe && loc >= 0 && loc + lp <= xl;
+        for (int32_t e = 0; in && e < n; ++e) in = g.xi[st + e] >= 0 && g.xi[st + e] < nt;
+        return in;
+    };
+    for (int32_t k = threadIdx.x; k < h[Q_NA]; k += GT) {
+        const int4 t = g.alist[h[Q_AOFF] + k];
+        if (t.x < 0 || t.x >= nt || !entries(t.y, t.w, pad8(t.w), t.z)) bad = 256;
+    }
+    for (int32_t z = threadIdx.x; z < nout; z += GT) {
+        const int4 t = g.outs[h[Q_ZOFF] + h[Q_T0] + z];
+        if (!entries(t.x, t.z, pad8(t.z), t.y)) bad = 512;
+    }
     for (int32_t z = threadIdx.x; z < nz; z += GT) {
-        const int32_t zo = h[Q_ZOFF];
-        if (g.zi[zo + z] < 0 || g.zi[zo + z] >= nt || g.zslot[zo + z] < 0 || g.zslot[zo + z] >= g.tlk[nt]) bad = 512;
+        const int32_t k = g.zslot[h[Q_ZOFF] + z];
+        if (k < 0 || k >= g.tlk[nt]) bad = 512;
     }
     for (int32_t l = threadIdx.x; l < pad32(nr); l += GT) {
         const int32_t q = g.perm[ro + l];
         if (q != 0xffff && q >= nr) bad = 1024;
     }
-    if (!top && g.halo)
+    if (g.halo)
         for (int32_t k = threadIdx.x; k < g.rh[R_N * b + R_NH]; k += GT) {
             const int32_t t = g.hl[g.rh[R_N * b + R_HOFF] + k];
             if (t < 0 || t >= g.tot[T_NR] || !g.xflag[t]) bad = 2048;
@@ -1229,18 +1434,21 @@ struct Mat<double> {
 // Placement: byte offsets into shared memory (-1: the array stays in global
 // memory).
 struct GridPlace {
-    int32_t o_p, o_w, o_t, o_tp, o_misc, o_inv, o_nar[2], o_all[2], o_D, o_r, o_x, o_perm, o_hl;
+    int32_t o_p, o_w, o_t, o_u, o_misc, o_X, o_tab, o_nar[2], o_all[2], o_D, o_r, o_x, o_perm, o_hl;
+    int32_t xe;   // entries of X on chip (o_X: their blocks, then their indices)
     int32_t bytes;
 };
 struct GridArgs {
-    int32_t P, nt, ntp, x_given, timing, halo, nslots;
+    int32_t P, nt, x_given, timing, halo, nslots;
     const int32_t *grp;        // per part: first and end part of its system, the system (NULL: one system)
     const double *gtol2;       // per system: tol^2, or below 0 for none to solve (NULL: tol2 for all)
-    const int32_t *hdr, *rh, *ws, *glen, *gso, *i_of_t, *zi, *zslot, *tlk, *hl;
+    const int32_t *hdr, *rh, *ws, *glen, *gso, *i_of_t, *zslot, *tlk, *hl;
+    const int4 *alist, *outs;   // the top: see k_gr_part_top
+    const int32_t *xi;
     const char *prog[2];
     const uint16_t *perm;
     const uint8_t *xflag;
-    const void *D, *inv;       // pivots and rows of the top's inverse, of the solve's type
+    const void *D, *X, *tD;    // pivots, the top's X and pivots, of the solve's type
     const void *jac;           // block-Jacobi inverses, part order planes
     const void *ma, *mb;       // the matrix's rows
     const void *F;             // right-hand side, internal order
@@ -1303,6 +1511,17 @@ struct V3<double, 24> {
         asm volatile("st.shared.f64 [%0+8], %1;" ::"r"(a), "d"(v[1]) : "memory");
         asm volatile("st.shared.f64 [%0+16], %1;" ::"r"(a), "d"(v[2]) : "memory");
     }
+};
+
+template <typename T>
+struct Cell;   // one component of a cell
+template <>
+struct Cell<float> {
+    static __device__ __forceinline__ void st(uint32_t a, float v) { asm volatile("st.shared.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory"); }
+};
+template <>
+struct Cell<double> {
+    static __device__ __forceinline__ void st(uint32_t a, double v) { asm volatile("st.shared.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory"); }
 };
 
 // Sums of products.  FP64: fused multiply-adds.  FP32: the product and the
@@ -1745,41 +1964,6 @@ __device__ __forceinline__ void pivots(const T *D, int32_t nv, uint32_t w)
     }
 }
 
-// Rows of the top's inverse, in FP64: one column of it per block by the top's
-// programs (levels as in the solve), stored as the row it is by symmetry:
-// row 3 k + c of output vertex k, one plane of ntp inputs per (c, component).
-template <typename T>
-__global__ void __launch_bounds__(GT, 1) k_gr_top_inverse(int32_t nt, int32_t ntp, const int32_t *ws, const char *fwd,
-                                                          const char *bwd, const double *D, T *inv)
-{
-    extern __shared__ __align__(16) unsigned char sm[];
-    __shared__ int32_t s_ws[2][W_N];
-    const uint32_t w = (uint32_t)__cvta_generic_to_shared(sm);
-    constexpr int B = SlotSize<double>::B;
-    for (int i = threadIdx.x; i < 2 * W_N; i += GT) s_ws[i / W_N][i % W_N] = ws[i];
-    __syncthreads();
-    const Prog f{s_ws[0], fwd, fwd + (size_t)B * s_ws[0][W_NARROW]}, r{s_ws[1], bwd, bwd + (size_t)B * s_ws[1][W_NARROW]};
-    for (int32_t col = blockIdx.x; col < 3 * nt; col += gridDim.x) {
-        for (int32_t i = threadIdx.x; i <= nt; i += GT) {
-            const double e[3] = {col == 3 * i ? 1.0 : 0.0, col == 3 * i + 1 ? 1.0 : 0.0, col == 3 * i + 2 ? 1.0 : 0.0};
-            V3<double, 24>::st(w + i * 24, e);   // cell nt: the spare one, zero
-        }
-        __syncthreads();
-        run<double, 24, true>(f, w);
-        pivots<double, 24>(D, nt, w);
-        __syncthreads();
-        run<double, 24, false>(r, w);
-        T *o = inv + (size_t)col * 3 * ntp;
-        for (int32_t i = threadIdx.x; i < ntp; i += GT) {
-            double z[3] = {0.0, 0.0, 0.0};
-            if (i < nt) V3<double, 24>::ld(w + i * 24, z);
-#pragma unroll
-            for (int c = 0; c < 3; ++c) o[(size_t)c * ntp + i] = (T)z[c];
-        }
-        __syncthreads();
-    }
-}
-
 // The scalars of a block's solve; warp 0 alone changes them.
 template <typename T>
 struct Solve {
@@ -1935,26 +2119,37 @@ __device__ __noinline__ void sums(const GridArgs &a, Solve<T> &Z, int op)
 
 // A part's numbers: its vertices, rows (with its top vertices), the top
 // vertices that it reaches and their offset, its first top vertex.  It needs
-// z of `nout` top vertices (those it reaches, then those it owns); a row of
-// their inverse, from tb to te (its own system's top vertices), is cut into
-// nch pieces, about one per warp.
+// z of `nout` top vertices (those it reaches, then those it owns), for which it
+// forms `na` rows of the top, `nl` of them long; [tb, te): its own system's top.
 struct PartDims {
-    int32_t nv, nr, ro, t0, nz, zo, nout, nch, chunk, tb, te;
+    int32_t nv, nr, ro, t0, nz, zo, nout, na, nl, tb, te;
 };
 __device__ __forceinline__ PartDims part_of(const GridArgs &a)
 {
     const int32_t *h = a.hdr + (size_t)Q_N * blockIdx.x;
-    PartDims g{h[Q_NV], h[Q_NR], h[Q_ROFF], h[Q_T0], h[Q_NZ], h[Q_ZOFF], 0, 1, 0, 0, a.nt};
+    PartDims g{h[Q_NV], h[Q_NR], h[Q_ROFF], h[Q_T0], h[Q_NZ], h[Q_ZOFF], 0, h[Q_NA], h[Q_NL], 0, a.nt};
     if (a.grp && a.nt > 0) {
         const int32_t *h0 = a.hdr + (size_t)Q_N * a.grp[3 * blockIdx.x], *h1 = a.hdr + (size_t)Q_N * (a.grp[3 * blockIdx.x + 1] - 1);
         g.tb = h0[Q_T0];
         g.te = h1[Q_T0] + h1[Q_NR] - h1[Q_NV];
     }
-    const int32_t npc = (pad32(g.te) - (g.tb & ~31) + 127) / 128;
     g.nout = g.nz + g.nr - g.nv;
-    g.nch = g.nout > 0 ? max(1, min(npc, GW / g.nout)) : 1;
-    g.chunk = (npc + g.nch - 1) / g.nch * 128;
     return g;
+}
+// The top's tables and X as the part reads them (in shared or global memory).
+template <typename T>
+struct Top {
+    const int4 *alist, *outs;
+    const T *X, *D;
+    const int32_t *xi;
+    bool local;   // X packed on chip
+};
+template <typename T>
+__device__ __forceinline__ Top<T> top_of(const GridArgs &a, const PartDims &g)
+{
+    const int32_t *h = a.hdr + (size_t)Q_N * blockIdx.x;
+    return Top<T>{a.alist + h[Q_AOFF], a.outs + g.zo + g.t0, reinterpret_cast<const T *>(a.X),
+                  reinterpret_cast<const T *>(a.tD), a.xi, false};
 }
 
 // One forest solve, in three steps (w: the right-hand side in, the solution
@@ -2021,54 +2216,85 @@ __device__ __forceinline__ bool gather_top(const GridArgs &a, const PartDims &g,
     return ok;
 }
 
-// Then (after a barrier) the top, as far as the part needs it: the rows of its
-// inverse times the top's right-hand side, a warp per row or piece of a row
-// (several blocks per lane in flight), then the pieces in order; then the
-// part's backward levels.
+// Then (after a barrier) the top, as far as the part needs it: u = D^-1 X r in
+// the rows that its outputs' columns name, a warp or 8 lanes per row; z = X^T u,
+// 8 lanes per output; then the part's backward levels.
 template <typename T, int VB>
-__device__ __forceinline__ void tree_down(const GridArgs &a, const PartDims &g, const Prog *s_prog, const T *inv, uint32_t w,
-                                          uint32_t tw, T *tp)
+__device__ __forceinline__ void tree_down(const PartDims &g, const Prog *s_prog, const Top<T> &top, uint32_t w, uint32_t tw, uint32_t tu)
 {
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int32_t nout = g.nout, nch = g.nch, chunk = g.chunk, nz = g.nz, zo = g.zo, t0 = g.t0, nr = g.nr, nv = g.nv,
-                  kb = g.tb & ~31, ke = pad32(g.te);
-    for (int32_t it = warp; it < nout * nch; it += GW) {
-        const int32_t o = it / nch, k0 = kb + (it - o * nch) * chunk, k1 = min(ke, k0 + chunk);
-        const int32_t i = o < nz ? __ldg(a.zi + zo + o) : t0 + o - nz;
-        const T *f = inv + (size_t)(a.pl.o_inv >= 0 ? o : i) * 9 * a.ntp + lane;
-        T z[3] = {0, 0, 0};
-        constexpr int N = sizeof(T) == 4 ? 4 : 2;
-        for (int32_t k = k0; k < k1; k += 32 * N) {
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, l8 = lane & 7;
+    const int32_t nout = g.nout, nl = g.nl, na = g.na, nz = g.nz, nr = g.nr, nv = g.nv, items = nl + (na - nl + 3) / 4;
+    const bool loc = top.local;
+    constexpr int N = sizeof(T) == 4 ? 4 : 2;   // blocks in flight per lane
+    for (int32_t it = warp; it < items; it += GW) {
+        const bool lng = it < nl;
+        const int32_t k = lng ? it : nl + 4 * (it - nl) + (lane >> 3), G = lng ? 32 : 8, l = lng ? lane : l8;
+        const int4 t = k < na ? top.alist[k] : make_int4(0, 0, 0, 0);
+        const int32_t len = t.w, lp = pad8(len), st = loc ? t.z : t.y;
+        const int32_t *xi = top.xi + st;
+        const T *x = top.X + 9 * (size_t)st;
+        // row l of D^-1 (its six entries: 00 01 02 11 12 22)
+        T d[3] = {0, 0, 0};
+        if (l < 3 && k < na) {
+            const T *D = top.D + (size_t)(t.x >> 5) * 192 + (t.x & 31);
+            d[0] = __ldg(D + 32 * l);
+            d[1] = __ldg(D + 32 * (l == 0 ? 1 : l + 2));
+            d[2] = __ldg(D + 32 * (l == 0 ? 2 : l + 3));
+        }
+        const int32_t most = __reduce_max_sync(0xffffffffu, len);
+        T y[3] = {0, 0, 0};
+        for (int32_t e0 = 0; e0 < most; e0 += G * N) {
             T m[N][9];
-#pragma unroll
-            for (int u = 0; u < N; ++u)
-#pragma unroll
-                for (int c = 0; c < 9; ++c) m[u][c] = k + 32 * u < k1 ? f[(size_t)c * a.ntp + k + 32 * u] : T(0);
+            int32_t i[N];
 #pragma unroll
             for (int u = 0; u < N; ++u) {
-                if (k + 32 * u >= k1) break;
-                T y[3];
-                V3<T, VB>::ld(tw + (k + lane + 32 * u) * VB, y);   // 0 outside [tb, te)
+                const int32_t e = e0 + G * u + l;
+                i[u] = e < len ? xi[e] : -1;
+#pragma unroll
+                for (int c = 0; c < 9; ++c) m[u][c] = e < len ? x[(size_t)c * lp + e] : T(0);
+            }
+#pragma unroll
+            for (int u = 0; u < N; ++u) {
+                if (e0 + G * u >= most) break;
+                T r[3] = {0, 0, 0};
+                if (i[u] >= 0) V3<T, VB>::ld(tw + i[u] * VB, r);
 #pragma unroll
                 for (int c = 0; c < 3; ++c)
-                    z[c] = fma(m[u][3 * c + 2], y[2], fma(m[u][3 * c + 1], y[1], fma(m[u][3 * c], y[0], z[c])));
+                    y[c] = fma(m[u][3 * c + 2], r[2], fma(m[u][3 * c + 1], r[1], fma(m[u][3 * c], r[0], y[c])));
             }
         }
+        if (lng)
 #pragma unroll
-        for (int b = 16; b > 0; b >>= 1)
+            for (int b = 16; b > 4; b >>= 1)
 #pragma unroll
-            for (int c = 0; c < 3; ++c) z[c] += __shfl_xor_sync(0xffffffffu, z[c], b);
-        if (lane == 0) {
-            tp[3 * it] = z[0]; tp[3 * it + 1] = z[1]; tp[3 * it + 2] = z[2];
-        }
+                for (int c = 0; c < 3; ++c) y[c] += __shfl_xor_sync(0xffffffffu, y[c], b);
+#pragma unroll
+        for (int b = 4; b > 0; b >>= 1)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) y[c] += __shfl_xor_sync(0xffffffffu, y[c], b);
+        if (l < 3 && k < na) Cell<T>::st(tu + t.x * VB + l * sizeof(T), fma(d[2], y[2], fma(d[1], y[1], d[0] * y[0])));
     }
     __syncthreads();
-    for (int32_t o = tid; o < nout; o += GT) {
+    for (int32_t base = 4 * warp; base < nout; base += 4 * GW) {
+        const int32_t o = base + (lane >> 3);
+        const int4 t = o < nout ? top.outs[o] : make_int4(0, 0, 0, 0);
+        const int32_t len = t.z, lp = pad8(len), st = loc ? t.y : t.x;
+        const int32_t *xi = top.xi + st;
+        const T *x = top.X + 9 * (size_t)st;
         T z[3] = {0, 0, 0};
-        for (int32_t k = o * nch; k < (o + 1) * nch; ++k) {
-            z[0] += tp[3 * k]; z[1] += tp[3 * k + 1]; z[2] += tp[3 * k + 2];
+        for (int32_t e = l8; e < len; e += 8) {
+            T u[3];
+            V3<T, VB>::ld(tu + xi[e] * VB, u);
+#pragma unroll
+            for (int c = 0; c < 3; ++c)
+                z[c] = fma(x[(size_t)(6 + c) * lp + e], u[2], fma(x[(size_t)(3 + c) * lp + e], u[1], fma(x[(size_t)c * lp + e], u[0], z[c])));
         }
-        V3<T, VB>::st(w + (o < nz ? nr + o : nv + o - nz) * VB, z);
+        __syncwarp();
+#pragma unroll
+        for (int b = 4; b > 0; b >>= 1)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) z[c] += __shfl_xor_sync(0xffffffffu, z[c], b);
+        if (l8 == 0 && o < nout) V3<T, VB>::st(w + (o < nz ? nr + o : nv + o - nz) * VB, z);
     }
     __syncthreads();
     run<T, VB, false>(s_prog[1], w);
@@ -2114,7 +2340,8 @@ __global__ void __launch_bounds__(GT, 1) k_pcg_grid(const __grid_constant__ Grid
         gso[i] = a.gso[ro / 32 + i];
     }
     const int32_t *hl = put(a.hl + a.rh[R_N * blockIdx.x + R_HOFF], a.pl.o_hl, a.halo ? nh : 0);
-    const T *D = nullptr, *inv = nullptr;
+    const T *D = nullptr;
+    Top<T> top{};
     if (PREC == 0) {
         D = put(reinterpret_cast<const T *>(a.D) + 6 * (size_t)ro, a.pl.o_D, 6 * pad32(nv));
         constexpr int B = SlotSize<T>::B;
@@ -2134,20 +2361,24 @@ __global__ void __launch_bounds__(GT, 1) k_pcg_grid(const __grid_constant__ Grid
             const T zero[3] = {0, 0, 0};
             V3<T, VB>::st(w + (nr + g.nz) * VB, zero);
         }
-        for (int i = tid; i < a.ntp; i += GT) {   // lanes beside the system's top vertices
-            const T zero[3] = {0, 0, 0};
-            V3<T, VB>::st(tw + i * VB, zero);
+        top = top_of<T>(a, g);
+        if (a.pl.o_tab >= 0) {
+            top.alist = put(top.alist, a.pl.o_tab, g.na);
+            top.outs = put(top.outs, a.pl.o_tab + 16 * g.na, g.nout);
         }
-        // the rows of the top's inverse that the part needs, when they fit
-        inv = reinterpret_cast<const T *>(a.inv);
-        if (a.pl.o_inv >= 0) {
-            T *d = reinterpret_cast<T *>(sm + a.pl.o_inv);
-            for (int32_t o = 0; o < g.nout; ++o) {
-                const int32_t i = o < g.nz ? __ldg(a.zi + g.zo + o) : g.t0 + o - g.nz;
-                const T *f = inv + (size_t)i * 9 * a.ntp;
-                for (int32_t k = tid; k < 9 * a.ntp; k += GT) d[(size_t)o * 9 * a.ntp + k] = f[k];
+        // the rows and columns of X that the part needs, when they fit
+        if (a.pl.o_X >= 0) {
+            T *xd = reinterpret_cast<T *>(sm + a.pl.o_X);
+            int32_t *xi = reinterpret_cast<int32_t *>(sm + a.pl.o_X + 9 * sizeof(T) * (size_t)a.pl.xe);
+            for (int32_t k = warp; k < g.na + g.nout; k += GW) {
+                const int4 t = k < g.na ? a.alist[h[Q_AOFF] + k] : a.outs[g.zo + g.t0 + k - g.na];
+                const int32_t from = k < g.na ? t.y : t.x, at = k < g.na ? t.z : t.y, n = pad8(k < g.na ? t.w : t.z);
+                for (int32_t e = lane; e < n; e += 32) xi[at + e] = top.xi[from + e];
+                for (int32_t e = lane; e < 9 * n; e += 32) xd[9 * (size_t)at + e] = top.X[9 * (size_t)from + e];
             }
-            inv = d;
+            top.X = xd;
+            top.xi = xi;
+            top.local = true;
         }
     }
     T *r = a.pl.o_r >= 0 ? reinterpret_cast<T *>(sm + a.pl.o_r) : reinterpret_cast<T *>(a.r) + 3 * (size_t)ro;
@@ -2328,7 +2559,7 @@ __global__ void __launch_bounds__(GT, 1) k_pcg_grid(const __grid_constant__ Grid
             break;
         }
         if (PREC == 0) {
-            tree_down<T, VB>(a, g, s_prog, inv, w, tw, reinterpret_cast<T *>(sm + a.pl.o_tp));
+            tree_down<T, VB>(g, s_prog, top, w, tw, sm0 + a.pl.o_u);
         }
         if (PREC == 0 || phase <= 0) {
             Acc<T> acc;
@@ -2427,14 +2658,13 @@ __global__ void __launch_bounds__(GT, 1) k_apply_grid(const __grid_constant__ Gr
     }
     const T zero[3] = {0, 0, 0};
     if (tid == 0) V3<T, VB>::st(w + (g.nr + g.nz) * VB, zero);   // the spare cell
-    for (int i = a.nt + tid; i < a.ntp; i += GT) V3<T, VB>::st(tw + i * VB, zero);
     unsigned long long *trx = a.lx + (size_t)Pkt<T>::W * a.nslots;
     tree_up<T, VB>(a, g, s_prog, reinterpret_cast<const T *>(a.D) + 6 * (size_t)g.ro, w, trx, 1u);
     if (!gather_top<T, VB>(a, g, tw, trx, 1u, 0)) s_bad = 1;
     __syncthreads();
     const bool bad = s_bad != 0;
     if (!bad)
-        tree_down<T, VB>(a, g, s_prog, reinterpret_cast<const T *>(a.inv), w, tw, reinterpret_cast<T *>(sm + a.pl.o_tp));
+        tree_down<T, VB>(g, s_prog, top_of<T>(a, g), w, tw, sm0 + a.pl.o_u);
     for (int32_t b = tid; b < g.nr; b += N * GT) {
         int32_t v[N];
 #pragma unroll
@@ -2479,15 +2709,15 @@ bool place(const GridLayout &G, int32_t mnh, size_t sz, size_t vb, bool tree, bo
     pl->o_p = need(3 * sz * (mnr + (halo ? (size_t)mnh : 0)));
     pl->o_w = need(vb * (size_t)(tree ? t[T_MDZ] + 1 : t[T_MNR]));
     pl->o_t = need(vb * pad32((int32_t)nt));
-    pl->o_tp = need(3 * sz * (tree ? (size_t)std::max(GW, t[T_MNO]) : 0));
+    pl->o_u = need(vb * pad32((int32_t)nt));
     pl->o_misc = need(8 * (mnr / 32 + 1));
     if (at > (size_t)GRID_SMEM) return false;
     for (int q = 0; q < 2; ++q) pl->o_nar[q] = pl->o_all[q] = -1;
-    pl->o_D = pl->o_inv = -1;
+    pl->o_D = pl->o_X = pl->o_tab = -1;
     pl->o_perm = opt(2 * (size_t)pad32((int32_t)mnr));
     pl->o_hl = halo ? opt(4 * (size_t)mnh) : -1;
     if (tree) {
-        pl->o_inv = opt(9 * sz * (size_t)pad32((int32_t)nt) * (size_t)t[T_MNO]);
+        pl->o_tab = opt(16 * ((size_t)t[T_MNA] + (size_t)t[T_MNO]));
         // the whole programs when they fit beside r and x, else the narrow levels
         const size_t all = B * ((size_t)t[T_MSF] + (size_t)t[T_MSB]) + 6 * sz * mnr + 64;
         if (at + all <= (size_t)GRID_SMEM)
@@ -2499,6 +2729,8 @@ bool place(const GridLayout &G, int32_t mnh, size_t sz, size_t vb, bool tree, bo
     pl->o_x = opt(3 * sz * mnr);
     if (tree) {
         pl->o_D = opt(6 * sz * (size_t)pad32((int32_t)mnr));
+        pl->xe = t[T_MX];
+        pl->o_X = opt((9 * sz + 4) * (size_t)t[T_MX]);
         for (int q = 0; q < 2; ++q)
             if (pl->o_all[q] < 0) {
                 // more room after all: one whole program
@@ -2522,10 +2754,10 @@ bool place_apply(const GridLayout &G, size_t sz, size_t vb, GridPlace *pl)
     };
     const size_t B = sz == 4 ? SlotSize<float>::B : SlotSize<double>::B;
     *pl = GridPlace{};
-    pl->o_inv = -1;
+    pl->o_X = pl->o_tab = -1;
     pl->o_w = need(vb * (size_t)(t[T_MDZ] + 1));
     pl->o_t = need(vb * (size_t)pad32(t[T_NT]));
-    pl->o_tp = need(3 * sz * (size_t)std::max(GW, t[T_MNO]));
+    pl->o_u = need(vb * (size_t)pad32(t[T_NT]));
     if (at > (size_t)GRID_SMEM) return false;
     for (int q = 0; q < 2; ++q) {
         const size_t b = B * (size_t)(q ? t[T_MNB] : t[T_MNF]);
@@ -2646,25 +2878,16 @@ sgp_status numeric(sgp_ctx *ctx, GridLayout &G, const sgp_factor *F, const GBuil
     const int32_t *t = G.tot;
     const double *L = bp<const double>(F->L), *Di = bp<const double>(F->Dinv);
     const int32_t nf = 32 * t[T_SF], nb = 32 * t[T_SB], nr = t[T_NR], nt = t[T_NT], B = SGP_BLOCK;
-    T *D, *inv;
-    double *tD;
-    const int32_t ntp = pad32(nt), us[2] = {G.top_slots[0], G.top_slots[1]};
+    T *D, *X, *tD;
     SGP_TRY(ensure(ctx, G.D, 6 * (size_t)nr, &D));
-    SGP_TRY(ensure(ctx, G.inv, 9 * (size_t)ntp * nt, &inv));
-    SGP_TRY(ensure(ctx, G.tD, 6 * (size_t)ntp, &tD));
+    SGP_TRY(ensure(ctx, G.X, 9 * ((size_t)t[T_RE] + (size_t)t[T_CE]), &X));
+    SGP_TRY(ensure(ctx, G.tD, 6 * (size_t)pad32(nt), &tD));
     LAUNCH(ctx, (k_gr_blocks<T, false>), grid_for(nf, B), B, 0, nf, (const int32_t *)g.msrc[0], L, g.prog[0]);
     LAUNCH(ctx, (k_gr_blocks<T, true>), grid_for(nb, B), B, 0, nb, (const int32_t *)g.msrc[1], L, g.prog[1]);
     LAUNCH(ctx, k_gr_pivots<T>, grid_for(nr, B), B, 0, nr, (const int32_t *)g.d_src, Di, D);
     if (nt == 0) return SGP_OK;
-    LAUNCH(ctx, (k_gr_blocks<double, false>), grid_for(32 * us[0], B), B, 0, 32 * us[0], (const int32_t *)g.tmsrc[0], L,
-           g.tprog[0]);
-    LAUNCH(ctx, (k_gr_blocks<double, true>), grid_for(32 * us[1], B), B, 0, 32 * us[1], (const int32_t *)g.tmsrc[1], L,
-           g.tprog[1]);
-    LAUNCH(ctx, k_gr_pivots<double>, grid_for(nt, B), B, 0, nt, td_src, Di, tD);
-    SGP_CUDA(ctx, cudaFuncSetAttribute(k_gr_top_inverse<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 24 * (NTOP + 1)));
-    LAUNCH(ctx, k_gr_top_inverse<T>, std::min(3 * nt, ctx->num_sms * 4), GT, 24 * (size_t)(nt + 1), nt, ntp,
-           (const int32_t *)(g.ws + (size_t)G.P * 2 * W_N), (const char *)g.tprog[0], (const char *)g.tprog[1],
-           (const double *)tD, inv);
+    LAUNCH(ctx, k_gr_top_fill<T>, nt, 128, 0, g, X);
+    LAUNCH(ctx, k_gr_pivots<T>, grid_for(nt, B), B, 0, nt, td_src, Di, tD);
     return SGP_OK;
 }
 
@@ -2823,15 +3046,25 @@ sgp_status grid_build(sgp_ctx *ctx, sgp_factor *F, const sgp_matrix *M)
     SGP_TRY(S.take(NP, &g.sgf));
     SGP_TRY(S.take(PB, &g.nseg));
     SGP_TRY(S.take(PB * 2 * LMAX * NCLS, &g.kb));
+    SGP_TRY(S.take(NTOP, &g.clen));
+    SGP_TRY(S.take(NTOP, &g.rlen));
+    SGP_TRY(S.take(NTOP, &g.cptr));
+    SGP_TRY(S.take(NTOP, &g.rptr));
+    SGP_TRY(S.take((size_t)NTOP * CMAX, &g.cidx));
+    SGP_TRY(S.take((size_t)NTOP * CMAX * 9, &g.cx));
+    SGP_CUDA(ctx, cudaMemsetAsync(g.rlen, 0, sizeof(int32_t) * NTOP, ctx->stream));
     g.lp = lp; g.seg = seg; g.sp = sp; g.lpos = lpos;
     if (f32) g.col32 = reinterpret_cast<const float2 *>(bp<const float4>(M->blk32) + 2 * M->m);
     SGP_CUDA(ctx, cudaMemsetAsync(g.tot, 0, sizeof(int32_t) * T_N, ctx->stream));
     LAUNCH(ctx, k_gr_rows, 1, 256, 0, P, NI, d_ipart, nblk, (const int32_t *)off, g.hdr, g.tot);
     const unsigned gy = (unsigned)std::max(1, std::min(8, U / GT));
     SGP_TRY(sgp_launch(ctx, "k_gr_row_maps", k_gr_row_maps, dim3(P, gy), dim3(GT), 0, g));
-    LAUNCH(ctx, k_gr_part_count, P + 1, GT, 0, g);
+    LAUNCH(ctx, k_gr_part_count, P, GT, 0, g);
     LAUNCH(ctx, k_gr_offsets1, 1, 256, 0, P, g.hdr, g.tot);
-    LAUNCH(ctx, k_gr_segments, P + 1, GT, 0, g);
+    LAUNCH(ctx, k_gr_cols, 3 * NTOP / 96, 96, 0, g, bp<const double>(F->L));
+    LAUNCH(ctx, k_gr_top_offsets, 1, 1024, 0, g);
+    LAUNCH(ctx, k_gr_part_top<false>, P, GT, 0, g);
+    LAUNCH(ctx, k_gr_segments, P, GT, 0, g);
     GridRows &R = G.rows;
     SGP_TRY(rows_count(ctx, R, g, M, NRmax));
     LAUNCH(ctx, k_gr_offsets2, 1, 256, 0, P, g.hdr, g.tot, (const int32_t *)g.ws);
@@ -2843,8 +3076,6 @@ sgp_status grid_build(sgp_ctx *ctx, sgp_factor *F, const sgp_matrix *M)
     SGP_TRY(read_back(ctx, hs.top, g.hdr + (size_t)Q_N * P, sizeof(hs.top)));
     SGP_TRY(read_back(ctx, R.tot, g.rh + R_N * P, sizeof(R.tot)));
     memcpy(G.tot, hs.t, sizeof(hs.t));
-    G.top_slots[0] = hs.top[Q_NSF];
-    G.top_slots[1] = hs.top[Q_NSB];
     if (G.tot[T_ERR] || G.tot[T_MDZ] > 8190) return SGP_OK;
     GridPlace pl;
     const bool rows = rows_place(G, R, M, f32, true), apply = !f32 && place_apply(G, 8, 24, &pl);
@@ -2854,23 +3085,22 @@ sgp_status grid_build(sgp_ctx *ctx, sgp_factor *F, const sgp_matrix *M)
         const size_t slots = (size_t)G.tot[q ? T_SB : T_SF];
         SGP_TRY(ensure(ctx, G.prog[q], slots * (f32 ? SlotSize<float>::B : SlotSize<double>::B), &g.prog[q]));
         SGP_TRY(S.take(32 * slots, &g.msrc[q]));
-        SGP_TRY(S.take((size_t)G.top_slots[q] * SlotSize<double>::B, &g.tprog[q]));
-        SGP_TRY(S.take(32 * (size_t)G.top_slots[q], &g.tmsrc[q]));
     }
-    SGP_TRY(ensure(ctx, G.zi, G.tot[T_Z], &g.zi));
+    SGP_TRY(ensure(ctx, G.alist, G.tot[T_A], &g.alist));
+    SGP_TRY(ensure(ctx, G.outs, (size_t)G.tot[T_Z] + (size_t)G.tot[T_NT], &g.outs));
+    SGP_TRY(ensure(ctx, G.xi, (size_t)G.tot[T_RE] + (size_t)G.tot[T_CE], &g.xi));
     SGP_TRY(ensure(ctx, G.zslot, G.tot[T_Z], &g.zslot));
     SGP_TRY(ensure(ctx, G.tlk, (size_t)G.tot[T_NT] + 1, &g.tlk));
-    SGP_TRY(sgp_launch(ctx, "k_gr_program", f32 ? k_gr_program<float> : k_gr_program<double>, dim3(P, 2), dim3(GT), 0, g, 0));
-    if (G.tot[T_NT] > 0)
-        SGP_TRY(sgp_launch(ctx, "k_gr_program", k_gr_program<double>, dim3(1, 2), dim3(GT), 0, g, P));
+    SGP_TRY(sgp_launch(ctx, "k_gr_program", f32 ? k_gr_program<float> : k_gr_program<double>, dim3(P, 2), dim3(GT), 0, g));
+    LAUNCH(ctx, k_gr_part_top<true>, P, GT, 0, g);
     LAUNCH(ctx, k_gr_slots, 1, 1024, 0, g);
     if (rows) SGP_TRY(rows_fill(ctx, G, R, g, M, f32));
-    LAUNCH(ctx, k_gr_check, P + 1, GT, 0, g);
     const int32_t *td_src = sp + hs.top[Q_SOFF];
     if (f32)
         SGP_TRY(numeric<float>(ctx, G, F, g, td_src));
     else
         SGP_TRY(numeric<double>(ctx, G, F, g, td_src));
+    LAUNCH(ctx, k_gr_check, P, GT, 0, g);
     SGP_TRY(read_back(ctx, hs.t, g.tot, sizeof(hs.t)));
     if (hs.t[T_ERR]) return sgp_fail(ctx, SGP_ERR_CUDA, "tree_factor: inconsistent grid layout (0x%x)", hs.t[T_ERR]);
     G.prec = F->precision;
@@ -2961,8 +3191,8 @@ void grid_rows_release(GridRows &R)
 }
 void grid_release(GridLayout &G)
 {
-    for (DBuf *d : {&G.hdr, &G.dtot, &G.ws, &G.zi, &G.zslot, &G.tlk, &G.i_of_t, &G.t_of_i, &G.prog[0], &G.prog[1], &G.D,
-                    &G.inv, &G.tD, &G.apply})
+    for (DBuf *d : {&G.hdr, &G.dtot, &G.ws, &G.alist, &G.outs, &G.xi, &G.zslot, &G.tlk, &G.i_of_t, &G.t_of_i, &G.prog[0], &G.prog[1], &G.D,
+                    &G.X, &G.tD, &G.apply})
         if (d->p) cudaFree(d->p);
     for (DBuf &d : G.scr)
         if (d.p) cudaFree(d.p);
@@ -3010,6 +3240,13 @@ size_t grid_work_bytes(const GridLayout &G, size_t sz, int ng)
            sizeof(Scal) * (size_t)ng;
 }
 
+static void top_args(const GridLayout &G, GridArgs &a)
+{
+    a.alist = bp<const int4>(G.alist); a.outs = bp<const int4>(G.outs);
+    a.xi = bp<const int32_t>(G.xi);
+    a.X = G.X.p; a.tD = G.tD.p;
+}
+
 // x = P^-1 b of an FP64 factor in one launch, without a host synchronisation;
 // a wait that gives up leaves NaN.  orig_of: the caller's order, or NULL for
 // the internal one; nothing is done when *done is set.
@@ -3024,12 +3261,13 @@ sgp_status grid_apply(sgp_ctx *ctx, const sgp_factor *F, const DBuf &ws, const d
     const int32_t *t = G.tot;
     GridArgs a{};
     if (!place_apply(G, 8, 24, &a.pl)) return sgp_fail(ctx, SGP_ERR_CUDA, "tree solve: the grid layout does not fit");
-    a.P = G.P; a.nt = t[T_NT]; a.ntp = pad32(a.nt); a.nslots = t[T_Z];
+    a.P = G.P; a.nt = t[T_NT]; a.nslots = t[T_Z];
     a.hdr = bp<const int32_t>(G.hdr); a.ws = bp<const int32_t>(G.ws);
     a.i_of_t = bp<const int32_t>(G.i_of_t);
-    a.zi = bp<const int32_t>(G.zi); a.zslot = bp<const int32_t>(G.zslot); a.tlk = bp<const int32_t>(G.tlk);
+    top_args(G, a);
+    a.zslot = bp<const int32_t>(G.zslot); a.tlk = bp<const int32_t>(G.tlk);
     for (int q = 0; q < 2; ++q) a.prog[q] = bp<const char>(G.prog[q]);
-    a.D = G.D.p; a.inv = G.inv.p;
+    a.D = G.D.p;
     a.F = b; a.x = x;
     a.err = bp<int>(ws);
     a.lx = reinterpret_cast<unsigned long long *>(ws.p) + 2;
@@ -3080,14 +3318,15 @@ sgp_status grid_pcg(sgp_ctx *ctx, const sgp_matrix *M, const GridLayout &G, cons
     if (a.pl.o_r < 0) a.r = take(3 * sizeof(T) * nr);
     if (a.pl.o_x < 0) a.xt = take(3 * sizeof(T) * nr);
     a.P = G.P; a.nt = tree ? t[T_NT] : 0; a.x_given = x_given; a.timing = ctx->timing; a.halo = R.halo;
-    a.ntp = pad32(a.nt); a.nslots = t[T_Z];
+    a.nslots = t[T_Z];
     a.hdr = bp<const int32_t>(G.hdr); a.rh = bp<const int32_t>(R.rh); a.ws = bp<const int32_t>(G.ws);
     a.glen = bp<const int32_t>(R.glen); a.gso = bp<const int32_t>(R.gso); a.i_of_t = bp<const int32_t>(G.i_of_t);
-    a.zi = bp<const int32_t>(G.zi); a.zslot = bp<const int32_t>(G.zslot); a.tlk = bp<const int32_t>(G.tlk);
+    top_args(G, a);
+    a.zslot = bp<const int32_t>(G.zslot); a.tlk = bp<const int32_t>(G.tlk);
     a.hl = bp<const int32_t>(R.hl);
     a.perm = bp<const uint16_t>(R.perm); a.xflag = bp<const uint8_t>(R.xflag);
     for (int q = 0; q < 2; ++q) a.prog[q] = bp<const char>(G.prog[q]);
-    a.D = a.jac = G.D.p; a.inv = G.inv.p; a.ma = R.ma.p; a.mb = R.mb.p;
+    a.D = a.jac = G.D.p; a.ma = R.ma.p; a.mb = R.mb.p;
     a.F = F; a.x = x;
     a.gamma0 = M->gamma0;
     a.tol2 = stopE ? -1.0 : tol * tol;

@@ -57,9 +57,10 @@ struct GridLayout {
     int ok = 0, prec = 0;
     int64_t nr_max = 0;
     int32_t P = 0, LV = 0;
-    int32_t tot[24] = {0}, top_slots[2] = {0, 0};   // totals and maxima over the parts; slots of the top's programs
-    DBuf hdr, dtot, ws, zi, zslot, tlk, i_of_t, t_of_i;
-    DBuf prog[2], D, inv, tD;
+    int32_t tot[32] = {0};                          // totals and maxima over the parts
+    DBuf hdr, dtot, ws, zslot, tlk, i_of_t, t_of_i;
+    DBuf prog[2], D;
+    DBuf alist, outs, xi, X, tD;                    // the top: its tables, X = L^-1 and pivots
     DBuf apply;                                     // error word and packets of a forest solve alone
     size_t apply_bytes = 0;
     DBuf scr[SGP_GRID_SCRATCH];
