@@ -63,7 +63,10 @@ __device__ __forceinline__ void pq_finish(Scal *sc, double pq)
 // 172 us.
 // DOT: inside a PCG step, with v^T y; the last block sets alpha = rho / v^T y
 // (in place of k_spmv_pq<double, 1, 1>, 238 us at 1e6 cells: FP64 steps of
-// 700,000 and 800,000 cells 129.7 -> 111.5 and 143.9 -> 124.9 ms).
+// 700,000 and 800,000 cells 129.7 -> 111.5 and 143.9 -> 124.9 ms).  Which lane
+// gets which of a block's rows of one length depends on timing (atomics), so a
+// row's term of v^T y goes to its place in shared memory and the terms are
+// summed in row order: the same bits in every run.
 template <int R, int NT, bool DOT>
 __global__ void __launch_bounds__(NT, 1024 / NT) k_product64(Blk<double> B, const int32_t *__restrict__ row_ptr, double gamma0,
                                                   int64_t n, const double *__restrict__ v,
@@ -71,8 +74,8 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_product64(Blk<double> B, cons
                                                   double *partials, Scal *sc)
 {
     if (DOT && sc->done) return;
-    double dot = 0.0;
     __shared__ int32_t cnt[64], row[R];
+    __shared__ double term[DOT ? R : 1];
     const int tid = threadIdx.x;
     const int64_t i0 = blockIdx.x * (int64_t)R;
     constexpr int K = R / NT;
@@ -104,7 +107,9 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_product64(Blk<double> B, cons
     __syncthreads();
     for (int k = 0; k < K; ++k) {
         // a warp's groups of 32 rows: long and short ones
-        const int64_t i = i0 + row[k & 1 ? (k + 1) * NT - 32 - (tid & ~31) + (tid & 31) : k * NT + tid];
+        const int32_t at = row[k & 1 ? (k + 1) * NT - 32 - (tid & ~31) + (tid & 31) : k * NT + tid];
+        const int64_t i = i0 + at;
+        if (DOT && i >= n) term[at] = 0.0;
         if (i >= n) continue;
         const double v0 = v[3 * i], v1 = v[3 * i + 1], v2 = v[3 * i + 2];
         double y0 = gamma0 * v0, y1 = gamma0 * v1, y2 = gamma0 * v2;
@@ -143,10 +148,14 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_product64(Blk<double> B, cons
         y0 += z0; y1 += z1; y2 += z2;
         const int64_t o = orig_of ? orig_of[i] : i;
         y[3 * o] = y0; y[3 * o + 1] = y1; y[3 * o + 2] = y2;
-        if (DOT) dot += fma(v2, y2, fma(v1, y1, v0 * y0));
+        if (DOT) term[at] = fma(v2, y2, fma(v1, y1, v0 * y0));
     }
     if (DOT) {
         __shared__ double sh[NT / 32];
+        __syncthreads();
+        double dot = 0.0;
+#pragma unroll
+        for (int k = 0; k < K; ++k) dot += term[k * NT + tid];
         const double s = block_sum<NT>(dot, sh);
         if (tid == 0) partials[blockIdx.x] = s;
         if (last_block(&sc->cnt)) {
