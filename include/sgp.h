@@ -240,7 +240,10 @@ sgp_status sgp_local_spanning_forest(sgp_ctx *ctx, const sgp_matrix *matrix, con
 sgp_status sgp_tree_factor(sgp_ctx *ctx, const sgp_matrix *matrix, const sgp_tree *tree,
                            sgp_factor **factor);
 /* x = P^{-1} b in FP64 (forward substitution, diagonal solve, backward
- * substitution, Appendix B.1).  b_dev, x_dev: n x 3 float64; may alias. */
+ * substitution, Appendix B.1).  b_dev, x_dev: n x 3 float64; may alias.
+ * Asynchronous.  A bounded device wait that gives up (see SGP_ERR_TIMEOUT)
+ * leaves NaN in x and is reported as TIMEOUT by the context's next
+ * sgp_tree_apply, solve or network call that finds it. */
 sgp_status sgp_tree_apply(sgp_ctx *ctx, const sgp_factor *factor, const double *b_dev,
                           double *x_dev);
 /* Shape of the factor: contraction levels (rounds == levels: each level

@@ -479,16 +479,24 @@ sgp_status sgp_create(sgp_ctx **out, int device, void *stream)
     if (ns && atoi(ns)) ctx->small_solve = 0;
     const char *nf = getenv("SGP_NO_FUSE");
     if (nf && atoi(nf)) ctx->fused = 0;
+    const char *wp = getenv("SGP_WAIT_POLLS");
+    if (wp) ctx->wait_polls = std::max(0, atoi(wp));
     if (scratch_ensure(ctx, 1 << 20) != SGP_OK || cudaMalloc(&ctx->d_flags, 4096) != cudaSuccess ||
-        cudaMemset(ctx->d_flags, 0, 4096) != cudaSuccess) {
+        cudaMemset(ctx->d_flags, 0, 4096) != cudaSuccess ||
+        cudaHostAlloc(&ctx->h_gave_up, 64, cudaHostAllocMapped) != cudaSuccess ||
+        cudaHostGetDevicePointer(&ctx->d_gave_up, ctx->h_gave_up, 0) != cudaSuccess) {
         cudaGetLastError();
         if (ctx->d_scratch) cudaFree(ctx->d_scratch);
+        if (ctx->d_flags) cudaFree(ctx->d_flags);
+        if (ctx->h_gave_up) cudaFreeHost(ctx->h_gave_up);
         delete ctx;
         return SGP_ERR_OOM;
     }
+    *ctx->h_gave_up = 0;
     if (noalloc_prepare(ctx) != SGP_OK) {
         cudaFree(ctx->d_scratch);
         cudaFree(ctx->d_flags);
+        cudaFreeHost(ctx->h_gave_up);
         delete ctx;
         return SGP_ERR_CUDA;
     }
@@ -506,6 +514,7 @@ void sgp_destroy(sgp_ctx *ctx)
     if (ctx->d_flags) cudaFree(ctx->d_flags);
     if (ctx->d_scan) cudaFree(ctx->d_scan);
     if (ctx->h_stage) cudaFreeHost(ctx->h_stage);
+    if (ctx->h_gave_up) cudaFreeHost(ctx->h_gave_up);
     for (auto e : ctx->ev_free) cudaEventDestroy(e);
     for (int k = 0; k < SGP_KT_COUNT; ++k)
         for (auto e : ctx->ev_pending[k]) cudaEventDestroy(e);

@@ -643,6 +643,8 @@ sgp_status sgp_pcg_solve_batched(sgp_ctx *ctx, const sgp_matrix *M, const sgp_fa
             SGP_TRY(pcg_b_run<double>(ctx, M, Fac, opts->precond, b, G, F, v, opts->x0_given, opts->tol, nullptr,
                                       opts->maxit, r, p, q, w));
             SGP_TRY(read_back(ctx, hs.data(), d_sc, sizeof(BScal) * n_inst));
+            if (gave_up(ctx))
+                for (auto &h : hs) h.status = SGP_ERR_TIMEOUT;
         }
         for (int64_t s = 0; s < n_inst; ++s) {
             inf[s].iterations = hs[s].it;
@@ -719,8 +721,8 @@ sgp_status sgp_pcg_solve_batched(sgp_ctx *ctx, const sgp_matrix *M, const sgp_fa
             for (int64_t s = 0; s < n_inst; ++s)
                 if (active[s]) {
                     inf[s].iterations += hs[s].it;
-                    if (hs[s].status == SGP_ERR_NOT_SPD) {
-                        inf[s].status = SGP_ERR_NOT_SPD;
+                    if (hs[s].status == SGP_ERR_NOT_SPD || hs[s].status == SGP_ERR_TIMEOUT) {
+                        inf[s].status = hs[s].status;
                         nrm[s] = 0.0;
                         active[s] = 0;
                     }
@@ -743,6 +745,7 @@ sgp_status sgp_pcg_solve_batched(sgp_ctx *ctx, const sgp_matrix *M, const sgp_fa
     }
     if (infos) std::memcpy(infos, inf.data(), sizeof(sgp_solve_info) * n_inst);
     if (rc == SGP_ERR_NOT_SPD) return sgp_fail(ctx, rc, "pcg_batched: breakdown in an instance");
+    if (rc == SGP_ERR_TIMEOUT) return sgp_fail(ctx, rc, "pcg_batched: a bounded device wait gave up");
     if (rc != SGP_OK) return sgp_fail(ctx, rc, "pcg_batched: an instance did not converge");
     return SGP_OK;
 }

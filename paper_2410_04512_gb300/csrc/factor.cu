@@ -1185,6 +1185,8 @@ sgp_status sgp_tree_apply(sgp_ctx *ctx, const sgp_factor *F, const double *b, do
     if (F->n == 0) return SGP_OK;
     SGP_CUDA(ctx, cudaSetDevice(ctx->device));
     // (in place is fine in one launch, as every part writes the rows it has read)
+    if (gave_up(ctx))
+        return sgp_fail(ctx, SGP_ERR_TIMEOUT, "tree_apply: a bounded device wait gave up in an earlier forest solve");
     const bool apart = b == x || b + 3 * F->n <= x || x + 3 * F->n <= b;
     if (apart && grid_apply_ready(ctx, F)) return grid_apply(ctx, F, F->gl.apply, b, x, bp<const int32_t>(F->orig_of), nullptr);
     // caller order -> internal order (the factor's workspace) -> caller order

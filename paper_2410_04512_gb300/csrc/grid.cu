@@ -1459,6 +1459,8 @@ struct GridArgs {
     long long maxit;
     int stopE;
     int *err;
+    int *gave_up;              // a forest solve alone: the context's word (host memory) for a wait that gave up
+    int polls;                 // polls after which a wait gives up
     Scal *sc;
     unsigned long long *ns;    // phase times (timing)
     GridPlace pl;
@@ -1628,7 +1630,6 @@ __device__ __forceinline__ void st_word(unsigned long long *p, unsigned long lon
 // arrival are one memory access: no fence, no separate flag, and a torn read
 // is seen as such.  A cell's vector takes 4 words in FP32 (the last unused)
 // and 6 in FP64.
-constexpr int WAIT_MAX = 1 << 21;   // polls: about two seconds
 template <typename T>
 struct Pkt;
 template <>
@@ -1674,20 +1675,20 @@ struct Pkt<double> {
         return ok;
     }
 };
-// gives up (returns true) after WAIT_MAX polls, or when another block has
-__device__ __forceinline__ bool give_up(int it, int *err)
+// gives up (returns true) after a.polls polls, or when another block has
+__device__ __forceinline__ bool give_up(int it, const GridArgs &a)
 {
-    if (it >= WAIT_MAX || ((it & 1023) == 1023 && *(volatile int *)err != 0)) {
-        atomicOr(err, 1);
+    if (it >= a.polls || ((it & 1023) == 1023 && *(volatile int *)a.err != 0)) {
+        atomicOr(a.err, 1);
         return true;
     }
     return false;
 }
 template <typename T>
-__device__ __forceinline__ bool wait_packet(const unsigned long long *p, unsigned ep, T *v, int *err)
+__device__ __forceinline__ bool wait_packet(const unsigned long long *p, unsigned ep, T *v, const GridArgs &a)
 {
     for (int it = 0; !Pkt<T>::get(p, ep, v); ++it)
-        if (give_up(it, err)) return false;
+        if (give_up(it, a)) return false;
     return true;
 }
 
@@ -1697,10 +1698,10 @@ __device__ __forceinline__ bool wait_packet(const unsigned long long *p, unsigne
 // after all blocks have written e - 1, that is, after they have read e - 2.
 constexpr int PK = (PMAX + 31) / 32;
 template <typename T, int NV>
-__device__ __forceinline__ bool exchange(unsigned long long *pk, int p0, int P, unsigned epoch, int *err, Acc<T> *v)
+__device__ __forceinline__ bool exchange(const GridArgs &g, int p0, int P, unsigned epoch, Acc<T> *v)
 {
     const int lane = threadIdx.x & 31;
-    unsigned long long *set = pk + (size_t)(epoch & 1u) * PMAX * 4;
+    unsigned long long *set = g.pk + (size_t)(epoch & 1u) * PMAX * 4;
     const unsigned long long e = (unsigned long long)epoch << 32;
     if (lane == 0) {
 #pragma unroll
@@ -1727,7 +1728,7 @@ __device__ __forceinline__ bool exchange(unsigned long long *pk, int p0, int P, 
 #pragma unroll
             for (int k = 0; k < NV; ++k) off |= ((unsigned)(a[k][u] >> 32) ^ epoch) | ((unsigned)(b[k][u] >> 32) ^ epoch);
         if (!__any_sync(0xffffffffu, off != 0)) break;
-        if (__any_sync(0xffffffffu, give_up(it, err))) {
+        if (__any_sync(0xffffffffu, give_up(it, g))) {
             ok = false;
             break;
         }
@@ -2106,7 +2107,7 @@ __device__ __noinline__ void sums(const GridArgs &a, Solve<T> &Z, int op)
         if (lane < GW) v[1].join(Z.red[1][lane]);
         v[1].warp();
     }
-    const bool ok = two ? exchange<T, 2>(a.pk, Z.p0, Z.np, epoch, a.err, v) : exchange<T, 1>(a.pk, Z.p0, Z.np, epoch, a.err, v);
+    const bool ok = two ? exchange<T, 2>(a, Z.p0, Z.np, epoch, v) : exchange<T, 1>(a, Z.p0, Z.np, epoch, v);
     if (lane) return;
     Z.epoch = epoch;
     if (!ok) {
@@ -2199,7 +2200,7 @@ __device__ __forceinline__ bool gather_top(const GridArgs &a, const PartDims &g,
             const bool a0 = Pkt<T>::get(pv, ep, v), a1 = Pkt<T>::get(p0, ep, y0),
                        a2 = Pkt<T>::get(p1, ep, y1);
             if (a0 && a1 && a2) break;
-            ok = !give_up(it, a.err);
+            ok = !give_up(it, a);
         }
         if (k0 < k1) {
             v[0] += y0[0]; v[1] += y0[1]; v[2] += y0[2];
@@ -2208,7 +2209,7 @@ __device__ __forceinline__ bool gather_top(const GridArgs &a, const PartDims &g,
             v[0] += y1[0]; v[1] += y1[1]; v[2] += y1[2];
         }
         for (int32_t k = k0 + 2; k < k1 && ok; ++k) {
-            ok = wait_packet<T>(a.lx + (size_t)Pkt<T>::W * k, ep, y0, a.err);
+            ok = wait_packet<T>(a.lx + (size_t)Pkt<T>::W * k, ep, y0, a);
             v[0] += y0[0]; v[1] += y0[1]; v[2] += y0[2];
         }
         V3<T, VB>::st(tw + i * VB, v);
@@ -2451,7 +2452,7 @@ __global__ void __launch_bounds__(GT, 1) k_pcg_grid(const __grid_constant__ Grid
                 for (int32_t i = tid; i < nr; i += GT)
                     if (a.xflag[ro + i]) Pkt<T>::put(a.px + (size_t)Pkt<T>::W * (ro + i), e, ps + 3 * i);
                 for (int32_t k = tid; k < nh; k += GT)
-                    if (!wait_packet<T>(a.px + (size_t)Pkt<T>::W * hl[k], ep, ps + 3 * (nr + k), a.err)) Z.bad = 1;
+                    if (!wait_packet<T>(a.px + (size_t)Pkt<T>::W * hl[k], ep, ps + 3 * (nr + k), a)) Z.bad = 1;
                 __syncthreads();
             } else {
                 T *o = reinterpret_cast<T *>(a.pg) + 3 * (size_t)ro;
@@ -2663,6 +2664,7 @@ __global__ void __launch_bounds__(GT, 1) k_apply_grid(const __grid_constant__ Gr
     if (!gather_top<T, VB>(a, g, tw, trx, 1u, 0)) s_bad = 1;
     __syncthreads();
     const bool bad = s_bad != 0;
+    if (bad && tid == 0) *(volatile int *)a.gave_up = 1;
     if (!bad)
         tree_down<T, VB>(g, s_prog, top_of<T>(a, g), w, tw, sm0 + a.pl.o_u);
     for (int32_t b = tid; b < g.nr; b += N * GT) {
@@ -3248,7 +3250,7 @@ static void top_args(const GridLayout &G, GridArgs &a)
 }
 
 // x = P^-1 b of an FP64 factor in one launch, without a host synchronisation;
-// a wait that gives up leaves NaN.  orig_of: the caller's order, or NULL for
+// a wait that gives up leaves NaN and sets the context's word (gave_up).  orig_of: the caller's order, or NULL for
 // the internal one; nothing is done when *done is set.
 bool grid_apply_ready(const sgp_ctx *ctx, const sgp_factor *F)
 {
@@ -3270,6 +3272,8 @@ sgp_status grid_apply(sgp_ctx *ctx, const sgp_factor *F, const DBuf &ws, const d
     a.D = G.D.p;
     a.F = b; a.x = x;
     a.err = bp<int>(ws);
+    a.gave_up = ctx->d_gave_up;
+    a.polls = ctx->wait_polls;
     a.lx = reinterpret_cast<unsigned long long *>(ws.p) + 2;
     SGP_CUDA(ctx, cudaMemsetAsync(ws.p, 0, G.apply_bytes, ctx->stream));
     void *args[] = {&a, &orig_of, &done};
@@ -3335,6 +3339,7 @@ sgp_status grid_pcg(sgp_ctx *ctx, const sgp_matrix *M, const GridLayout &G, cons
     a.maxit = maxit;
     a.stopE = stopE;
     a.err = &out->err;
+    a.polls = ctx->wait_polls;
     a.sc = out->sc;
     if (groups) {
         a.grp = groups->grp;

@@ -571,6 +571,13 @@ static sgp_status mpnn_ensure(sgp_ctx *ctx, sgp_mpnn *N, int64_t n)
     return SGP_OK;
 }
 
+// A forest solve whose wait gave up left NaN in the basis: reported by the calls
+// that wait for the stream.
+static sgp_status forest_check(sgp_ctx *ctx)
+{
+    return gave_up(ctx) ? sgp_fail(ctx, SGP_ERR_TIMEOUT, "mpnn: a bounded device wait gave up in a forest solve") : SGP_OK;
+}
+
 static unsigned red_blocks(int64_t cnt)
 {
     return (unsigned)std::max<int64_t>(1, std::min<int64_t>(1024, (cnt + TB - 1) / TB));
@@ -661,6 +668,7 @@ sgp_status sgp_mpnn_params(sgp_ctx *ctx, const sgp_mpnn *N, float *params, float
     if (params) SGP_CUDA(ctx, cudaMemcpyAsync(params, N->p.p, sizeof(float) * NPARAM, cudaMemcpyDeviceToHost, ctx->stream));
     if (grads) SGP_CUDA(ctx, cudaMemcpyAsync(grads, N->g.p, sizeof(float) * NPARAM, cudaMemcpyDeviceToHost, ctx->stream));
     SGP_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+    SGP_TRY(forest_check(ctx));
     return SGP_OK;
 }
 
@@ -786,7 +794,10 @@ sgp_status sgp_mpnn_backward(sgp_ctx *ctx, sgp_mpnn *N, const double *v_target, 
         LAUNCH(ctx, k_mp_agg_t, grid_for(16 * n, TB), TB, 0, n, row_ptr, col, (const float *)du, h, dh);
     }
     SGP_TRY((wgrad<DIN, 0, H>(ctx, N, n, dh, x, nullptr, OFF_WIN, OFF_BIN)));
-    if (loss) SGP_TRY(read_back(ctx, loss, lossout, sizeof(double)));
+    if (loss) {
+        SGP_TRY(read_back(ctx, loss, lossout, sizeof(double)));
+        SGP_TRY(forest_check(ctx));
+    }
     return SGP_OK;
 }
 
@@ -858,5 +869,5 @@ extern "C" sgp_status sgp_warm_start(sgp_ctx *ctx, sgp_mpnn *N, const sgp_matrix
     LAUNCH(ctx, k_to_caller<double>, grid_for(n, TB), TB, 0, n, bp<const int32_t>(M->orig_of), (const double *)w,
            v0);
     if (used) *used = u;
-    return SGP_OK;
+    return forest_check(ctx);   // (a read-back lies behind the forest solve)
 }

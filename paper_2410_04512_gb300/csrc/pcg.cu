@@ -1286,9 +1286,13 @@ sgp_status pcg_run(sgp_ctx *ctx, const sgp_matrix *M, const sgp_factor *Fac, int
         return grid_pcg<T>(ctx, M, *G, G->rows, precond, F, reinterpret_cast<T *>(x), x_given, tol, maxit, gwork, hs, mu,
                            stopE);
     const bool tree = precond == SGP_PRECOND_TREE && ctx->fused && Ft && xt && bins_tree_ready<T>(Fac, M);
-    if (!tree)
-        return pcg_core<T, X>(ctx, M, Fac, precond, make_blk<T>(M), bp<const int32_t>(M->row_ptr), M->n, false, F,
-                              x, x_given, tol, maxit, r, p, q, w, partials, sc, hs, mu, stopE);
+    if (!tree) {
+        SGP_TRY((pcg_core<T, X>(ctx, M, Fac, precond, make_blk<T>(M), bp<const int32_t>(M->row_ptr), M->n, false, F,
+                                x, x_given, tol, maxit, r, p, q, w, partials, sc, hs, mu, stopE)));
+        // (NaN from a forest solve whose wait gave up reads as a breakdown)
+        if (gave_up(ctx)) hs->status = SGP_ERR_TIMEOUT;
+        return SGP_OK;
+    }
     SGP_TRY(bins_to_tree<T>(ctx, Fac, F, Ft));
     if (x_given) SGP_TRY(bins_to_tree<T>(ctx, Fac, reinterpret_cast<const T *>(x), xt));
     SGP_TRY((pcg_core<T, T>(ctx, M, Fac, precond, tree_blk<T>(Fac), bp<const int32_t>(Fac->bl.rpt), Fac->bl.NT,
@@ -1692,6 +1696,7 @@ sgp_status sgp_fcg_solve(sgp_ctx *ctx, const sgp_matrix *M, const sgp_aug *A, co
             SGP_TRY((pcg_core<double, double>(ctx, P, Fac, SGP_PRECOND_TREE, make_blk<double>(P),
                                               bp<const int32_t>(P->row_ptr), n, false, (const double *)r, z, 0, itol,
                                               inner_maxit, ri, pi, qi, wi, partials, sci, &hi)));
+        if (gave_up(ctx)) hi.status = SGP_ERR_TIMEOUT;
         inner += hi.it;
         if (hi.status == SGP_ERR_NOT_SPD || hi.status == SGP_ERR_TIMEOUT) {
             h.status = hi.status;

@@ -77,6 +77,10 @@ struct sgp_ctx {
     // pinned staging for small device->host reads
     void *h_stage = nullptr;
     size_t h_stage_bytes = 0;
+    // set (in host memory) by a forest solve one of whose bounded waits gave up;
+    // and the polls after which a wait does (about two seconds)
+    int *h_gave_up = nullptr, *d_gave_up = nullptr;
+    int wait_polls = 1 << 21;
     // kernel timing
     int timing = 0;
     double kt_ms[SGP_KT_COUNT] = {};
@@ -211,6 +215,14 @@ static inline T *bp(const DBuf &b) { return reinterpret_cast<T *>(b.p); }
 
 // Copy `bytes` from device to host through the pinned stage and synchronise.
 sgp_status read_back(sgp_ctx *ctx, void *host, const void *dev, size_t bytes);
+// A forest solve of this context, complete by now, gave up; forgets it.
+static inline bool gave_up(sgp_ctx *ctx)
+{
+    volatile int *w = ctx->h_gave_up;
+    const bool g = *w != 0;
+    if (g) *w = 0;
+    return g;
+}
 // Ensure ctx->d_scratch has at least `bytes` (used by reductions and scans).
 sgp_status scratch_ensure(sgp_ctx *ctx, size_t bytes);
 
