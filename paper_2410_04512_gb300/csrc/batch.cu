@@ -557,9 +557,11 @@ sgp_status sgp_pcg_solve_batched(sgp_ctx *ctx, const sgp_matrix *M, const sgp_fa
     // the persistent solve, all systems in one launch, where the factor's layout
     // has their boundaries
     std::vector<int32_t> grp;
-    const bool grid = opts->precond == SGP_PRECOND_TREE &&
-                      (mixed ? grid_ready<float>(ctx, Fac, M) : grid_ready<double>(ctx, Fac, M)) &&
-                      grid_groups(Fac->gl, n_inst, offsets, grp);
+    const GridLayout *G0 = nullptr;
+    const GridRows *R0 = nullptr;
+    if (opts->precond == SGP_PRECOND_TREE && Fac->gl.ok && grid_groups(Fac->gl, n_inst, offsets, grp))
+        SGP_TRY(mixed ? grid_serves<float>(ctx, Fac, M, &G0, &R0) : grid_serves<double>(ctx, Fac, M, &G0, &R0));
+    const bool grid = G0 != nullptr;
     const size_t gw = grid ? grid_work_bytes(Fac->gl, mixed ? 4 : 8, (int)n_inst) + sizeof(int32_t) * grp.size() + 1024 : 0;
     size_t need = gw + 6 * v64 + (mixed ? 6 * v32 : 0) + sizeof(double) * 2 * nch + sizeof(BScal) * n_inst +
                   sizeof(double) * 6 * n_inst + tbl + 18 * 4096;
@@ -636,7 +638,7 @@ sgp_status sgp_pcg_solve_batched(sgp_ctx *ctx, const sgp_matrix *M, const sgp_fa
     if (!mixed) {
         if (grid) {
             if (!opts->x0_given) SGP_CUDA(ctx, cudaMemsetAsync(v, 0, v64, ctx->stream));
-            SGP_TRY(grid_pcg<double>(ctx, M, Fac->gl, Fac->gl.rows, SGP_PRECOND_TREE, F, v, opts->x0_given, opts->tol,
+            SGP_TRY(grid_pcg<double>(ctx, M, *G0, *R0, SGP_PRECOND_TREE, F, v, opts->x0_given, opts->tol,
                                      opts->maxit, gwork, gs.data(), 0.0, 0, &groups));
             take_scalars(hs, gs);
         } else {
@@ -710,7 +712,7 @@ sgp_status sgp_pcg_solve_batched(sgp_ctx *ctx, const sgp_matrix *M, const sgp_fa
             LAUNCH(ctx, k_b_scale, G, BB, 0, b, (const double *)r, (const double *)d_scale, r32, d32);
             if (grid) {
                 groups.tol2 = d_tol2;
-                SGP_TRY(grid_pcg<float>(ctx, M, Fac->gl, Fac->gl.rows, SGP_PRECOND_TREE, (const float *)r32, d32, 0, itol,
+                SGP_TRY(grid_pcg<float>(ctx, M, *G0, *R0, SGP_PRECOND_TREE, (const float *)r32, d32, 0, itol,
                                         opts->maxit, gwork, gs.data(), 0.0, 0, &groups));
                 take_scalars(hs, gs);
             } else {

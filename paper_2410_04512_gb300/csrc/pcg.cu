@@ -1263,27 +1263,20 @@ sgp_status pcg_core(sgp_ctx *ctx, const sgp_matrix *M, const sgp_factor *Fac, in
     return SGP_OK;
 }
 
-// The layout of the persistent solve that serves this run, or NULL.
-template <typename T>
-const GridLayout *grid_of(const sgp_ctx *ctx, const sgp_matrix *M, const sgp_factor *Fac, int precond)
-{
-    if (precond == SGP_PRECOND_TREE) return grid_ready<T>(ctx, Fac, M) ? &Fac->gl : nullptr;
-    const GridLayout &G = ctx->grid_plain;   // written for this call
-    return ctx->fused && ctx->bin_cap == 0 && G.ok ? &G : nullptr;
-}
-
-// One PCG run on Gamma x = F in the matrix's internal order.  With the
+// One PCG run on Gamma x = F in the matrix's internal order: in the persistent
+// launch on the layout G and the rows R when there are such.  Else, with the
 // tree preconditioner and a binned factor built from this assembly, the run
 // takes F (and x) to the factor's tree order, solves there with the fused
 // steps, and brings x back; Ft and xt are tree-order workspaces (NT cells).
 template <typename T, typename X>
 sgp_status pcg_run(sgp_ctx *ctx, const sgp_matrix *M, const sgp_factor *Fac, int precond, const T *F, X *x,
                    int x_given, double tol, int64_t maxit, T *r, T *p, T *q, T *w, T *Ft, T *xt,
-                   double *partials, Scal *sc, void *gwork, Scal *hs, double mu = 0.0, int stopE = 0)
+                   double *partials, Scal *sc, const GridLayout *G, const GridRows *R, void *gwork, Scal *hs,
+                   double mu = 0.0, int stopE = 0)
 {
     static_assert(sizeof(X) == sizeof(T), "iterate and vectors share one precision");
-    if (const GridLayout *G = grid_of<T>(ctx, M, Fac, precond))
-        return grid_pcg<T>(ctx, M, *G, G->rows, precond, F, reinterpret_cast<T *>(x), x_given, tol, maxit, gwork, hs, mu,
+    if (G)
+        return grid_pcg<T>(ctx, M, *G, *R, precond, F, reinterpret_cast<T *>(x), x_given, tol, maxit, gwork, hs, mu,
                            stopE);
     const bool tree = precond == SGP_PRECOND_TREE && ctx->fused && Ft && xt && bins_tree_ready<T>(Fac, M);
     if (!tree) {
@@ -1458,15 +1451,22 @@ sgp_status sgp_pcg_solve(sgp_ctx *ctx, const sgp_matrix *M, const sgp_factor *Fa
     size_t need = 8 * v64 + (mixed ? 8 * v32 : 0) + sizeof(double) * 2 * MAXP + 2 * sizeof(Scal) + 8192;
     // the persistent solve's layout: the factor's, or (row-wise
     // preconditioners) parts of the matrix's rows
-    if (opts->precond != SGP_PRECOND_TREE && ctx->fused && ctx->bin_cap == 0) {
+    const GridLayout *G0 = nullptr;
+    const GridRows *R0 = nullptr;
+    if (opts->precond == SGP_PRECOND_TREE) {
+        SGP_TRY(mixed ? grid_serves<float>(ctx, Fac, M, &G0, &R0) : grid_serves<double>(ctx, Fac, M, &G0, &R0));
+    } else if (ctx->fused && ctx->bin_cap == 0) {
         const double *jac = nullptr;
         if (opts->precond == SGP_PRECOND_BLOCK_JACOBI) {
             SGP_TRY(matrix_block_jacobi(ctx, const_cast<sgp_matrix *>(M)));
             jac = bp<const double>(M->jac);
         }
         SGP_TRY(grid_plain(ctx, M, mixed, jac, ctx->grid_plain));
+        if (ctx->grid_plain.ok) {
+            G0 = &ctx->grid_plain;
+            R0 = &G0->rows;
+        }
     }
-    const GridLayout *G0 = mixed ? grid_of<float>(ctx, M, Fac, opts->precond) : grid_of<double>(ctx, M, Fac, opts->precond);
     const size_t gw = G0 ? grid_work_bytes(*G0, mixed ? 4 : 8) : 0;
     SGP_TRY(scratch_ensure(ctx, need + gw + 4096));
     char *base = reinterpret_cast<char *>(ctx->d_scratch) + 256;
@@ -1507,7 +1507,7 @@ sgp_status sgp_pcg_solve(sgp_ctx *ctx, const sgp_matrix *M, const sgp_factor *Fa
     double hres[2] = {0, 0};
     if (!mixed) {
         SGP_TRY(pcg_run<double, double>(ctx, M, Fac, opts->precond, F, v, opts->x0_given, opts->tol,
-                                        opts->maxit, r, p, q, w, Ft64, xt64, partials, sc, gwork, &hs, mu,
+                                        opts->maxit, r, p, q, w, Ft64, xt64, partials, sc, G0, R0, gwork, &hs, mu,
                                         stopE ? 1 : 0));
         inf.iterations = hs.it;
         inf.err_bound = (mu > 0.0 && hs.gsum > 0.0) ? std::sqrt(std::max(hs.est, 0.0) / hs.gsum) : 0.0;
@@ -1568,7 +1568,7 @@ sgp_status sgp_pcg_solve(sgp_ctx *ctx, const sgp_matrix *M, const sgp_factor *Fa
             const double itol_k = std::max(itol, std::min(need, 0.5));
             SGP_TRY(pcg_run<float, float>(ctx, M, Fac, opts->precond, (const float *)r32, d32, 0, itol_k,
                                           opts->maxit - total, s32, p32, q32, w32, Ft32, xt32, partials, sc,
-                                          gwork, &hs));
+                                          G0, R0, gwork, &hs));
             total += hs.it;
             ++outer;
             if (hs.status == SGP_ERR_NOT_SPD || hs.status == SGP_ERR_TIMEOUT) {

@@ -268,9 +268,9 @@ sgp_status bins_check(sgp_ctx *ctx, const sgp_factor *F);
 bool small_solve_fits(const sgp_ctx *ctx, const sgp_factor *F);
 
 // The grid solve (grid.cu): a whole PCG run in one persistent launch.
-// grid_build runs at the end of a factor build; grid_ready tells whether it
-// serves precision T of this matrix; grid_rows puts another matrix on a
-// factor's parts, grid_plain cuts a matrix into parts of rows; grid_pcg runs
+// grid_build runs at the end of a factor build; grid_serves gives the layout
+// and rows that serve a matrix in precision T; grid_rows puts another matrix on
+// a factor's parts, grid_plain cuts a matrix into parts of rows; grid_pcg runs
 // it on internal-order vectors with `work` (grid_work_bytes) and returns the
 // final scalars.
 // Several systems in one solve (device arrays): grp, per part the system's
@@ -281,15 +281,13 @@ struct GridGroups {
     const int32_t *grp = nullptr;
     const double *tol2 = nullptr;
 };
-struct GridLayout;
-struct GridRows;
 sgp_status grid_build(sgp_ctx *ctx, sgp_factor *F, const sgp_matrix *M);
 sgp_status grid_rows(sgp_ctx *ctx, const sgp_factor *F, const sgp_matrix *M, GridRows &R);
 sgp_status grid_plain(sgp_ctx *ctx, const sgp_matrix *M, bool f32, const double *jac, GridLayout &G);
 void grid_release(GridLayout &G);
 void grid_rows_release(GridRows &R);
 template <typename T>
-bool grid_ready(const sgp_ctx *ctx, const sgp_factor *F, const sgp_matrix *M);
+sgp_status grid_serves(sgp_ctx *ctx, const sgp_factor *F, const sgp_matrix *M, const GridLayout **G, const GridRows **R);
 bool grid_apply_ready(const sgp_ctx *ctx, const sgp_factor *F);
 // (ws: the packets' buffer, at least gl.apply_bytes)
 sgp_status grid_apply(sgp_ctx *ctx, const sgp_factor *F, const DBuf &ws, const double *b, double *x, const int32_t *orig_of,
