@@ -46,7 +46,7 @@ struct DBuf {
 // The rows of one matrix (generation mgen) on the parts of a grid layout; tot: slots / 32, halo cells, the largest halo.
 struct GridRows {
     int ok = 0, halo = 0, vb = 16;   // vb: bytes per cell of the on-chip vectors
-    uint64_t mgen = 0;
+    uint64_t mgen = 0, fgen = 0;     // (fgen: of the layout's factor, for the rows of another matrix)
     int32_t tot[4] = {0};
     DBuf rh, glen, gso, perm, xflag, hl, ma, mb, hb, hpre;
 };
@@ -54,7 +54,7 @@ struct GridRows {
 // forest the parts' programs and the top, in one precision.
 #define SGP_GRID_SCRATCH 48
 struct GridLayout {
-    int ok = 0, prec = 0;
+    int ok = 0, prec = 0, diag = 0;   // diag: parts of rows with block-Jacobi inverses
     int64_t nr_max = 0;
     int32_t P = 0, LV = 0;
     int32_t tot[32] = {0};                          // totals and maxima over the parts
@@ -115,9 +115,9 @@ struct sgp_ctx {
     std::vector<KtRec> *capture_sink = nullptr;
     std::vector<GraphEntry *> graphs;
     uint64_t graph_clock = 0;
-    // persistent solves whose layout belongs to one call, written anew by each:
-    // the parts of rows of the row-wise preconditioners, and P' of a flexible
-    // solve on its factor's parts
+    // persistent solves' layouts of the last call: the parts of rows of the
+    // row-wise preconditioners, and the rows of another matrix (P' of a flexible
+    // solve, another assembly) on its factor's parts
     GridLayout grid_plain;
     GridRows grid_rows;
     DBuf grid_apply;   // packets of the forest solves inside this context's solves

@@ -73,3 +73,55 @@ def test_batch_with_a_kept_factor(cuda_device, precision):
         lo, hi = int(b.off[s]), int(b.off[s + 1])
         if hi > lo:
             assert rel_err(out[0][lo:hi], out[1][lo:hi]) <= 1e-8
+
+
+@pytest.mark.parametrize("precision", [sgp.PREC_F64, sgp.PREC_MIXED])
+@pytest.mark.parametrize("precond", [sgp.PRECOND_BLOCK_JACOBI, sgp.PRECOND_NONE])
+def test_rows_are_laid_out_once_per_assembly(cuda_device, precond, precision):
+    """The parts of rows of a row-wise solve are kept for the next solve of the
+    same assembly (fewer launches, the same bits) and for no other: another
+    preconditioner or the same handle assembled anew."""
+    c = workloads.ball(n=20011, seed=2113, gamma0=1e-3)
+    F = dev_tensor(c.forces())
+    cx = sgp.Context(0)
+    s = GpuSystem(cx, c, precision=precision, tree=False)
+
+    def solve(ctx, M, pre=precond):
+        ctx.launch_count(reset=True)
+        v, info = ctx.pcg_solve(M, None, F, tol=1e-10, precond=pre, precision=precision)
+        assert info.status == 0
+        return v.clone(), ctx.launch_count()
+
+    v1, l1 = solve(cx, s.M)
+    v2, l2 = solve(cx, s.M)
+    assert l2 < l1 and torch.equal(v1, v2)
+    other = sgp.PRECOND_NONE + sgp.PRECOND_BLOCK_JACOBI - precond
+    va, _ = solve(cx, s.M, other)
+    vb, _ = solve(sgp.Context(0), s.M, other)
+    assert torch.equal(va, vb)
+    M = cx.friction_assemble(s.graph, s.pos, 1.3 * s.gp, 0.8 * s.gq, c.gamma0, precision, s.M)   # the same handle
+    va, _ = solve(cx, M)
+    vb, _ = solve(sgp.Context(0), M)
+    assert torch.equal(va, vb) and not torch.equal(va, v1)
+
+
+def test_flexible_solve_lays_out_its_rows_once(cuda_device):
+    """P' on the factor's parts: kept for the next flexible solve, built anew
+    with the factor or the augmented forest."""
+    c = workloads.ball(n=5003, seed=2114, gamma0=1e-3)
+    F = dev_tensor(c.forces())
+    cx = sgp.Context(0)
+    s = GpuSystem(cx, c)
+    aug = cx.augment_tree(s.M, s.T)
+    out = []
+    for k in range(4):
+        if k == 2:
+            cx.tree_factor(s.M, s.T, s.Fac)
+        if k == 3:
+            cx.augment_tree(s.M, s.T, 0, aug)
+        cx.launch_count(reset=True)
+        v, info = cx.fcg_solve(s.M, aug, s.Fac, F, tol=1e-9)
+        assert info.status == 0
+        out.append((v.clone(), cx.launch_count()))
+    assert out[1][1] < out[0][1] == out[2][1] == out[3][1]
+    assert all(torch.equal(v, out[0][0]) for v, _ in out)
