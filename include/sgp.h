@@ -458,9 +458,12 @@ sgp_status sgp_set_tuning(sgp_ctx *ctx, const sgp_tuning *tuning);
  * is the time of one PCG iteration when iterations > 0 (each timed solve
  * runs exactly that many iterations; opts->tol is ignored), or, when
  * iterations == 0, the time of a whole solve to opts->tol plus the factor
- * build of the candidate (the cost of one time step).  The choice is stored
+ * build of the candidate (the cost of one time step).  Where the persistent
+ * launch or the one-block solve serves the timed solves, the knobs that it
+ * does not read (all but bin_cap; for the one-block solve all but bin_cap and
+ * tail_cap) stay as they are.  The choice is stored
  * in the context and copied to `out` (may be NULL; ms_per_iteration then
- * holds the winning objective).  F_dev is only read.  On failure the previous
+ * holds the winning objective, and a knob left at 0 reads as its default).  F_dev is only read.  On failure the previous
  * tuning is restored.  Synchronises. */
 sgp_status sgp_autotune(sgp_ctx *ctx, const sgp_matrix *matrix, const sgp_tree *tree, sgp_factor **factor,
                         int64_t n_instances, const int64_t *offsets, const double *F_dev,

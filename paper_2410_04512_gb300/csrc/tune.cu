@@ -51,6 +51,29 @@ struct Run {
         *ms_per_it = best;
         return SGP_OK;
     }
+    // The timed solves run in one launch, which reads no knob but bin_cap (and
+    // tail_cap, when one thread block runs them): there is nothing to choose
+    // between, and the smallest of equal times would be left to chance.
+    sgp_status in_one_launch(bool *persistent, bool *one_block)
+    {
+        const bool mixed = opts.precision == SGP_PREC_MIXED;
+        *persistent = *one_block = false;
+        if (opts.precond == SGP_PRECOND_TREE) {
+            const GridLayout *G = nullptr;
+            const GridRows *R = nullptr;
+            std::vector<int32_t> grp;
+            *one_block = n_inst == 0 && mixed && small_solve_fits(ctx, *Fh);
+            if (n_inst == 0 || grid_groups((*Fh)->gl, n_inst, offsets, grp))
+                SGP_TRY(mixed ? grid_serves<float>(ctx, *Fh, M, &G, &R) : grid_serves<double>(ctx, *Fh, M, &G, &R));
+            *persistent = G != nullptr;
+        } else {
+            double ms;
+            SGP_TRY(time_it(&ms));
+            *persistent = n_inst == 0 && ctx->fused && ctx->bin_cap == 0 && ctx->grid_plain.ok &&
+                          ctx->grid_plain.rows.mgen == M->gen;
+        }
+        return SGP_OK;
+    }
 };
 
 }  // namespace
@@ -142,7 +165,9 @@ sgp_status sgp_autotune(sgp_ctx *ctx, const sgp_matrix *M, const sgp_tree *T, sg
     if (cudaEventCreate(&run.e0) != cudaSuccess || cudaEventCreate(&run.e1) != cudaSuccess)
         return finish(sgp_fail(ctx, SGP_ERR_CUDA, "autotune: event creation failed"));
 
-    // 1. tail size, then bin size (each candidate rebuilds the factor)
+    // 1. tail size, then bin size (each candidate rebuilds the factor); the
+    // persistent launch has no tail
+    bool persistent = false, one_block = false;
     if (tree) {
         auto pick = [&](int *knob, const int *cand, int nc) -> sgp_status {
             int best = *knob;
@@ -158,13 +183,23 @@ sgp_status sgp_autotune(sgp_ctx *ctx, const sgp_matrix *M, const sgp_tree *T, sg
             return SGP_OK;
         };
         const int caps[] = {0, 256, 512, 1024, 2048, 4096, -1};
-        if ((st = pick(&ctx->tail_cap, caps, 7)) != SGP_OK) return finish(st);
+        if ((st = build()) != SGP_OK || (st = run.in_one_launch(&persistent, &one_block)) != SGP_OK) return finish(st);
+        const bool tail = !persistent;
+        if (tail && (st = pick(&ctx->tail_cap, caps, 7)) != SGP_OK) return finish(st);
         const int bins[] = {0, -1, 512, 1024, 2048};
         if ((st = pick(&ctx->bin_cap, bins, 5)) != SGP_OK) return finish(st);
-        if ((st = build()) != SGP_OK) return finish(st);
+        if ((st = build()) != SGP_OK || (st = run.in_one_launch(&persistent, &one_block)) != SGP_OK) return finish(st);
+        if (!tail && !persistent) {   // the bins or the level kernels were faster: they have one
+            if ((st = pick(&ctx->tail_cap, caps, 7)) != SGP_OK || (st = build()) != SGP_OK ||
+                (st = run.in_one_launch(&persistent, &one_block)) != SGP_OK)
+                return finish(st);
+        }
+    } else {
+        if ((st = run.in_one_launch(&persistent, &one_block)) != SGP_OK) return finish(st);
+        if (persistent && (st = run.time_it(&best_ms)) != SGP_OK) return finish(st);
     }
     // 2. lanes per block row of the product and rows in flight per lane
-    {
+    if (!persistent && !one_block) {
         const int lprs[] = {1, 2, 4, 8};
         int best_lpr = ctx->spmv_lpr, best_ilp = ctx->spmv_ilp;
         best_ms = 1e300;
@@ -181,7 +216,7 @@ sgp_status sgp_autotune(sgp_ctx *ctx, const sgp_matrix *M, const sgp_tree *T, sg
         ctx->spmv_ilp = best_ilp;
     }
     // 3. rows per work item of the batched solver
-    if (n_instances > 0) {
+    if (n_instances > 0 && !persistent) {
         const int chunks[] = {512, 1024, 2048, 4096, 8192};
         int best_ch = ctx->batch_chunk;
         best_ms = 1e300;
@@ -195,6 +230,10 @@ sgp_status sgp_autotune(sgp_ctx *ctx, const sgp_matrix *M, const sgp_tree *T, sg
     }
     if (out) {
         sgp_get_tuning(ctx, out);
+        // knobs left at their defaults: the values those stand for
+        if (!out->spmv_lpr) out->spmv_lpr = opts->precision == SGP_PREC_MIXED ? 2 : 1;
+        if (!out->spmv_ilp) out->spmv_ilp = 1;
+        if (!out->batch_chunk && n_instances > 0) out->batch_chunk = 2048;
         out->ms_per_iteration = best_ms;
     }
     return finish(SGP_OK);
