@@ -1,6 +1,8 @@
 // api.cu -- context, errors, device buffers, scans and kernel timing.
 #include "sgp_internal.cuh"
 
+#include <cuda.h>
+
 #include <atomic>
 #include <cstdlib>
 
@@ -242,9 +244,30 @@ sgp_status kt_end(sgp_ctx *ctx, int kclass, cudaEvent_t start)
     return SGP_OK;
 }
 
+// The SMs that a launch on the context's stream can have: the device's (an MPS
+// client's share of them), or those of the green context the stream belongs to.
+// The persistent solves wait for one another's blocks and take at most one per SM.
+static bool stream_sms(sgp_ctx *ctx)
+{
+    if (cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, ctx->device) != cudaSuccess) return false;
+    void *get = nullptr, *res = nullptr;
+    cudaDriverEntryPointQueryResult q1, q2;
+    if (cudaGetDriverEntryPointByVersion("cuStreamGetGreenCtx", &get, CUDART_VERSION, cudaEnableDefault, &q1) != cudaSuccess ||
+        cudaGetDriverEntryPointByVersion("cuGreenCtxGetDevResource", &res, CUDART_VERSION, cudaEnableDefault, &q2) != cudaSuccess ||
+        q1 != cudaDriverEntryPointSuccess || q2 != cudaDriverEntryPointSuccess) {
+        cudaGetLastError();
+        return true;   // a driver without green contexts
+    }
+    CUgreenCtx g = nullptr;
+    CUdevResource r{};
+    if (reinterpret_cast<decltype(&cuStreamGetGreenCtx)>(get)((CUstream)ctx->stream, &g) == CUDA_SUCCESS && g &&
+        reinterpret_cast<decltype(&cuGreenCtxGetDevResource)>(res)(g, &r, CU_DEV_RESOURCE_TYPE_SM) == CUDA_SUCCESS)
+        ctx->num_sms = (int)r.sm.smCount;
+    return ctx->num_sms > 0;
+}
+
 sgp_status resident_grid(sgp_ctx *ctx, const void *kernel, int block, int64_t want, unsigned *grid)
 {
-    if (!ctx->num_sms) SGP_CUDA(ctx, cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, ctx->device));
     int per_sm = 0;
     for (auto &kv : ctx->occupancy)
         if (kv.first == kernel) per_sm = kv.second;
@@ -493,7 +516,7 @@ sgp_status sgp_create(sgp_ctx **out, int device, void *stream)
         return SGP_ERR_OOM;
     }
     *ctx->h_gave_up = 0;
-    if (noalloc_prepare(ctx) != SGP_OK) {
+    if (noalloc_prepare(ctx) != SGP_OK || !stream_sms(ctx)) {
         cudaFree(ctx->d_scratch);
         cudaFree(ctx->d_flags);
         cudaFreeHost(ctx->h_gave_up);

@@ -2793,12 +2793,9 @@ sgp_status ensure(sgp_ctx *ctx, DBuf &b, size_t count, U **p)
 }
 
 // Parts for n rows: one block per SM, at least `umin` rows each.
-sgp_status part_count(sgp_ctx *ctx, int32_t n, int32_t umin, int32_t *P)
+int32_t part_count(const sgp_ctx *ctx, int32_t n, int32_t umin)
 {
-    if (!ctx->num_sms)
-        SGP_CUDA(ctx, cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, ctx->device));
-    *P = std::max(1, std::min(std::min(ctx->num_sms, PMAX), (n + umin - 1) / umin));
-    return SGP_OK;
+    return std::max(1, std::min(std::min(ctx->num_sms, PMAX), (n + umin - 1) / umin));
 }
 
 // The rows of a matrix on the parts of a layout, up to the counts (they go to
@@ -2908,8 +2905,7 @@ sgp_status grid_build(sgp_ctx *ctx, sgp_factor *F, const sgp_matrix *M)
     // At least 128 rows per part.  Measured (us per iteration, FP64 lattice of
     // 10,000 cells): 41.3 with 64 rows and 152 parts, 38.9 with 128, 42.9 with
     // 256, 53.9 with 512: more parts share the FP64 work, fewer exchange less.
-    int32_t P = 1;
-    SGP_TRY(part_count(ctx, n, 128, &P));
+    int32_t P = part_count(ctx, n, 128);
     int32_t U = (n + P - 1) / P;
     // a batch: no part holds rows of two instances, and U is the smallest at
     // which the instances' parts fit the device
@@ -3158,8 +3154,7 @@ sgp_status grid_plain(sgp_ctx *ctx, const sgp_matrix *M, bool f32, const double 
     G.prec = prec;
     G.diag = diag;
     // FP64 is bound by its issue rate: all SMs from 64 rows each on; FP32 from 128
-    int32_t P = 1;
-    SGP_TRY(part_count(ctx, n, f32 ? 128 : 64, &P));
+    int32_t P = part_count(ctx, n, f32 ? 128 : 64);
     const int32_t U = (n + P - 1) / P;
     P = (n + U - 1) / U;
     if ((size_t)U * (f32 ? 24 : 48) > (size_t)GRID_SMEM) {
@@ -3224,6 +3219,7 @@ void grid_release(GridLayout &G)
 // What serves a tree-preconditioned run in precision T: the factor's layout and
 // the matrix's rows on its parts, the factor's own or, for another assembly (a
 // factor kept for several steps), put there now; NULL where nothing does.
+// (A layout cut for more SMs than the context's stream has cannot be resident.)
 // MIXED solve of 1e5 cells with a factor of another assembly: 31.2 -> 11.2 ms
 // (its own 10.7; bins 25.5); 1e6: 92.8 -> 54.8 (52.4; 77.5).
 template <typename T>
@@ -3231,7 +3227,7 @@ sgp_status grid_serves(sgp_ctx *ctx, const sgp_factor *F, const sgp_matrix *M, c
 {
     *G = nullptr;
     *R = nullptr;
-    if (!ctx->fused || !F || !F->gl.ok || !F->gl.rows.ok || F->gl.prec != (sizeof(T) == 4 ? SGP_PREC_MIXED : SGP_PREC_F64))
+    if (!ctx->fused || !F || !F->gl.ok || !F->gl.rows.ok || F->gl.P > ctx->num_sms || F->gl.prec != (sizeof(T) == 4 ? SGP_PREC_MIXED : SGP_PREC_F64))
         return SGP_OK;
     const GridRows *r = &F->gl.rows;
     if (r->mgen != M->gen) {
@@ -3289,7 +3285,7 @@ static void top_args(const GridLayout &G, GridArgs &a)
 // the internal one; nothing is done when *done is set.
 bool grid_apply_ready(const sgp_ctx *ctx, const sgp_factor *F)
 {
-    return ctx->fused && F->gl.ok && F->gl.prec == SGP_PREC_F64 && F->gl.apply_bytes > 0;
+    return ctx->fused && F->gl.ok && F->gl.prec == SGP_PREC_F64 && F->gl.apply_bytes > 0 && F->gl.P <= ctx->num_sms;
 }
 sgp_status grid_apply(sgp_ctx *ctx, const sgp_factor *F, const DBuf &ws, const double *b, double *x, const int32_t *orig_of,
                       const int *done)

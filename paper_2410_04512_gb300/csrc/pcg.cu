@@ -1631,7 +1631,7 @@ sgp_status sgp_fcg_solve(sgp_ctx *ctx, const sgp_matrix *M, const sgp_aug *A, co
     const double itol = opts->inner_tol > 0.0 ? opts->inner_tol : 0.1;
     const size_t v64 = sizeof(double) * 3 * n;
     // the inner solves: P' on the parts of the factor's persistent solve
-    bool grid = ctx->fused && Fac->gl.ok && Fac->gl.prec == SGP_PREC_F64;
+    bool grid = ctx->fused && Fac->gl.ok && Fac->gl.prec == SGP_PREC_F64 && Fac->gl.P <= ctx->num_sms;
     if (grid) {
         SGP_TRY(grid_rows(ctx, Fac, A->P, ctx->grid_rows));
         grid = ctx->grid_rows.ok != 0;
