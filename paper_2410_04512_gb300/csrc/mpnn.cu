@@ -20,6 +20,8 @@
 // reduced per block and then in block order (deterministic).
 #include <cuda_bf16.h>
 
+#include <cfloat>
+
 #include "sgp_internal.cuh"
 
 sgp_status spmv64(sgp_ctx *ctx, const sgp_matrix *M, const double *v, double *y);
@@ -63,29 +65,30 @@ __global__ void k_mp_norm_sum(int64_t n, const double *__restrict__ b1, double *
         if (threadIdx.x == 0) {
             const double mean = t / (double)(n > 0 ? n : 1);
             out[0] = mean;
-            out[1] = 1.0 / (mean > 0.0 ? mean : 1.0);
+            out[1] = fmin(1.0 / (mean > 0.0 ? mean : 1.0), DBL_MAX);
         }
     }
 }
 
 // FP64 bound: the scale comes as a reciprocal, as a division is some ten
-// instructions (seven of them per cell: 26 us at 1e5 cells, 15 so).
+// instructions (seven of them per cell: 26 us at 1e5 cells, 15 so).  Twice in
+// turn, not as a square, which leaves the range of doubles at 1e154.
 __global__ void k_mp_features(int64_t n, const double *__restrict__ b0, const double *__restrict__ b1,
                               const double *__restrict__ b2, const int32_t *__restrict__ row_ptr,
                               const double *__restrict__ mean_b1, float *x)
 {
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
-    const double s = mean_b1[1], s2 = s * s;
+    const double s = mean_b1[1];
     const double *a = b0 + 3 * i, *b = b1 + 3 * i, *c = b2 + 3 * i;
     auto dot = [](const double *u, const double *v) { return u[0] * v[0] + u[1] * v[1] + u[2] * v[2]; };
     float *o = x + DIN * i;
     o[0] = (float)(sqrt(dot(a, a)) * s);
     o[1] = (float)(sqrt(dot(b, b)) * s);
     o[2] = (float)(sqrt(dot(c, c)) * s);
-    o[3] = (float)(dot(a, b) * s2);
-    o[4] = (float)(dot(a, c) * s2);
-    o[5] = (float)(dot(b, c) * s2);
+    o[3] = (float)(dot(a, b) * s * s);
+    o[4] = (float)(dot(a, c) * s * s);
+    o[5] = (float)(dot(b, c) * s * s);
     o[6] = (float)((row_ptr[i + 1] - row_ptr[i]) * (1.0 / 6.0));
     o[7] = 1.0f;
 }
