@@ -596,7 +596,7 @@ static sgp_status dense_tiles(sgp_ctx *ctx, int64_t n, const float *X1, const fl
     SGP_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     const int64_t want = (n + 16 * NU - 1) / (16 * NU);
     // two blocks per SM (registers)
-    const unsigned G = (unsigned)std::max<int64_t>(1, std::min<int64_t>(want, 2 * 152));
+    const unsigned G = (unsigned)std::max<int64_t>(1, std::min<int64_t>(want, 2 * ctx->num_sms));
     LAUNCH(ctx, kern, G, TB, smem, n, X1, X2, W, b, row_ptr, Y);
     return SGP_OK;
 }
@@ -605,7 +605,7 @@ template <int D1, int D2, int DOUT, bool TRANS, bool RELU>
 static sgp_status dense(sgp_ctx *ctx, int64_t n, const float *X1, const float *X2, const __nv_bfloat16 *W,
                         const __nv_bfloat16 *b, const int32_t *row_ptr, float *Y)
 {
-    return n >= 2 * 152 * 128 ? dense_tiles<D1, D2, DOUT, TRANS, RELU, 8>(ctx, n, X1, X2, W, b, row_ptr, Y)
+    return n >= 2 * (int64_t)ctx->num_sms * 128 ? dense_tiles<D1, D2, DOUT, TRANS, RELU, 8>(ctx, n, X1, X2, W, b, row_ptr, Y)
                               : dense_tiles<D1, D2, DOUT, TRANS, RELU, 4>(ctx, n, X1, X2, W, b, row_ptr, Y);
 }
 
