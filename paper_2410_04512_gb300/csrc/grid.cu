@@ -42,6 +42,7 @@
 // 34 us (76), FP64 spheroid of 3e5 125 us (282), FP32 spheroid of 1e6 122 us
 // (181); block Jacobi, FP64, 2e5 cells 54 us (81).
 #include <algorithm>
+#include <cmath>
 #include <cstddef>
 #include <cstring>
 #include <type_traits>
@@ -1273,16 +1274,26 @@ __global__ void __launch_bounds__(1024) k_gr_slots(GBuild g)
 
 // ---- numeric layout
 // D^-1 in groups of 32 rows, one plane of 32 values per entry (a source of
-// -1 gives a zero block)
+// -1 gives a zero block).  FP32: times a power of two near gamma0^(1/2).  PCG's
+// iterates do not depend on the preconditioner's size, but r^T z and p^T q do
+// (1 / gamma0 and less), and FP32 sums of them leave FP32's range where FP64
+// ones do not: coefficients of 1e-34 broke down.  So both stay near |r|^2 times
+// a power between -1/2 and 1/2 of gamma0.
 template <typename T>
-__global__ void k_gr_pivots(int32_t cnt, const int32_t *__restrict__ src, const double *__restrict__ from, T *to)
+T pivot_scale(const sgp_matrix *M)
+{
+    return sizeof(T) == 4 ? (T)std::ldexp(1.0, std::ilogb(M->gamma0) / 2) : T(1);
+}
+template <typename T>
+__global__ void k_gr_pivots(int32_t cnt, const int32_t *__restrict__ src, const double *__restrict__ from, double scale,
+                            T *to)
 {
     int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= cnt) return;
     const int32_t s = src[i];
     T *o = to + (size_t)(i >> 5) * 192 + (i & 31);
 #pragma unroll
-    for (int a = 0; a < 6; ++a) o[32 * a] = s >= 0 ? (T)from[(size_t)6 * s + a] : T(0);
+    for (int a = 0; a < 6; ++a) o[32 * a] = s >= 0 ? (T)(scale * from[(size_t)6 * s + a]) : T(0);
 }
 // The programs' blocks: -L of the lane's pair, transposed in the backward
 // program (TR); FP64 lanes hold one row.
@@ -2872,8 +2883,10 @@ sgp_status rows_fill(sgp_ctx *ctx, const GridLayout &G, GridRows &R, GBuild &g, 
 }
 
 template <typename T>
-sgp_status numeric(sgp_ctx *ctx, GridLayout &G, const sgp_factor *F, const GBuild &g, const int32_t *td_src)
+sgp_status numeric(sgp_ctx *ctx, GridLayout &G, const sgp_factor *F, const sgp_matrix *M, const GBuild &g,
+                   const int32_t *td_src)
 {
+    const double scale = pivot_scale<T>(M);
     const int32_t *t = G.tot;
     const double *L = bp<const double>(F->L), *Di = bp<const double>(F->Dinv);
     const int32_t nf = 32 * t[T_SF], nb = 32 * t[T_SB], nr = t[T_NR], nt = t[T_NT], B = SGP_BLOCK;
@@ -2883,10 +2896,10 @@ sgp_status numeric(sgp_ctx *ctx, GridLayout &G, const sgp_factor *F, const GBuil
     SGP_TRY(ensure(ctx, G.tD, 6 * (size_t)pad32(nt), &tD));
     LAUNCH(ctx, (k_gr_blocks<T, false>), grid_for(nf, B), B, 0, nf, (const int32_t *)g.msrc[0], L, g.prog[0]);
     LAUNCH(ctx, (k_gr_blocks<T, true>), grid_for(nb, B), B, 0, nb, (const int32_t *)g.msrc[1], L, g.prog[1]);
-    LAUNCH(ctx, k_gr_pivots<T>, grid_for(nr, B), B, 0, nr, (const int32_t *)g.d_src, Di, D);
+    LAUNCH(ctx, k_gr_pivots<T>, grid_for(nr, B), B, 0, nr, (const int32_t *)g.d_src, Di, scale, D);
     if (nt == 0) return SGP_OK;
     LAUNCH(ctx, k_gr_top_fill<T>, nt, 128, 0, g, X);
-    LAUNCH(ctx, k_gr_pivots<T>, grid_for(nt, B), B, 0, nt, td_src, Di, tD);
+    LAUNCH(ctx, k_gr_pivots<T>, grid_for(nt, B), B, 0, nt, td_src, Di, scale, tD);
     return SGP_OK;
 }
 
@@ -3094,9 +3107,9 @@ sgp_status grid_build(sgp_ctx *ctx, sgp_factor *F, const sgp_matrix *M)
     if (rows) SGP_TRY(rows_fill(ctx, G, R, g, M, f32));
     const int32_t *td_src = sp + hs.top[Q_SOFF];
     if (f32)
-        SGP_TRY(numeric<float>(ctx, G, F, g, td_src));
+        SGP_TRY(numeric<float>(ctx, G, F, M, g, td_src));
     else
-        SGP_TRY(numeric<double>(ctx, G, F, g, td_src));
+        SGP_TRY(numeric<double>(ctx, G, F, M, g, td_src));
     LAUNCH(ctx, k_gr_check, P, GT, 0, g);
     SGP_TRY(read_back(ctx, hs.t, g.tot, sizeof(hs.t)));
     if (hs.t[T_ERR]) return sgp_fail(ctx, SGP_ERR_CUDA, "tree_factor: inconsistent grid layout (0x%x)", hs.t[T_ERR]);
@@ -3190,10 +3203,10 @@ sgp_status grid_plain(sgp_ctx *ctx, const sgp_matrix *M, bool f32, const double 
         SGP_TRY(buf_ensure(ctx, G.D, (f32 ? 4 : 8) * 6 * (size_t)nr));
         if (f32)
             LAUNCH(ctx, k_gr_pivots<float>, grid_for(nr, SGP_BLOCK), SGP_BLOCK, 0, nr, bp<const int32_t>(G.i_of_t), jac,
-                   bp<float>(G.D));
+                   (double)pivot_scale<float>(M), bp<float>(G.D));
         else
             LAUNCH(ctx, k_gr_pivots<double>, grid_for(nr, SGP_BLOCK), SGP_BLOCK, 0, nr, bp<const int32_t>(G.i_of_t), jac,
-                   bp<double>(G.D));
+                   (double)pivot_scale<double>(M), bp<double>(G.D));
     }
     R.mgen = M->gen;
     G.ok = 1;
