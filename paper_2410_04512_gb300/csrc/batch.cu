@@ -559,7 +559,7 @@ sgp_status sgp_pcg_solve_batched(sgp_ctx *ctx, const sgp_matrix *M, const sgp_fa
     std::vector<int32_t> grp;
     const GridLayout *G0 = nullptr;
     const GridRows *R0 = nullptr;
-    if (opts->precond == SGP_PRECOND_TREE && Fac->gl.ok && grid_groups(Fac->gl, n_inst, offsets, grp))
+    if (opts->precond == SGP_PRECOND_TREE && grid_groups(Fac->gl, n_inst, offsets, grp))
         SGP_TRY(mixed ? grid_serves<float>(ctx, Fac, M, &G0, &R0) : grid_serves<double>(ctx, Fac, M, &G0, &R0));
     const bool grid = G0 != nullptr;
     const size_t gw = grid ? grid_work_bytes(Fac->gl, mixed ? 4 : 8, (int)n_inst) + sizeof(int32_t) * grp.size() + 1024 : 0;

@@ -3256,10 +3256,11 @@ template sgp_status grid_serves<float>(sgp_ctx *, const sgp_factor *, const sgp_
 template sgp_status grid_serves<double>(sgp_ctx *, const sgp_factor *, const sgp_matrix *, const GridLayout **, const GridRows **);
 
 // The systems of a batched solve, offsets[0..n_inst], on the parts of a
-// factor: per part its system's parts and the system.  False where a system
-// does not begin and end with instances of the layout.
+// factor: per part its system's parts and the system.  False without a layout,
+// or where a system does not begin and end with instances of the layout.
 bool grid_groups(const GridLayout &G, int64_t n_inst, const int64_t *offsets, std::vector<int32_t> &grp)
 {
+    if (!G.ok) return false;
     grp.assign(3 * (size_t)G.P, 0);
     for (int64_t s = 0; s < n_inst; ++s) {
         if (offsets[s] == offsets[s + 1]) continue;

@@ -14,6 +14,14 @@ pytestmark = pytest.mark.gpu
 DEAD = ("spmv_lpr", "spmv_ilp", "tail_cap", "batch_chunk")
 
 
+def test_batch_of_more_instances_than_blocks(cuda_device):
+    """No persistent launch and no layout: every knob is timed."""
+    cx = sgp.Context(0)
+    b = GpuBatch(cx, [5] * 170, precision=sgp.PREC_MIXED)
+    t = cx.autotune(b.M, b.T, b.Fh, dev_tensor(b.F), offsets=b.off, precision=sgp.PREC_MIXED, iterations=3)
+    assert t["batch_chunk"] in (512, 1024, 2048, 4096, 8192) and cx.get_tuning()["batch_chunk"] == t["batch_chunk"]
+
+
 @pytest.mark.parametrize("start", [{}, {"spmv_lpr": 4, "spmv_ilp": 2, "tail_cap": 512, "batch_chunk": 1024}])
 @pytest.mark.parametrize("what", ["tree", "jacobi", "batch"])
 def test_unread_knobs_stay(cuda_device, what, start):
