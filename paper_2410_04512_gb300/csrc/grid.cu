@@ -1274,15 +1274,18 @@ __global__ void __launch_bounds__(1024) k_gr_slots(GBuild g)
 
 // ---- numeric layout
 // D^-1 in groups of 32 rows, one plane of 32 values per entry (a source of
-// -1 gives a zero block).  FP32: times a power of two near gamma0^(1/2).  PCG's
-// iterates do not depend on the preconditioner's size, but r^T z and p^T q do
-// (1 / gamma0 and less), and FP32 sums of them leave FP32's range where FP64
-// ones do not: coefficients of 1e-34 broke down.  So both stay near |r|^2 times
-// a power between -1/2 and 1/2 of gamma0.
+// -1 gives a zero block).  FP32: times a power of two where gamma0 is far from
+// 1.  PCG's iterates do not depend on the preconditioner's size, but r^T z and
+// p^T q do (|r|^2 / gamma0 and less), and FP32 sums of them leave FP32's range
+// where FP64 ones do not: coefficients of 1e-34 broke down.  With 1 / gamma0
+// held to 2^80 at most and 2^-40 at least, both stay inside for coefficients
+// from 1e-34 to 1e34.  (A gamma0 that is small beside the contacts alone needs no
+// scale, and a small one does it no harm.)
 template <typename T>
-T pivot_scale(const sgp_matrix *M)
+double pivot_scale(const sgp_matrix *M)
 {
-    return sizeof(T) == 4 ? (T)std::ldexp(1.0, std::ilogb(M->gamma0) / 2) : T(1);
+    const int e = std::ilogb(M->gamma0), k = e < -80 ? e + 80 : e > 40 ? e - 40 : 0;
+    return sizeof(T) == 4 ? std::ldexp(1.0, k) : 1.0;
 }
 template <typename T>
 __global__ void k_gr_pivots(int32_t cnt, const int32_t *__restrict__ src, const double *__restrict__ from, double scale,
@@ -3203,10 +3206,10 @@ sgp_status grid_plain(sgp_ctx *ctx, const sgp_matrix *M, bool f32, const double 
         SGP_TRY(buf_ensure(ctx, G.D, (f32 ? 4 : 8) * 6 * (size_t)nr));
         if (f32)
             LAUNCH(ctx, k_gr_pivots<float>, grid_for(nr, SGP_BLOCK), SGP_BLOCK, 0, nr, bp<const int32_t>(G.i_of_t), jac,
-                   (double)pivot_scale<float>(M), bp<float>(G.D));
+                   pivot_scale<float>(M), bp<float>(G.D));
         else
             LAUNCH(ctx, k_gr_pivots<double>, grid_for(nr, SGP_BLOCK), SGP_BLOCK, 0, nr, bp<const int32_t>(G.i_of_t), jac,
-                   (double)pivot_scale<double>(M), bp<double>(G.D));
+                   pivot_scale<double>(M), bp<double>(G.D));
     }
     R.mgen = M->gen;
     G.ok = 1;
