@@ -95,3 +95,16 @@ def test_large_parts_of_rows(cuda_device, precond, precision):
         assert float((out[0][0] - out[1][0]).norm() / out[1][0].norm()) <= 1e-6
     else:
         assert 0.5 * out[1][1] <= out[0][1] <= 2.0 * out[1][1]
+
+
+def test_no_layout_where_none_can_fit(cuda_device):
+    """Too many cells for the SMs there are: the factor is built without a
+    launch for the persistent solve."""
+    n = 1_300_021
+    counts = []
+    for cap in (0, -1):
+        s = System(cap, n, sgp.PREC_F64)
+        s.cx.launch_count(reset=True)
+        s.cx.tree_factor(s.M, s.T, s.Fac)
+        counts.append(s.cx.launch_count())
+    assert counts[0] == counts[1]
