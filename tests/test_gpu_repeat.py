@@ -11,6 +11,7 @@ import torch
 import paper_2410_04512_gb300 as sgp
 import workloads
 from gpu_common import GpuSystem, dev_tensor
+from test_gpu_batched import GpuBatch
 
 pytestmark = pytest.mark.gpu
 
@@ -30,3 +31,37 @@ def test_multi_launch_fp64_steps_repeat(cuda_device, precond):
         if first is None:
             first = v.clone()
         assert torch.equal(v, first)
+
+
+@pytest.mark.parametrize("precision", [sgp.PREC_F64, sgp.PREC_MIXED])
+@pytest.mark.parametrize("what", ["tree", "jacobi", "none", "batch", "network", "apply"])
+def test_persistent_launches_repeat(cuda_device, what, precision):
+    """The same bits again, and after the factor is built again."""
+    cx = sgp.Context(0)
+    if what == "batch":
+        b = GpuBatch(cx, [3000, 2600, 0, 4000], precision=precision)
+        F = dev_tensor(b.F)
+        M, T, Fac = b.M, b.T, b.Fh
+
+        def run():
+            return cx.pcg_solve_batched(M, Fac, b.off, F, tol=1e-10, precision=precision)[0]
+    else:
+        c = workloads.ball(n=61003, seed=2110, gamma0=1e-3)
+        F = dev_tensor(c.forces())
+        s = GpuSystem(cx, c, precision=precision)
+        M, T, Fac = s.M, s.T, s.Fac
+        pre = {"tree": sgp.PRECOND_TREE, "jacobi": sgp.PRECOND_BLOCK_JACOBI, "none": sgp.PRECOND_NONE}.get(what)
+        net = cx.mpnn_create((0.1 * np.random.default_rng(1).standard_normal(sgp.MPNN_PARAMS)).astype(np.float32))
+
+        def run():
+            if what == "apply":
+                return cx.tree_apply(Fac, F)
+            if what == "network":
+                return cx.mpnn_forward(net, M, Fac, F)
+            return cx.pcg_solve(M, Fac, F, tol=1e-10, precond=pre, precision=precision)[0]
+
+    first = run().clone()
+    for k in range(4):
+        if k == 2:
+            cx.tree_factor(M, T, Fac)
+        assert torch.equal(run(), first)
