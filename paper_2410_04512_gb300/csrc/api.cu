@@ -65,18 +65,25 @@ sgp_status scratch_ensure(sgp_ctx *ctx, size_t bytes)
     return SGP_OK;
 }
 
+// the pinned page of a context
+constexpr size_t PINNED = 4096;
+
 sgp_status read_back(sgp_ctx *ctx, void *host, const void *dev, size_t bytes)
 {
+    void *stage = ctx->h_stage;
     if (bytes > ctx->h_stage_bytes) {
-        if (ctx->h_stage) cudaFreeHost(ctx->h_stage);
-        ctx->h_stage = nullptr;
-        size_t want = bytes < 4096 ? 4096 : bytes;
-        SGP_CUDA(ctx, cudaMallocHost(&ctx->h_stage, want));
-        ctx->h_stage_bytes = want;
+        if (bytes > ctx->h_large_bytes) {
+            if (ctx->h_large) cudaFreeHost(ctx->h_large);
+            ctx->h_large = nullptr;
+            ctx->h_large_bytes = 0;
+            SGP_CUDA(ctx, cudaMallocHost(&ctx->h_large, bytes));
+            ctx->h_large_bytes = bytes;
+        }
+        stage = ctx->h_large;
     }
-    SGP_CUDA(ctx, cudaMemcpyAsync(ctx->h_stage, dev, bytes, cudaMemcpyDeviceToHost, ctx->stream));
+    SGP_CUDA(ctx, cudaMemcpyAsync(stage, dev, bytes, cudaMemcpyDeviceToHost, ctx->stream));
     SGP_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-    memcpy(host, ctx->h_stage, bytes);
+    memcpy(host, stage, bytes);
     SGP_TRY(kt_collect(ctx));
     return SGP_OK;
 }
@@ -506,7 +513,7 @@ sgp_status sgp_create(sgp_ctx **out, int device, void *stream)
     if (wp) ctx->wait_polls = std::max(0, atoi(wp));
     if (scratch_ensure(ctx, 1 << 20) != SGP_OK || cudaMalloc(&ctx->d_flags, 4096) != cudaSuccess ||
         cudaMemset(ctx->d_flags, 0, 4096) != cudaSuccess ||
-        cudaHostAlloc(&ctx->h_gave_up, 64, cudaHostAllocMapped) != cudaSuccess ||
+        cudaHostAlloc(&ctx->h_gave_up, PINNED, cudaHostAllocMapped) != cudaSuccess ||
         cudaHostGetDevicePointer(&ctx->d_gave_up, ctx->h_gave_up, 0) != cudaSuccess) {
         cudaGetLastError();
         if (ctx->d_scratch) cudaFree(ctx->d_scratch);
@@ -516,6 +523,8 @@ sgp_status sgp_create(sgp_ctx **out, int device, void *stream)
         return SGP_ERR_OOM;
     }
     *ctx->h_gave_up = 0;
+    ctx->h_stage = reinterpret_cast<char *>(ctx->h_gave_up) + 64;
+    ctx->h_stage_bytes = PINNED - 64;
     if (noalloc_prepare(ctx) != SGP_OK || !stream_sms(ctx)) {
         cudaFree(ctx->d_scratch);
         cudaFree(ctx->d_flags);
@@ -536,7 +545,7 @@ void sgp_destroy(sgp_ctx *ctx)
     if (ctx->d_scratch) cudaFree(ctx->d_scratch);
     if (ctx->d_flags) cudaFree(ctx->d_flags);
     if (ctx->d_scan) cudaFree(ctx->d_scan);
-    if (ctx->h_stage) cudaFreeHost(ctx->h_stage);
+    if (ctx->h_large) cudaFreeHost(ctx->h_large);
     if (ctx->h_gave_up) cudaFreeHost(ctx->h_gave_up);
     for (auto e : ctx->ev_free) cudaEventDestroy(e);
     for (int k = 0; k < SGP_KT_COUNT; ++k)

@@ -74,12 +74,13 @@ struct sgp_ctx {
     cudaStream_t stream = nullptr;
     std::string err;
     int64_t launches = 0;
-    // pinned staging for small device->host reads
-    void *h_stage = nullptr;
-    size_t h_stage_bytes = 0;
-    // set (in host memory) by a forest solve one of whose bounded waits gave up;
-    // and the polls after which a wait does (about two seconds)
+    // a pinned page: the word that a forest solve sets when one of its bounded
+    // waits gives up, then staging for small device->host reads (h_large: for
+    // larger ones); and the polls after which a wait gives up (about two seconds)
     int *h_gave_up = nullptr, *d_gave_up = nullptr;
+    char *h_stage = nullptr;
+    void *h_large = nullptr;
+    size_t h_stage_bytes = 0, h_large_bytes = 0;
     int wait_polls = 1 << 21;
     // kernel timing
     int timing = 0;
