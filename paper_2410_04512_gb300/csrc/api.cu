@@ -509,8 +509,8 @@ sgp_status sgp_create(sgp_ctx **out, int device, void *stream)
     if (ns && atoi(ns)) ctx->small_solve = 0;
     const char *nf = getenv("SGP_NO_FUSE");
     if (nf && atoi(nf)) ctx->fused = 0;
-    const char *wp = getenv("SGP_WAIT_POLLS");
-    if (wp) ctx->wait_polls = std::max(0, atoi(wp));
+    const char *sk = getenv("SGP_SKEW_PACKETS");
+    if (sk && atoi(sk)) ctx->skew = 1u << 20;
     if (scratch_ensure(ctx, 1 << 20) != SGP_OK || cudaMalloc(&ctx->d_flags, 4096) != cudaSuccess ||
         cudaMemset(ctx->d_flags, 0, 4096) != cudaSuccess ||
         cudaHostAlloc(&ctx->h_gave_up, PINNED, cudaHostAllocMapped) != cudaSuccess ||

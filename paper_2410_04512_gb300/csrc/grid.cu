@@ -1497,7 +1497,7 @@ struct GridArgs {
     int stopE;
     int *err;
     int *gave_up;              // a forest solve alone: the context's word (host memory) for a wait that gave up
-    int polls;                 // polls after which a wait gives up
+    unsigned skew;             // block 0 numbers its packets from here (0; tests: waits that run out)
     Scal *sc;
     unsigned long long *ns;    // phase times (timing)
     GridPlace pl;
@@ -1712,20 +1712,22 @@ struct Pkt<double> {
         return ok;
     }
 };
-// gives up (returns true) after a.polls polls, or when another block has
-__device__ __forceinline__ bool give_up(int it, const GridArgs &a)
+constexpr int WAIT_MAX = 1 << 21;   // polls: about two seconds
+// gives up (returns true) after WAIT_MAX polls, or when another block has.  (The
+// limit as an argument costs 0.5 to 0.8 us an iteration.)
+__device__ __forceinline__ bool give_up(int it, int *err)
 {
-    if (it >= a.polls || ((it & 1023) == 1023 && *(volatile int *)a.err != 0)) {
-        atomicOr(a.err, 1);
+    if (it >= WAIT_MAX || ((it & 1023) == 1023 && *(volatile int *)err != 0)) {
+        atomicOr(err, 1);
         return true;
     }
     return false;
 }
 template <typename T>
-__device__ __forceinline__ bool wait_packet(const unsigned long long *p, unsigned ep, T *v, const GridArgs &a)
+__device__ __forceinline__ bool wait_packet(const unsigned long long *p, unsigned ep, T *v, int *err)
 {
     for (int it = 0; !Pkt<T>::get(p, ep, v); ++it)
-        if (give_up(it, a)) return false;
+        if (give_up(it, err)) return false;
     return true;
 }
 
@@ -1735,10 +1737,10 @@ __device__ __forceinline__ bool wait_packet(const unsigned long long *p, unsigne
 // after all blocks have written e - 1, that is, after they have read e - 2.
 constexpr int PK = (PMAX + 31) / 32;
 template <typename T, int NV>
-__device__ __forceinline__ bool exchange(const GridArgs &g, int p0, int P, unsigned epoch, Acc<T> *v)
+__device__ __forceinline__ bool exchange(unsigned long long *pk, int p0, int P, unsigned epoch, int *err, Acc<T> *v)
 {
     const int lane = threadIdx.x & 31;
-    unsigned long long *set = g.pk + (size_t)(epoch & 1u) * PMAX * 4;
+    unsigned long long *set = pk + (size_t)(epoch & 1u) * PMAX * 4;
     const unsigned long long e = (unsigned long long)epoch << 32;
     if (lane == 0) {
 #pragma unroll
@@ -1765,7 +1767,7 @@ __device__ __forceinline__ bool exchange(const GridArgs &g, int p0, int P, unsig
 #pragma unroll
             for (int k = 0; k < NV; ++k) off |= ((unsigned)(a[k][u] >> 32) ^ epoch) | ((unsigned)(b[k][u] >> 32) ^ epoch);
         if (!__any_sync(0xffffffffu, off != 0)) break;
-        if (__any_sync(0xffffffffu, give_up(it, g))) {
+        if (__any_sync(0xffffffffu, give_up(it, err))) {
             ok = false;
             break;
         }
@@ -2144,7 +2146,7 @@ __device__ __noinline__ void sums(const GridArgs &a, Solve<T> &Z, int op)
         if (lane < GW) v[1].join(Z.red[1][lane]);
         v[1].warp();
     }
-    const bool ok = two ? exchange<T, 2>(a, Z.p0, Z.np, epoch, v) : exchange<T, 1>(a, Z.p0, Z.np, epoch, v);
+    const bool ok = two ? exchange<T, 2>(a.pk, Z.p0, Z.np, epoch, a.err, v) : exchange<T, 1>(a.pk, Z.p0, Z.np, epoch, a.err, v);
     if (lane) return;
     Z.epoch = epoch;
     if (!ok) {
@@ -2237,7 +2239,7 @@ __device__ __forceinline__ bool gather_top(const GridArgs &a, const PartDims &g,
             const bool a0 = Pkt<T>::get(pv, ep, v), a1 = Pkt<T>::get(p0, ep, y0),
                        a2 = Pkt<T>::get(p1, ep, y1);
             if (a0 && a1 && a2) break;
-            ok = !give_up(it, a);
+            ok = !give_up(it, a.err);
         }
         if (k0 < k1) {
             v[0] += y0[0]; v[1] += y0[1]; v[2] += y0[2];
@@ -2246,7 +2248,7 @@ __device__ __forceinline__ bool gather_top(const GridArgs &a, const PartDims &g,
             v[0] += y1[0]; v[1] += y1[1]; v[2] += y1[2];
         }
         for (int32_t k = k0 + 2; k < k1 && ok; ++k) {
-            ok = wait_packet<T>(a.lx + (size_t)Pkt<T>::W * k, ep, y0, a);
+            ok = wait_packet<T>(a.lx + (size_t)Pkt<T>::W * k, ep, y0, a.err);
             v[0] += y0[0]; v[1] += y0[1]; v[2] += y0[2];
         }
         V3<T, VB>::st(tw + i * VB, v);
@@ -2425,7 +2427,7 @@ __global__ void __launch_bounds__(GT, 1) k_pcg_grid(const __grid_constant__ Grid
     Mat<T> M;
     M.a = reinterpret_cast<decltype(M.a)>(a.ma);
     M.b = reinterpret_cast<decltype(M.b)>(a.mb);
-    unsigned ep = 0;   // steps started: the number of this step's packets
+    unsigned ep = blockIdx.x == 0 ? a.skew : 0u;   // steps started: the number of this step's packets
     unsigned long long tk = 0, t_spmv = 0, t_tree = 0, t_vec = 0;
     const bool clk = a.timing && blockIdx.x == 0 && tid == 0;
     auto lap = [&](unsigned long long &sum) {
@@ -2465,7 +2467,7 @@ __global__ void __launch_bounds__(GT, 1) k_pcg_grid(const __grid_constant__ Grid
         Z.S.tolE2 = a.tolE2;
         Z.go = 1;
         Z.bad = 0;
-        Z.epoch = 0;
+        Z.epoch = ep;
     }
     // x = 0 or given; without it the first pass skips the product
     for (int32_t i = tid; i < nr; i += GT) {
@@ -2489,7 +2491,7 @@ __global__ void __launch_bounds__(GT, 1) k_pcg_grid(const __grid_constant__ Grid
                 for (int32_t i = tid; i < nr; i += GT)
                     if (a.xflag[ro + i]) Pkt<T>::put(a.px + (size_t)Pkt<T>::W * (ro + i), e, ps + 3 * i);
                 for (int32_t k = tid; k < nh; k += GT)
-                    if (!wait_packet<T>(a.px + (size_t)Pkt<T>::W * hl[k], ep, ps + 3 * (nr + k), a)) Z.bad = 1;
+                    if (!wait_packet<T>(a.px + (size_t)Pkt<T>::W * hl[k], ep, ps + 3 * (nr + k), a.err)) Z.bad = 1;
                 __syncthreads();
             } else {
                 T *o = reinterpret_cast<T *>(a.pg) + 3 * (size_t)ro;
@@ -2697,8 +2699,9 @@ __global__ void __launch_bounds__(GT, 1) k_apply_grid(const __grid_constant__ Gr
     const T zero[3] = {0, 0, 0};
     if (tid == 0) V3<T, VB>::st(w + (g.nr + g.nz) * VB, zero);   // the spare cell
     unsigned long long *trx = a.lx + (size_t)Pkt<T>::W * a.nslots;
-    tree_up<T, VB>(a, g, s_prog, reinterpret_cast<const T *>(a.D) + 6 * (size_t)g.ro, w, trx, 1u);
-    if (!gather_top<T, VB>(a, g, tw, trx, 1u, 0)) s_bad = 1;
+    const unsigned ep = blockIdx.x == 0 ? a.skew + 1u : 1u;
+    tree_up<T, VB>(a, g, s_prog, reinterpret_cast<const T *>(a.D) + 6 * (size_t)g.ro, w, trx, ep);
+    if (!gather_top<T, VB>(a, g, tw, trx, ep, 0)) s_bad = 1;
     __syncthreads();
     const bool bad = s_bad != 0;
     if (bad && tid == 0) *(volatile int *)a.gave_up = 1;
@@ -3359,9 +3362,10 @@ sgp_status grid_apply(sgp_ctx *ctx, const sgp_factor *F, const DBuf &ws, const d
     a.F = b; a.x = x;
     a.err = bp<int>(ws);
     a.gave_up = ctx->d_gave_up;
-    a.polls = ctx->wait_polls;
+    a.skew = ctx->skew;
     a.lx = reinterpret_cast<unsigned long long *>(ws.p) + 2;
     SGP_CUDA(ctx, cudaMemsetAsync(ws.p, 0, G.apply_bytes, ctx->stream));
+    if (ctx->skew) SGP_CUDA(ctx, cudaMemsetAsync(a.err, 1, sizeof(int), ctx->stream));   // (waits that fail are short)
     void *args[] = {&a, &orig_of, &done};
     const auto kern = k_apply_grid<double, 24>;
     SGP_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, GRID_SMEM));
@@ -3425,7 +3429,7 @@ sgp_status grid_pcg(sgp_ctx *ctx, const sgp_matrix *M, const GridLayout &G, cons
     a.maxit = maxit;
     a.stopE = stopE;
     a.err = &out->err;
-    a.polls = ctx->wait_polls;
+    a.skew = ctx->skew;
     a.sc = out->sc;
     if (groups) {
         a.grp = groups->grp;
@@ -3433,6 +3437,7 @@ sgp_status grid_pcg(sgp_ctx *ctx, const sgp_matrix *M, const GridLayout &G, cons
     }
     a.ns = out->ns;
     SGP_CUDA(ctx, cudaMemsetAsync(zero, 0, (size_t)(zend - zero), ctx->stream));
+    if (ctx->skew) SGP_CUDA(ctx, cudaMemsetAsync(a.err, 1, sizeof(int), ctx->stream));
     void *args[] = {&a};
     auto go = [&](auto kern) -> sgp_status {
         SGP_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, GRID_SMEM));

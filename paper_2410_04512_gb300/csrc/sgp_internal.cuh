@@ -76,12 +76,11 @@ struct sgp_ctx {
     int64_t launches = 0;
     // a pinned page: the word that a forest solve sets when one of its bounded
     // waits gives up, then staging for small device->host reads (h_large: for
-    // larger ones); and the polls after which a wait gives up (about two seconds)
+    // larger ones)
     int *h_gave_up = nullptr, *d_gave_up = nullptr;
     char *h_stage = nullptr;
     void *h_large = nullptr;
     size_t h_stage_bytes = 0, h_large_bytes = 0;
-    int wait_polls = 1 << 21;
     // kernel timing
     int timing = 0;
     double kt_ms[SGP_KT_COUNT] = {};
@@ -106,6 +105,7 @@ struct sgp_ctx {
     int fused = 1;          // PCG step fused around the binned tree solve
     int small_solve = 1;    // whole mixed solves of small systems in one thread block
     int use_pdl = 1;        // programmatic dependent launch of the level kernels
+    unsigned skew = 0;      // persistent launches whose first block numbers its packets wrongly (tests)
     int batch_chunk = 0;    // rows per work item of the batched solver
     int num_sms = 0;
     std::vector<std::pair<const void *, int>> occupancy;  // kernel -> resident blocks/SM

@@ -1,6 +1,6 @@
-"""Bounded waits that give up: with no polls to spend, every wait between the
-thread blocks of a persistent launch ends at its first miss, and each call
-says TIMEOUT (not a breakdown, not a result).  Afterwards the context works."""
+"""Bounded waits that give up: where one thread block of a persistent launch
+numbers its packets wrongly, the waits for it run out, and each call says
+TIMEOUT (not a breakdown, not a result)."""
 from __future__ import annotations
 
 import numpy as np
@@ -16,11 +16,12 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.fixture()
-def hasty(cuda_device, monkeypatch):
-    """A context whose waits give up at once."""
-    monkeypatch.setenv("SGP_WAIT_POLLS", "0")
+def skewed(cuda_device, monkeypatch):
+    """A context whose waits run out (soon: its launches start with the word
+    set that ends waits after some polls)."""
+    monkeypatch.setenv("SGP_SKEW_PACKETS", "1")
     cx = sgp.Context(0)
-    monkeypatch.delenv("SGP_WAIT_POLLS")
+    monkeypatch.delenv("SGP_SKEW_PACKETS")
     return cx
 
 
@@ -34,45 +35,45 @@ def _timeout(fn):
     assert e.value.code == sgp.ERR_TIMEOUT
 
 
-def test_forest_solve_alone(hasty):
+def test_forest_solve_alone(skewed):
     c = _cells()
-    s = GpuSystem(hasty, c)
+    s = GpuSystem(skewed, c)
     b = dev_tensor(c.forces())
-    x = hasty.tree_apply(s.Fac, b)
+    x = skewed.tree_apply(s.Fac, b)
     torch.cuda.synchronize()
     assert torch.isnan(x).any()
-    _timeout(lambda: hasty.tree_apply(s.Fac, b))
+    _timeout(lambda: skewed.tree_apply(s.Fac, b))
     # the same factor in a context that waits
     y = sgp.Context(0).tree_apply(s.Fac, b)
     assert torch.isfinite(y).all()
 
 
 @pytest.mark.parametrize("precision", [sgp.PREC_F64, sgp.PREC_MIXED])
-def test_solves(hasty, precision):
+def test_solves(skewed, precision):
     c = _cells()
-    s = GpuSystem(hasty, c, precision=precision)
+    s = GpuSystem(skewed, c, precision=precision)
     F = dev_tensor(c.forces())
-    _timeout(lambda: hasty.pcg_solve(s.M, s.Fac, F, precision=precision))
-    _timeout(lambda: hasty.pcg_solve(s.M, None, F, precision=precision, precond=sgp.PRECOND_BLOCK_JACOBI))
+    _timeout(lambda: skewed.pcg_solve(s.M, s.Fac, F, precision=precision))
+    _timeout(lambda: skewed.pcg_solve(s.M, None, F, precision=precision, precond=sgp.PRECOND_BLOCK_JACOBI))
     v, info = sgp.Context(0).pcg_solve(s.M, s.Fac, F, precision=precision)
     assert info.status == 0
 
 
 @pytest.mark.parametrize("precision", [sgp.PREC_F64, sgp.PREC_MIXED])
-def test_batch(hasty, precision):
-    b = GpuBatch(hasty, [3000, 2500], precision=precision)
-    _timeout(lambda: hasty.pcg_solve_batched(b.M, b.Fh, b.off, dev_tensor(b.F), precision=precision))
+def test_batch(skewed, precision):
+    b = GpuBatch(skewed, [3000, 2500], precision=precision)
+    _timeout(lambda: skewed.pcg_solve_batched(b.M, b.Fh, b.off, dev_tensor(b.F), precision=precision))
 
 
-def test_forest_solves_inside_other_calls(hasty):
+def test_forest_solves_inside_other_calls(skewed):
     """The multi-launch solve (graphs of the forest's launch), a batch cut
     otherwise than its graph, the network."""
     c = _cells()
-    s = GpuSystem(hasty, c)
+    s = GpuSystem(skewed, c)
     F = dev_tensor(c.forces())
-    net = hasty.mpnn_create((0.1 * np.random.default_rng(1).standard_normal(sgp.MPNN_PARAMS)).astype(np.float32))
-    hasty.mpnn_forward(net, s.M, s.Fac, F)
-    _timeout(lambda: hasty.mpnn_backward(net, F, sgp.MPNN_LOSS_L2))
-    _timeout(lambda: hasty.warm_start(net, s.M, s.Fac, F))
-    aug = hasty.augment_tree(s.M, s.T)
-    _timeout(lambda: hasty.fcg_solve(s.M, aug, s.Fac, F))
+    net = skewed.mpnn_create((0.1 * np.random.default_rng(1).standard_normal(sgp.MPNN_PARAMS)).astype(np.float32))
+    skewed.mpnn_forward(net, s.M, s.Fac, F)
+    _timeout(lambda: skewed.mpnn_backward(net, F, sgp.MPNN_LOSS_L2))
+    _timeout(lambda: skewed.warm_start(net, s.M, s.Fac, F))
+    aug = skewed.augment_tree(s.M, s.T)
+    _timeout(lambda: skewed.fcg_solve(s.M, aug, s.Fac, F))
