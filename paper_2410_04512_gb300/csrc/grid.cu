@@ -67,13 +67,12 @@ constexpr int NCLS = 8;          // segment classes: 8 sources or more, 7, ... 1
 
 // header of a part (entry P: the top); Q_NSF, Q_NSB: slots of its programs;
 // Q_NA, Q_NL: rows of the top that it forms and how many are long; Q_XR, Q_XC:
-// entries of those rows and of the columns of its outputs (padded); Q_COFF:
-// where the latter's row numbers start
+// entries of those rows and of the columns of its outputs (padded)
 enum { Q_SOFF, Q_NV, Q_ROFF, Q_NR, Q_T0, Q_NP, Q_POFF, Q_NZ, Q_ZOFF, Q_DOFF, Q_NSF, Q_SF, Q_NSB, Q_SB,
-       Q_NA, Q_AOFF, Q_NL, Q_XR, Q_XC, Q_COFF, Q_N = 24 };
+       Q_NA, Q_AOFF, Q_NL, Q_XR, Q_XC, Q_N = 24 };
 // totals and maxima over the parts
 enum { T_NT, T_NR, T_P, T_Z, T_D, T_SF, T_SB, T_MNR, T_MNZ, T_MSF, T_MSB, T_MDZ, T_MNF, T_MNB, T_MNO,
-       T_RE, T_CE, T_A, T_MNA, T_MX, T_CI, T_ERR, T_N = 32 };
+       T_RE, T_CE, T_A, T_MNA, T_MX, T_ERR, T_N = 32 };
 // a matrix's rows on the parts: slots and halo cells of each part with their
 // offsets; behind the parts the totals and the largest halo
 enum { R_NS, R_SLOT, R_NH, R_HOFF, R_N };
@@ -513,8 +512,7 @@ struct GBuild {
     int32_t *clen, *rlen, *cptr, *rptr;      // the top's X: entries of its columns and rows, and where they start
     int32_t *cidx;                           // rows of every column's entries, CMAX per column
     double *cx;                              // and their blocks
-    int32_t *xi;                             // rows of X: the column of every entry
-    int32_t *ci;                             // per part, columns of its outputs: every entry's row, as the part numbers them
+    int32_t *xi;                             // the other index of every entry: rows, then columns
     int4 *alist, *outs;                      // per part: rows of X, outputs (see k_gr_part_top)
     int identity, halo;
 };
@@ -619,7 +617,6 @@ __global__ void __launch_bounds__(256) k_gr_offsets2(int32_t P, int32_t *hdr, in
     hdr_scan(P, hdr, tot, Q_NSF, Q_SF, T_SF, 0, sh);
     hdr_scan(P, hdr, tot, Q_NSB, Q_SB, T_SB, 0, sh);
     hdr_scan(P, hdr, tot, Q_NA, Q_AOFF, T_A, 0, sh);
-    hdr_scan(P, hdr, tot, Q_XC, Q_COFF, T_CI, 0, sh);
     if (threadIdx.x < P) {
         const int32_t *h = hdr + (size_t)Q_N * threadIdx.x;
         atomicMax(tot + T_MNR, h[Q_NR]);
@@ -1155,13 +1152,11 @@ __global__ void __launch_bounds__(1024) k_gr_top_offsets(GBuild g)
 // chip the part's rows, then its columns, are packed ("local" starts).
 //   alist: row, start, local start, length
 //   outs:  column's start, local start, length
-//   ci:    the columns' entries' rows, by their place in alist
 template <bool FILL>
 __global__ void __launch_bounds__(GT) k_gr_part_top(GBuild g)
 {
     __shared__ int32_t sh[GW];
     __shared__ uint8_t in[NTOP];
-    __shared__ uint16_t place[FILL ? NTOP : 1];
     const int b = blockIdx.x;
     int32_t *h = g.hdr + (size_t)Q_N * b;
     if (g.tot[T_ERR]) return;   // (nothing of this launch writes it)
@@ -1199,26 +1194,10 @@ __global__ void __launch_bounds__(GT) k_gr_part_top(GBuild g)
         int32_t tl, ts, tx;
         const int32_t l = nl + gscan<GT>(n > TLONG, sh, &tl), k = ns + gscan<GT>(n > 0 && n <= TLONG, sh, &ts),
                       x0 = xr + gscan<GT>(pad8(n), sh, &tx);
-        if (FILL && n > 0) {
-            const int32_t at = n > TLONG ? l : h[Q_NL] + k;
-            g.alist[h[Q_AOFF] + at] = make_int4(j, g.rptr[j], x0, n);
-            place[j] = (uint16_t)at;
-        }
+        if (FILL && n > 0) g.alist[h[Q_AOFF] + (n > TLONG ? l : h[Q_NL] + k)] = make_int4(j, g.rptr[j], x0, n);
         nl += tl;
         ns += ts;
         xr += tx;
-    }
-    if (FILL) {
-        __syncthreads();
-        int32_t *ci = g.ci + h[Q_COFF] - h[Q_XR];   // by local starts
-        for (int32_t i = threadIdx.x; i < nt; i += GT) {
-            const bool own = i >= t0 && i - t0 < nout - nz, reach = vm[i] != 0;
-            for (int q = 0; q < 2; ++q) {
-                if (!(q ? own : reach)) continue;
-                const int4 t = outs[q ? nz + i - t0 : vm[i] - 1];   // (this thread's own)
-                for (int32_t e = 0; e < pad8(t.z); ++e) ci[t.y + e] = e < t.z ? place[g.cidx[(size_t)i * CMAX + e]] : 0;
-            }
-        }
     }
     if (!FILL && threadIdx.x == 0) {
         h[Q_NA] = nl + ns;
@@ -1256,6 +1235,7 @@ __global__ void __launch_bounds__(128) k_gr_top_fill(GBuild g, T *X)
         }
         const int32_t cs = re + g.cptr[j], n = g.clen[j], lc = pad8(n);
         for (int32_t e = threadIdx.x; e < n; e += 128) {
+            g.xi[cs + e] = g.cidx[(size_t)j * CMAX + e];
             const double *x = g.cx + ((size_t)j * CMAX + e) * 9;
             T *o = X + 9 * (size_t)cs + e;
 #pragma unroll
@@ -1407,7 +1387,7 @@ __global__ void __launch_bounds__(GT) k_gr_check(GBuild g)
 {
     const int b = blockIdx.x;
     int bad = 0;
-    const int32_t nt = g.tot[T_NT], re = g.tot[T_RE], ce = g.tot[T_CE];
+    const int32_t nt = g.tot[T_NT], xe = g.tot[T_RE] + g.tot[T_CE];
     const int32_t *h = g.hdr + (size_t)Q_N * b;
     const int32_t nv = h[Q_NV], nr = h[Q_NR], nz = h[Q_NZ], nd = nr + nz, ro = h[Q_ROFF], nout = nz + nr - nv,
                   xl = h[Q_XR] + h[Q_XC];
@@ -1423,20 +1403,18 @@ __global__ void __launch_bounds__(GT) k_gr_check(GBuild g)
             if (ws[k] < 0 || ws[k] > ws[k + 1] || ws[k + 1] > ns) bad = 64;
     }
     // the top: every row and column that the part reads, and its entries
-    auto entries = [&](int32_t st0, int32_t st, int32_t end, int32_t n, int32_t loc0, int32_t loc, int32_t lend,
-                       const int32_t *x, int32_t lim) {
-        const int32_t lp = pad8(n);
-        bool in = n >= 0 && st >= st0 && st + lp <= end && loc >= loc0 && loc + lp <= lend;
-        for (int32_t e = 0; in && e < n; ++e) in = x[e] >= 0 && x[e] < lim;
+    auto entries = [&](int32_t st, int32_t n, int32_t lp, int32_t loc) {
+        bool in = n >= 0 && n <= lp && st >= 0 && st + lp <= xe && loc >= 0 && loc + lp <= xl;
+        for (int32_t e = 0; in && e < n; ++e) in = g.xi[st + e] >= 0 && g.xi[st + e] < nt;
         return in;
     };
     for (int32_t k = threadIdx.x; k < h[Q_NA]; k += GT) {
         const int4 t = g.alist[h[Q_AOFF] + k];
-        if (t.x < 0 || t.x >= nt || !entries(0, t.y, re, t.w, 0, t.z, h[Q_XR], g.xi + t.y, nt)) bad = 256;
+        if (t.x < 0 || t.x >= nt || !entries(t.y, t.w, pad8(t.w), t.z)) bad = 256;
     }
     for (int32_t z = threadIdx.x; z < nout; z += GT) {
         const int4 t = g.outs[h[Q_ZOFF] + h[Q_T0] + z];
-        if (!entries(re, t.x, re + ce, t.z, h[Q_XR], t.y, xl, g.ci + h[Q_COFF] - h[Q_XR] + t.y, h[Q_NA])) bad = 512;
+        if (!entries(t.x, t.z, pad8(t.z), t.y)) bad = 512;
     }
     for (int32_t z = threadIdx.x; z < nz; z += GT) {
         const int32_t k = g.zslot[h[Q_ZOFF] + z];
@@ -1481,7 +1459,7 @@ struct GridArgs {
     const double *gtol2;       // per system: tol^2, or below 0 for none to solve (NULL: tol2 for all)
     const int32_t *hdr, *rh, *ws, *glen, *gso, *i_of_t, *zslot, *tlk, *hl;
     const int4 *alist, *outs;   // the top: see k_gr_part_top
-    const int32_t *xi, *ci;
+    const int32_t *xi;
     const char *prog[2];
     const uint16_t *perm;
     const uint8_t *xflag;
@@ -2181,7 +2159,7 @@ template <typename T>
 struct Top {
     const int4 *alist, *outs;
     const T *X, *D;
-    const int32_t *xi, *ci;   // (ci by local starts)
+    const int32_t *xi;
     bool local;   // X packed on chip
 };
 template <typename T>
@@ -2189,7 +2167,7 @@ __device__ __forceinline__ Top<T> top_of(const GridArgs &a, const PartDims &g)
 {
     const int32_t *h = a.hdr + (size_t)Q_N * blockIdx.x;
     return Top<T>{a.alist + h[Q_AOFF], a.outs + g.zo + g.t0, reinterpret_cast<const T *>(a.X),
-                  reinterpret_cast<const T *>(a.tD), a.xi, a.ci + h[Q_COFF] - h[Q_XR], false};
+                  reinterpret_cast<const T *>(a.tD), a.xi, false};
 }
 
 // One forest solve, in three steps (w: the right-hand side in, the solution
@@ -2312,19 +2290,19 @@ __device__ __forceinline__ void tree_down(const PartDims &g, const Prog *s_prog,
         for (int b = 4; b > 0; b >>= 1)
 #pragma unroll
             for (int c = 0; c < 3; ++c) y[c] += __shfl_xor_sync(0xffffffffu, y[c], b);
-        if (l < 3 && k < na) Cell<T>::st(tu + k * VB + l * sizeof(T), fma(d[2], y[2], fma(d[1], y[1], d[0] * y[0])));
+        if (l < 3 && k < na) Cell<T>::st(tu + t.x * VB + l * sizeof(T), fma(d[2], y[2], fma(d[1], y[1], d[0] * y[0])));
     }
     __syncthreads();
     for (int32_t base = 4 * warp; base < nout; base += 4 * GW) {
         const int32_t o = base + (lane >> 3);
         const int4 t = o < nout ? top.outs[o] : make_int4(0, 0, 0, 0);
         const int32_t len = t.z, lp = pad8(len), st = loc ? t.y : t.x;
-        const int32_t *ci = top.ci + t.y;
+        const int32_t *xi = top.xi + st;
         const T *x = top.X + 9 * (size_t)st;
         T z[3] = {0, 0, 0};
         for (int32_t e = l8; e < len; e += 8) {
             T u[3];
-            V3<T, VB>::ld(tu + ci[e] * VB, u);
+            V3<T, VB>::ld(tu + xi[e] * VB, u);
 #pragma unroll
             for (int c = 0; c < 3; ++c)
                 z[c] = fma(x[(size_t)(6 + c) * lp + e], u[2], fma(x[(size_t)(3 + c) * lp + e], u[1], fma(x[(size_t)c * lp + e], u[0], z[c])));
@@ -2413,11 +2391,11 @@ __global__ void __launch_bounds__(GT, 1) k_pcg_grid(const __grid_constant__ Grid
             for (int32_t k = warp; k < g.na + g.nout; k += GW) {
                 const int4 t = k < g.na ? a.alist[h[Q_AOFF] + k] : a.outs[g.zo + g.t0 + k - g.na];
                 const int32_t from = k < g.na ? t.y : t.x, at = k < g.na ? t.z : t.y, n = pad8(k < g.na ? t.w : t.z);
-                for (int32_t e = lane; e < n; e += 32) xi[at + e] = k < g.na ? top.xi[from + e] : top.ci[at + e];
+                for (int32_t e = lane; e < n; e += 32) xi[at + e] = top.xi[from + e];
                 for (int32_t e = lane; e < 9 * n; e += 32) xd[9 * (size_t)at + e] = top.X[9 * (size_t)from + e];
             }
             top.X = xd;
-            top.xi = top.ci = xi;
+            top.xi = xi;
             top.local = true;
         }
     }
@@ -2600,6 +2578,10 @@ __global__ void __launch_bounds__(GT, 1) k_pcg_grid(const __grid_constant__ Grid
         }
         if (PREC == 0) {
             tree_down<T, VB>(g, s_prog, top, w, tw, sm0 + a.pl.o_u);
+            if (sizeof(T) == 8 && a.pl.o_u == a.pl.o_p && phase > 0) {   // p's first rows again
+                const T *o = reinterpret_cast<const T *>(a.pg) + 3 * (size_t)ro;
+                for (int32_t i = tid; i < min(3 * nr, a.nt * (int)(VB / sizeof(T))); i += GT) ps[i] = __ldcg(o + i);
+            }
         }
         if (PREC == 0 || phase <= 0) {
             Acc<T> acc;
@@ -2751,10 +2733,13 @@ bool place(const GridLayout &G, int32_t mnh, size_t sz, size_t vb, bool tree, bo
     pl->o_p = need(3 * sz * (mnr + (halo ? (size_t)mnh : 0)));
     pl->o_w = need(vb * (size_t)(tree ? t[T_MDZ] + 1 : t[T_MNR]));
     pl->o_t = need(vb * nt);
-    // (u by the part's own rows: with one place per top vertex the FP64 solve
-    // ended at 550,000 cells, so at 600,000)
-    pl->o_u = need(tree ? vb * (size_t)t[T_MNA] : 0);
-    pl->o_misc = need(8 * (mnr / 32 + 1));
+    // the top's D^-1 X r; where it does not fit beside the rest and p is in
+    // memory too (no halo on chip), in the place of p's first rows (sizes of
+    // 530,000 to 640,000 cells, by their largest part; FP32 ends at NREC cells)
+    const size_t misc = 8 * (mnr / 32 + 1);
+    const bool in_p = tree && !halo && sz == 8 && at + vb * nt + misc + 32 > (size_t)GRID_SMEM && vb * nt <= 3 * sz * mnr;
+    pl->o_u = in_p ? pl->o_p : need(vb * nt);
+    pl->o_misc = need(misc);
     if (at > (size_t)GRID_SMEM) return false;
     for (int q = 0; q < 2; ++q) pl->o_nar[q] = pl->o_all[q] = -1;
     pl->o_D = pl->o_X = pl->o_tab = -1;
@@ -2801,7 +2786,7 @@ bool place_apply(const GridLayout &G, size_t sz, size_t vb, GridPlace *pl)
     pl->o_X = pl->o_tab = -1;
     pl->o_w = need(vb * (size_t)(t[T_MDZ] + 1));
     pl->o_t = need(vb * (size_t)t[T_NT]);
-    pl->o_u = need(vb * (size_t)t[T_MNA]);
+    pl->o_u = need(vb * (size_t)t[T_NT]);
     if (at > (size_t)GRID_SMEM) return false;
     for (int q = 0; q < 2; ++q) {
         const size_t b = B * (size_t)(q ? t[T_MNB] : t[T_MNF]);
@@ -3140,8 +3125,7 @@ sgp_status grid_build(sgp_ctx *ctx, sgp_factor *F, const sgp_matrix *M)
     }
     SGP_TRY(ensure(ctx, G.alist, G.tot[T_A], &g.alist));
     SGP_TRY(ensure(ctx, G.outs, (size_t)G.tot[T_Z] + (size_t)G.tot[T_NT], &g.outs));
-    SGP_TRY(ensure(ctx, G.xi, G.tot[T_RE], &g.xi));
-    SGP_TRY(ensure(ctx, G.ci, G.tot[T_CI], &g.ci));
+    SGP_TRY(ensure(ctx, G.xi, (size_t)G.tot[T_RE] + (size_t)G.tot[T_CE], &g.xi));
     SGP_TRY(ensure(ctx, G.zslot, G.tot[T_Z], &g.zslot));
     SGP_TRY(ensure(ctx, G.tlk, (size_t)G.tot[T_NT] + 1, &g.tlk));
     SGP_TRY(sgp_launch(ctx, "k_gr_program", f32 ? k_gr_program<float> : k_gr_program<double>, dim3(P, 2), dim3(GT), 0, g));
@@ -3263,7 +3247,7 @@ void grid_rows_release(GridRows &R)
 }
 void grid_release(GridLayout &G)
 {
-    for (DBuf *d : {&G.hdr, &G.dtot, &G.ws, &G.alist, &G.outs, &G.xi, &G.ci, &G.zslot, &G.tlk, &G.i_of_t, &G.t_of_i, &G.prog[0], &G.prog[1], &G.D,
+    for (DBuf *d : {&G.hdr, &G.dtot, &G.ws, &G.alist, &G.outs, &G.xi, &G.zslot, &G.tlk, &G.i_of_t, &G.t_of_i, &G.prog[0], &G.prog[1], &G.D,
                     &G.X, &G.tD, &G.apply})
         if (d->p) cudaFree(d->p);
     for (DBuf &d : G.scr)
@@ -3334,7 +3318,6 @@ static void top_args(const GridLayout &G, GridArgs &a)
 {
     a.alist = bp<const int4>(G.alist); a.outs = bp<const int4>(G.outs);
     a.xi = bp<const int32_t>(G.xi);
-    a.ci = bp<const int32_t>(G.ci);
     a.X = G.X.p; a.tD = G.tD.p;
 }
 

@@ -60,7 +60,7 @@ struct GridLayout {
     int32_t tot[32] = {0};                          // totals and maxima over the parts
     DBuf hdr, dtot, ws, zslot, tlk, i_of_t, t_of_i;
     DBuf prog[2], D;
-    DBuf alist, outs, xi, ci, X, tD;                    // the top: its tables, X = L^-1 and pivots
+    DBuf alist, outs, xi, X, tD;                    // the top: its tables, X = L^-1 and pivots
     DBuf apply;                                     // error word and packets of a forest solve alone
     size_t apply_bytes = 0;
     DBuf scr[SGP_GRID_SCRATCH];
