@@ -257,18 +257,28 @@ sgp_status kt_end(sgp_ctx *ctx, int kclass, cudaEvent_t start)
 static bool stream_sms(sgp_ctx *ctx)
 {
     if (cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, ctx->device) != cudaSuccess) return false;
-    void *get = nullptr, *res = nullptr;
-    cudaDriverEntryPointQueryResult q1, q2;
-    if (cudaGetDriverEntryPointByVersion("cuStreamGetGreenCtx", &get, CUDART_VERSION, cudaEnableDefault, &q1) != cudaSuccess ||
-        cudaGetDriverEntryPointByVersion("cuGreenCtxGetDevResource", &res, CUDART_VERSION, cudaEnableDefault, &q2) != cudaSuccess ||
-        q1 != cudaDriverEntryPointSuccess || q2 != cudaDriverEntryPointSuccess) {
-        cudaGetLastError();
-        return true;   // a driver without green contexts
-    }
+    // the driver's functions, looked up once per process (0.1 ms)
+    static const struct Green {
+        decltype(&cuStreamGetGreenCtx) of = nullptr;
+        decltype(&cuGreenCtxGetDevResource) resource = nullptr;
+        Green()
+        {
+            void *f = nullptr, *g = nullptr;
+            cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound, r = q;
+            if (cudaGetDriverEntryPointByVersion("cuStreamGetGreenCtx", &f, CUDART_VERSION, cudaEnableDefault, &q) == cudaSuccess &&
+                cudaGetDriverEntryPointByVersion("cuGreenCtxGetDevResource", &g, CUDART_VERSION, cudaEnableDefault, &r) == cudaSuccess &&
+                q == cudaDriverEntryPointSuccess && r == cudaDriverEntryPointSuccess) {
+                of = reinterpret_cast<decltype(of)>(f);
+                resource = reinterpret_cast<decltype(resource)>(g);
+            } else {
+                cudaGetLastError();   // a driver without green contexts
+            }
+        }
+    } green;
     CUgreenCtx g = nullptr;
     CUdevResource r{};
-    if (reinterpret_cast<decltype(&cuStreamGetGreenCtx)>(get)((CUstream)ctx->stream, &g) == CUDA_SUCCESS && g &&
-        reinterpret_cast<decltype(&cuGreenCtxGetDevResource)>(res)(g, &r, CU_DEV_RESOURCE_TYPE_SM) == CUDA_SUCCESS)
+    if (green.of && green.of((CUstream)ctx->stream, &g) == CUDA_SUCCESS && g &&
+        green.resource(g, &r, CU_DEV_RESOURCE_TYPE_SM) == CUDA_SUCCESS)
         ctx->num_sms = (int)r.sm.smCount;
     return ctx->num_sms > 0;
 }
