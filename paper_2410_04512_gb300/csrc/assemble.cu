@@ -45,11 +45,19 @@ __global__ void k_slot_place(const int32_t *__restrict__ ij, int64_t m, const in
 // every edge (i, j), its slot in row int_of[i] and in row int_of[j].
 __global__ void k_sort_rows(const int32_t *__restrict__ row_ptr, int64_t n, const int32_t *__restrict__ ij,
                             const int32_t *__restrict__ int_of, int32_t *col, int32_t *slot_edge,
-                            int32_t *edge_slot, int32_t *edge_slot_j)
+                            int32_t *edge_slot, int32_t *edge_slot_j, int32_t *lengths)
 {
     int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (r >= n) return;
     const int32_t b0 = row_ptr[r], k = row_ptr[r + 1] - b0;
+    // of a sixteenth of the warps: their longest rows, and all their slots
+    if ((r >> 5 & 15) == 0 && (r | 31) < n) {
+        const int32_t most = __reduce_max_sync(0xffffffffu, k), sum = __reduce_add_sync(0xffffffffu, k);
+        if ((threadIdx.x & 31) == 0) {
+            atomicAdd(lengths, most);
+            atomicAdd(lengths + 1, sum);
+        }
+    }
     for (int32_t a = 1; a < k; ++a) {
         const int32_t c = col[b0 + a], se = slot_edge[b0 + a];
         int32_t b = a - 1;
@@ -247,7 +255,7 @@ sgp_status sgp_friction_assemble(sgp_ctx *ctx, const sgp_graph *G, const double 
     }
     const int32_t *int_of = bp<const int32_t>(M->int_of);
     int *err = ctx->d_flags;
-    SGP_CUDA(ctx, cudaMemsetAsync(err, 0, sizeof(int), ctx->stream));
+    SGP_CUDA(ctx, cudaMemsetAsync(err, 0, 3 * sizeof(int), ctx->stream));   // errors, row lengths
     SGP_CUDA(ctx, cudaMemsetAsync(cnt, 0, sizeof(int32_t) * (n + 1), ctx->stream));
     SGP_CUDA(ctx, cudaMemsetAsync(cursor, 0, sizeof(int32_t) * (n + 1), ctx->stream));
     LAUNCH(ctx, k_slot_count, grid_for(m, SGP_BLOCK), SGP_BLOCK, 0, ij, m, int_of, cnt);
@@ -256,13 +264,15 @@ sgp_status sgp_friction_assemble(sgp_ctx *ctx, const sgp_graph *G, const double 
            col, slot_edge);
     int32_t *edge_slot_j = bp<int32_t>(M->edge_slot_j);
     LAUNCH(ctx, k_sort_rows, grid_for(n, SGP_BLOCK), SGP_BLOCK, 0, (const int32_t *)row_ptr, n, ij, int_of, col,
-           slot_edge, edge_slot, edge_slot_j);
+           slot_edge, edge_slot, edge_slot_j, err + 1);
     LAUNCH(ctx, k_edge_weight, grid_for(m, SGP_BLOCK), SGP_BLOCK, 0, m, gpar, gperp, bp<double>(M->w), err);
     LAUNCH(ctx, k_blocks, grid_for(m, SGP_BLOCK), SGP_BLOCK, 0, ij, pos, gpar, gperp,
            (const int32_t *)edge_slot, (const int32_t *)edge_slot_j, (const int32_t *)col, m, ns,
            bp<double>(M->blk), blk32, err);
-    int herr = 0;
-    SGP_TRY(read_back(ctx, &herr, err, sizeof(int)));
+    int h[3] = {0, 0, 0};
+    SGP_TRY(read_back(ctx, h, err, sizeof(h)));
+    const int herr = h[0];
+    M->regular = h[2] > 0 && 32.0 * h[1] < 1.4 * h[2];
     if (herr & 1)
         return sgp_fail(ctx, SGP_ERR_INVALID_ARG,
                         "friction_assemble: friction coefficients must be positive and finite");

@@ -1047,13 +1047,19 @@ namespace {
 // wasted, so one lane per row; FP32 is bound by memory, where more lanes per
 // row give longer contiguous loads.
 template <typename T>
-sgp_status launch_spmv_pq(sgp_ctx *ctx, Blk<T> B, const int32_t *row_ptr, T g0, int64_t n, const T *p,
+sgp_status launch_spmv_pq(sgp_ctx *ctx, Blk<T> B, const int32_t *row_ptr, bool regular, T g0, int64_t n, const T *p,
                           T *q, double *partials, Scal *sc)
 {
     // FP64 with a lane per row: rows by length (from 100,000 rows on, see
-    // product64; as many partials as blocks)
+    // product64; as many partials as blocks), unless they are about equally long
+    // in their own order already, which keeps neighbours' loads together.  The
+    // longest of 32 rows over their mean decides, below 1.4; us a product of
+    // 500,000 cells by length and in order: 1.01 (sheet) 111 and 91, 1.29 (with
+    // noise) 101 and 89, 1.52 90 and 88, 1.62 (lattice) 107 and 116, 1.87 (cube)
+    // 121 and 147, 1.99 (ball) 106 and 132; 4e6 cells, 1.01: 625 and 582; 120,000,
+    // 1.51: 29 and 33
     if constexpr (sizeof(T) == 8)
-        if (ctx->spmv_lpr <= 1 && ctx->spmv_ilp <= 1 && n >= 100000 && n <= (int64_t)1024 * MAXP) {
+        if (!regular && ctx->spmv_lpr <= 1 && ctx->spmv_ilp <= 1 && n >= 100000 && n <= (int64_t)1024 * MAXP) {
             LAUNCH(ctx, (k_product64<1024, 512, true>), (unsigned)((n + 1023) / 1024), 512, 0, B, row_ptr, g0, n, p,
                    (const int32_t *)nullptr, q, partials, sc);
             return SGP_OK;
@@ -1167,7 +1173,7 @@ sgp_status pcg_core(sgp_ctx *ctx, const sgp_matrix *M, const sgp_factor *Fac, in
         if (fused) {
             for (int it = 0; it < count; ++it) {
                 SGP_TRY(kt_begin(ctx, SGP_KT_SPMV, &ev));
-                SGP_TRY(launch_spmv_pq<T>(ctx, B, row_ptr, g0, n, (const T *)p, q, partials, sc));
+                SGP_TRY(launch_spmv_pq<T>(ctx, B, row_ptr, M->regular, g0, n, (const T *)p, q, partials, sc));
                 SGP_TRY(kt_end(ctx, SGP_KT_SPMV, ev));
                 SGP_TRY(kt_begin(ctx, SGP_KT_TREE_SOLVE, &ev));
                 SGP_TRY(bins_pcg_step<T>(ctx, Fac, r, (const T *)q, w, sc));
@@ -1180,7 +1186,7 @@ sgp_status pcg_core(sgp_ctx *ctx, const sgp_matrix *M, const sgp_factor *Fac, in
         }
         for (int it = 0; it < count; ++it) {
             SGP_TRY(kt_begin(ctx, SGP_KT_SPMV, &ev));
-            SGP_TRY(launch_spmv_pq<T>(ctx, B, row_ptr, g0, n, (const T *)p, q, partials, sc));
+            SGP_TRY(launch_spmv_pq<T>(ctx, B, row_ptr, M->regular, g0, n, (const T *)p, q, partials, sc));
             SGP_TRY(kt_end(ctx, SGP_KT_SPMV, ev));
             SGP_TRY(kt_begin(ctx, SGP_KT_PCG_VECTOR, &ev));
             if (precond == SGP_PRECOND_TREE)
@@ -1716,7 +1722,7 @@ sgp_status sgp_fcg_solve(sgp_ctx *ctx, const sgp_matrix *M, const sgp_aug *A, co
         }
         SGP_TRY(kt_end(ctx, SGP_KT_PCG_VECTOR, ev));
         SGP_TRY(kt_begin(ctx, SGP_KT_SPMV, &ev));
-        SGP_TRY(launch_spmv_pq<double>(ctx, B64, row_ptr, M->gamma0, n, (const double *)p, q, partials, sco));
+        SGP_TRY(launch_spmv_pq<double>(ctx, B64, row_ptr, M->regular, M->gamma0, n, (const double *)p, q, partials, sco));
         SGP_TRY(kt_end(ctx, SGP_KT_SPMV, ev));
         SGP_TRY(kt_begin(ctx, SGP_KT_PCG_VECTOR, &ev));
         LAUNCH(ctx, k_fcg_upd, G, RB, 0, n3, (const double *)p, (const double *)q, x, r, partials, sco);

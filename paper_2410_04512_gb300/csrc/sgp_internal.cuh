@@ -326,6 +326,7 @@ struct sgp_matrix {
     double gamma0 = 0;
     int32_t precision = SGP_PREC_F64;
     int batched = 0;   // assembled from a batched graph (solved per instance)
+    int regular = 0;   // rows of 32 neighbours in order are about as long as their longest
     std::vector<int64_t> inst_row;   // its instances' offsets
     DBuf ij;         // m x 2 int32 (copy of the graph's edge list)
     DBuf row_ptr;    // n + 1 int32 over 2m directed slots, columns ascending in a row

@@ -65,3 +65,23 @@ def test_persistent_launches_repeat(cuda_device, what, precision):
         if k == 2:
             cx.tree_factor(M, T, Fac)
         assert torch.equal(run(), first)
+
+
+@pytest.mark.parametrize("geometry", ["ball", "sheet"])
+def test_multi_launch_fp64_steps_repeat_and_agree(cuda_device, geometry):
+    """Rows of many lengths (a ball: dealt to lanes by length) and rows about
+    equally long (a sheet: in their own order): the same bits in every run, and
+    20 unpreconditioned steps equal to the one-launch solve's but for the order
+    of sums (1e-10 of the iterate)."""
+    c = workloads.ball(n=120011, seed=2120, gamma0=1e-3) if geometry == "ball" else workloads.hex_sheet(nx=331, ny=311, seed=3)
+    F = dev_tensor(c.forces())
+    out = []
+    for cap in (0, -1):
+        cx = sgp.Context(0)
+        cx.set_tuning(bin_cap=cap)
+        s = GpuSystem(cx, c, tree=False)
+        kw = dict(tol=1e-300, maxit=20, precond=sgp.PRECOND_NONE, raise_on_error=False)
+        out.append(cx.pcg_solve(s.M, None, F, **kw)[0].clone())
+        for _ in range(4):
+            assert torch.equal(cx.pcg_solve(s.M, None, F, **kw)[0], out[-1])
+    assert float((out[0] - out[1]).norm() / out[1].norm()) <= 1e-10
