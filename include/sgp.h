@@ -255,8 +255,10 @@ sgp_status sgp_factor_info(const sgp_factor *factor, int32_t *rounds, int32_t *l
 /* Layout of the factor's binned solve: number of bins, vertices of the top
  * part (solved by one thread block), products sent from bins to the top
  * ("leaks"), the subtree bound, and whether the FP32 and FP64 applications
- * use it (1) or run one launch per contraction level (0: the layout is off
- * or does not fit in shared memory).  Any pointer may be NULL. */
+ * use it (1) or not (0: the layout is off or does not fit in shared memory,
+ * and one launch per contraction level serves; or the factor has parts for the
+ * persistent launch, see sgp_tuning's bin_cap, and no bins are built: all
+ * zeros).  Any pointer may be NULL. */
 sgp_status sgp_factor_layout(const sgp_factor *factor, int32_t *bins, int32_t *top, int32_t *leaks,
                              int32_t *bin_cap, int32_t *fp32, int32_t *fp64);
 void sgp_factor_destroy(sgp_factor *factor);
@@ -275,7 +277,9 @@ void sgp_factor_destroy(sgp_factor *factor);
  * H is P^{-1} from `factor` (required for SGP_PRECOND_TREE), the block-Jacobi
  * inverse (computed inside the call) or I.  MIXED runs FP64 iterative
  * refinement: r = F - Gamma v in FP64, an FP32 inner PCG on r/|r| to
- * inner_tol (FP64 dot products), v += |r| d, until |r| <= tol |F|.  A
+ * inner_tol, v += |r| d, until |r| <= tol |F|; its dot products are FP64 sums
+ * or, in the persistent launch (see sgp_tuning's bin_cap), sums of exact
+ * products in pairs of floats (some 48 bits).  A
  * MIXED tree-preconditioned solve of a small system (every contraction level
  * in the factor's one-block tail and its vectors within one block's shared
  * memory: about a thousand cells) runs the whole refinement in one launch
@@ -291,9 +295,12 @@ sgp_status sgp_pcg_solve(sgp_ctx *ctx, const sgp_matrix *matrix, const sgp_facto
 /* Batched PCG: every instance s of a block-diagonal matrix (assembled from a
  * batched collision graph with the same offsets) is solved for its own
  * Gamma_ss v_s = F_s with its own scalars (alpha, beta, rho) and its own
- * stopping test |r_s| <= tol |F_s|; all instances share each kernel launch
- * and the tree factor of the whole batch.  Converged instances drop out of
- * the products and vector updates.  Iterations are replayed as CUDA graphs.
+ * stopping test |r_s| <= tol |F_s|; all instances share the tree factor of the
+ * whole batch and each kernel launch.  With the tree preconditioner and no more
+ * instances than SMs a run is one persistent launch, in which every instance
+ * iterates and stops on thread blocks of its own; otherwise iterations are
+ * replayed as CUDA graphs and converged instances drop out of the products
+ * and vector updates.
  * opts as for sgp_pcg_solve (maxit per instance).  infos (host, n_instances
  * entries, may be NULL) receives each instance's statistics.  Returns the
  * first failing status (NOT_SPD before NO_CONVERGENCE); INVALID_ARG if an
@@ -431,13 +438,15 @@ typedef struct {
     int32_t bin_cap;     /* the tree solve's thread-block bins: contraction subtrees
                             of at most bin_cap vertices are solved by one thread
                             block each (three launches per application); 0 =
-                            default (systems whose parts fit on chip, about 1e6
-                            cells in MIXED and 5e5 in FP64, and batches of no
-                            more instances than SMs: a whole PCG run is one
-                            persistent launch, with every preconditioner; FP64
-                            forest solves alone too, up to about 7e5 cells;
-                            otherwise bins of 1024 for the FP32 solve of a MIXED
-                            factor, one launch per contraction level for FP64),
+                            default (systems whose parts fit on chip, about
+                            1.1e6 cells in MIXED and 6e5 in FP64, and batches
+                            of no more instances than SMs: a whole PCG run is
+                            one persistent launch, with every preconditioner,
+                            also with the factor of another assembly of the same
+                            cells; FP64 forest solves alone too, up to about
+                            9.5e5 cells; otherwise bins of 1024 for the FP32
+                            solve of a MIXED factor, one launch per contraction
+                            level for FP64),
                             -1 = off in both precisions, 64..8192 = that cap in
                             both precisions; read when a factor is built */
     double ms_per_iteration; /* sgp_autotune: the winning objective (ms per PCG

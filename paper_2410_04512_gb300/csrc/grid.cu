@@ -38,8 +38,8 @@
 // cells also the stream of matrix rows and blocks from HBM.
 // Measured per iteration against the multi-launch paths it replaces (product,
 // vector kernels and level kernels or bins; tol 1e-10): FP64 lattice of 1e4
-// cells 31 us (104), FP32 spheroid of 1e5 26.4 us (63), FP32 sheet of 2.5e5
-// 34 us (76), FP64 spheroid of 3e5 125 us (282), FP32 spheroid of 1e6 122 us
+// cells 30.6 us (104), FP32 spheroid of 1e5 27.5 us (63), FP32 sheet of 2.5e5
+// 34 us (76), FP64 spheroid of 3e5 121 us (282), FP32 spheroid of 1e6 122 us
 // (181); block Jacobi, FP64, 2e5 cells 54 us (81).
 #include <algorithm>
 #include <cmath>
@@ -2968,7 +2968,7 @@ sgp_status grid_build(sgp_ctx *ctx, sgp_factor *F, const sgp_matrix *M)
     const auto too_large = [&](int32_t rows) { return (size_t)rows * 24 > (size_t)GRID_SMEM || rows > NREC; };
     if (too_large(U)) return SGP_OK;
     // The subtree bound trades the number of top vertices (every block reads
-    // its rows of their inverse) and the length of the narrow levels against
+    // its rows and columns of their L^-1) and the length of the narrow levels against
     // what balancing can do (a part cannot be smaller than its largest
     // subtree).  Measured, us per iteration: FP64, U = 127 rows per part: 31.8
     // with bmax = U, 31.1 with 3U/2, 30.7 with 2U; U = 395: U/2 61, 3U/4 50, 3U/2
